@@ -171,7 +171,8 @@ int sort_species(pic_sim *s, int i)
         launch_permute_f32(view32(s, i, p.cur), view32(s, i, o), perm, p.d_count, p.n_hi, s->g.dim, s->st);
     p.cur = o;
     if (p.items) {
-        build_tile_items(p.tile_start, s->g.ntiles, s->g.dim, p.item_cnt, p.item_scan, p.items, p.nitems, s->st);
+        build_tile_items(p.tile_start, s->g.ntiles, tile_chunk(s->g, p.has_qed_arrays(), p.n_hi), p.item_cnt,
+                         p.item_scan, p.items, p.nitems, s->st);
         p.items_valid = true;
     }
     CK(cudaGetLastError());
@@ -180,11 +181,11 @@ int sort_species(pic_sim *s, int i)
 
 bool use_tile_push(const pic_sim *s, const SpeciesState &p)
 {
-    // the tiled kernels stage order-2 stencils; order 4 runs on the simple kernels
+    // (3D order 4 runs on the simple kernels)
     if (s->push_variant == PIC_PUSH_SIMPLE || !p.items_valid || s->precision != PIC_PREC_FP32_CELLOFF ||
-        s->g.order != 2 || p.kind != PIC_KIND_MASSIVE)
+        p.kind != PIC_KIND_MASSIVE)
         return false;
-    if (s->g.dim == 3) return tile3d_push_supported(s->g);
+    if (s->g.dim == 3) return s->g.order == 2 && tile3d_push_supported(s->g);
     return s->g.dim == 2 && s->g.tile_log2[0] == s->g.tile_log2[1] &&
            (s->g.tile_log2[0] == 3 || s->g.tile_log2[0] == 4);
 }
@@ -355,7 +356,7 @@ void push_species(pic_sim *s, int i, float *F)
         if (use_tile_photon_push(s, p)) {
             // the photons sorted into work items on the tiled kernel, then
             // those emitted since, as items of consecutive photons
-            const long long max_items = (long long)tile_items_capacity(p.n_hi, s->g.ntiles, s->g.dim);
+            const long long max_items = (long long)tile_items_capacity(p.n_hi, s->g.ntiles);
             if (q.on && q.net) cudaMemsetAsync(q.cq_n, 0, sizeof(uint32_t), s->st);  // the candidates' queue
             launch_push_photon_tile2d(P, p.items, p.nitems, max_items, F, s->g, push_const(s, p), q, s->d_err, s->st);
             // the photons appended since the sort: items of consecutive
@@ -376,13 +377,13 @@ void push_species(pic_sim *s, int i, float *F)
         if (use_tile_push(s, p)) {
             // the particles sorted into work items on the tiled kernel, those
             // appended since (pairs) on the one-thread-per-particle kernel
-            const long long max_items = (long long)tile_items_capacity(p.n_hi, s->g.ntiles, s->g.dim);
+            const long long max_items = (long long)tile_items_capacity(p.n_hi, s->g.ntiles);
             if (s->g.dim == 3)
                 launch_push_tile3d(P, p.items, p.nitems, max_items, F, s->g, push_const(s, p), s->d_err, s->d_eabs,
                                    p.defer + 1, p.defer, s->st, &q);
             else
-                launch_push_tile2d(P, p.items, p.nitems, max_items, F, s->g, push_const(s, p), s->d_err,
-                                   s->d_eabs, s->st, true, &q);
+                launch_push_qed_tile2d(P, p.items, p.nitems, max_items, F, s->g, push_const(s, p), s->d_err,
+                                       s->d_eabs, s->st, q);
             launch_push_qed_f32(P, F, s->g, push_const(s, p), q, s->d_err, s->d_eabs, s->st,
                                 p.tile_start + s->g.ntiles);
         } else {
@@ -391,7 +392,7 @@ void push_species(pic_sim *s, int i, float *F)
         return;
     }
     if (use_tile_push(s, p)) {
-        const long long max_items = (long long)tile_items_capacity(p.n_hi, s->g.ntiles, s->g.dim);
+        const long long max_items = (long long)tile_items_capacity(p.n_hi, s->g.ntiles);
         if (s->g.dim == 3)
             launch_push_tile3d(view32(s, i, p.cur), p.items, p.nitems, max_items, F, s->g, push_const(s, p), s->d_err,
                                s->d_eabs, p.defer + 1, p.defer, s->st);
@@ -686,7 +687,7 @@ int pic_create(const pic_grid *grid, double dt, const pic_species *species, int 
         rc = rc ? rc : dalloc(s, (void **)&p.d_count, sizeof(long long));
         rc = rc ? rc : dalloc(s, (void **)&p.tile_start, (size_t)(g.ntiles + 1) * sizeof(uint32_t));
         if (prec == PIC_PREC_FP32_CELLOFF && (g.dim == 2 || (g.dim == 3 && tile3d_push_supported(g)))) {
-            p.items_cap = (long long)tile_items_capacity(p.cap, g.ntiles, g.dim);
+            p.items_cap = (long long)tile_items_capacity(p.cap, g.ntiles);
             rc = rc ? rc : dalloc(s, (void **)&p.items, (size_t)p.items_cap * sizeof(TileItem));
             rc = rc ? rc : dalloc(s, (void **)&p.nitems, sizeof(uint32_t));
             rc = rc ? rc : dalloc(s, (void **)&p.item_cnt, (size_t)(g.ntiles + 1) * sizeof(uint32_t));

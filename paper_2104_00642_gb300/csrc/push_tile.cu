@@ -1,4 +1,6 @@
-// push_tile.cu -- tiled particle push for 2D grids (FP32 cell+offset form).
+// push_tile.cu -- tiled particle pushes of the QED species for 2D grids (FP32
+// cell+offset form), and the tile sort's work items (push_tile2d.cu has the
+// push without QED).
 //
 // Particles are counting-sorted by tile (T x T cells) every K steps.  Each
 // work item is a chunk of at most kChunk particles that sat in one tile at the
@@ -13,6 +15,7 @@
 // A particle that drifted so far since the sort that its stencil leaves the
 // box is handled on the global path (gather from HBM, global atomics), so the
 // result does not depend on the sort interval.
+#include <algorithm>
 #include <cstring>
 
 #include "push_qed_dev.cuh"
@@ -110,34 +113,12 @@ struct AccGlobal {
     }
 };
 
-// warp-aggregated current into the shared box: the lanes of grp share the
-// window origin; each value is summed over the group with one warp
-// reduction and added by the group's first lane with one shared atomic
-// (in the fixed-point units of AccShared; a group sum of at most 32
-// particles stays far inside int32)
-struct AccWarp {
-    int *base;
-    int cs, rs;
-    float scale;
-    unsigned grp;
-    bool lead;
-    __device__ __forceinline__ void add(int c, int a, int b, float v)
-    {
-        const int s = __reduce_add_sync(grp, __float2int_rn(v * scale));
-        if (lead && s) atomicAdd(base + c * cs + b * rs + a, s);
-    }
-};
-
 // With use_tma the field box of an item is one TMA tile copy (tmap: the six
 // field components as a 3D tensor, x fastest), issued by one thread and
 // overlapping the zeroing of the current box and the particle staging.
 //
-// AGG (warp-aggregated deposit): the 32 lanes of a warp take 32 consecutive
-// particles of the item (the sort orders a tile's particles by cell, so they
-// share cells: their gathers read the same nodes -- shared-memory broadcasts --
-// and lanes with the same deposit window are summed before one atomic per
-// value).  Without AGG lane l walks the l-th of 32 contiguous segments, so
-// the lanes of an atomic hit different cells.
+// Lane l walks the l-th of 32 contiguous segments of the item's (cell-sorted)
+// particles, so the lanes of an atomic hit different cells.
 //
 // QM (QED leptons): 1 = the Monte Carlo of Sec. IV with the
 // tables (Method I or II), 2 = with the surrogate network inside its chi
@@ -145,9 +126,9 @@ struct AccWarp {
 // the drifts, as in the one-thread-per-particle QED push.  The event flag
 // of every particle of the items is written (0 for dead ones); particles
 // appended after the sort are left to that kernel.
-template <int T, bool AGG, int QM>
+template <int T, int QM>
 __global__ void __launch_bounds__(kTileThreads, QM == 2 ? 3 : kTileMinBlocks)
-    k_push_tile2d(PartF32 P, const TileItem *__restrict__ items, const uint32_t *__restrict__ nitems,
+    k_push_qed_tile2d(PartF32 P, const TileItem *__restrict__ items, const uint32_t *__restrict__ nitems,
                   float *__restrict__ F, Grid g, PushConst pc, int *err, double *e_abs,
                   const __grid_constant__ CUtensorMap tmap, int use_tma, QedParams q)
 {
@@ -217,7 +198,7 @@ __global__ void __launch_bounds__(kTileThreads, QM == 2 ? 3 : kTileMinBlocks)
         // (asynchronous 4-byte copies: no register round trip)
         for (int i = threadIdx.x; i < m.count; i += blockDim.x) {
             const int l = __float2int_rz(((float)i + 0.5f) * invS), j = i - l * S;
-            const int pos = AGG ? i : j * 33 + l;
+            const int pos = j * 33 + l;
             const int p = m.start + i;  // capacities are below 2^31
             cp_async4(sPc + pos, P.cell + p);
             cp_async4(sP + 0 * kPSlot + pos, P.off[0] + p);
@@ -241,19 +222,12 @@ __global__ void __launch_bounds__(kTileThreads, QM == 2 ? 3 : kTileMinBlocks)
         // 3. particles
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         constexpr int kWarps = kTileThreads / 32;
-        // passes of the warp over the item: warp-uniform, so the lanes stay
-        // together for the warp-collective deposit of AGG
-        const int npass = AGG ? (m.count + kTileThreads - 1) / kTileThreads : (S + kWarps - 1) / kWarps;
+        // passes of the warp over the item (warp-uniform: the network's
+        // evaluation and the whole-warp deposit are collective)
+        const int npass = (S + kWarps - 1) / kWarps;
         for (int pass = 0; pass < npass; pass++) {
-            int li, pos;
-            if (AGG) {
-                li = pass * kTileThreads + warp * 32 + lane;
-                pos = li;
-            } else {
-                const int j = pass * kWarps + warp;
-                li = j < S ? lane * S + j : m.count;
-                pos = j * 33 + lane;
-            }
+            const int j = pass * kWarps + warp;
+            const int li = j < S ? lane * S + j : m.count, pos = j * 33 + lane;
             const uint32_t cp = li < m.count ? sPc[pos] : kDead;
             bool act = cp != kDead;  // a live particle of this item
             int c[2] = {0, 0}, c1[2] = {0, 0}, u0[2] = {0, 0};
@@ -293,7 +267,7 @@ __global__ void __launch_bounds__(kTileThreads, QM == 2 ? 3 : kTileMinBlocks)
             const long long pg = (long long)m.start + li;
             uint32_t event = 0;
             float4 evd = make_float4(0.f, 0.f, 0.f, 0.f);
-            if constexpr (QM != 0) qed_lepton_f32<QM == 2>(q, sNet, act, pg, eb, ux, uy, uz, err, event, evd);
+            qed_lepton_f32<QM == 2>(q, sNet, act, pg, eb, ux, uy, uz, err, event, evd);
             if (act) {
                 ig1 = inv_gamma_fast(ux, uy, uz);
                 const float d0 = hdx0 * ux * ig1, d1 = hdx1 * uy * ig1;
@@ -333,37 +307,24 @@ __global__ void __launch_bounds__(kTileThreads, QM == 2 ? 3 : kTileMinBlocks)
                 AccGlobal acc{Fg + JX * V + (long long)u0[1] * rs + u0[0], V, rs};
                 esirkepov2d(S0, dS, cjx, cjy, jvz, acc);
             }
-            if (AGG) {
-                const unsigned smask = __ballot_sync(0xffffffffu, din);
-                if (din) {
-                    const int key = (u0[1] - by0) * B::WX + (u0[0] - bx0);
-                    const unsigned grp = __match_any_sync(smask, key);
-                    AccWarp acc{sJ + key, B::N, B::WX, jscale, grp, lane == __ffs(grp) - 1};
-                    esirkepov2d(S0, dS, cjx, cjy, jvz, acc);
-                }
-            } else {
-                // A warp whose 32 lanes all deposit on one window (a dense
-                // beam: the whole chunk in one cell, so lane striding cannot
-                // spread the lanes over cells) sums each value over the warp
-                // with one reduction and adds it with one atomic; otherwise
-                // every lane adds its own values (lanes on different cells).
-                // The fixed-point scale is folded into the three coefficients.
-                const int key = din ? (u0[1] - by0) * B::WX + (u0[0] - bx0) : -1;
-                int same = 0;
-                // (checked in the QED variants, whose beams are dense; a plain
-                // plasma of tens of particles per cell never fills a warp's
-                // lanes with one window, and the check costs ~3 % there)
-                if constexpr (QM != 0) __match_all_sync(0xffffffffu, key, &same);
-                if (same && key >= 0) {
-                    AccWarpAll acc{sJ + key, B::N, B::WX, lane == 0};
-                    esirkepov2d(S0, dS, sjx, sjy, jvz * jscale, acc);
-                } else if (din) {
-                    AccSharedUnits acc{sJ + key, B::N, B::WX};
-                    esirkepov2d(S0, dS, sjx, sjy, jvz * jscale, acc);
-                }
+            // A warp whose 32 lanes all deposit on one window (a dense
+            // beam: the whole chunk in one cell, so lane striding cannot
+            // spread the lanes over cells) sums each value over the warp
+            // with one reduction and adds it with one atomic; otherwise
+            // every lane adds its own values (lanes on different cells).
+            // The fixed-point scale is folded into the three coefficients.
+            const int key = din ? (u0[1] - by0) * B::WX + (u0[0] - bx0) : -1;
+            int same = 0;
+            __match_all_sync(0xffffffffu, key, &same);
+            if (same && key >= 0) {
+                AccWarpAll acc{sJ + key, B::N, B::WX, lane == 0};
+                esirkepov2d(S0, dS, sjx, sjy, jvz * jscale, acc);
+            } else if (din) {
+                AccSharedUnits acc{sJ + key, B::N, B::WX};
+                esirkepov2d(S0, dS, sjx, sjy, jvz * jscale, acc);
             }
             if (!act) {
-                if (QM != 0 && li < m.count) q.ev[pg] = 0;
+                if (li < m.count) q.ev[pg] = 0;
                 continue;
             }
             // boundaries
@@ -386,10 +347,8 @@ __global__ void __launch_bounds__(kTileThreads, QM == 2 ? 3 : kTileMinBlocks)
             } else {
                 sPc[pos] = pack_cell(g, cc[0], cc[1], 0);
             }
-            if constexpr (QM != 0) {
-                q.ev[pg] = event;
-                if (event) reinterpret_cast<float4 *>(q.evk)[pg] = evd;
-            }
+            q.ev[pg] = event;
+            if (event) reinterpret_cast<float4 *>(q.evk)[pg] = evd;
             // the new state goes back to the particle's own staging slot and
             // leaves in array order below: lane-strided global stores would
             // touch 32 sectors per instruction
@@ -404,7 +363,7 @@ __global__ void __launch_bounds__(kTileThreads, QM == 2 ? 3 : kTileMinBlocks)
         // keep their staged values)
         for (int i = threadIdx.x; i < m.count; i += blockDim.x) {
             const int l = __float2int_rz(((float)i + 0.5f) * invS), j = i - l * S;
-            const int pos = AGG ? i : j * 33 + l;
+            const int pos = j * 33 + l;
             const int p = m.start + i;
             P.cell[p] = sPc[pos];
             P.off[0][p] = sP[pos];
@@ -679,9 +638,18 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks)
 }
 
 // ---------------------------------------------------------------------
-// work items: chunks of at most `chunk` particles of one tile
+// work items: a tile's particles in about equal pieces of at most `chunk`,
+// each but the last a multiple of `grain` (the particles of one pass of the
+// CTA that takes it)
 // ---------------------------------------------------------------------
-__global__ void k_item_counts(const uint32_t *__restrict__ starts, long long ntiles, uint32_t chunk, uint32_t *cnt)
+__device__ __forceinline__ uint32_t item_size(uint32_t n, uint32_t chunk, uint32_t grain)
+{
+    const uint32_t k = (n + chunk - 1) / chunk;
+    return k ? ((n + k - 1) / k + grain - 1) / grain * grain : chunk;
+}
+
+__global__ void k_item_counts(const uint32_t *__restrict__ starts, long long ntiles, uint32_t chunk, uint32_t grain,
+                              uint32_t *cnt)
 {
     long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t > ntiles) return;
@@ -689,45 +657,53 @@ __global__ void k_item_counts(const uint32_t *__restrict__ starts, long long nti
         cnt[t] = 0;
         return;
     }
-    uint32_t n = starts[t + 1] - starts[t];
-    cnt[t] = (n + chunk - 1) / chunk;
+    const uint32_t n = starts[t + 1] - starts[t], s = item_size(n, chunk, grain);
+    cnt[t] = (n + s - 1) / s;
 }
 
 __global__ void k_item_write(const uint32_t *__restrict__ starts, const uint32_t *__restrict__ off, long long ntiles,
-                             uint32_t chunk, TileItem *items, uint32_t *nitems)
+                             uint32_t chunk, uint32_t grain, TileItem *items, uint32_t *nitems)
 {
     long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= ntiles) {
         if (t == ntiles) *nitems = off[ntiles];
         return;
     }
-    uint32_t s = starts[t], n = starts[t + 1] - s;
-    uint32_t o = off[t];
-    for (uint32_t q = 0; q * chunk < n; q++) {
+    const uint32_t s = starts[t], n = starts[t + 1] - s, o = off[t], sz = item_size(n, chunk, grain);
+    for (uint32_t q = 0; q * sz < n; q++) {
         TileItem m;
         m.tile = (int)t;
-        m.start = (int)(s + q * chunk);
-        m.count = (int)min(chunk, n - q * chunk);
+        m.start = (int)(s + q * sz);
+        m.count = (int)min(sz, n - q * sz);
         m.pad = 0;
         items[o + q] = m;
     }
 }
 
-int tile_chunk(int dim) { return dim == 3 ? kChunk3 : kChunk; }
-
-size_t tile_items_capacity(long long cap, long long ntiles, int dim)
+// Particles per work item at most.  2D without QED: kChunkMax (the records
+// fit) while that leaves each of the 456 resident CTAs an item and a half,
+// less for fewer particles.  (A hot plasma of 1,048,576 particles: 59 us a
+// push with items of 352, 48 with 512 or 1024; an item's fixed cost is the
+// flush of its current box, ~210 instructions a warp.)
+int tile_chunk(const Grid &g, bool qed, long long n)
 {
-    return (size_t)(ntiles + cap / tile_chunk(dim) + 2);
+    if (g.dim == 3) return kChunk3;
+    if (qed) return kChunk;
+    for (int c = kChunkMax; c > kPushThreads; c /= 2)
+        if (2 * n >= 3ll * 456 * c) return c;
+    return kPushThreads;
 }
 
-void build_tile_items(const uint32_t *starts, long long ntiles, int dim, uint32_t *cnt_scratch,
+size_t tile_items_capacity(long long cap, long long ntiles) { return (size_t)(ntiles + cap / 256 + 2); }
+
+void build_tile_items(const uint32_t *starts, long long ntiles, int chunk, uint32_t *cnt_scratch,
                       uint32_t *scan_scratch, TileItem *items, uint32_t *nitems, cudaStream_t st)
 {
-    const uint32_t chunk = (uint32_t)tile_chunk(dim);
+    const uint32_t c = (uint32_t)chunk, grain = chunk % kPushThreads == 0 ? kPushThreads : 32u;
     note_launch(2);
-    k_item_counts<<<div_up(ntiles + 1, 256), 256, 0, st>>>(starts, ntiles, chunk, cnt_scratch);
+    k_item_counts<<<div_up(ntiles + 1, 256), 256, 0, st>>>(starts, ntiles, c, grain, cnt_scratch);
     scan_exclusive(cnt_scratch, cnt_scratch, ntiles + 1, scan_scratch, st);
-    k_item_write<<<div_up(ntiles + 1, 256), 256, 0, st>>>(starts, cnt_scratch, ntiles, chunk, items, nitems);
+    k_item_write<<<div_up(ntiles + 1, 256), 256, 0, st>>>(starts, cnt_scratch, ntiles, c, grain, items, nitems);
 }
 
 bool tile_push_supported(const Grid &g, int tile_edge)
@@ -735,7 +711,7 @@ bool tile_push_supported(const Grid &g, int tile_edge)
     return g.dim == 2 && (1 << g.tile_log2[0]) == tile_edge && (1 << g.tile_log2[1]) == tile_edge;
 }
 
-template <int T, bool AGG, int QM>
+template <int T, int QM>
 static void launch_T(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items, float *F,
                      const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st, const QedParams &q)
 {
@@ -743,7 +719,7 @@ static void launch_T(const PartF32 &P, const TileItem *items, const uint32_t *ni
     constexpr int smem = ((Box2<T>::SMEM + 15) & ~15) + 128 + (QM == 2 ? kMlpStageBytes : 0);
     static bool attr = false;
     if (!attr) {
-        cudaFuncSetAttribute(k_push_tile2d<T, AGG, QM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaFuncSetAttribute(k_push_qed_tile2d<T, QM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         attr = true;
     }
     static int nsm = 0;
@@ -760,38 +736,32 @@ static void launch_T(const PartF32 &P, const TileItem *items, const uint32_t *ni
     if (!tma) memset(&tmap, 0, sizeof tmap);
     static int per_sm = 0;  // resident CTAs per SM
     if (!per_sm) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_push_tile2d<T, AGG, QM>, kTileThreads, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_push_qed_tile2d<T, QM>, kTileThreads, smem);
         if (per_sm < 1) per_sm = 1;
     }
     long long grid = std::min<long long>(max_items, (long long)nsm * per_sm);  // one resident wave
     if (grid < 1) grid = 1;
     note_launch();
-    k_push_tile2d<T, AGG, QM><<<(int)grid, kTileThreads, smem, st>>>(P, items, nitems, F, g, pc, err, e_abs, tmap,
-                                                                    tma ? 1 : 0, q);
+    k_push_qed_tile2d<T, QM><<<(int)grid, kTileThreads, smem, st>>>(P, items, nitems, F, g, pc, err, e_abs, tmap,
+                                                                   tma ? 1 : 0, q);
 }
 
 template <int T>
-static void launch_variant(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
-                           float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st,
-                           bool agg, const QedParams *q)
+static void launch_lepton(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
+                          float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st,
+                          const QedParams &q)
 {
-    if (q && q->on) {
-        if (q->net) launch_T<T, false, 2>(P, items, nitems, max_items, F, g, pc, err, e_abs, st, *q);
-        else launch_T<T, false, 1>(P, items, nitems, max_items, F, g, pc, err, e_abs, st, *q);
-        return;
-    }
-    const QedParams none{};
-    if (agg) launch_T<T, true, 0>(P, items, nitems, max_items, F, g, pc, err, e_abs, st, none);
-    else launch_T<T, false, 0>(P, items, nitems, max_items, F, g, pc, err, e_abs, st, none);
+    if (q.net) launch_T<T, 2>(P, items, nitems, max_items, F, g, pc, err, e_abs, st, q);
+    else launch_T<T, 1>(P, items, nitems, max_items, F, g, pc, err, e_abs, st, q);
 }
 
-void launch_push_tile2d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
-                        float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st,
-                        bool agg, const QedParams *q)
+void launch_push_qed_tile2d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
+                            float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st,
+                            const QedParams &q)
 {
     if (P.n == 0) return;
-    if ((1 << g.tile_log2[0]) == 16) launch_variant<16>(P, items, nitems, max_items, F, g, pc, err, e_abs, st, agg, q);
-    else launch_variant<8>(P, items, nitems, max_items, F, g, pc, err, e_abs, st, agg, q);
+    if ((1 << g.tile_log2[0]) == 16) launch_lepton<16>(P, items, nitems, max_items, F, g, pc, err, e_abs, st, q);
+    else launch_lepton<8>(P, items, nitems, max_items, F, g, pc, err, e_abs, st, q);
 }
 
 template <int T, bool SURR>

@@ -7,9 +7,11 @@ namespace pic {
 
 struct QedParams;
 
-constexpr int kChunk = 384;        // particles per work item at most
-constexpr int kTileThreads = 128;  // threads per CTA of the tiled push
-constexpr int kTileMinBlocks = 6;  // CTAs per SM: 80 registers, 35 KB shared memory each (measured best)
+constexpr int kChunkMax = 1024;    // particles per work item at most (2D)
+constexpr int kPushThreads = 256;  // threads per CTA of the 2D push
+constexpr int kChunk = 384;        // particles per work item at most (2D, QED species)
+constexpr int kTileThreads = 128;  // threads per CTA of the QED species' pushes and the 3D push
+constexpr int kTileMinBlocks = 6;  // CTAs per SM of the 2D QED pushes: 80 registers, 35 KB shared memory each (measured best)
 
 struct TileItem {
     int tile, start, count, pad;
@@ -19,17 +21,23 @@ struct TileItem {
 // 256-1024 on the 8-ppc thermal workload: smaller items balance the CTAs)
 constexpr int kChunk3 = 256;
 
-size_t tile_items_capacity(long long cap, long long ntiles, int dim);
-void build_tile_items(const uint32_t *starts, long long ntiles, int dim, uint32_t *cnt_scratch,
+// particles per work item at most, for n particles of a species on grid g
+// (qed: photons and the leptons of the Monte Carlo)
+int tile_chunk(const Grid &g, bool qed, long long n);
+size_t tile_items_capacity(long long cap, long long ntiles);
+void build_tile_items(const uint32_t *starts, long long ntiles, int chunk, uint32_t *cnt_scratch,
                       uint32_t *scan_scratch, TileItem *items, uint32_t *nitems, cudaStream_t st);
 bool tile_push_supported(const Grid &g, int tile_edge);
-// (agg: the warp-aggregated deposit, lanes on consecutive particles;
-// q: a QED lepton species' Monte Carlo, fused in (lane-strided, agg
-// ignored) -- nullptr or q->on == 0 for none; the particles appended since
-// the sort, and their event flags, are left to launch_push_qed_f32)
+// 2D, shape orders 2 and 4 (agg: the warp-aggregated deposit, order 2); and
+// with a QED lepton species' Monte Carlo q fused in (order 2; q.on; the
+// particles appended since the sort, and their event flags, are left to
+// launch_push_qed_f32)
 void launch_push_tile2d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
                         float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st,
-                        bool agg, const QedParams *q = nullptr);
+                        bool agg);
+void launch_push_qed_tile2d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
+                            float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st,
+                            const QedParams &q);
 // the tiled photon push (2D, FP32; tiles of 8 or 16 cells): the photons of
 // the work items, their pair Monte Carlo with q; the photons appended since
 // the sort are left to launch_push_photon_f32

@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kTileThreads, QM == 2 ? 3 : 5)
     const float k = pc.qmdt2_f;
     const float cjx = pc.cJ_f[0], cjy = pc.cJ_f[1], cjz = pc.cJ_f[2];
     // fixed-point unit of the shared current box: 2^20 units per C, C the
-    // largest value one particle adds to a node (see AccShared)
+    // largest value one particle adds to a node
     const float cmax = fmaxf(fmaxf(fabsf(cjx), fabsf(cjy)), fabsf(cjz));
     const float jscale = 1048576.0f / fmaxf(cmax, 1e-30f);
     const float junit = 1.0f / jscale;

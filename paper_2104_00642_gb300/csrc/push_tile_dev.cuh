@@ -23,26 +23,11 @@ __device__ __forceinline__ int union4(int i0, const float *w0, int i1, const flo
 }
 
 // current into the shared box as 32-bit fixed point (integer shared-memory
-// atomics are native; float ones are not).  A chunk has at most kChunk
-// particles and each adds at most C = |q w| max(dx_d/dt) in magnitude to a
-// node, so with 2^20/C units per C a node holds at most 2^30: no overflow.
-// Rounding each value to the unit costs at most 2^-21 C per particle and
-// node, below 1e-6 of the node's sum of |contributions| scale.
-struct AccShared {
-    int *base;  // component 0 at (ux, uy) of the window
-    int cs, rs;
-    float scale;
-    __device__ __forceinline__ void add(int c, int a, int b, float v)
-    {
-        // no zero test: a branch per node costs more than the occasional
-        // zero add, and the warp issues the atomic for its other lanes anyway
-        atomicAdd(base + c * cs + b * rs + a, __float2int_rn(v * scale));
-    }
-};
-
-// as AccShared with the values already in fixed-point units (the caller
-// folded the scale into the deposit's coefficients: one multiply fewer per
-// node)
+// atomics are native; float ones are not), the values already in the units of
+// the box (the caller folds the scale into the deposit's coefficients).  Where
+// the units are fixed per launch they are 2^20 per C, C = |q w| max(dx_d/dt):
+// an item's particles (at most 1024, each adding at most C in magnitude to a
+// node) keep a node below 2^30, and rounding a value costs at most 2^-21 C.
 struct AccSharedUnits {
     int *base;
     int cs, rs;

@@ -185,7 +185,8 @@ bool use_tile_push(const pic_sim *s, const SpeciesState &p)
     if (s->push_variant == PIC_PUSH_SIMPLE || !p.items_valid || s->precision != PIC_PREC_FP32_CELLOFF ||
         p.kind != PIC_KIND_MASSIVE)
         return false;
-    if (s->g.dim == 3) return s->g.order == 2 && tile3d_push_supported(s->g);
+    if (s->g.dim == 3)
+        return s->g.order == 2 && (s->qed_on && p.qed ? tile3d_qed_push_supported(s->g) : tile3d_push_supported(s->g));
     return s->g.dim == 2 && s->g.tile_log2[0] == s->g.tile_log2[1] &&
            (s->g.tile_log2[0] == 3 || s->g.tile_log2[0] == 4);
 }
@@ -379,8 +380,8 @@ void push_species(pic_sim *s, int i, float *F)
             // appended since (pairs) on the one-thread-per-particle kernel
             const long long max_items = (long long)tile_items_capacity(p.n_hi, s->g.ntiles);
             if (s->g.dim == 3)
-                launch_push_tile3d(P, p.items, p.nitems, max_items, F, s->g, push_const(s, p), s->d_err, s->d_eabs,
-                                   p.defer + 1, p.defer, s->st, &q);
+                launch_push_qed_tile3d(P, p.items, p.nitems, max_items, F, s->g, push_const(s, p), s->d_err,
+                                       s->d_eabs, s->st, q);
             else
                 launch_push_qed_tile2d(P, p.items, p.nitems, max_items, F, s->g, push_const(s, p), s->d_err,
                                        s->d_eabs, s->st, q);

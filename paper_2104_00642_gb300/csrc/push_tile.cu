@@ -687,9 +687,11 @@ __global__ void k_item_write(const uint32_t *__restrict__ starts, const uint32_t
 // flush of its current box, ~210 instructions a warp.)
 int tile_chunk(const Grid &g, bool qed, long long n)
 {
-    if (g.dim == 3) return kChunk3;
+    if (g.dim == 3) return qed ? kChunk3 : kChunk3Max;
     if (qed) return kChunk;
-    for (int c = kChunkMax; c > kPushThreads; c /= 2)
+    // (order 4 spreads a particle over 25 nodes: half the particles an item
+    // keep its fixed-point units as fine against them)
+    for (int c = g.order == 4 ? kChunkMax / 2 : kChunkMax; c > kPushThreads; c /= 2)
         if (2 * n >= 3ll * 456 * c) return c;
     return kPushThreads;
 }

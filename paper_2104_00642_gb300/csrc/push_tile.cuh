@@ -17,8 +17,9 @@ struct TileItem {
     int tile, start, count, pad;
 };
 
-// 3D items (the 3D push stages no particle state; 256 measured best among
-// 256-1024 on the 8-ppc thermal workload: smaller items balance the CTAs)
+// 3D items: a 4^3 tile of the 8-ppc thermal workload in one item (512 +- 23
+// particles); QED leptons: 256 measured best among 256-1024 on that workload
+constexpr int kChunk3Max = 640;
 constexpr int kChunk3 = 256;
 
 // particles per work item at most, for n particles of a species on grid g
@@ -51,15 +52,19 @@ void launch_tail_items(const PartF32 &P, const uint32_t *first, const Grid &g, T
                        cudaStream_t st);
 // the surrogate's candidate conversions queued by the tiled photon push (q.cq)
 void launch_photon_resolve(const QedParams &q, const PartF32 &P, int *err, cudaStream_t st);
-// 3D: tiles of 4^3 cells, every n_d a multiple of 4
+// 3D, tiles of 4^3 cells (defer: a list of capacity >= the particle count,
+// ndefer its device count; the particles the tiled kernel defers are pushed
+// after it on the global path)
 bool tile3d_push_supported(const Grid &g);
-// (defer: a list of capacity >= the particle count, ndefer its device count;
-// the particles the tiled kernel defers are pushed after it on the global
-// path.  q: a QED lepton species' Monte Carlo, fused in -- nullptr or
-// q->on == 0 for none; nothing is deferred then, and the particles appended
-// since the sort are left to launch_push_qed_f32)
 void launch_push_tile3d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
                         float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, uint32_t *defer,
-                        uint32_t *ndefer, cudaStream_t st, const QedParams *q = nullptr);
+                        uint32_t *ndefer, cudaStream_t st);
+// and with a QED lepton species' Monte Carlo q fused in (q.on; every n_d a
+// multiple of 4); nothing is deferred, and the particles appended since the
+// sort are left to launch_push_qed_f32
+bool tile3d_qed_push_supported(const Grid &g);
+void launch_push_qed_tile3d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
+                            float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st,
+                            const QedParams &q);
 
 }  // namespace pic

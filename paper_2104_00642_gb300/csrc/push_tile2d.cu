@@ -23,19 +23,6 @@
 
 namespace pic {
 
-// drift_f32 with selects instead of branches (a warp of a hot plasma always
-// has lanes on both sides of a branch, three drifts per axis and particle):
-// the offset o + h u ginv, h = dt/(2 dx), with face crossing
-__device__ __forceinline__ void drift_sel_f32(int &c, float &o, float h, float u, float ginv)
-{
-    const float on = fmaf(h * u, ginv, o);
-    const bool up = on >= 1.0f, dn = on < 0.0f;
-    const float w = dn ? on + 1.0f : on;  // in (0, 1], or on itself
-    const bool face = dn && w >= 1.0f;    // a tiny negative offset rounded up to 1: the particle sits on the face
-    o = up ? on - 1.0f : (face ? 0.0f : w);
-    c += (up ? 1 : 0) - (dn && !face ? 1 : 0);
-}
-
 template <int T>
 struct Box2p {
     static constexpr int WX = T + 12;  // x: [t0-4, t0+T+8), a multiple of 4 floats
@@ -141,73 +128,67 @@ struct AccWarp {
     }
 };
 
-// The deposits of one item's records: n records, the r-th at slot first +
-// dir r of the record arrays.  CROSS: the nearest node moved along an axis
-// (union window of ORDER + 2 nodes); else start and end share the window of
-// ORDER + 1 nodes.
+// One row of the deposits: records lane S + j, S rows of 32.  CROSS: the
+// nearest node moved along an axis (filed from the back; union window of
+// ORDER + 2 nodes); else start and end share the window of ORDER + 1 nodes.
 //
-// Lane striding: the records are cut into 32 contiguous segments of S and
-// lane l of every warp walks segment l.  Records of one cell lie together
-// (the particles are cell-sorted), so the 32 lanes of one shared atomic are
-// on 32 different cells, whatever the order in the tile; S is odd, so the
-// record reads are conflict-free too.
+// Lane striding: the n records are cut into 32 contiguous segments of S and
+// lane l of every row is on segment l.  Records of one cell lie together (the
+// particles are cell-sorted), so the 32 lanes of one shared atomic are on 32
+// different cells, whatever the order in the tile; S is odd, so the record
+// reads are conflict-free too.
 template <int T, int ORDER, bool AGG, bool CROSS>
-__device__ __forceinline__ void deposit_records2d(const float *sR, int *sJ, int first, int dir, int n, float sjx,
-                                                  float sjy, float sqw)
+__device__ __forceinline__ void deposit_row2d(const float *sR, int *sJ, int j, int S, int n, float sjx, float sjy,
+                                              float sqw)
 {
     using B = Box2p<T>;
     constexpr int W = ORDER + (CROSS ? 2 : 1), PN = ORDER + 1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = kPushThreads / 32;
-    const int S = AGG ? (n + 31) >> 5 : ((n + 31) >> 5) | 1;
-    for (int j = warp; j < S; j += nwarps) {
-        const int r = AGG ? j * 32 + lane : lane * S + j;
-        const bool valid = r < n;
-        const int slot = first + dir * r;
-        int key = -1;
-        float jvz = 0.f;
-        float S0[2][W], dS[2][W];
-        if (valid) {
-            const uint32_t pk = __float_as_uint(sR[5 * kChunkMax + slot]);
-            key = (int)(pk & 0xffffu);
-            jvz = sqw * sR[4 * kChunkMax + slot];
+    const int lane = threadIdx.x & 31;
+    const int r = AGG ? j * 32 + lane : lane * S + j;
+    const bool valid = r < n;
+    const int slot = CROSS ? kChunkMax - 1 - r : r;
+    int key = -1;
+    float jvz = 0.f;
+    float S0[2][W], dS[2][W];
+    if (valid) {
+        const uint32_t pk = __float_as_uint(sR[5 * kChunkMax + slot]);
+        key = (int)(pk & 0xffffu);
+        jvz = sqw * sR[4 * kChunkMax + slot];
 #pragma unroll
-            for (int d = 0; d < 2; d++) {
-                const float oh = sR[d * kChunkMax + slot], oe = sR[(2 + d) * kChunkMax + slot];
-                float w0[PN], w1[PN];
-                int i;
-                axis_wn_f32<ORDER>(0, oh, i, w0);
-                axis_wn_f32<ORDER>(0, oe, i, w1);
-                if constexpr (CROSS) {
-                    const bool o0 = (pk >> (16 + 2 * d)) & 1u, o1 = (pk >> (17 + 2 * d)) & 1u;
+        for (int d = 0; d < 2; d++) {
+            const float oh = sR[d * kChunkMax + slot], oe = sR[(2 + d) * kChunkMax + slot];
+            float w0[PN], w1[PN];
+            int i;
+            axis_wn_f32<ORDER>(0, oh, i, w0);
+            axis_wn_f32<ORDER>(0, oe, i, w1);
+            if constexpr (CROSS) {
+                const bool o0 = (pk >> (16 + 2 * d)) & 1u, o1 = (pk >> (17 + 2 * d)) & 1u;
 #pragma unroll
-                    for (int k = 0; k < W; k++) {
-                        const float s0 = o0 ? (k >= 1 ? w0[k - 1] : 0.f) : (k < PN ? w0[k] : 0.f);
-                        const float s1 = o1 ? (k >= 1 ? w1[k - 1] : 0.f) : (k < PN ? w1[k] : 0.f);
-                        S0[d][k] = s0;
-                        dS[d][k] = s1 - s0;
-                    }
-                } else {
+                for (int k = 0; k < W; k++) {
+                    const float s0 = o0 ? (k >= 1 ? w0[k - 1] : 0.f) : (k < PN ? w0[k] : 0.f);
+                    const float s1 = o1 ? (k >= 1 ? w1[k - 1] : 0.f) : (k < PN ? w1[k] : 0.f);
+                    S0[d][k] = s0;
+                    dS[d][k] = s1 - s0;
+                }
+            } else {
 #pragma unroll
-                    for (int k = 0; k < W; k++) {
-                        S0[d][k] = w0[k];
-                        dS[d][k] = w1[k] - w0[k];
-                    }
+                for (int k = 0; k < W; k++) {
+                    S0[d][k] = w0[k];
+                    dS[d][k] = w1[k] - w0[k];
                 }
             }
         }
-        if constexpr (AGG) {
-            const unsigned smask = __ballot_sync(0xffffffffu, valid);
-            if (valid) {
-                const unsigned grp = __match_any_sync(smask, key);
-                AccWarp acc{sJ + key, B::NJ, B::RJ, grp, lane == __ffs(grp) - 1};
-                esirkepov2d<W>(S0, dS, sjx, sjy, jvz, acc);
-            }
-        } else {
-            if (valid) {
-                AccSharedUnits acc{sJ + key, B::NJ, B::RJ};
-                esirkepov2d<W>(S0, dS, sjx, sjy, jvz, acc);
-            }
+    }
+    if constexpr (AGG) {
+        const unsigned smask = __ballot_sync(0xffffffffu, valid);
+        if (valid) {
+            const unsigned grp = __match_any_sync(smask, key);
+            AccWarp acc{sJ + key, B::NJ, B::RJ, grp, lane == __ffs(grp) - 1};
+            esirkepov2d<W>(S0, dS, sjx, sjy, jvz, acc);
         }
+    } else if (valid) {
+        AccSharedUnits acc{sJ + key, B::NJ, B::RJ};
+        esirkepov2d<W>(S0, dS, sjx, sjy, jvz, acc);
     }
 }
 
@@ -229,8 +210,9 @@ __device__ __forceinline__ void deposit_records2d(const float *sR, int *sJ, int 
 // one-thread-per-particle kernel -> 39 us.
 //
 // Fixed point: the units of the item's current box come from its particles,
-// 2^31 per |q w| sum(max_d |v_d|).  No node can hold more: a particle adds at
-// most |q w v_d| max(W) to a node, and wrapped intermediate sums are exact.
+// about 2^31 for the sum over them of the most that each can add to one node
+// (|q w v_d| times the shapes' largest values), so no node can overflow, and
+// wrapped intermediate sums are exact.
 //
 // The field box of an item is one TMA tile copy (tmap: the six field
 // components as a 3D tensor, x fastest) issued by one thread: of the CTA's
@@ -249,8 +231,8 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     constexpr int H = ORDER / 2, PN = ORDER + 1;
     extern __shared__ __align__(16) float smem_raw[];
     __shared__ uint64_t mbar;
-    __shared__ int sCnt[2];                      // records filed from the front (node unmoved) and the back
-    __shared__ float sSum[kPushThreads / 32];    // sum of max_d |v_d| per warp
+    __shared__ int sCnt[3];                      // records filed from the front (node unmoved) and the back; rows taken
+    __shared__ float sSum[3][kPushThreads / 32];  // sum of |v_d| per warp
     // the TMA destination starts on a 128-byte boundary
     // (offset from the shared array itself, so that the compiler keeps every
     // access below in the shared address space)
@@ -274,7 +256,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         tma_load_3d(sF, &tmap, tile % g.ntile[0] * T - 4 + g.G[0], tile / g.ntile[0] * T - 4 + g.G[1], 0, &mbar);
     };
     if (threadIdx.x == 0) {
-        sCnt[0] = sCnt[1] = 0;
+        sCnt[0] = sCnt[1] = sCnt[2] = 0;
         if (use_tma) {
             mbar_init(&mbar, 1);
             if ((int)blockIdx.x < nit) stage_box(items[blockIdx.x].tile);
@@ -324,10 +306,10 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             if (threadIdx.x == 0) atomicOr(err, ERR_TIMEOUT);
             return;
         }
-        // push phase, in block-wide passes (warp-uniform: the records are
-        // filed by the warp)
-        float vsum = 0.f;
-        for (uint32_t pbase = m.start; pbase < pend; pbase += kPushThreads, p += kPushThreads) {
+        // push phase (the records are filed by the warp; a warp without
+        // particles skips its passes)
+        float vsum[3] = {0.f, 0.f, 0.f};
+        for (uint32_t pbase = m.start + 32 * warp; pbase < pend; pbase += kPushThreads, p += kPushThreads) {
             const uint32_t cp = ncell;
             float ux = nst[2], uy = nst[3], uz = nst[4];
             float o[2] = {nst[0], nst[1]};
@@ -429,7 +411,9 @@ __global__ void __launch_bounds__(kPushThreads, 3)
                 for (int d = 0; d < 2; d++)
                     pk |= (uint32_t)(icn[d] - H - u0[d]) << (16 + 2 * d) | (uint32_t)(i1[d] - H - u0[d]) << (17 + 2 * d);
                 sR[5 * kChunkMax + slot] = __uint_as_float(pk);
-                vsum += fmaxf(fmaxf(fabsf(ux), fabsf(uy)), fabsf(uz)) * ig1;
+                vsum[0] += fabsf(ux) * ig1;
+                vsum[1] += fabsf(uy) * ig1;
+                vsum[2] += fabsf(vz);
             }
             if (!act) continue;
             // boundaries
@@ -454,24 +438,27 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             P.u[1][p] = uy;
             P.u[2][p] = uz;
         }
-#pragma unroll
-        for (int s = 16; s > 0; s >>= 1) vsum += __shfl_xor_sync(0xffffffffu, vsum, s);
-        if (lane == 0) sSum[warp] = vsum;
+        warp_sums(vsum, sSum);
         __syncthreads();
         // the next item's field box, while this one's records are deposited
         if (use_tma && threadIdx.x == 0 && it + (int)gridDim.x < nit) stage_box(items[it + gridDim.x].tile);
         // deposit phase
-        float vs = 0.f;
-#pragma unroll
-        for (int w = 0; w < kPushThreads / 32; w++) vs += sSum[w];
-        const float jscale = 2147483648.0f / fmaxf(fabsf(qw) * vs, 1e-28f);
-        const float sjx = cjx * jscale, sjy = cjy * jscale, sqw = qw * jscale;
-        deposit_records2d<T, ORDER, AGG, false>(sR, sJ, 0, 1, sCnt[0], sjx, sjy, sqw);
-        deposit_records2d<T, ORDER, AGG, true>(sR, sJ, kChunkMax - 1, -1, sCnt[1], sjx, sjy, sqw);
+        // (the largest share of a particle's current on one node, per unit of
+        // |q w v_d|: along x and y the prefix of the shape difference times the
+        // other axis' shape, along z both shapes; then 1/2^31 of the sum)
+        constexpr float kW = ORDER == 2 ? 0.75f : 115.0f / 192.0f, kP = ORDER == 2 ? 1.0f : 2.0f / 3.0f;
+        const float scx = box_units(sSum[0], fabsf(qw) * (kP * kW)), scy = box_units(sSum[1], fabsf(qw) * (kP * kW)),
+                    scz = box_units(sSum[2], fabsf(qw) * (kW * kW));
+        const float sjx = cjx * scx, sjy = cjy * scy, sqw = qw * scz;
+        const int nk = sCnt[0], nc = sCnt[1], Sk = deposit_rows(nk), Sc = deposit_rows(nc);
+        for (int j = next_row(&sCnt[2]); j < Sc + Sk; j = next_row(&sCnt[2])) {
+            if (j < Sc) deposit_row2d<T, ORDER, AGG, true>(sR, sJ, j, Sc, nc, sjx, sjy, sqw);
+            else deposit_row2d<T, ORDER, AGG, false>(sR, sJ, j - Sc, Sk, nk, sjx, sjy, sqw);
+        }
         __syncthreads();
-        if (threadIdx.x == 0) sCnt[0] = sCnt[1] = 0;
+        if (threadIdx.x == 0) sCnt[0] = sCnt[1] = sCnt[2] = 0;
         // flush the current box, four values at a time, and leave it zero
-        const float junit = 1.0f / jscale;
+        const float unit[3] = {1.0f / scx, 1.0f / scy, 1.0f / scz};
         for (int v4 = threadIdx.x; v4 < 3 * B::WY * (B::WX / 4); v4 += kPushThreads) {
             const int row = v4 / (B::WX / 4), x = 4 * (v4 - row * (B::WX / 4));
             const int c = row / B::WY, y = row - c * B::WY;
@@ -479,6 +466,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             const int4 iv = *cellv;
             if ((iv.x | iv.y | iv.z | iv.w) == 0) continue;
             *cellv = make_int4(0, 0, 0, 0);
+            const float junit = c == 0 ? unit[0] : (c == 1 ? unit[1] : unit[2]);
             const float4 v = make_float4(iv.x * junit, iv.y * junit, iv.z * junit, iv.w * junit);
             const int gx = bx0 + x, gy = by0 + y;
             if (gx < -g.G[0] || gx + 3 >= g.n[0] + g.G[0] || gy < -g.G[1] || gy >= g.n[1] + g.G[1]) {

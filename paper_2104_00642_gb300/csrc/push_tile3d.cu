@@ -1,43 +1,43 @@
-// push_tile3d.cu -- tiled particle push for 3D grids (FP32 cell+offset
-// form): the scheme of push_tile.cu with a 3D box.
+// push_tile3d.cu -- tiled particle push for 3D grids (FP32 cell+offset form,
+// shape order 2, without QED): the two phases of push_tile2d.cu with a 3D box.
 #include <algorithm>
 #include <cstring>
 
-#include "push_qed_dev.cuh"
 #include "push_tile_dev.cuh"
 #include "tma.cuh"
 
 namespace pic {
 
-// ---------------------------------------------------------------------
-// 3D: tiles of T^3 cells, the same scheme with a 3D box
-//   x: [t0-4, t0+T+4) (float4-aligned rows), y and z: [t0-3, t0+T+3);
-// the box of a tile that touches the domain edge stays inside the padded
-// field box (ghost layers of 4), so staging and flush need no edge tests.
-// Consecutive lanes take consecutive particles of an item (coalesced loads
-// of the particle state, which is not staged in 3D).
-// ---------------------------------------------------------------------
+// Tiles of T^3 cells.  The box holds x in [t0-4, t0+T+4) (float4-aligned
+// rows) and y, z in [t0-3, t0+T+4): a particle within two cells below or one
+// above its tile's faces after the half drift finds all its nodes there.  In
+// x the box of an edge tile stays inside the padded rows; rows and planes of
+// a ragged grid's last tiles may lie past them (staged as zero, never
+// deposited on: a cell below n reaches node n+2, the padding node n+3).
 template <int T>
-struct Box3 {
-    static constexpr int WX = T + 8, WY = T + 6, WZ = T + 6;
+struct Box3p {
+    static constexpr int WX = T + 8, WY = T + 7, WZ = T + 7;
     static constexpr int RS = WX, PS = WX * WY, N = WX * WY * WZ;
-    static constexpr int SMEM = 9 * N * (int)sizeof(float);  // fields (6) + current (3)
+    // fields (6), current (3), deposit records (7 words per particle)
+    static constexpr int SMEM = (9 * N + 7 * kChunk3Max) * (int)sizeof(float);
 };
 
 // element k of a small register array without dynamic indexing (selects)
-__device__ __forceinline__ float sel3(const float *v, int k) { return k == 0 ? v[0] : (k == 1 ? v[1] : v[2]); }
-__device__ __forceinline__ float sel4(const float *v, int k)
+template <int W>
+__device__ __forceinline__ float sel(const float *v, int k)
 {
-    return k == 0 ? v[0] : (k == 1 ? v[1] : (k == 2 ? v[2] : v[3]));
+    float r = v[0];
+#pragma unroll
+    for (int i = 1; i < W; i++) r = k == i ? v[i] : r;
+    return r;
 }
 
-// Eq. (19) in 3D on the shared box.  The z loop is kept rolled: the 3D push
-// body is large, and a fully unrolled one stalls on instruction fetch.
+// Eq. (19) in 3D on the shared box
 template <int T>
 __device__ __forceinline__ void gather3d_box(const float *__restrict__ P, const int *o0, const int *icn,
                                              const float (*wn)[3], const int *ich, const float (*wh)[3], float *eb)
 {
-    using B = Box3<T>;
+    using B = Box3p<T>;
 #pragma unroll
     for (int c = 0; c < 6; c++) {
         const int sx = stag(c, 0), sy = stag(c, 1), sz = stag(c, 2);
@@ -49,7 +49,7 @@ __device__ __forceinline__ void gather3d_box(const float *__restrict__ P, const 
         const float *wz = sz ? wh[2] : wn[2];
         const float *q = P + c * B::N + iz * B::PS + iy * B::RS + ix;
         float acc = 0.f;
-#pragma unroll 1
+#pragma unroll
         for (int cz = 0; cz < 3; cz++) {
             float sb = 0.f;
 #pragma unroll
@@ -60,293 +60,297 @@ __device__ __forceinline__ void gather3d_box(const float *__restrict__ P, const 
                 s += wx[2] * r[2];
                 sb += wy[b] * s;
             }
-            acc += sel3(wz, cz) * sb;
+            acc += wz[cz] * sb;
         }
         eb[c] = acc;
     }
 }
 
-// Esirkepov in 3D on the union window (Eqs. (20)-(22)): W_x = dSx (ty tz +
-// dSy dSz / 12) with t = S0 + dS/2 (= S0y S0z + (dSy S0z + S0y dSz)/2 +
-// dSy dSz/3), cyclic for y and z; J_d is cJ_d times the prefix sum of W_d
-// along d (three nonzero nodes of the four).  Shared int32 fixed point.
-template <int T>
-__device__ __forceinline__ void esirkepov3d_box(int *base, const float (*S0)[4], const float (*dS)[4], float cjx,
-                                                float cjy, float cjz, float scale)
+// Esirkepov in 3D on a window of W nodes a side (Eqs. (20)-(22)): W_x = dSx
+// (ty tz + dSy dSz / 12) with t = S0 + dS/2 (= S0y S0z + (dSy S0z + S0y
+// dSz)/2 + dSy dSz/3), cyclic for y and z; J_d is cJ_d times the prefix sum of
+// W_d along d (W - 1 nonzero nodes).  Shared int32 fixed point; the
+// coefficients carry the units.
+template <int T, int W>
+__device__ __forceinline__ void esirkepov3d_box(int *base, const float (*S0)[W], const float (*dS)[W], const float *cj)
 {
-    using B = Box3<T>;
-    float t[3][4], p[3][3];
+    using B = Box3p<T>;
+    float t[3][W], p[3][W - 1];
 #pragma unroll
     for (int d = 0; d < 3; d++) {
 #pragma unroll
-        for (int k = 0; k < 4; k++) t[d][k] = S0[d][k] + 0.5f * dS[d][k];
+        for (int k = 0; k < W; k++) t[d][k] = S0[d][k] + 0.5f * dS[d][k];
         p[d][0] = dS[d][0];
-        p[d][1] = p[d][0] + dS[d][1];
-        p[d][2] = p[d][1] + dS[d][2];
+#pragma unroll
+        for (int k = 1; k < W - 1; k++) p[d][k] = p[d][k - 1] + dS[d][k];
     }
-    const float cj[3] = {cjx * scale, cjy * scale, cjz * scale};
     const float r12 = 1.0f / 12.0f;
-    // the outermost loop of each component stays rolled (code size, as in
-    // gather3d_box); its index picks the z (or y) shape by selects
+    // the outermost loop of each component stays rolled (code size: an
+    // unrolled body stalls on instruction fetch); its index picks the z (or
+    // y) shape by selects
 #pragma unroll 1
-    for (int c = 0; c < 4; c++) {
-        const float tzc = sel4(t[2], c), dzc = sel4(dS[2], c) * r12;
+    for (int c = 0; c < W; c++) {
+        const float tzc = sel<W>(t[2], c), dzc = sel<W>(dS[2], c) * r12;
         int *bc = base + c * B::PS;
 #pragma unroll
-        for (int b = 0; b < 4; b++) {
+        for (int b = 0; b < W; b++) {
             const float wx = fmaf(t[1][b], tzc, dS[1][b] * dzc) * cj[0];
 #pragma unroll
-            for (int a = 0; a < 3; a++) atomicAdd(bc + b * B::RS + a, __float2int_rn(p[0][a] * wx));
+            for (int a = 0; a < W - 1; a++) atomicAdd(bc + b * B::RS + a, __float2int_rn(p[0][a] * wx));
         }
 #pragma unroll
-        for (int a = 0; a < 4; a++) {
+        for (int a = 0; a < W; a++) {
             const float wy = fmaf(t[0][a], tzc, dS[0][a] * dzc) * cj[1];
 #pragma unroll
-            for (int b = 0; b < 3; b++) atomicAdd(bc + B::N + b * B::RS + a, __float2int_rn(p[1][b] * wy));
+            for (int b = 0; b < W - 1; b++) atomicAdd(bc + B::N + b * B::RS + a, __float2int_rn(p[1][b] * wy));
         }
     }
 #pragma unroll 1
-    for (int b = 0; b < 4; b++) {
-        const float tyb = sel4(t[1], b), dyb = sel4(dS[1], b) * r12;
+    for (int b = 0; b < W; b++) {
+        const float tyb = sel<W>(t[1], b), dyb = sel<W>(dS[1], b) * r12;
         int *bb = base + 2 * B::N + b * B::RS;
 #pragma unroll
-        for (int a = 0; a < 4; a++) {
+        for (int a = 0; a < W; a++) {
             const float wz = fmaf(t[0][a], tyb, dS[0][a] * dyb) * cj[2];
 #pragma unroll
-            for (int c = 0; c < 3; c++) atomicAdd(bb + c * B::PS + a, __float2int_rn(p[2][c] * wz));
+            for (int c = 0; c < W - 1; c++) atomicAdd(bb + c * B::PS + a, __float2int_rn(p[2][c] * wz));
         }
     }
 }
 
-// the QED variants' slow paths, out of line (rare: a particle that drifted
-// out of its tile's box since the sort): the gather from HBM and the
-// deposit with global atomics on the 5-node window
-static __device__ __noinline__ void gather3d_global(const float *F, const Grid &g, const int *icn,
-                                                   const float (*wn)[3], const int *ich, const float (*wh)[3],
-                                                   float *eb)
+// one row of the deposits (as deposit_row2d of push_tile2d.cu)
+template <int T, bool CROSS>
+__device__ __forceinline__ void deposit_row3d(const float *sR, int *sJ, int j, int S, int n, const float *cj)
 {
-    gather<float, 3>(F, g, icn, wn, ich, wh, eb);
-}
-
-static __device__ __noinline__ bool deposit3d_global(float *F, const Grid &g, const PushConst &pc, const int *ch,
-                                                     const float *oh, const int *c, const float *o, float uy,
-                                                     float uz, float ig1)
-{
-    float S0[3][5], dS[3][5];
-    int base[3];
-    bool ok = true;
+    constexpr int W = CROSS ? 4 : 3;
+    const int r = (int)(threadIdx.x & 31u) * S + j;
+    if (r >= n) return;
+    const int slot = CROSS ? kChunk3Max - 1 - r : r;
+    const uint32_t pk = __float_as_uint(sR[6 * kChunk3Max + slot]);
+    float S0[3][W], dS[3][W];
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-        int i0, i1;
         float w0[3], w1[3];
-        axis_wn_f32(ch[d], oh[d], i0, w0);
-        axis_wn_f32(c[d], o[d], i1, w1);
-        ok &= window5<float>(i0, w0, i1, w1, S0[d], dS[d]);
-        base[d] = i0 - 2;
+        int i;
+        axis_wn_f32(0, sR[d * kChunk3Max + slot], i, w0);
+        axis_wn_f32(0, sR[(3 + d) * kChunk3Max + slot], i, w1);
+        const bool o0 = CROSS && ((pk >> (16 + 2 * d)) & 1u), o1 = CROSS && ((pk >> (17 + 2 * d)) & 1u);
+#pragma unroll
+        for (int k = 0; k < W; k++) {
+            const float s0 = o0 ? (k >= 1 ? w0[k - 1] : 0.f) : (k < 3 ? w0[k < 3 ? k : 0] : 0.f);
+            const float s1 = o1 ? (k >= 1 ? w1[k - 1] : 0.f) : (k < 3 ? w1[k < 3 ? k : 0] : 0.f);
+            S0[d][k] = s0;
+            dS[d][k] = s1 - s0;
+        }
     }
-    if (!ok) return false;
-    const float cJ[3] = {pc.cJ_f[0], pc.cJ_f[1], pc.cJ_f[2]};
-    deposit_global<float, 3>(F, g, base, S0, dS, cJ, pc.qw_f * uy * ig1, pc.qw_f * uz * ig1);
-    return true;
+    esirkepov3d_box<T, W>(sJ + (pk & 0xffffu), S0, dS, cj);
 }
 
-// A particle whose stencil leaves its tile's box (it drifted since the sort)
-// is not pushed here (QM == 0): its index goes to a list, and the list is
-// pushed afterwards on the global path (launch_push_list_f32).  Nothing of
-// the particle is written before that decision, and a warp never waits on
-// one lane's slow path.
+// One item in the two phases of k_push_tile2d (push_tile2d.cu): push with
+// consecutive lanes on consecutive particles, then the lane-strided deposit of
+// the records, those whose nearest node did not move on 3^3 windows (54
+// atomics), the others on 4^3 (144); units of the current box from the item's
+// particles.
 //
-// QM (QED leptons): 1 = the Monte Carlo of Sec. IV with the tables, 2 = with
-// the surrogate network (its image after the boxes), as in the 2D kernel;
-// a particle whose stencil left the box takes the global gather and deposit
-// in place (its optical depth has moved on).  Particles are taken in
-// block-wide passes so that the network's warp-collective evaluation sees
-// every lane; the event flag of every particle of the items is written.
-template <int T, int QM>
-__global__ void __launch_bounds__(kTileThreads, QM == 2 ? 3 : 5)
+// Bound: the shared-memory pipe (78 %; 162 field loads and 54 to 144 atomics a
+// particle, about two wavefronts each) and issue (57 %).  256^3-style thermal
+// plasma, 16,777,216 particles at 200 keV: 2.63 ms a push in one pass over
+// consecutive lanes (eight lanes on one cell) and its deferred list, now 1.73
+// ms; 856,440 particles on a 61 x 45 x 39 grid: 757 us one thread per
+// particle, now 130 us.  The box's row above the tile is two cells deep: 7 %
+// fewer cells (six rows and planes around the tile) deferred enough particles
+// to cost 1.96 ms.
+//
+// A particle whose stencil leaves its tile's box (it drifted since the sort)
+// is not pushed here: its index goes to a list, and the list is pushed
+// afterwards on the global path (launch_push_list_f32).  Nothing of the
+// particle is written before that decision, and a warp never waits on one
+// lane's slow path.
+template <int T>
+__global__ void __launch_bounds__(kPushThreads, 3)
     k_push_tile3d(PartF32 P, const TileItem *__restrict__ items, const uint32_t *__restrict__ nitems,
                   float *__restrict__ F, Grid g, PushConst pc, int *err, double *e_abs, uint32_t *defer,
-                  uint32_t *ndefer, const __grid_constant__ CUtensorMap tmap, int use_tma, QedParams q)
+                  uint32_t *ndefer, const __grid_constant__ CUtensorMap tmap, int use_tma)
 {
-    using B = Box3<T>;
+    using B = Box3p<T>;
     extern __shared__ __align__(16) float smem_raw[];
     __shared__ uint64_t mbar;
+    __shared__ int sCnt[3];                    // records filed from the front (node unmoved) and the back; rows taken
+    __shared__ float sSum[3][kPushThreads / 32];  // sum of |v_d| per warp
     // the TMA destination starts on a 128-byte boundary
     // (offset from the shared array itself, so that the compiler keeps every
     // access below in the shared address space)
     float *smem = smem_raw + ((128u - ((uint32_t)__cvta_generic_to_shared(smem_raw) & 127u)) & 127u) / 4u;
     float *sF = smem;                                    // 6 components
     int *sJ = reinterpret_cast<int *>(smem + 6 * B::N);  // 3 components, fixed point
-    unsigned char *sNet = reinterpret_cast<unsigned char *>(smem) + B::SMEM;  // QM == 2: the network
-    if constexpr (QM == 2) mlp_stage(sNet, q.net, kMlpStageBytes);
+    float *sR = smem + 9 * B::N;                         // records: oh (3), oe (3), window
     const int nit = (int)*nitems;
     const long long V = g.vol;
     const float hdx[3] = {pc.hdx_f[0], pc.hdx_f[1], pc.hdx_f[2]};
     const float k = pc.qmdt2_f;
-    const float cjx = pc.cJ_f[0], cjy = pc.cJ_f[1], cjz = pc.cJ_f[2];
-    // fixed-point unit of the shared current box: 2^20 units per C, C the
-    // largest value one particle adds to a node
-    const float cmax = fmaxf(fmaxf(fabsf(cjx), fabsf(cjy)), fabsf(cjz));
-    const float jscale = 1048576.0f / fmaxf(cmax, 1e-30f);
-    const float junit = 1.0f / jscale;
     float *Fg = F + g.origin;
     const int rs = (int)g.sy, ps = (int)g.sz;
-    if (use_tma && threadIdx.x == 0) mbar_init(&mbar, 1);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto corner = [&](int tile, int *o) {
+        o[0] = tile % g.ntile[0] * T - 4;
+        o[1] = tile / g.ntile[0] % g.ntile[1] * T - 3;
+        o[2] = tile / (g.ntile[0] * g.ntile[1]) * T - 3;
+    };
+    auto stage_box = [&](int tile) {  // one thread; padded x coordinate a multiple of 4 floats, as TMA requires
+        int o[3];
+        corner(tile, o);
+        fence_proxy_async_smem();
+        mbar_arrive_expect_tx(&mbar, 6 * B::N * (int)sizeof(float));
+        tma_load_4d(sF, &tmap, o[0] + g.G[0], o[1] + g.G[1], o[2] + g.G[2], 0, &mbar);
+    };
+    if (threadIdx.x == 0) {
+        sCnt[0] = sCnt[1] = sCnt[2] = 0;
+        if (use_tma) {
+            mbar_init(&mbar, 1);
+            if ((int)blockIdx.x < nit) stage_box(items[blockIdx.x].tile);
+        }
+    }
+    for (int e4 = threadIdx.x; e4 < 3 * B::N / 4; e4 += kPushThreads)
+        reinterpret_cast<int4 *>(sJ)[e4] = make_int4(0, 0, 0, 0);
     __syncthreads();
     uint32_t phase = 0;
     for (int it = blockIdx.x; it < nit; it += gridDim.x) {
         const TileItem m = items[it];
-        const int tx = m.tile % g.ntile[0], ty = (m.tile / g.ntile[0]) % g.ntile[1],
-                  tz = m.tile / (g.ntile[0] * g.ntile[1]);
-        const int o0[3] = {tx * T - 4, ty * T - 3, tz * T - 3};
-        // 1-2. stage fields (one TMA tile: x padded coordinate tx*T, a
-        // multiple of 4 floats; else float4 rows), zero the current box
-        if (use_tma) {
-            if (threadIdx.x == 0) {
-                fence_proxy_async_smem();
-                mbar_arrive_expect_tx(&mbar, 6 * B::N * (int)sizeof(float));
-                tma_load_4d(sF, &tmap, o0[0] + g.G[0], o0[1] + g.G[1], o0[2] + g.G[2], 0, &mbar);
+        int o0[3];
+        corner(m.tile, o0);
+        // the first pass's particle state, ahead of the wait for the field box
+        uint32_t p = (uint32_t)m.start + threadIdx.x;  // capacities are below 2^31
+        const uint32_t pend = (uint32_t)(m.start + m.count);
+        uint32_t ncell = kDead;
+        float nst[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        auto fetch = [&](uint32_t pn) {
+            ncell = kDead;
+            if (pn < pend) {
+                ncell = P.cell[pn];
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    nst[d] = P.off[d][pn];
+                    nst[3 + d] = P.u[d][pn];
+                }
             }
-        } else {
-            for (int e4 = threadIdx.x; e4 < 6 * B::N / 4; e4 += blockDim.x) {
-                const int e = 4 * e4;
-                const int c = e / B::N, r = e - c * B::N;
-                const int z = r / B::PS, y = (r - z * B::PS) / B::RS, x = r - z * B::PS - y * B::RS;
-                const float *src = Fg + c * V + (long long)(o0[2] + z) * ps + (long long)(o0[1] + y) * rs + o0[0] + x;
-                reinterpret_cast<float4 *>(sF)[e4] = __ldg(reinterpret_cast<const float4 *>(src));
-            }
-        }
-        for (int e4 = threadIdx.x; e4 < 3 * B::N / 4; e4 += blockDim.x)
-            reinterpret_cast<int4 *>(sJ)[e4] = make_int4(0, 0, 0, 0);
+        };
+        fetch(p);
         bool landed = true;
         if (use_tma) {
-            landed = mbar_wait(&mbar, phase, 1 << 22);
+            landed = mbar_wait(&mbar, phase, 1 << 22);  // bounded: a copy that never lands is reported
             phase ^= 1u;
+        } else {
+            for (int e = threadIdx.x; e < 6 * B::N; e += kPushThreads) {
+                const int c = e / B::N, r = e - c * B::N;
+                const int z = r / B::PS, y = (r - z * B::PS) / B::RS, x = r - z * B::PS - y * B::RS;
+                const int gx = o0[0] + x, gy = o0[1] + y, gz = o0[2] + z;
+                float v = 0.f;
+                if (gx < g.n[0] + g.G[0] && gy < g.n[1] + g.G[1] && gz < g.n[2] + g.G[2])
+                    v = __ldg(Fg + c * V + (long long)gz * ps + (long long)gy * rs + gx);
+                sF[e] = v;
+            }
         }
         if (__syncthreads_or(!landed)) {
             if (threadIdx.x == 0) atomicOr(err, ERR_TIMEOUT);
             return;
         }
-        // 3. particles, in block-wide passes (warp-uniform), consecutive lanes
-        // on consecutive particles: the particle state is read straight from
-        // HBM, coalesced (lane striding, as in 2D, measured 5 % slower here:
-        // without a staging buffer its loads scatter)
-        for (int pbase = 0; pbase < m.count; pbase += blockDim.x) {
-            const int li = pbase + threadIdx.x;
-            const int p = m.start + li;
-            const bool mine = li < m.count;
-            const uint32_t cp = mine ? P.cell[p] : kDead;
+        // push phase (a warp without particles skips its passes)
+        float vsum[3] = {0.f, 0.f, 0.f};
+        for (uint32_t pbase = m.start + 32 * warp; pbase < pend; pbase += kPushThreads, p += kPushThreads) {
+            const uint32_t cp = ncell;
+            float o[3] = {nst[0], nst[1], nst[2]};
+            float ux = nst[3], uy = nst[4], uz = nst[5];
+            fetch(p + kPushThreads);
             bool act = cp != kDead;
-            int c[3] = {0, 0, 0}, ch[3] = {0, 0, 0}, c1[3] = {0, 0, 0};
-            float o[3] = {0.f, 0.f, 0.f}, oh[3] = {0.f, 0.f, 0.f}, o1[3] = {0.f, 0.f, 0.f};
-            float ux = 0.f, uy = 0.f, uz = 0.f, ig1 = 0.f;
-            float eb[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            int c[3] = {0, 0, 0}, c1[3] = {0, 0, 0}, u0[3] = {0, 0, 0};
+            float oh[3] = {0.f, 0.f, 0.f}, o1[3] = {0.f, 0.f, 0.f};
+            int icn[3] = {0, 0, 0}, i1[3] = {0, 0, 0};
+            float ig1 = 0.f;
+            bool din = false, cross = false;
             if (act) {
                 unpack_cell(g, cp, c[0], c[1], c[2]);
-                o[0] = P.off[0][p];
-                o[1] = P.off[1][p];
-                o[2] = P.off[2][p];
-                ux = P.u[0][p];
-                uy = P.u[1][p];
-                uz = P.u[2][p];
                 const float ig = inv_gamma_fast(ux, uy, uz);
                 const float u[3] = {ux, uy, uz};
-#pragma unroll
-                for (int d = 0; d < 3; d++) drift_f32(c[d], o[d], hdx[d] * u[d] * ig);
-                int icn[3], ich[3];
+                int ich[3];
                 float wn[3][3], wh[3][3];
                 bool gin = true;
 #pragma unroll
                 for (int d = 0; d < 3; d++) {
-                    ch[d] = c[d];
+                    drift_sel_f32(c[d], o[d], hdx[d], u[d], ig);
                     oh[d] = o[d];
                     axis_w_f32(c[d], o[d], icn[d], wn[d], ich[d], wh[d]);
-                    const int W = d == 0 ? B::WX : B::WY;
-                    gin &= ch[d] - 1 >= o0[d] && ch[d] + 2 < o0[d] + W;
+                    gin &= c[d] - 1 >= o0[d] && c[d] + 2 < o0[d] + (d == 0 ? B::WX : B::WY);
                 }
-                if (QM == 0 && !gin) {
-                    defer[atomicAdd(ndefer, 1u)] = (uint32_t)p;
-                    act = false;  // pushed by the list, from its unchanged state
-                } else {
-                    if (gin) gather3d_box<T>(sF, o0, icn, wn, ich, wh, eb);
-                    else gather3d_global(F, g, icn, wn, ich, wh, eb);
+                if (gin) {
+                    float eb[6];
+                    gather3d_box<T>(sF, o0, icn, wn, ich, wh, eb);
                     if (pc.pusher) vay<float>(ux, uy, uz, k * eb[0], k * eb[1], k * eb[2], k * eb[3], k * eb[4], k * eb[5]);
                     else boris_fast(ux, uy, uz, k * eb[0], k * eb[1], k * eb[2], k * eb[3], k * eb[4], k * eb[5]);
+                    ig1 = inv_gamma_fast(ux, uy, uz);
+                    const float un[3] = {ux, uy, uz};
+                    // Esirkepov on x^{n+1/2} -> x^{n+3/2}: the window of both end points
+                    bool ok = true;
+                    din = true;
+#pragma unroll
+                    for (int d = 0; d < 3; d++) {
+                        drift_sel_f32(c[d], o[d], hdx[d], un[d], ig1);
+                        c1[d] = c[d];
+                        o1[d] = o[d];
+                        drift_sel_f32(c[d], o[d], hdx[d], un[d], ig1);
+                        i1[d] = c[d] + (o[d] >= 0.5f ? 1 : 0);
+                        ok &= (i1[d] - icn[d] >= -1 && i1[d] - icn[d] <= 1);
+                        cross |= i1[d] != icn[d];
+                        u0[d] = min(icn[d], i1[d]) - 1;
+                        din &= u0[d] >= o0[d] && u0[d] + 3 < o0[d] + (d == 0 ? B::WX : B::WY);
+                    }
+                    // a non-finite momentum (a NaN or infinite field) is reported and the particle
+                    // removed before anything uses its position: NaN positions would give no valid
+                    // cell or node index to the gather, the deposit or the diagnostics (and would
+                    // otherwise be reported as a Courant violation)
+                    if (!isfinite(ux + uy + uz)) {
+                        atomicOr(err, ERR_NONFINITE);
+                        P.cell[p] = kDead;
+                        act = din = false;
+                    } else if (!ok) {
+                        atomicOr(err, ERR_CFL);
+                        act = din = false;  // keeps its stored state
+                    }
                 }
+                if (act && !din) defer[atomicAdd(ndefer, 1u)] = p;  // pushed by the list from its unchanged state
             }
-            // QED (every lane of the block: the network's evaluation is warp-collective)
-            uint32_t event = 0;
-            float4 evd = make_float4(0.f, 0.f, 0.f, 0.f);
-            if constexpr (QM != 0) qed_lepton_f32<QM == 2>(q, sNet, act, p, eb, ux, uy, uz, err, event, evd);
-            bool dep = false;  // deposited (so the state is written)
-            if (act) {
-                ig1 = inv_gamma_fast(ux, uy, uz);
-                const float dd[3] = {hdx[0] * ux * ig1, hdx[1] * uy * ig1, hdx[2] * uz * ig1};
+            // file the deposit record: from the front, or (node moved) from the back
+            const unsigned mk = __ballot_sync(0xffffffffu, din && !cross), mc = __ballot_sync(0xffffffffu, din && cross);
+            int at = 0;
+            if (lane == 0 && mk) at = atomicAdd(&sCnt[0], __popc(mk));
+            if (lane == 1 && mc) at = atomicAdd(&sCnt[1], __popc(mc));
+            const int a0 = __shfl_sync(0xffffffffu, at, 0), a1 = __shfl_sync(0xffffffffu, at, 1);
+            if (!din) continue;
+            const unsigned lt = (1u << lane) - 1u;
+            const int slot = cross ? kChunk3Max - 1 - a1 - __popc(mc & lt) : a0 + __popc(mk & lt);
+            uint32_t pk = (uint32_t)((u0[2] - o0[2]) * B::PS + (u0[1] - o0[1]) * B::RS + (u0[0] - o0[0]));
 #pragma unroll
-                for (int d = 0; d < 3; d++) drift_f32(c[d], o[d], dd[d]);
-#pragma unroll
-                for (int d = 0; d < 3; d++) {
-                    c1[d] = c[d];
-                    o1[d] = o[d];
-                }
-#pragma unroll
-                for (int d = 0; d < 3; d++) drift_f32(c[d], o[d], dd[d]);
-                // Esirkepov on x^{n+1/2} -> x^{n+3/2}
-                int i0[3], i1[3];
-                float w0[3][3], w1[3][3];
-                bool ok = true, din = true;
-                float S0[3][4], dS[3][4];
-                int u0[3];
-#pragma unroll
-                for (int d = 0; d < 3; d++) {
-                    axis_wn_f32(ch[d], oh[d], i0[d], w0[d]);
-                    axis_wn_f32(c[d], o[d], i1[d], w1[d]);
-                    ok &= (i1[d] - i0[d] >= -1 && i1[d] - i0[d] <= 1);
-                    u0[d] = union4(i0[d], w0[d], i1[d], w1[d], S0[d], dS[d]);
-                    const int W = d == 0 ? B::WX : B::WY;
-                    din &= u0[d] >= o0[d] && u0[d] + 3 < o0[d] + W;
-                }
-                // a non-finite momentum (a NaN or infinite field) is reported and the particle
-                // removed before anything uses its position: NaN positions would give no valid
-                // cell or node index to the gather, the deposit or the diagnostics (and would
-                // otherwise be reported as a Courant violation)
-                if (!isfinite(ux + uy + uz)) {
-                    atomicOr(err, ERR_NONFINITE);
-                    P.cell[p] = kDead;
-                } else if (!ok) {
-                    atomicOr(err, ERR_CFL);
-                } else if (din) {
-                    esirkepov3d_box<T>(sJ + (u0[2] - o0[2]) * B::PS + (u0[1] - o0[1]) * B::RS + (u0[0] - o0[0]), S0,
-                                       dS, cjx, cjy, cjz, jscale);
-                    dep = true;
-                } else if (QM == 0) {
-                    defer[atomicAdd(ndefer, 1u)] = (uint32_t)p;  // pushed by the list from its unchanged state
-                } else {
-                    dep = deposit3d_global(F, g, pc, ch, oh, c, o, uy, uz, ig1);
-                    if (!dep) atomicOr(err, ERR_CFL);
-                }
+            for (int d = 0; d < 3; d++) {
+                sR[d * kChunk3Max + slot] = oh[d];
+                sR[(3 + d) * kChunk3Max + slot] = o[d];
+                pk |= (uint32_t)(icn[d] - 1 - u0[d]) << (16 + 2 * d) | (uint32_t)(i1[d] - 1 - u0[d]) << (17 + 2 * d);
             }
-            if (!dep) {
-                if (QM != 0 && mine) q.ev[p] = 0;
-                continue;
-            }
+            sR[6 * kChunk3Max + slot] = __uint_as_float(pk);
+            vsum[0] += fabsf(ux) * ig1;
+            vsum[1] += fabsf(uy) * ig1;
+            vsum[2] += fabsf(uz) * ig1;
             // boundaries
             int cc[3] = {c1[0], c1[1], c1[2]};
             bool dead = false;
 #pragma unroll
             for (int d = 0; d < 3; d++) {
-                if (g.bc[d] == PERIODIC) {
-                    if (cc[d] < 0) cc[d] += g.n[d];
-                    else if (cc[d] >= g.n[d]) cc[d] -= g.n[d];
-                } else if (cc[d] < 0 || cc[d] >= g.n[d]) {
-                    dead = true;
-                }
+                const bool lo = cc[d] < 0, hi = cc[d] >= g.n[d], per = g.bc[d] == PERIODIC;
+                dead |= !per && (lo || hi);
+                cc[d] += per ? (lo ? g.n[d] : (hi ? -g.n[d] : 0)) : 0;
             }
             if (dead) {
                 P.cell[p] = kDead;
                 double uu = (double)ux * ux + (double)uy * uy + (double)uz * uz;
                 atomicAdd(e_abs, pc.wmdV * uu / (sqrt(1.0 + uu) + 1.0));
-                event = 0;  // an emitter absorbed in the same step records no photon
             } else {
                 P.cell[p] = pack_cell(g, cc[0], cc[1], cc[2]);
             }
@@ -355,76 +359,79 @@ __global__ void __launch_bounds__(kTileThreads, QM == 2 ? 3 : 5)
             P.u[0][p] = ux;
             P.u[1][p] = uy;
             P.u[2][p] = uz;
-            if constexpr (QM != 0) {
-                q.ev[p] = event;
-                if (event) reinterpret_cast<float4 *>(q.evk)[p] = evd;
-            }
+        }
+        warp_sums(vsum, sSum);
+        __syncthreads();
+        // the next item's field box, while this one's records are deposited
+        if (use_tma && threadIdx.x == 0 && it + (int)gridDim.x < nit) stage_box(items[it + gridDim.x].tile);
+        // deposit phase
+        // (a node's share of a particle's |q w v_d|: at most the square of the
+        // largest weight, 3/4)
+        float sc[3], cj[3];
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            sc[d] = box_units(sSum[d], fabsf(pc.qw_f) * 0.5625f);
+            cj[d] = pc.cJ_f[d] * sc[d];
+        }
+        const int nk = sCnt[0], nc = sCnt[1], Sk = deposit_rows(nk), Sc = deposit_rows(nc);
+        for (int j = next_row(&sCnt[2]); j < Sc + Sk; j = next_row(&sCnt[2])) {
+            if (j < Sc) deposit_row3d<T, true>(sR, sJ, j, Sc, nc, cj);
+            else deposit_row3d<T, false>(sR, sJ, j - Sc, Sk, nk, cj);
         }
         __syncthreads();
-        // 4. flush the current box, four values at a time
-        for (int e4 = threadIdx.x; e4 < 3 * B::N / 4; e4 += blockDim.x) {
+        if (threadIdx.x == 0) sCnt[0] = sCnt[1] = sCnt[2] = 0;
+        // flush the current box, four values at a time, and leave it zero (rows
+        // past a ragged grid's padding hold zeros only)
+        const float unit[3] = {1.0f / sc[0], 1.0f / sc[1], 1.0f / sc[2]};
+        for (int e4 = threadIdx.x; e4 < 3 * B::N / 4; e4 += kPushThreads) {
             const int4 iv = reinterpret_cast<const int4 *>(sJ)[e4];
             if ((iv.x | iv.y | iv.z | iv.w) == 0) continue;
+            reinterpret_cast<int4 *>(sJ)[e4] = make_int4(0, 0, 0, 0);
             const int e = 4 * e4;
             const int c = e / B::N, r = e - c * B::N;
             const int z = r / B::PS, y = (r - z * B::PS) / B::RS, x = r - z * B::PS - y * B::RS;
+            const float junit = c == 0 ? unit[0] : (c == 1 ? unit[1] : unit[2]);
             float *dst = Fg + (JX + c) * V + (long long)(o0[2] + z) * ps + (long long)(o0[1] + y) * rs + o0[0] + x;
             atomicAdd(reinterpret_cast<float4 *>(dst), make_float4(iv.x * junit, iv.y * junit, iv.z * junit, iv.w * junit));
         }
-        __syncthreads();
+        // (the next item's first barrier orders the flush before its records)
     }
-}
-
-template <int QM>
-static void launch_tile3d_T(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
-                            float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, uint32_t *defer,
-                            uint32_t *ndefer, cudaStream_t st, const QedParams &q)
-{
-    constexpr int T = 4;
-    constexpr int smem = Box3<T>::SMEM + 128 + (QM == 2 ? kMlpStageBytes : 0);  // + alignment of the TMA destination
-    static bool attr = false;
-    static int nsm = 0, per_sm = 0;
-    if (!attr) {
-        cudaFuncSetAttribute(k_push_tile3d<T, QM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_push_tile3d<T, QM>, kTileThreads, smem);
-        if (per_sm < 1) per_sm = 1;
-        attr = true;
-    }
-    // the six field components as one 4D tensor (x, y, z, component)
-    CUtensorMap tmap;
-    const int box[4] = {Box3<T>::WX, Box3<T>::WY, Box3<T>::WZ, 6};
-    const bool tma = tma_encode_field_map3(&tmap, F, g.ext, g.sy, g.sz, g.vol, 6, box);
-    if (!tma) memset(&tmap, 0, sizeof tmap);
-    long long grid = std::min<long long>(max_items, (long long)nsm * per_sm);  // one resident wave
-    if (grid < 1) grid = 1;
-    note_launch();
-    k_push_tile3d<T, QM><<<(int)grid, kTileThreads, smem, st>>>(P, items, nitems, F, g, pc, err, e_abs, defer, ndefer,
-                                                                 tmap, tma ? 1 : 0, q);
 }
 
 void launch_push_tile3d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
                         float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, uint32_t *defer,
-                        uint32_t *ndefer, cudaStream_t st, const QedParams *q)
+                        uint32_t *ndefer, cudaStream_t st)
 {
     if (P.n == 0) return;
-    if (q && q->on) {  // QED leptons: no deferral (see k_push_tile3d)
-        if (q->net) launch_tile3d_T<2>(P, items, nitems, max_items, F, g, pc, err, e_abs, defer, ndefer, st, *q);
-        else launch_tile3d_T<1>(P, items, nitems, max_items, F, g, pc, err, e_abs, defer, ndefer, st, *q);
-        return;
+    constexpr int T = 4;
+    constexpr int smem = Box3p<T>::SMEM + 128;  // + alignment of the TMA destination
+    static int nsm = 0, per_sm = 0;
+    if (!per_sm) {
+        cudaFuncSetAttribute(k_push_tile3d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_push_tile3d<T>, kPushThreads, smem);
+        if (per_sm < 1) per_sm = 1;
     }
+    // the six field components as one 4D tensor (x, y, z, component)
+    CUtensorMap tmap;
+    const int box[4] = {Box3p<T>::WX, Box3p<T>::WY, Box3p<T>::WZ, 6};
+    const bool tma = tma_encode_field_map3(&tmap, F, g.ext, g.sy, g.sz, g.vol, 6, box);
+    if (!tma) memset(&tmap, 0, sizeof tmap);
+    long long grid = std::min<long long>(max_items, (long long)nsm * per_sm);  // one resident wave
+    if (grid < 1) grid = 1;
     cudaMemsetAsync(ndefer, 0, sizeof(uint32_t), st);
-    const QedParams none{};
-    launch_tile3d_T<0>(P, items, nitems, max_items, F, g, pc, err, e_abs, defer, ndefer, st, none);
+    note_launch();
+    k_push_tile3d<T><<<(int)grid, kPushThreads, smem, st>>>(P, items, nitems, F, g, pc, err, e_abs, defer, ndefer, tmap,
+                                                            tma ? 1 : 0);
     launch_push_list_f32(P, defer, ndefer, P.n, F, g, pc, err, e_abs, st);
 }
 
 bool tile3d_push_supported(const Grid &g)
 {
     for (int d = 0; d < 3; d++)
-        if (g.tile_log2[d] != 2 || g.n[d] % 4 != 0 || g.G[d] != 4) return false;
+        if (g.tile_log2[d] != 2 || g.G[d] != 4) return false;
     return g.dim == 3;
 }
 

@@ -51,6 +51,54 @@ struct AccWarpAll {
     }
 };
 
+// drift_f32 with selects instead of branches (a warp of a hot plasma always
+// has lanes on both sides of a branch, three drifts per axis and particle):
+// the offset o + h u ginv, h = dt/(2 dx), with face crossing
+__device__ __forceinline__ void drift_sel_f32(int &c, float &o, float h, float u, float ginv)
+{
+    const float on = fmaf(h * u, ginv, o);
+    const bool up = on >= 1.0f, dn = on < 0.0f;
+    const float w = dn ? on + 1.0f : on;  // in (0, 1], or on itself
+    const bool face = dn && w >= 1.0f;    // a tiny negative offset rounded up to 1: the particle sits on the face
+    o = up ? on - 1.0f : (face ? 0.0f : w);
+    c += (up ? 1 : 0) - (dn && !face ? 1 : 0);
+}
+
+// per-warp sums of |v_d| over the records a thread filed
+__device__ __forceinline__ void warp_sums(float *v, float (*sum)[kPushThreads / 32])
+{
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) v[d] += __shfl_xor_sync(0xffffffffu, v[d], s);
+        if ((threadIdx.x & 31u) == 0) sum[d][threadIdx.x >> 5] = v[d];
+    }
+}
+
+// fixed-point units per unit of current for an item whose particles' sum of
+// |v_d| is in sum (per warp), each adding at most most |v_d| to a node: 2^31
+// less a margin for the roundings (at most half a unit per particle, and
+// FP32's in the sums)
+__device__ __forceinline__ float box_units(const float *sum, float most)
+{
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < kPushThreads / 32; w++) v += sum[w];
+    return 2.14e9f / fmaxf(most * v, 1e-28f);
+}
+
+// the deposit phase's rows of 32 records (an odd number: see deposit_row2d),
+// taken by the CTA's warps as they come free, the costlier ones first: a
+// fixed share of the rows left warps waiting at the barrier (2.5 of 11 warps
+// stalled there in the 3D push, 9 rows on 8 warps)
+__device__ __forceinline__ int deposit_rows(int n) { return n ? ((n + 31) >> 5) | 1 : 0; }
+__device__ __forceinline__ int next_row(int *taken)
+{
+    int j = 0;
+    if ((threadIdx.x & 31u) == 0) j = atomicAdd(taken, 1);
+    return __shfl_sync(0xffffffffu, j, 0);
+}
+
 // Boris (Eqs. (13)-(16)) with the FP32 reciprocal square root and divide
 // of the special-function unit (a few ulp, far inside the FP32 tolerance)
 __device__ __forceinline__ void boris_fast(float &ux, float &uy, float &uz, float ex, float ey, float ez, float bx,

@@ -62,3 +62,19 @@ def test_tile2d_order4_one_step_matches_oracle(tile, n, nppc, crowd, bc):
             setattr(s, k, getattr(s, k)[:1].copy())
     _crowd(w, crowd, 3, 7)
     _one_step(w, F, 4, (tile, tile, 1))
+
+
+@pytest.mark.parametrize("n,nppc,crowd,bc", [((13, 10, 9), 3, 0.0, (P, P, P)),    # ragged in every axis
+                                             ((16, 12, 8), 2, 0.6, (P, P, P)),    # a tile of more than 640 particles
+                                             ((11, 14, 17), 1, 0.0, (A, P, A)),   # absorbing faces on ragged tiles
+                                             ((28, 9, 8), 0, 0.0, (P, P, P))])    # one particle (pitch = padded row)
+def test_tile3d_ragged_one_step_matches_oracle(n, nppc, crowd, bc):
+    dx = (0.1, 0.12, 0.11)
+    dt = 0.9 / np.sqrt(sum(1.0 / d ** 2 for d in dx))
+    w, F = random_state(3, n, dx, dt, max(nppc, 1), seed=650 + n[0], umax=0.9, bc=bc)
+    if nppc == 0:
+        s = w.species[0]
+        for k in ("x", "y", "z", "ux", "uy", "uz"):
+            setattr(s, k, getattr(s, k)[-1:].copy())
+    _crowd(w, crowd, 3, 9)
+    _one_step(w, F, 2, (4, 4, 4))

@@ -216,46 +216,37 @@ void out_box(const Grid &g, long long *m)
         m[d] = d >= g.dim ? 1 : (g.bc[d] == ABSORB ? g.n[d] + 1 : g.n[d]);
 }
 
+// one component to and from the host in the exchange layout, staged in a
+// dense device block: s->rho (the diagnostics' array, free between them), or
+// a temporary one when rho itself leaves
 template <typename R>
 int copy_comp_out(pic_sim *s, const R *dev, double *host_out)
 {
-    const Grid &g = s->g;
-    std::vector<R> h((size_t)g.vol);
-    CK(cudaMemcpyAsync(h.data(), dev, (size_t)g.vol * sizeof(R), cudaMemcpyDeviceToHost, s->st));
-    CK(cudaStreamSynchronize(s->st));
     long long m[3];
-    out_box(g, m);
-    for (long long k = 0; k < m[2]; k++)
-        for (long long j = 0; j < m[1]; j++)
-            for (long long i = 0; i < m[0]; i++)
-                host_out[(k * m[1] + j) * m[0] + i] = (double)h[(size_t)goff(g, (int)i, (int)j, (int)k)];
+    out_box(s->g, m);
+    const size_t bytes = (size_t)(m[0] * m[1] * m[2]) * sizeof(double);
+    double *stage = s->rho, *tmp = nullptr;
+    if ((const void *)dev == (const void *)s->rho) {
+        if (int rc = talloc(s, (void **)&tmp, bytes)) return rc;
+        stage = tmp;
+    }
+    field_pack<R>(dev, s->g, m, stage, s->st);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(host_out, stage, bytes, cudaMemcpyDeviceToHost, s->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
+    tfree(s, tmp);
+    if (e != cudaSuccess) return fail(s, PIC_ERR_CUDA, "field copy: %s", cudaGetErrorString(e));
     return PIC_OK;
 }
 
 template <typename R>
 int copy_comp_in(pic_sim *s, R *dev, const double *host_in)
 {
-    const Grid &g = s->g;
-    std::vector<R> h((size_t)g.vol);
-    CK(cudaMemcpyAsync(h.data(), dev, (size_t)g.vol * sizeof(R), cudaMemcpyDeviceToHost, s->st));
-    CK(cudaStreamSynchronize(s->st));
     long long m[3];
-    out_box(g, m);
-    // every padded cell whose (periodic image of the) index lies in the box
-    for (int k = -g.G[2]; k < g.n[2] + g.G[2]; k++)
-        for (int j = -g.G[1]; j < g.n[1] + g.G[1]; j++)
-            for (int i = -g.G[0]; i < g.n[0] + g.G[0]; i++) {
-                int p[3] = {i, j, k};
-                bool in = true;
-                for (int d = 0; d < 3 && in; d++) {
-                    if (d >= g.dim) continue;
-                    if (g.bc[d] == PERIODIC) p[d] = ((p[d] % g.n[d]) + g.n[d]) % g.n[d];
-                    else if (p[d] < 0 || p[d] >= m[d]) in = false;
-                }
-                if (!in) continue;
-                h[(size_t)goff(g, i, j, k)] = (R)host_in[((long long)p[2] * m[1] + p[1]) * m[0] + p[0]];
-            }
-    CK(cudaMemcpyAsync(dev, h.data(), (size_t)g.vol * sizeof(R), cudaMemcpyHostToDevice, s->st));
+    out_box(s->g, m);
+    CK(cudaMemcpyAsync(s->rho, host_in, (size_t)(m[0] * m[1] * m[2]) * sizeof(double), cudaMemcpyHostToDevice, s->st));
+    field_unpack<R>(s->rho, s->g, m, dev, s->st);
+    CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s->st));
     return PIC_OK;
 }
@@ -714,13 +705,14 @@ int pic_create(const pic_grid *grid, double dt, const pic_species *species, int 
     }
     rc = rc ? rc : dalloc(s, &s->sort_scratch, sort_scratch_bytes(maxcap));
     rc = rc ? rc : dalloc(s, (void **)&s->diag_scratch, diag_scratch_doubles() * sizeof(double));
-    rc = rc ? rc : dalloc(s, (void **)&s->diag_out, 16 * sizeof(double));
+    rc = rc ? rc : dalloc(s, (void **)&s->diag_out, 32 * sizeof(double));
     rc = rc ? rc : dalloc(s, (void **)&s->d_err, sizeof(int));
     rc = rc ? rc : dalloc(s, (void **)&s->d_eabs, sizeof(double));
     rc = rc ? rc : dalloc(s, (void **)&s->d_elost, sizeof(double));
     if (!rc) {
         cudaError_t z = cudaMemsetAsync(s->F, 0, (size_t)NCOMP * g.vol * R, s->st);
         if (z == cudaSuccess) z = cudaMemsetAsync(s->d_err, 0, sizeof(int), s->st);
+        if (z == cudaSuccess) z = cudaMemsetAsync(s->diag_scratch, 0, diag_scratch_doubles() * sizeof(double), s->st);
         if (z == cudaSuccess) z = cudaMemsetAsync(s->d_eabs, 0, sizeof(double), s->st);
         if (z == cudaSuccess) z = cudaMemsetAsync(s->d_elost, 0, sizeof(double), s->st);
         for (int i = 0; i < nsp && z == cudaSuccess; i++)
@@ -1195,43 +1187,45 @@ int pic_diagnostics(pic_sim *s, pic_diag *d)
         dV *= g.dx[a];
         vol *= g.dx[a] * g.n[a];
     }
-    double h[16] = {0};
-    // field energy
+    // every reduction into its own slots of diag_out, read back once
+    double *out = s->diag_out;
     if (s->precision == PIC_PREC_FP64_PLAIN)
-        diag_field_energy<double>((const double *)s->F, g, s->diag_scratch, s->diag_out, s->st);
+        diag_field_energy<double>((const double *)s->F, g, s->diag_scratch, out, s->st);
     else
-        diag_field_energy<float>((const float *)s->F, g, s->diag_scratch, s->diag_out, s->st);
-    CK(cudaMemcpyAsync(h, s->diag_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, s->st));
+        diag_field_energy<float>((const float *)s->F, g, s->diag_scratch, out, s->st);
+    for (int i = 0; i < s->nsp; i++) {
+        const bool photon = s->sp[i].kind == PIC_KIND_PHOTON;
+        if (s->precision == PIC_PREC_FP64_PLAIN)
+            diag_kinetic_f64(view64(s, i, s->sp[i].cur), photon, s->diag_scratch, out + 2 + 2 * i, s->st);
+        else
+            diag_kinetic_f32(view32(s, i, s->sp[i].cur), photon, s->diag_scratch, out + 2 + 2 * i, s->st);
+    }
+    int rc = compute_rho(s);
+    if (rc) return rc;
+    double *tail = out + 2 + 2 * s->nsp;
+    if (s->precision == PIC_PREC_FP64_PLAIN)
+        diag_gauss<double>((const double *)s->F, s->rho, g, s->rho_bg, s->d_eabs, s->d_elost, s->diag_scratch, tail, s->st);
+    else
+        diag_gauss<float>((const float *)s->F, s->rho, g, s->rho_bg, s->d_eabs, s->d_elost, s->diag_scratch, tail, s->st);
+    CK(cudaGetLastError());
+    double h[2 + 2 * PIC_MAX_SPECIES + 3] = {0};
+    CK(cudaMemcpyAsync(h, out, (size_t)(2 + 2 * s->nsp + 3) * sizeof(double), cudaMemcpyDeviceToHost, s->st));
     CK(cudaStreamSynchronize(s->st));
     d->U_E = 0.5 * h[0] * dV;
     d->U_B = 0.5 * h[1] * dV;
     double charge = 0.0;
     for (int i = 0; i < s->nsp; i++) {
-        SpeciesState &p = s->sp[i];
-        if (s->precision == PIC_PREC_FP64_PLAIN)
-            diag_kinetic_f64(view64(s, i, p.cur), p.kind == PIC_KIND_PHOTON, s->diag_scratch, s->diag_out, s->st);
-        else
-            diag_kinetic_f32(view32(s, i, p.cur), p.kind == PIC_KIND_PHOTON, s->diag_scratch, s->diag_out, s->st);
-        CK(cudaMemcpyAsync(h, s->diag_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, s->st));
-        CK(cudaStreamSynchronize(s->st));
-        d->U_kin[i] = h[0] * p.w * (p.kind == PIC_KIND_PHOTON ? 1.0 : p.m) * dV;
-        d->n_alive[i] = (int64_t)llround(h[1]);
-        charge += p.q * p.w * h[1] * dV;
+        const SpeciesState &p = s->sp[i];
+        const double *k = h + 2 + 2 * i;
+        d->U_kin[i] = k[0] * p.w * (p.kind == PIC_KIND_PHOTON ? 1.0 : p.m) * dV;
+        d->n_alive[i] = (int64_t)llround(k[1]);
+        charge += p.q * p.w * k[1] * dV;
     }
     d->charge = charge + s->rho_bg * vol;
-    int rc = compute_rho(s);
-    if (rc) return rc;
-    if (s->precision == PIC_PREC_FP64_PLAIN)
-        diag_gauss<double>((const double *)s->F, s->rho, g, s->rho_bg, s->diag_scratch, s->diag_out, s->st);
-    else
-        diag_gauss<float>((const float *)s->F, s->rho, g, s->rho_bg, s->diag_scratch, s->diag_out, s->st);
-    CK(cudaMemcpyAsync(h, s->diag_out, sizeof(double), cudaMemcpyDeviceToHost, s->st));
-    CK(cudaMemcpyAsync(h + 1, s->d_eabs, sizeof(double), cudaMemcpyDeviceToHost, s->st));
-    CK(cudaStreamSynchronize(s->st));
-    CK(cudaGetLastError());
-    d->gauss_max = h[0];
-    d->E_absorbed = h[1];
-    CK(cudaMemcpy(&d->E_photon_lost, s->d_elost, sizeof(double), cudaMemcpyDeviceToHost));
+    const double *t = h + 2 + 2 * s->nsp;
+    d->gauss_max = t[0];
+    d->E_absorbed = t[1];
+    d->E_photon_lost = t[2];
     d->step = s->step;
     d->t = (double)s->step * g.dt;
     bool finite = std::isfinite(d->U_E) && std::isfinite(d->U_B) && std::isfinite(d->gauss_max);

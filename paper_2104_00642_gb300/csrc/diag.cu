@@ -5,8 +5,16 @@
 //
 // Sums use a fixed reduction tree: a fixed grid of blocks, each reducing a
 // fixed strided set of elements in a fixed shuffle order into one partial,
-// then one block summing the partials in index order, so results do not
-// depend on scheduling.
+// and the block that finishes last summing the partials in index order, so
+// results do not depend on scheduling.
+//
+// FP64 runs at 1/73 of the FP32 rate here and bounds these kernels: the roots
+// and quotients are Newton iterations from an FP32 seed, FP32 inputs become
+// FP64 by moving their bits, and nothing is divided by dx per particle
+// (charge density of 1,048,576 particles in 2D: 326 -> 212 us; species
+// without charge deposit none).
+#include <algorithm>
+
 #include "diag.cuh"
 #include "push_dev.cuh"
 
@@ -28,91 +36,12 @@ __device__ __forceinline__ double warp_max(double v)
     return v;
 }
 
-// NV values per thread reduced to partial[blockIdx.x * NV + q]
 template <int NV, bool MAX>
-__device__ __forceinline__ void block_reduce_store(double *v, double *partial)
+__device__ __forceinline__ void block_reduce_store(const double *v, double *to)
 {
     __shared__ double sh[NV][kRedThreads / 32];
     int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < NV; q++) {
-        double x = MAX ? warp_max(v[q]) : warp_sum(v[q]);
-        if (lane == 0) sh[q][warp] = x;
-    }
     __syncthreads();
-    if (threadIdx.x < 32) {
-#pragma unroll
-        for (int q = 0; q < NV; q++) {
-            double x = lane < kRedThreads / 32 ? sh[q][lane] : (MAX ? 0.0 : 0.0);
-            x = MAX ? warp_max(x) : warp_sum(x);
-            if (lane == 0) partial[blockIdx.x * NV + q] = x;
-        }
-    }
-}
-
-template <typename R>
-__global__ void __launch_bounds__(kRedThreads) k_field_energy(const R *__restrict__ F, Grid g, double *partial)
-{
-    long long tot = (long long)g.n[0] * g.n[1] * g.n[2];
-    double v[2] = {0.0, 0.0};
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < tot;
-         t += (long long)gridDim.x * blockDim.x) {
-        int i = (int)(t % g.n[0]);
-        long long r = t / g.n[0];
-        int j = (int)(r % g.n[1]);
-        int k = (int)(r / g.n[1]);
-        long long o = goff(g, i, j, k);
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            double e = (double)F[(EX + c) * g.vol + o], b = (double)F[(BX + c) * g.vol + o];
-            v[0] += e * e;
-            v[1] += b * b;
-        }
-    }
-    block_reduce_store<2, false>(v, partial);
-}
-
-// sum of (gamma - 1) = u^2 / (gamma + 1) per particle, or of |k| for photons
-__global__ void __launch_bounds__(kRedThreads) k_kinetic_f32(PartF32 P, int photon, double *partial)
-{
-    double v[2] = {0.0, 0.0};
-    long long n = *P.dn;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
-        if (P.cell[p] == kDead) continue;
-        double ux = P.u[0][p], uy = P.u[1][p], uz = P.u[2][p];
-        double uu = ux * ux + uy * uy + uz * uz;
-        v[0] += photon ? sqrt(uu) : uu / (sqrt(1.0 + uu) + 1.0);
-        v[1] += 1.0;
-    }
-    block_reduce_store<2, false>(v, partial);
-}
-
-__global__ void __launch_bounds__(kRedThreads) k_kinetic_f64(PartF64 P, int photon, double *partial)
-{
-    double v[2] = {0.0, 0.0};
-    long long n = *P.dn;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
-        if (P.cell[p] == kDead) continue;
-        double ux = P.u[0][p], uy = P.u[1][p], uz = P.u[2][p];
-        double uu = ux * ux + uy * uy + uz * uz;
-        v[0] += photon ? sqrt(uu) : uu / (sqrt(1.0 + uu) + 1.0);
-        v[1] += 1.0;
-    }
-    block_reduce_store<2, false>(v, partial);
-}
-
-// sums partial[b*NV + q] over b in index order (one block, fixed tree)
-template <int NV, bool MAX>
-__global__ void __launch_bounds__(kRedThreads) k_final(const double *__restrict__ partial, int nparts, double *out)
-{
-    double v[NV];
-#pragma unroll
-    for (int q = 0; q < NV; q++) v[q] = 0.0;
-    for (int b = threadIdx.x; b < nparts; b += blockDim.x)
-#pragma unroll
-        for (int q = 0; q < NV; q++) v[q] = MAX ? fmax(v[q], partial[b * NV + q]) : v[q] + partial[b * NV + q];
-    __shared__ double sh[NV][kRedThreads / 32];
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < NV; q++) {
         double x = MAX ? warp_max(v[q]) : warp_sum(v[q]);
@@ -124,15 +53,125 @@ __global__ void __launch_bounds__(kRedThreads) k_final(const double *__restrict_
         for (int q = 0; q < NV; q++) {
             double x = lane < kRedThreads / 32 ? sh[q][lane] : 0.0;
             x = MAX ? warp_max(x) : warp_sum(x);
-            if (lane == 0) out[q] = x;
+            if (lane == 0) to[q] = x;
         }
     }
 }
 
+// NV values per thread to the grid's totals in out: one partial per block,
+// summed by the block that arrives last (*done counts the arrivals and is
+// left zero; a second launch for the last sum cost 5 us)
+template <int NV, bool MAX>
+__device__ __forceinline__ void grid_reduce(const double *v, double *partial, unsigned *done, double *out)
+{
+    __shared__ bool last;
+    block_reduce_store<NV, MAX>(v, partial + (size_t)blockIdx.x * NV);
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double t[NV];
+#pragma unroll
+    for (int q = 0; q < NV; q++) t[q] = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += kRedThreads)
+#pragma unroll
+        for (int q = 0; q < NV; q++) {
+            const double x = __ldcg(partial + (size_t)b * NV + q);
+            t[q] = MAX ? fmax(t[q], x) : t[q] + x;
+        }
+    block_reduce_store<NV, MAX>(t, out);
+    if (threadIdx.x == 0) *done = 0u;
+}
+
+// a float as a double, by its bits (zero, denormals, infinities and NaN by
+// the conversion)
+__device__ __forceinline__ double widen(float f)
+{
+    const uint32_t b = __float_as_uint(f), e = (b >> 23) & 0xffu;
+    if (e - 1u >= 254u) return (double)f;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
+// 1/sqrt(a) for a >= 1: the FP32 root of a's leading bits, then two Newton
+// steps (7e-7 -> 7e-13 -> rounding); beyond FP32's range the library's root
+__device__ __forceinline__ double rsqrt_fp64(double a)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(a);
+    if (hi >= 0x46000000u) return 1.0 / sqrt(a);  // a >= 2^97, infinity, NaN
+    double r = widen(rsqrtf(__uint_as_float((hi - 0x38000000u) << 3)));
+    const double h = 0.5 * a;
+    r = fma(r, fma(-h, r * r, 0.5), r);
+    return fma(r, fma(-h, r * r, 0.5), r);
+}
+
+// 1/b for 1 <= b < 2^97, the same way
+__device__ __forceinline__ double rcp_fp64(double b)
+{
+    double q = widen(__frcp_rn(__uint_as_float(((uint32_t)__double2hiint(b) - 0x38000000u) << 3)));
+    q = fma(q, fma(-b, q, 1.0), q);
+    return fma(q, fma(-b, q, 1.0), q);
+}
+
+// cell t of the interior, x fastest (the padded grid holds fewer than 2^31 cells)
+__device__ __forceinline__ long long interior(const Grid &g, uint32_t t)
+{
+    const uint32_t r = t / (uint32_t)g.n[0];
+    const int i = (int)(t - r * (uint32_t)g.n[0]);
+    const int k = (int)(r / (uint32_t)g.n[1]);
+    return goff(g, i, (int)(r - (uint32_t)k * (uint32_t)g.n[1]), k);
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kRedThreads) k_field_energy(const R *__restrict__ F, Grid g, double *partial,
+                                                              unsigned *done, double *out)
+{
+    const uint32_t tot = (uint32_t)g.n[0] * g.n[1] * g.n[2];
+    double v[2] = {0.0, 0.0};
+    for (uint32_t t = blockIdx.x * kRedThreads + threadIdx.x; t < tot; t += gridDim.x * kRedThreads) {
+        const long long o = interior(g, t);
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            const double e = widen(F[(EX + c) * g.vol + o]), b = widen(F[(BX + c) * g.vol + o]);
+            v[0] += e * e;
+            v[1] += b * b;
+        }
+    }
+    grid_reduce<2, false>(v, partial, done, out);
+}
+
+// sum of (gamma - 1) = u^2 / (gamma + 1) per particle, or of |k| for photons
+template <class P_t>
+__global__ void __launch_bounds__(kRedThreads) k_kinetic(P_t P, int photon, double *partial, unsigned *done, double *out)
+{
+    double v[2] = {0.0, 0.0};
+    long long live = 0;
+    const long long n = *P.dn;
+    for (long long p = (long long)blockIdx.x * kRedThreads + threadIdx.x; p < n; p += (long long)gridDim.x * kRedThreads) {
+        if (P.cell[p] == kDead) continue;
+        const double ux = widen(P.u[0][p]), uy = widen(P.u[1][p]), uz = widen(P.u[2][p]);
+        const double uu = ux * ux + uy * uy + uz * uz;
+        if (photon) {
+            v[0] += sqrt(uu);
+        } else {
+            const double a = 1.0 + uu;
+            if ((uint32_t)__double2hiint(a) >= 0x46000000u) v[0] += uu / (sqrt(a) + 1.0);
+            else v[0] += uu * rcp_fp64(fma(a, rsqrt_fp64(a), 1.0));
+        }
+        live++;
+    }
+    v[1] = (double)live;
+    grid_reduce<2, false>(v, partial, done, out);
+}
+
 // charge density of one species: q w W (W_2 or W_4, the shape the deposit
-// uses) at x -/+ (dt/2) v, half each
+// uses) at x -/+ (dt/2) v, half each.  X: position in cells (a cell index and
+// the offset from it)
 template <int DIM, int ORDER>
-__device__ __forceinline__ void rho_add(double *rho, const Grid &g, const double *X, double qw2)
+__device__ __forceinline__ void rho_add(double *rho, const Grid &g, const int *c, const double *X, double qw2)
 {
     constexpr int P = ORDER + 1, H = ORDER / 2;
     // a non-finite position has no node; the pushes remove particles whose
@@ -143,115 +182,129 @@ __device__ __forceinline__ void rho_add(double *rho, const Grid &g, const double
     int ic[3] = {0, 0, 0};
     double w[3][P];
 #pragma unroll
-    for (int d = 0; d < 3; d++) {
-        if (d < DIM) {
-            ic[d] = (int)floor(X[d] + 0.5);
-            if constexpr (ORDER == 4) w4<double>(X[d] - (double)ic[d], w[d]);
-            else w2<double>(X[d] - (double)ic[d], w[d]);
-        } else {
+    for (int d = 0; d < DIM; d++) {
+        const double f = floor(X[d] + 0.5);
+        ic[d] = c[d] + (int)f - H;
+        if constexpr (ORDER == 4) w4<double>(X[d] - f, w[d]);
+        else w2<double>(X[d] - f, w[d]);
+    }
+    double *base = rho + goff(g, ic[0], ic[1], ic[2]);
 #pragma unroll
-            for (int a = 0; a < P; a++) w[d][a] = a == H ? 1.0 : 0.0;
+    for (int k = 0; k < (DIM > 2 ? P : 1); k++) {
+        const double wz = DIM > 2 ? qw2 * w[2][k] : qw2;
+#pragma unroll
+        for (int b = 0; b < (DIM > 1 ? P : 1); b++) {
+            const double wy = DIM > 1 ? wz * w[1][b] : wz;
+#pragma unroll
+            for (int a = 0; a < P; a++) atomicAdd(base + (k * g.sz + b * g.sy + a), wy * w[0][a]);
         }
     }
-#pragma unroll
-    for (int c = 0; c < (DIM > 2 ? P : 1); c++)
-#pragma unroll
-        for (int b = 0; b < (DIM > 1 ? P : 1); b++)
-#pragma unroll
-            for (int a = 0; a < P; a++) {
-                int jb = DIM > 1 ? b : H, kc = DIM > 2 ? c : H;
-                double wt = w[0][a] * w[1][jb] * w[2][kc];
-                atomicAdd(rho + goff(g, ic[0] + a - H, DIM > 1 ? ic[1] + b - H : 0, DIM > 2 ? ic[2] + c - H : 0),
-                          qw2 * wt);
-            }
+}
+
+// the particle of a thread: a warp takes 256 consecutive particles in eight
+// rounds, its lanes eight apart, so that the lanes of one atomic are on
+// several cells (the particles are cell-sorted; lanes on one node queue up)
+__device__ __forceinline__ long long rho_particle()
+{
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    return (t & ~255ll) | ((t & 31) << 3) | ((t >> 5) & 7);
 }
 
 template <int DIM, int ORDER>
-__global__ void k_rho_f32(PartF32 P, Grid g, double hdt, double qw2, double *rho)
+__global__ void __launch_bounds__(256) k_rho_f32(PartF32 P, Grid g, double hdt, double qw2, double *rho)
 {
-    long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long p = rho_particle();
     if (p >= *P.dn) return;
-    uint32_t cp = P.cell[p];
+    const uint32_t cp = P.cell[p];
     if (cp == kDead) return;
     int c[3];
     unpack_cell(g, cp, c[0], c[1], c[2]);
-    double ux = P.u[0][p], uy = P.u[1][p], uz = P.u[2][p];
-    double ig = 1.0 / sqrt(1.0 + ux * ux + uy * uy + uz * uz);
-    double u[3] = {ux, uy, uz};
+    const double u[3] = {widen(P.u[0][p]), widen(P.u[1][p]), widen(P.u[2][p])};
+    const double h = hdt * rsqrt_fp64(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    double o[3] = {0, 0, 0}, d[3] = {0, 0, 0};
+#pragma unroll
+    for (int a = 0; a < DIM; a++) {
+        o[a] = widen(P.off[a][p]);
+        d[a] = h * u[a] * g.rdx_d[a];
+    }
+#pragma unroll
     for (int side = -1; side <= 1; side += 2) {
-        double X[3] = {0, 0, 0};
-        for (int d = 0; d < DIM; d++) X[d] = (double)c[d] + (double)P.off[d][p] + side * hdt * u[d] * ig / g.dx[d];
-        rho_add<DIM, ORDER>(rho, g, X, qw2);
+        const double X[3] = {o[0] + side * d[0], o[1] + side * d[1], o[2] + side * d[2]};
+        rho_add<DIM, ORDER>(rho, g, c, X, qw2);
     }
 }
 
 template <int DIM, int ORDER>
-__global__ void k_rho_f64(PartF64 P, Grid g, double hdt, double qw2, double *rho)
+__global__ void __launch_bounds__(256) k_rho_f64(PartF64 P, Grid g, double hdt, double qw2, double *rho)
 {
-    long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long p = rho_particle();
     if (p >= *P.dn) return;
     if (P.cell[p] == kDead) return;
-    double ux = P.u[0][p], uy = P.u[1][p], uz = P.u[2][p];
-    double ig = 1.0 / sqrt(1.0 + ux * ux + uy * uy + uz * uz);
-    double u[3] = {ux, uy, uz};
+    const double u[3] = {P.u[0][p], P.u[1][p], P.u[2][p]};
+    const double h = hdt * rsqrt_fp64(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    const int c[3] = {0, 0, 0};
+#pragma unroll
     for (int side = -1; side <= 1; side += 2) {
         double X[3] = {0, 0, 0};
-        for (int d = 0; d < DIM; d++) X[d] = (P.x[d][p] + side * hdt * u[d] * ig) / g.dx[d];
-        rho_add<DIM, ORDER>(rho, g, X, qw2);
+#pragma unroll
+        for (int a = 0; a < DIM; a++) X[a] = (P.x[a][p] + side * (h * u[a])) * g.rdx_d[a];
+        rho_add<DIM, ORDER>(rho, g, c, X, qw2);
     }
 }
 
 // max over interior nodes of |div E - rho - rho_bg|
+// (and the tallies the diagnostics report with it: out[1] = *t1, out[2] = *t2)
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads) k_gauss(const R *__restrict__ F, const double *__restrict__ rho, Grid g,
-                                                       double rho_bg, double *partial)
+                                                       double rho_bg, double *partial, unsigned *done, double *out,
+                                                       const double *t1, const double *t2)
 {
-    long long tot = (long long)g.n[0] * g.n[1] * g.n[2];
+    const uint32_t tot = (uint32_t)g.n[0] * g.n[1] * g.n[2];
     double v[1] = {0.0};
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < tot;
-         t += (long long)gridDim.x * blockDim.x) {
-        int i = (int)(t % g.n[0]);
-        long long r = t / g.n[0];
-        int j = (int)(r % g.n[1]);
-        int k = (int)(r / g.n[1]);
-        long long o = goff(g, i, j, k);
-        const R *Ex = F + EX * g.vol, *Ey = F + EY * g.vol, *Ez = F + EZ * g.vol;
-        double div = ((double)Ex[o] - (double)Ex[o - 1]) / g.dx[0];
-        if (g.dim > 1) div += ((double)Ey[o] - (double)Ey[o - g.sy]) / g.dx[1];
-        if (g.dim > 2) div += ((double)Ez[o] - (double)Ez[o - g.sz]) / g.dx[2];
+    const R *Ex = F + EX * g.vol, *Ey = F + EY * g.vol, *Ez = F + EZ * g.vol;
+    for (uint32_t t = blockIdx.x * kRedThreads + threadIdx.x; t < tot; t += gridDim.x * kRedThreads) {
+        const long long o = interior(g, t);
+        double div = (widen(Ex[o]) - widen(Ex[o - 1])) * g.rdx_d[0];
+        if (g.dim > 1) div += (widen(Ey[o]) - widen(Ey[o - g.sy])) * g.rdx_d[1];
+        if (g.dim > 2) div += (widen(Ez[o]) - widen(Ez[o - g.sz])) * g.rdx_d[2];
         v[0] = fmax(v[0], fabs(div - rho[o] - rho_bg));
     }
-    block_reduce_store<1, true>(v, partial);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        out[1] = *t1;
+        out[2] = *t2;
+    }
+    grid_reduce<1, true>(v, partial, done, out);
 }
 
 // ---------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------
-size_t diag_scratch_doubles() { return (size_t)kRedBlocks * 4 + 64; }
+// partials, then the arrival counter of grid_reduce (zero between launches)
+size_t diag_scratch_doubles() { return (size_t)kRedBlocks * 2 + 64; }
+static unsigned *done_of(double *scratch) { return reinterpret_cast<unsigned *>(scratch + (size_t)kRedBlocks * 2); }
+static int red_blocks(long long n) { return (int)std::max<long long>(1, std::min<long long>(kRedBlocks, div_up(n, kRedThreads))); }
+static long long interior_cells(const Grid &g) { return (long long)g.n[0] * g.n[1] * g.n[2]; }
 
 template <typename R>
 void diag_field_energy(const R *F, const Grid &g, double *scratch, double *out2, cudaStream_t st)
 {
-    k_field_energy<R><<<kRedBlocks, kRedThreads, 0, st>>>(F, g, scratch);
-    k_final<2, false><<<1, kRedThreads, 0, st>>>(scratch, kRedBlocks, out2);
+    k_field_energy<R><<<red_blocks(interior_cells(g)), kRedThreads, 0, st>>>(F, g, scratch, done_of(scratch), out2);
 }
 template void diag_field_energy<float>(const float *, const Grid &, double *, double *, cudaStream_t);
 template void diag_field_energy<double>(const double *, const Grid &, double *, double *, cudaStream_t);
 
 void diag_kinetic_f32(const PartF32 &P, bool photon, double *scratch, double *out2, cudaStream_t st)
 {
-    k_kinetic_f32<<<kRedBlocks, kRedThreads, 0, st>>>(P, photon ? 1 : 0, scratch);
-    k_final<2, false><<<1, kRedThreads, 0, st>>>(scratch, kRedBlocks, out2);
+    k_kinetic<<<red_blocks(P.n), kRedThreads, 0, st>>>(P, photon ? 1 : 0, scratch, done_of(scratch), out2);
 }
 void diag_kinetic_f64(const PartF64 &P, bool photon, double *scratch, double *out2, cudaStream_t st)
 {
-    k_kinetic_f64<<<kRedBlocks, kRedThreads, 0, st>>>(P, photon ? 1 : 0, scratch);
-    k_final<2, false><<<1, kRedThreads, 0, st>>>(scratch, kRedBlocks, out2);
+    k_kinetic<<<red_blocks(P.n), kRedThreads, 0, st>>>(P, photon ? 1 : 0, scratch, done_of(scratch), out2);
 }
 
 void diag_rho_f32(const PartF32 &P, const Grid &g, double qw, double *rho, cudaStream_t st)
 {
-    if (P.n == 0) return;
+    if (P.n == 0 || qw == 0.0) return;  // (photons: no charge)
     int nb = div_up(P.n, 256);
     double h = 0.5 * g.dt;
     if (g.order == 4) {
@@ -266,7 +319,7 @@ void diag_rho_f32(const PartF32 &P, const Grid &g, double qw, double *rho, cudaS
 }
 void diag_rho_f64(const PartF64 &P, const Grid &g, double qw, double *rho, cudaStream_t st)
 {
-    if (P.n == 0) return;
+    if (P.n == 0 || qw == 0.0) return;  // (photons: no charge)
     int nb = div_up(P.n, 256);
     double h = 0.5 * g.dt;
     if (g.order == 4) {
@@ -281,14 +334,71 @@ void diag_rho_f64(const PartF64 &P, const Grid &g, double qw, double *rho, cudaS
 }
 
 template <typename R>
-void diag_gauss(const R *F, const double *rho, const Grid &g, double rho_bg, double *scratch, double *out1,
-                cudaStream_t st)
+void diag_gauss(const R *F, const double *rho, const Grid &g, double rho_bg, const double *t1, const double *t2,
+                double *scratch, double *out3, cudaStream_t st)
 {
-    k_gauss<R><<<kRedBlocks, kRedThreads, 0, st>>>(F, rho, g, rho_bg, scratch);
-    k_final<1, true><<<1, kRedThreads, 0, st>>>(scratch, kRedBlocks, out1);
+    k_gauss<R><<<red_blocks(interior_cells(g)), kRedThreads, 0, st>>>(F, rho, g, rho_bg, scratch, done_of(scratch), out3,
+                                                                     t1, t2);
 }
-template void diag_gauss<float>(const float *, const double *, const Grid &, double, double *, double *, cudaStream_t);
-template void diag_gauss<double>(const double *, const double *, const Grid &, double, double *, double *,
-                                 cudaStream_t);
+template void diag_gauss<float>(const float *, const double *, const Grid &, double, const double *, const double *,
+                                double *, double *, cudaStream_t);
+template void diag_gauss<double>(const double *, const double *, const Grid &, double, const double *, const double *,
+                                 double *, double *, cudaStream_t);
+
+// ---------------------------------------------------------------------
+// exchange layout (FP64, x fastest, [0, N) or [0, N] per axis) <-> padded
+// component: one thread per padded cell of a row, so that a component crosses
+// to the host as one dense block and the host walks no arrays
+// ---------------------------------------------------------------------
+struct ExBox {
+    int m[3];
+};
+
+template <typename R>
+__global__ void __launch_bounds__(256) k_pack(const R *__restrict__ comp, Grid g, ExBox b, double *__restrict__ out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+    if (i >= b.m[0] || j >= b.m[1]) return;
+    out[((long long)k * b.m[1] + j) * b.m[0] + i] = (double)comp[goff(g, i, j, k)];
+}
+
+// every padded cell whose (periodic image of the) index lies in the box
+template <typename R>
+__global__ void __launch_bounds__(256) k_unpack(const double *__restrict__ in, Grid g, ExBox b, R *__restrict__ comp)
+{
+    int p[3] = {(int)(blockIdx.x * blockDim.x + threadIdx.x) - g.G[0], (int)(blockIdx.y * blockDim.y + threadIdx.y) - g.G[1],
+                (int)blockIdx.z - g.G[2]};
+    if (p[0] >= g.n[0] + g.G[0] || p[1] >= g.n[1] + g.G[1]) return;
+    const long long o = goff(g, p[0], p[1], p[2]);
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        if (d >= g.dim) continue;
+        if (g.bc[d] == PERIODIC) p[d] = (p[d] % g.n[d] + g.n[d]) % g.n[d];
+        else if (p[d] < 0 || p[d] >= b.m[d]) return;
+    }
+    comp[o] = (R)in[((long long)p[2] * b.m[1] + p[1]) * b.m[0] + p[0]];
+}
+
+static dim3 ex_block(const Grid &g) { return g.dim == 1 ? dim3(256, 1, 1) : dim3(64, 4, 1); }
+
+template <typename R>
+void field_pack(const R *comp, const Grid &g, const long long *m, double *out, cudaStream_t st)
+{
+    const ExBox b{{(int)m[0], (int)m[1], (int)m[2]}};
+    const dim3 blk = ex_block(g);
+    k_pack<R><<<dim3(div_up(m[0], blk.x), div_up(m[1], blk.y), (unsigned)m[2]), blk, 0, st>>>(comp, g, b, out);
+}
+template void field_pack<float>(const float *, const Grid &, const long long *, double *, cudaStream_t);
+template void field_pack<double>(const double *, const Grid &, const long long *, double *, cudaStream_t);
+
+template <typename R>
+void field_unpack(const double *in, const Grid &g, const long long *m, R *comp, cudaStream_t st)
+{
+    const ExBox b{{(int)m[0], (int)m[1], (int)m[2]}};
+    const dim3 blk = ex_block(g);
+    k_unpack<R><<<dim3(div_up(g.ext[0], blk.x), div_up(g.ext[1], blk.y), (unsigned)g.ext[2]), blk, 0, st>>>(in, g, b, comp);
+}
+template void field_unpack<float>(const double *, const Grid &, const long long *, float *, cudaStream_t);
+template void field_unpack<double>(const double *, const Grid &, const long long *, double *, cudaStream_t);
 
 }  // namespace pic

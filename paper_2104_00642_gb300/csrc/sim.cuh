@@ -77,7 +77,7 @@ struct pic_sim {
     pic::SpeciesState sp[PIC_MAX_SPECIES];
     void *sort_scratch = nullptr;
     double *diag_scratch = nullptr;
-    double *diag_out = nullptr;  // 16 doubles
+    double *diag_out = nullptr;  // 32 doubles
     int *d_err = nullptr;
     double *d_eabs = nullptr;
     long long step = 0;

@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "diag.cuh"
+#include "fp64_dev.cuh"
 #include "push_dev.cuh"
 
 namespace pic {
@@ -84,36 +85,6 @@ __device__ __forceinline__ void grid_reduce(const double *v, double *partial, un
         }
     block_reduce_store<NV, MAX>(t, out);
     if (threadIdx.x == 0) *done = 0u;
-}
-
-// a float as a double, by its bits (zero, denormals, infinities and NaN by
-// the conversion)
-__device__ __forceinline__ double widen(float f)
-{
-    const uint32_t b = __float_as_uint(f), e = (b >> 23) & 0xffu;
-    if (e - 1u >= 254u) return (double)f;
-    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
-}
-__device__ __forceinline__ double widen(double f) { return f; }
-
-// 1/sqrt(a) for a >= 1: the FP32 root of a's leading bits, then two Newton
-// steps (7e-7 -> 7e-13 -> rounding); beyond FP32's range the library's root
-__device__ __forceinline__ double rsqrt_fp64(double a)
-{
-    const uint32_t hi = (uint32_t)__double2hiint(a);
-    if (hi >= 0x46000000u) return 1.0 / sqrt(a);  // a >= 2^97, infinity, NaN
-    double r = widen(rsqrtf(__uint_as_float((hi - 0x38000000u) << 3)));
-    const double h = 0.5 * a;
-    r = fma(r, fma(-h, r * r, 0.5), r);
-    return fma(r, fma(-h, r * r, 0.5), r);
-}
-
-// 1/b for 1 <= b < 2^97, the same way
-__device__ __forceinline__ double rcp_fp64(double b)
-{
-    double q = widen(__frcp_rn(__uint_as_float(((uint32_t)__double2hiint(b) - 0x38000000u) << 3)));
-    q = fma(q, fma(-b, q, 1.0), q);
-    return fma(q, fma(-b, q, 1.0), q);
 }
 
 // cell t of the interior, x fastest (the padded grid holds fewer than 2^31 cells)

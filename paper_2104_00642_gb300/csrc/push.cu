@@ -32,7 +32,7 @@ template <int DIM, int ORDER>
 __global__ void __launch_bounds__(256) k_push_f32(PartF32 P, float *__restrict__ F, Grid g, PushConst pc,
                                                   int *err, double *e_abs)
 {
-    long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= *P.dn) return;
     push_one_f32<DIM, ORDER>(P, p, F, g, pc, err, e_abs);
 }
@@ -88,17 +88,14 @@ __device__ __forceinline__ void push_one_f32(const PartF32 &P, long long p, floa
 #pragma unroll
     for (int d = 0; d < DIM; d++) drift_f32(c[d], o[d], pc.hdx_f[d] * u[d] * ig1);
     // Esirkepov on x^{n+1/2} -> x^{n+3/2}
-    float S0[3][ORDER + 3], dS[3][ORDER + 3];
-    int base[3] = {0, 0, 0};
+    int i0[3] = {0, 0, 0}, i1[3] = {0, 0, 0};
+    float w0[3][ORDER + 1], w1[3][ORDER + 1];
     bool ok = true;
 #pragma unroll
     for (int d = 0; d < DIM; d++) {
-        int i0, i1;
-        float w0[ORDER + 1], w1[ORDER + 1];
-        axis_wn_f32<ORDER>(ch[d], oh[d], i0, w0);
-        axis_wn_f32<ORDER>(c[d], o[d], i1, w1);
-        ok &= window_n<float, ORDER>(i0, w0, i1, w1, S0[d], dS[d]);
-        base[d] = i0 - ORDER / 2 - 1;
+        axis_wn_f32<ORDER>(ch[d], oh[d], i0[d], w0[d]);
+        axis_wn_f32<ORDER>(c[d], o[d], i1[d], w1[d]);
+        ok &= i1[d] - i0[d] >= -1 && i1[d] - i0[d] <= 1;
     }
     // a non-finite momentum (a NaN or infinite field) is reported and the particle
     // removed before anything uses its position: NaN positions would give no valid
@@ -115,7 +112,7 @@ __device__ __forceinline__ void push_one_f32(const PartF32 &P, long long p, floa
     }
     const float cJ[3] = {pc.cJ_f[0], pc.cJ_f[1], pc.cJ_f[2]};
     const float qw = pc.qw_f;
-    deposit_global<float, DIM, ORDER>(F, g, base, S0, dS, cJ, qw * uy * ig1, qw * uz * ig1);
+    deposit_moved<float, DIM, ORDER>(F, g, i0, w0, i1, w1, cJ, qw * uy * ig1, qw * uz * ig1);
     // boundaries
     bool dead = false;
 #pragma unroll
@@ -144,52 +141,109 @@ __device__ __forceinline__ void push_one_f32(const PartF32 &P, long long p, floa
 // ---------------------------------------------------------------------
 // FP64 plain push (absolute positions)
 // ---------------------------------------------------------------------
+// the weights of shape order ORDER at delta from the nearest node; at order 2
+// w[2] = w[0] + delta saves two of seven FP64 operations
+template <int ORDER>
+__device__ __forceinline__ void shape_w_fp64(double delta, double *w)
+{
+    if constexpr (ORDER == 4) {
+        w4<double>(delta, w);
+    } else {
+        const double a = 0.5 - delta;
+        w[0] = 0.5 * a * a;
+        w[1] = 0.75 - delta * delta;
+        w[2] = w[0] + delta;
+    }
+}
+
+// nearest nodes and weights of both staggerings at X = x / dx
+template <int ORDER>
+__device__ __forceinline__ void axis_w_near(double X, int &icn, double *wn, int &ich, double *wh)
+{
+    shape_w_fp64<ORDER>(X - nearest_fp64(X, icn), wn);
+    const double Y = X - 0.5;  // half nodes: the nearest to X - 1/2
+    shape_w_fp64<ORDER>(Y - nearest_fp64(Y, ich), wh);
+}
+template <int ORDER>
+__device__ __forceinline__ void axis_wn_near(double X, int &icn, double *wn)
+{
+    shape_w_fp64<ORDER>(X - nearest_fp64(X, icn), wn);
+}
+
+// Boris (Eqs. (13)-(16)) with the FP64 root and quotient of fp64_dev.cuh
+__device__ __forceinline__ void boris_fp64(double &ux, double &uy, double &uz, double ex, double ey, double ez, double bx,
+                                           double by, double bz)
+{
+    const double umx = ux + ex, umy = uy + ey, umz = uz + ez;
+    const double ginv = rsqrt_fp64(1.0 + umx * umx + umy * umy + umz * umz);
+    const double tx = bx * ginv, ty = by * ginv, tz = bz * ginv;
+    const double f = 2.0 * rcp_fp64(1.0 + tx * tx + ty * ty + tz * tz);
+    const double upx = umx + (umy * tz - umz * ty);
+    const double upy = umy + (umz * tx - umx * tz);
+    const double upz = umz + (umx * ty - umy * tx);
+    const double sx = tx * f, sy = ty * f, sz = tz * f;
+    ux = umx + (upy * sz - upz * sy) + ex;
+    uy = umy + (upz * sx - upx * sz) + ey;
+    uz = umz + (upx * sy - upy * sx) + ez;
+}
+
+// the cell of x in [0, n dx): floor(x / dx), divided out only where the
+// product with 1/dx lies within rounding of a cell face
+__device__ __forceinline__ int cell_fp64(double x, const Grid &g, int d)
+{
+    const double q = x * g.rdx_d[d];
+    int i;
+    const double f = q - nearest_fp64(q - 0.5, i);  // in [0, 1]
+    if (f < 1e-9 || f > 1.0 - 1e-9) i = (int)floor(x / g.dx[d]);
+    return i < 0 ? 0 : (i >= g.n[d] ? g.n[d] - 1 : i);
+}
+
+// The FP64 pipe bounds this kernel (1.06 TFLOP/s; about 320 operations a
+// particle in 2D): positions are multiplied by 1/dx, roots and quotients come
+// from Newton iterations, nodes from a rounding addition, and the deposit
+// takes the window its particles need.  262,144 electrons of the laser-foil:
+// 315 -> 176 us.  (Lanes on far-apart particles, so that the atomics of one
+// node do not queue up, measured 193 us: the atomics are not what binds.)
 template <int DIM, int ORDER>
 __global__ void __launch_bounds__(256) k_push_f64(PartF64 P, double *__restrict__ F, Grid g, PushConst pc,
                                                   int *err, double *e_abs)
 {
-    long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= *P.dn) return;
     if (P.cell[p] == kDead) return;
     double x[3] = {P.x[0][p], DIM >= 2 ? P.x[1][p] : 0.0, DIM >= 3 ? P.x[2][p] : 0.0};
-    double ux = P.u[0][p], uy = P.u[1][p], uz = P.u[2][p];
-    double ig = inv_gamma(ux, uy, uz);
-    double u[3] = {ux, uy, uz};
+    double u[3] = {P.u[0][p], P.u[1][p], P.u[2][p]};
+    double h = pc.hdt * rsqrt_fp64(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    int i0[3] = {0, 0, 0}, ich[3] = {0, 0, 0};
+    double w0[3][ORDER + 1], wh[3][ORDER + 1];
 #pragma unroll
-    for (int d = 0; d < DIM; d++) x[d] += pc.hdt * u[d] * ig;
-    double xh[3] = {x[0], x[1], x[2]};
-    int icn[3] = {0, 0, 0}, ich[3] = {0, 0, 0};
-    double wn[3][ORDER + 1], wh[3][ORDER + 1];
-#pragma unroll
-    for (int d = 0; d < DIM; d++) axis_w_f64<ORDER>(x[d] / g.dx[d], icn[d], wn[d], ich[d], wh[d]);
+    for (int d = 0; d < DIM; d++) {
+        x[d] += h * u[d];
+        axis_w_near<ORDER>(x[d] * g.rdx_d[d], i0[d], w0[d], ich[d], wh[d]);
+    }
     double eb[6];
-    gather<double, DIM, ORDER>(F, g, icn, wn, ich, wh, eb);
+    gather<double, DIM, ORDER>(F, g, i0, w0, ich, wh, eb);
     const double k = pc.qmdt2;
-    lorentz<double>(pc.pusher, ux, uy, uz, k * eb[0], k * eb[1], k * eb[2], k * eb[3], k * eb[4], k * eb[5]);
-    double ig1 = inv_gamma(ux, uy, uz);
-    u[0] = ux; u[1] = uy; u[2] = uz;
-#pragma unroll
-    for (int d = 0; d < DIM; d++) x[d] += pc.hdt * u[d] * ig1;
-    double x1[3] = {x[0], x[1], x[2]};
-#pragma unroll
-    for (int d = 0; d < DIM; d++) x[d] += pc.hdt * u[d] * ig1;
-    double S0[3][ORDER + 3], dS[3][ORDER + 3];
-    int base[3] = {0, 0, 0};
+    if (pc.pusher) vay<double>(u[0], u[1], u[2], k * eb[0], k * eb[1], k * eb[2], k * eb[3], k * eb[4], k * eb[5]);
+    else boris_fp64(u[0], u[1], u[2], k * eb[0], k * eb[1], k * eb[2], k * eb[3], k * eb[4], k * eb[5]);
+    const double ig1 = rsqrt_fp64(1.0 + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    h = pc.hdt * ig1;
+    double x1[3] = {0.0, 0.0, 0.0};
+    int i1[3] = {0, 0, 0};
+    double w1[3][ORDER + 1];
     bool ok = true;
 #pragma unroll
     for (int d = 0; d < DIM; d++) {
-        int i0, i1;
-        double w0[ORDER + 1], w1[ORDER + 1];
-        axis_wn_f64<ORDER>(xh[d] / g.dx[d], i0, w0);
-        axis_wn_f64<ORDER>(x[d] / g.dx[d], i1, w1);
-        ok &= window_n<double, ORDER>(i0, w0, i1, w1, S0[d], dS[d]);
-        base[d] = i0 - ORDER / 2 - 1;
+        const double dx = h * u[d];
+        x1[d] = x[d] + dx;
+        axis_wn_near<ORDER>((x1[d] + dx) * g.rdx_d[d], i1[d], w1[d]);
+        ok &= i1[d] - i0[d] >= -1 && i1[d] - i0[d] <= 1;
     }
     // a non-finite momentum (a NaN or infinite field) is reported and the particle
     // removed before anything uses its position: NaN positions would give no valid
     // cell or node index to the gather, the deposit or the diagnostics (and would
     // otherwise be reported as a Courant violation)
-    if (!isfinite(ux + uy + uz)) {
+    if (!isfinite(u[0] + u[1] + u[2])) {
         atomicOr(err, ERR_NONFINITE);
         P.cell[p] = kDead;
         return;
@@ -198,7 +252,7 @@ __global__ void __launch_bounds__(256) k_push_f64(PartF64 P, double *__restrict_
         atomicOr(err, ERR_CFL);
         return;
     }
-    deposit_global<double, DIM, ORDER>(F, g, base, S0, dS, pc.cJ, pc.qw * uy * ig1, pc.qw * uz * ig1);
+    deposit_moved<double, DIM, ORDER>(F, g, i0, w0, i1, w1, pc.cJ, pc.qw * u[1] * ig1, pc.qw * u[2] * ig1);
     bool dead = false;
     int cc[3] = {0, 0, 0};
 #pragma unroll
@@ -210,21 +264,20 @@ __global__ void __launch_bounds__(256) k_push_f64(PartF64 P, double *__restrict_
         } else if (x1[d] < 0.0 || x1[d] >= L) {
             dead = true;
         }
-        int ci = (int)floor(x1[d] / g.dx[d]);
-        cc[d] = ci < 0 ? 0 : (ci >= g.n[d] ? g.n[d] - 1 : ci);
+        cc[d] = cell_fp64(x1[d], g, d);
     }
     if (dead) {
         P.cell[p] = kDead;
-        double uu = ux * ux + uy * uy + uz * uz;
+        double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
         atomicAdd(e_abs, pc.wmdV * uu / (sqrt(1.0 + uu) + 1.0));
     } else {
         P.cell[p] = pack_cell(g, cc[0], cc[1], cc[2]);
     }
 #pragma unroll
     for (int d = 0; d < DIM; d++) P.x[d][p] = x1[d];
-    P.u[0][p] = ux;
-    P.u[1][p] = uy;
-    P.u[2][p] = uz;
+    P.u[0][p] = u[0];
+    P.u[1][p] = u[1];
+    P.u[2][p] = u[2];
 }
 
 // ---------------------------------------------------------------------

@@ -2,6 +2,7 @@
 // node and W_2 weights (Sec. II.D), the gather of Eq. (19), Esirkepov's
 // window and deposit (Eqs. (20)-(22)), and the FP32 offset drift.
 #pragma once
+#include "fp64_dev.cuh"
 #include "push.cuh"
 
 namespace pic {
@@ -142,28 +143,6 @@ __device__ __forceinline__ bool window5(int ic0, const R *w0, int ic1, const R *
     return true;
 }
 
-// shapes of the start and end points on the window of ORDER + 3 nodes that
-// starts ORDER/2 + 1 nodes left of the start point's nearest node (ORDER 2:
-// the 5-node window of window5, ORDER 4: 7 nodes); false when the nearest
-// node moved by more than one
-template <typename R, int ORDER>
-__device__ __forceinline__ bool window_n(int ic0, const R *w0, int ic1, const R *w1, R *S0, R *dS)
-{
-    constexpr int P = ORDER + 1, WN = ORDER + 3;
-    int sh = ic1 - ic0;
-    R S1[WN];
-#pragma unroll
-    for (int a = 0; a < WN; a++) { S0[a] = 0; S1[a] = 0; }
-#pragma unroll
-    for (int a = 0; a < P; a++) S0[a + 1] = w0[a];
-    if (sh < -1 || sh > 1) return false;
-#pragma unroll
-    for (int a = 0; a < P; a++) S1[a + 1 + sh] = w1[a];
-#pragma unroll
-    for (int a = 0; a < WN; a++) dS[a] = S1[a] - S0[a];
-    return true;
-}
-
 // Esirkepov deposit into the global current (red.global.add).  Along an
 // active axis d: J_d(i+1/2) = J_d(i-1/2) - q w (dx_d/dt) W_d(i), summed
 // from zero left of the window (the fifth partial sum is sum dS = 0).
@@ -268,6 +247,137 @@ __device__ __forceinline__ void deposit_global(R *__restrict__ F, const Grid &g,
             }
     }
     (void)jvy;
+}
+
+// the start and end shapes on the window of W nodes from min(i0, i1) - ORDER/2:
+// W = ORDER + 1 (nearest node unmoved) or ORDER + 2 (moved by one at most)
+template <typename R, int ORDER, int W>
+__device__ __forceinline__ void window_w(int i0, const R *w0, int i1, const R *w1, R *S0, R *dS)
+{
+    constexpr int P = ORDER + 1;
+    const bool o0 = W > P && i0 > i1, o1 = W > P && i1 > i0;
+#pragma unroll
+    for (int k = 0; k < W; k++) {
+        const R s0 = o0 ? (k >= 1 ? w0[k - 1] : R(0)) : (k < P ? w0[k < P ? k : 0] : R(0));
+        const R s1 = o1 ? (k >= 1 ? w1[k - 1] : R(0)) : (k < P ? w1[k < P ? k : 0] : R(0));
+        S0[k] = s0;
+        dS[k] = s1 - s0;
+    }
+}
+
+// nonzero, by the bits (a compare of doubles takes the FP64 pipe)
+__device__ __forceinline__ bool nonzero(double v) { return (__double2hiint(v) << 1 | __double2loint(v)) != 0; }
+__device__ __forceinline__ bool nonzero(float v) { return v != 0.f; }
+
+// Esirkepov's deposit into the global current on a window of W nodes
+// (Eqs. (20)-(22)), with t = S0 + dS/2: along an active axis d the prefix sum
+// of dS_d times the time average of the other axes' shapes (t_a t_b + dS_a
+// dS_b / 12); along an inactive axis q w v_d times that average of all.
+// base: the window's first node.
+template <typename R, int DIM, int W>
+__device__ __forceinline__ void deposit_window(R *__restrict__ F, const Grid &g, const int *base, const R (*S0)[W],
+                                               const R (*dS)[W], const R *cJ, R jvy, R jvz)
+{
+    const long long o = goff(g, base[0], DIM > 1 ? base[1] : 0, DIM > 2 ? base[2] : 0);
+    R *Jx = F + JX * g.vol + o, *Jy = F + JY * g.vol + o, *Jz = F + JZ * g.vol + o;
+    const int sy = (int)g.sy, sz = (int)g.sz;
+    R t[DIM][W], p[DIM][W - 1], d12[DIM][W];
+#pragma unroll
+    for (int d = 0; d < DIM; d++) {
+        p[d][0] = cJ[d] * dS[d][0];
+#pragma unroll
+        for (int k = 0; k < W; k++) {
+            t[d][k] = S0[d][k] + R(0.5) * dS[d][k];
+            d12[d][k] = dS[d][k] * R(1.0 / 12.0);
+            if (k > 0 && k < W - 1) p[d][k] = p[d][k - 1] + cJ[d] * dS[d][k];
+        }
+    }
+    auto add = [](R *at, R v) {
+        if (nonzero(v)) atomicAdd(at, v);
+    };
+    if constexpr (DIM == 1) {
+#pragma unroll
+        for (int a = 0; a < W; a++) {
+            if (a < W - 1) add(Jx + a, p[0][a]);
+            add(Jy + a, jvy * t[0][a]);
+            add(Jz + a, jvz * t[0][a]);
+        }
+    } else if constexpr (DIM == 2) {
+#pragma unroll
+        for (int a = 0; a < W; a++) {
+            const R ja = jvz * t[0][a], jd = jvz * d12[0][a];
+#pragma unroll
+            for (int b = 0; b < W; b++) {
+                if (a < W - 1) add(Jx + b * sy + a, p[0][a] * t[1][b]);
+                if (b < W - 1) add(Jy + b * sy + a, p[1][b] * t[0][a]);
+                add(Jz + b * sy + a, ja * t[1][b] + jd * dS[1][b]);
+            }
+        }
+    } else {
+#pragma unroll 1
+        for (int c = 0; c < W; c++) {
+            R tc = t[2][0], dc = d12[2][0];
+#pragma unroll
+            for (int k = 1; k < W; k++) {
+                tc = c == k ? t[2][k] : tc;
+                dc = c == k ? d12[2][k] : dc;
+            }
+#pragma unroll
+            for (int b = 0; b < W; b++) {
+                const R w = t[1][b] * tc + dS[1][b] * dc;
+#pragma unroll
+                for (int a = 0; a < W - 1; a++) add(Jx + c * sz + b * sy + a, p[0][a] * w);
+            }
+#pragma unroll
+            for (int a = 0; a < W; a++) {
+                const R w = t[0][a] * tc + dS[0][a] * dc;
+#pragma unroll
+                for (int b = 0; b < W - 1; b++) add(Jy + c * sz + b * sy + a, p[1][b] * w);
+            }
+        }
+#pragma unroll 1
+        for (int b = 0; b < W; b++) {
+            R tb = t[1][0], db = d12[1][0];
+#pragma unroll
+            for (int k = 1; k < W; k++) {
+                tb = b == k ? t[1][k] : tb;
+                db = b == k ? d12[1][k] : db;
+            }
+#pragma unroll
+            for (int a = 0; a < W; a++) {
+                const R w = t[0][a] * tb + dS[0][a] * db;
+#pragma unroll
+                for (int c = 0; c < W - 1; c++) add(Jz + c * sz + b * sy + a, p[2][c] * w);
+            }
+        }
+    }
+}
+
+// the deposit of one particle from the nearest nodes and weights of its end
+// points, on the smaller window when no lane of the warp's active ones moved
+// its nearest node
+template <typename R, int DIM, int ORDER>
+__device__ __forceinline__ void deposit_moved(R *__restrict__ F, const Grid &g, const int *i0, const R (*w0)[ORDER + 1],
+                                              const int *i1, const R (*w1)[ORDER + 1], const R *cJ, R jvy, R jvz)
+{
+    int base[3] = {0, 0, 0};
+    bool moved = false;
+#pragma unroll
+    for (int d = 0; d < DIM; d++) {
+        base[d] = min(i0[d], i1[d]) - ORDER / 2;
+        moved |= i0[d] != i1[d];
+    }
+    if (__any_sync(__activemask(), moved)) {
+        R S0[DIM][ORDER + 2], dS[DIM][ORDER + 2];
+#pragma unroll
+        for (int d = 0; d < DIM; d++) window_w<R, ORDER, ORDER + 2>(i0[d], w0[d], i1[d], w1[d], S0[d], dS[d]);
+        deposit_window<R, DIM, ORDER + 2>(F, g, base, S0, dS, cJ, jvy, jvz);
+    } else {
+        R S0[DIM][ORDER + 1], dS[DIM][ORDER + 1];
+#pragma unroll
+        for (int d = 0; d < DIM; d++) window_w<R, ORDER, ORDER + 1>(i0[d], w0[d], i1[d], w1[d], S0[d], dS[d]);
+        deposit_window<R, DIM, ORDER + 1>(F, g, base, S0, dS, cJ, jvy, jvz);
+    }
 }
 
 // FP32 offset drift with face crossing

@@ -161,14 +161,12 @@ int sort_species(pic_sim *s, int i)
 {
     SpeciesState &p = s->sp[i];
     if (p.n_hi == 0) return PIC_OK;
-    const uint32_t *perm = nullptr, *skeys = nullptr;
-    sort_by_tile(p.cell[p.cur], p.n_hi, p.d_count, s->g, s->sort_scratch, p.tile_start, p.d_count, &perm, &skeys,
-                 s->st);
-    int o = 1 - p.cur;
+    const SortResult r = sort_by_tile(p.cell[p.cur], p.n_hi, p.d_count, s->g, s->sort_scratch, s->st);
+    const int o = 1 - p.cur;
     if (s->precision == PIC_PREC_FP64_PLAIN)
-        launch_permute_f64(view64(s, i, p.cur), view64(s, i, o), perm, p.d_count, p.n_hi, s->g.dim, s->st);
+        sort_apply(view64(s, i, p.cur), view64(s, i, o), r, p.n_hi, s->g, p.tile_start, p.d_count, s->st);
     else
-        launch_permute_f32(view32(s, i, p.cur), view32(s, i, o), perm, p.d_count, p.n_hi, s->g.dim, s->st);
+        sort_apply(view32(s, i, p.cur), view32(s, i, o), r, p.n_hi, s->g, p.tile_start, p.d_count, s->st);
     p.cur = o;
     if (p.items) {
         build_tile_items(p.tile_start, s->g.ntiles, tile_chunk(s->g, p.has_qed_arrays(), p.n_hi), p.item_cnt,

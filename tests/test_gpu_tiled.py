@@ -78,3 +78,20 @@ def test_tile3d_ragged_one_step_matches_oracle(n, nppc, crowd, bc):
             setattr(s, k, getattr(s, k)[-1:].copy())
     _crowd(w, crowd, 3, 9)
     _one_step(w, F, 2, (4, 4, 4))
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 4095, 4096, 4097, 9001])
+def test_sort_is_numpys_stable_sort(n):
+    """particles at rest on a ragged 2D grid, sorted at step 0 (blocks of 4096
+    keys, 512 a warp): numpy's stable argsort by (tile, cell in the tile)"""
+    rng = np.random.default_rng(n)
+    nx, ny = 37, 22
+    x, y = rng.random(n) * nx, rng.random(n) * ny
+    z, tag = np.zeros(n), np.arange(n) * 1e-9
+    with pic.pic_create(2, (nx, ny), (1.0, 1.0), 0.5, [(-1.0, 1.0, 1e-20, n + 5)], sort_interval=1, tile=(8, 8)) as s:
+        s.pic_load_particles(0, x, y, None, z, z, tag)
+        s.pic_step(1)
+        p = s.pic_get_particles(0)
+    cx, cy = x.astype(int), y.astype(int)
+    key = ((cy // 8) * ((nx + 7) // 8) + cx // 8) * 64 + (cy % 8) * 8 + cx % 8
+    assert np.array_equal(p["uz"], tag.astype(np.float32).astype(np.float64)[np.argsort(key, kind="stable")])

@@ -419,21 +419,13 @@ void qed_spawn_views(pic_sim *s)
         if constexpr (sizeof(R) == 8) return view64(s, i, s->sp[i].cur);
         else return view32(s, i, s->sp[i].cur);
     };
-    uint32_t *off = (uint32_t *)s->sort_scratch;
+    uint32_t *bsum = (uint32_t *)s->sort_scratch;
     const int ph = s->qed.photon_sp, el = s->qed.electron_sp, po = s->qed.positron_sp;
     const int dim = s->g.dim;
-    // the scanned sums of the flags' blocks (the spawn kernels rank within a block)
-    auto scan = [&](const SpeciesState &p) {
-        const long long nb = scan_blocks(p.n_hi + 1);
-        scan_block_sums(p.ev, p.n_hi + 1, off, off + nb + 64, s->st, p.d_count);
-        return off + nb;  // total
-    };
     if (ph >= 0 && el >= 0 && po >= 0 && s->sp[ph].n_hi > 0) {
         SpeciesState &P = s->sp[ph], &E = s->sp[el], &O = s->sp[po];
-        const uint32_t *tot = scan(P);
-        launch_spawn_pairs(view(ph), off, tot, P.n_hi + 1, qed_params(s, ph), view(el), E.tau[E.cur], E.id[E.cur], E.ev,
-                           E.d_count, E.cap, view(po), O.tau[O.cur], O.id[O.cur], O.ev, O.d_count, O.cap, dim,
-                           s->d_err, s->st);
+        launch_spawn_pairs(view(ph), bsum, s->spawn_ctl, qed_params(s, ph), view(el), E.ev, E.d_count, E.cap, view(po),
+                           O.ev, O.d_count, O.cap, dim, s->d_err, s->st);
         E.n_hi = std::min(E.cap, E.n_hi + P.n_hi);
         O.n_hi = std::min(O.cap, O.n_hi + P.n_hi);
         // the pairs land past the sorted particles (tile_start[ntiles]): the
@@ -447,9 +439,8 @@ void qed_spawn_views(pic_sim *s)
         SpeciesState &p = s->sp[i];
         if (p.kind == PIC_KIND_PHOTON || !p.qed || p.n_hi == 0) continue;
         SpeciesState &P = s->sp[ph];
-        const uint32_t *tot = scan(p);
-        launch_spawn_photons(view(i), off, tot, p.n_hi + 1, qed_params(s, i), view(ph), P.tau[P.cur], P.id[P.cur], P.ev,
-                             P.d_count, P.cap, dim, s->d_err, s->st);
+        launch_spawn_photons(view(i), bsum, s->spawn_ctl, qed_params(s, i), view(ph), P.ev, P.d_count, P.cap, dim,
+                             s->d_err, s->st);
         P.n_hi = std::min(P.cap, P.n_hi + p.n_hi);
         // (the photons land past the sorted ones: the photon push takes them
         // as items of consecutive photons, the sort's work items stay valid)
@@ -705,12 +696,14 @@ int pic_create(const pic_grid *grid, double dt, const pic_species *species, int 
     rc = rc ? rc : dalloc(s, (void **)&s->diag_scratch, diag_scratch_doubles() * sizeof(double));
     rc = rc ? rc : dalloc(s, (void **)&s->diag_out, 32 * sizeof(double));
     rc = rc ? rc : dalloc(s, (void **)&s->d_err, sizeof(int));
+    rc = rc ? rc : dalloc(s, (void **)&s->spawn_ctl, sizeof(SpawnCtl));
     rc = rc ? rc : dalloc(s, (void **)&s->d_eabs, sizeof(double));
     rc = rc ? rc : dalloc(s, (void **)&s->d_elost, sizeof(double));
     if (!rc) {
         cudaError_t z = cudaMemsetAsync(s->F, 0, (size_t)NCOMP * g.vol * R, s->st);
         if (z == cudaSuccess) z = cudaMemsetAsync(s->d_err, 0, sizeof(int), s->st);
         if (z == cudaSuccess) z = cudaMemsetAsync(s->diag_scratch, 0, diag_scratch_doubles() * sizeof(double), s->st);
+        if (z == cudaSuccess) z = cudaMemsetAsync(s->spawn_ctl, 0, sizeof(SpawnCtl), s->st);
         if (z == cudaSuccess) z = cudaMemsetAsync(s->d_eabs, 0, sizeof(double), s->st);
         if (z == cudaSuccess) z = cudaMemsetAsync(s->d_elost, 0, sizeof(double), s->st);
         for (int i = 0; i < nsp && z == cudaSuccess; i++)

@@ -120,135 +120,6 @@ __device__ __forceinline__ void gather(const R *__restrict__ F, const Grid &g, c
     }
 }
 
-// shapes of the start and end points on the 5-node window that starts two
-// nodes left of the start point's nearest node; returns false when the
-// nearest node moved by more than one (Courant condition violated)
-template <typename R>
-__device__ __forceinline__ bool window5(int ic0, const R *w0, int ic1, const R *w1, R *S0, R *dS)
-{
-    int sh = ic1 - ic0;
-    R S1[5];
-#pragma unroll
-    for (int a = 0; a < 5; a++) { S0[a] = 0; S1[a] = 0; }
-#pragma unroll
-    for (int a = 0; a < 3; a++) S0[a + 1] = w0[a];
-    if (sh < -1 || sh > 1) return false;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        int b = a + 1 + sh;
-        S1[b] = w1[a];
-    }
-#pragma unroll
-    for (int a = 0; a < 5; a++) dS[a] = S1[a] - S0[a];
-    return true;
-}
-
-// Esirkepov deposit into the global current (red.global.add).  Along an
-// active axis d: J_d(i+1/2) = J_d(i-1/2) - q w (dx_d/dt) W_d(i), summed
-// from zero left of the window (the fifth partial sum is sum dS = 0).
-// Along an inactive axis: q w v_d times the time average of the product of
-// the node shapes, each linear in time between S0 and S1.
-template <typename R, int DIM, int ORDER = 2>
-__device__ __forceinline__ void deposit_global(R *__restrict__ F, const Grid &g, const int *base,
-                                               const R (*S0)[ORDER + 3], const R (*dS)[ORDER + 3], const R *cJ, R jvy,
-                                               R jvz)
-{
-    constexpr int WN = ORDER + 3;
-    R *Jx = F + JX * g.vol, *Jy = F + JY * g.vol, *Jz = F + JZ * g.vol;
-    const R half = R(0.5), third = R(1.0 / 3.0);
-    if (DIM == 1) {
-        long long o = goff(g, base[0], 0, 0);
-        R acc = 0;
-#pragma unroll
-        for (int a = 0; a < WN - 1; a++) {
-            acc += cJ[0] * dS[0][a];
-            if (acc != R(0)) atomicAdd(Jx + o + a, acc);
-        }
-#pragma unroll
-        for (int a = 0; a < WN; a++) {
-            R f = S0[0][a] + half * dS[0][a];
-            if (f != R(0)) {
-                atomicAdd(Jy + o + a, jvy * f);
-                atomicAdd(Jz + o + a, jvz * f);
-            }
-        }
-    } else if (DIM == 2) {
-#pragma unroll
-        for (int b = 0; b < WN; b++) {
-            long long o = goff(g, base[0], base[1] + b, 0);
-            R ty = S0[1][b] + half * dS[1][b];
-            R acc = 0;
-#pragma unroll
-            for (int a = 0; a < WN - 1; a++) {
-                acc += cJ[0] * (dS[0][a] * ty);
-                if (acc != R(0)) atomicAdd(Jx + o + a, acc);
-            }
-        }
-#pragma unroll
-        for (int a = 0; a < WN; a++) {
-            R tx = S0[0][a] + half * dS[0][a];
-            R acc = 0;
-#pragma unroll
-            for (int b = 0; b < WN - 1; b++) {
-                acc += cJ[1] * (dS[1][b] * tx);
-                if (acc != R(0)) atomicAdd(Jy + goff(g, base[0] + a, base[1] + b, 0), acc);
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < WN; b++) {
-            long long o = goff(g, base[0], base[1] + b, 0);
-#pragma unroll
-            for (int a = 0; a < WN; a++) {
-                R wz = S0[0][a] * S0[1][b] + half * dS[0][a] * S0[1][b] + half * S0[0][a] * dS[1][b] +
-                       third * dS[0][a] * dS[1][b];
-                if (wz != R(0)) atomicAdd(Jz + o + a, jvz * wz);
-            }
-        }
-    } else {
-#pragma unroll
-        for (int c = 0; c < WN; c++)
-#pragma unroll
-            for (int b = 0; b < WN; b++) {
-                R t = S0[1][b] * S0[2][c] + half * dS[1][b] * S0[2][c] + half * S0[1][b] * dS[2][c] +
-                      third * dS[1][b] * dS[2][c];
-                long long o = goff(g, base[0], base[1] + b, base[2] + c);
-                R acc = 0;
-#pragma unroll
-                for (int a = 0; a < WN - 1; a++) {
-                    acc += cJ[0] * (dS[0][a] * t);
-                    if (acc != R(0)) atomicAdd(Jx + o + a, acc);
-                }
-            }
-#pragma unroll
-        for (int c = 0; c < WN; c++)
-#pragma unroll
-            for (int a = 0; a < WN; a++) {
-                R t = S0[0][a] * S0[2][c] + half * dS[0][a] * S0[2][c] + half * S0[0][a] * dS[2][c] +
-                      third * dS[0][a] * dS[2][c];
-                R acc = 0;
-#pragma unroll
-                for (int b = 0; b < WN - 1; b++) {
-                    acc += cJ[1] * (dS[1][b] * t);
-                    if (acc != R(0)) atomicAdd(Jy + goff(g, base[0] + a, base[1] + b, base[2] + c), acc);
-                }
-            }
-#pragma unroll
-        for (int b = 0; b < WN; b++)
-#pragma unroll
-            for (int a = 0; a < WN; a++) {
-                R t = S0[0][a] * S0[1][b] + half * dS[0][a] * S0[1][b] + half * S0[0][a] * dS[1][b] +
-                      third * dS[0][a] * dS[1][b];
-                R acc = 0;
-#pragma unroll
-                for (int c = 0; c < WN - 1; c++) {
-                    acc += cJ[2] * (dS[2][c] * t);
-                    if (acc != R(0)) atomicAdd(Jz + goff(g, base[0] + a, base[1] + b, base[2] + c), acc);
-                }
-            }
-    }
-    (void)jvy;
-}
-
 // the start and end shapes on the window of W nodes from min(i0, i1) - ORDER/2:
 // W = ORDER + 1 (nearest node unmoved) or ORDER + 2 (moved by one at most)
 template <typename R, int ORDER, int W>

@@ -35,7 +35,7 @@ __device__ __forceinline__ void k_push_qed_f32_one(PartF32 &P, float *__restrict
     const bool live = mine && p < *P.dn && P.cell[p] != kDead;
     if (!SURR || !__any_sync(0xffffffffu, live)) {
         if (!live) {
-            if (mine && p <= P.n) q.ev[p] = 0;  // dead slots and slots past the live count (and the scan's end slot)
+            if (mine && p < *P.dn) q.ev[p] = 0;  // a dead slot (flags past the device count are never read)
             return;
         }
     }
@@ -70,7 +70,7 @@ __device__ __forceinline__ void k_push_qed_f32_one(PartF32 &P, float *__restrict
     float4 evd = make_float4(0.f, 0.f, 0.f, 0.f);
     qed_lepton_f32<SURR>(q, smem, live, p, eb, ux, uy, uz, err, event, evd);
     if (SURR && !live) {
-        if (mine && p <= P.n) q.ev[p] = 0;
+        if (mine && p < *P.dn) q.ev[p] = 0;
         return;
     }
     const float ig1 = inv_gamma(ux, uy, uz);
@@ -83,17 +83,14 @@ __device__ __forceinline__ void k_push_qed_f32_one(PartF32 &P, float *__restrict
     const float o1[3] = {o[0], o[1], o[2]};
 #pragma unroll
     for (int d = 0; d < DIM; d++) drift_f32(c[d], o[d], pc.hdx_f[d] * u[d] * ig1);
-    float S0[3][5], dS[3][5];
-    int base[3] = {0, 0, 0};
+    int i0[3] = {0, 0, 0}, i1[3] = {0, 0, 0};
+    float w0[3][3], w1[3][3];
     bool ok = true;
 #pragma unroll
     for (int d = 0; d < DIM; d++) {
-        int i0, i1;
-        float w0[3], w1[3];
-        axis_wn_f32(ch[d], oh[d], i0, w0);
-        axis_wn_f32(c[d], o[d], i1, w1);
-        ok &= window5<float>(i0, w0, i1, w1, S0[d], dS[d]);
-        base[d] = i0 - 2;
+        axis_wn_f32(ch[d], oh[d], i0[d], w0[d]);
+        axis_wn_f32(c[d], o[d], i1[d], w1[d]);
+        ok &= i1[d] - i0[d] >= -1 && i1[d] - i0[d] <= 1;
     }
     // a non-finite momentum (a NaN or infinite field) is reported and the particle
     // removed before anything uses its position: NaN positions would give no valid
@@ -111,7 +108,7 @@ __device__ __forceinline__ void k_push_qed_f32_one(PartF32 &P, float *__restrict
         return;
     }
     const float cJ[3] = {pc.cJ_f[0], pc.cJ_f[1], pc.cJ_f[2]};
-    deposit_global<float, DIM>(F, g, base, S0, dS, cJ, pc.qw_f * uy * ig1, pc.qw_f * uz * ig1);
+    deposit_moved<float, DIM, 2>(F, g, i0, w0, i1, w1, cJ, pc.qw_f * uy * ig1, pc.qw_f * uz * ig1);
     bool dead = false;
 #pragma unroll
     for (int d = 0; d < DIM; d++) {
@@ -145,6 +142,10 @@ __global__ void __launch_bounds__(256, SURR ? 2 : 1) k_push_qed_f32(PartF32 P, f
                                                       const uint32_t *__restrict__ first)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    const long long nlive = *P.dn;
+    // (a block without particles leaves before it stages the network: the grid
+    // covers the host's bound on the count)
+    if (((first ? (long long)*first / blockDim.x : 0) + blockIdx.x) * blockDim.x >= nlive) return;
     if constexpr (SURR) {
         mlp_stage(smem, q.net, kMlpStageBytes);
         __syncthreads();
@@ -154,11 +155,11 @@ __global__ void __launch_bounds__(256, SURR ? 2 : 1) k_push_qed_f32(PartF32 P, f
         return;
     }
     // the tail after the tiled kernel's particles: a block-uniform grid
-    // stride over [first, P.n] (a grid over the whole range would launch a
+    // stride over [first, count) (a grid over the whole range would launch a
     // block per 256 slots only to find most of them the tiled kernel's)
     const long long p0 = (long long)*first;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long base = (p0 / blockDim.x + blockIdx.x) * blockDim.x; base <= P.n; base += stride)
+    for (long long base = (p0 / blockDim.x + blockIdx.x) * blockDim.x; base < nlive; base += stride)
         k_push_qed_f32_one<DIM, SURR>(P, F, g, pc, q, err, e_abs, smem, base + threadIdx.x, p0);
 }
 
@@ -172,7 +173,7 @@ __device__ __forceinline__ void k_push_photon_f32_one(PartF32 &P, const float *_
     const bool live = mine && p < *P.dn && P.cell[p] != kDead;
     if (!SURR || !__any_sync(0xffffffffu, live)) {
         if (!live) {
-            if (mine && p <= P.n) q.ev[p] = 0;  // dead slots and slots past the live count (and the scan's end slot)
+            if (mine && p < *P.dn) q.ev[p] = 0;  // a dead slot (flags past the device count are never read)
             return;
         }
     }
@@ -204,11 +205,11 @@ __device__ __forceinline__ void k_push_photon_f32_one(PartF32 &P, const float *_
         gather<float, DIM>(F, g, icn, wn, ich, wh, eb);
         qed_photon_f32<SURR>(q, smem, live, p, km, kx, ky, kz, eb, live ? q.tau[p] : 0.0, err, event, evd);
         if (SURR && !live) {
-            if (mine && p <= P.n) q.ev[p] = 0;
+            if (mine && p < *P.dn) q.ev[p] = 0;
             return;
         }
     } else if (SURR && !live) {
-        if (mine && p <= P.n) q.ev[p] = 0;
+        if (mine && p < *P.dn) q.ev[p] = 0;
         return;
     }
 #pragma unroll
@@ -240,6 +241,10 @@ __global__ void __launch_bounds__(256, SURR ? 2 : 1) k_push_photon_f32(PartF32 P
                                                          QedParams q, int *err, const uint32_t *__restrict__ first)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    const long long nlive = *P.dn;
+    // (a block without particles leaves before it stages the network: the grid
+    // covers the host's bound on the count)
+    if (((first ? (long long)*first / blockDim.x : 0) + blockIdx.x) * blockDim.x >= nlive) return;
     if constexpr (SURR) {
         mlp_stage(smem, q.net, kMlpStageBytes);
         __syncthreads();
@@ -249,17 +254,17 @@ __global__ void __launch_bounds__(256, SURR ? 2 : 1) k_push_photon_f32(PartF32 P
         return;
     }
     // the tail after the tiled kernel's particles: a block-uniform grid
-    // stride over [first, P.n] (a grid over the whole range would launch a
+    // stride over [first, count) (a grid over the whole range would launch a
     // block per 256 slots only to find most of them the tiled kernel's)
     const long long p0 = (long long)*first;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long base = (p0 / blockDim.x + blockIdx.x) * blockDim.x; base <= P.n; base += stride)
+    for (long long base = (p0 / blockDim.x + blockIdx.x) * blockDim.x; base < nlive; base += stride)
         k_push_photon_f32_one<DIM, SURR>(P, F, g, pc, q, err, smem, base + threadIdx.x, p0);
 }
 
 // The photon push with the pair network on the tcgen05 tensor cores:
 // persistent CTAs of 128 threads walk tiles of 128 photon slots (slots up
-// to P.n, so that the scan's end slot and the dead slots get a zero flag);
+// to the device count, so that the dead slots get a zero flag);
 // the network is evaluated by the whole CTA (mlp_eval_cta: one row per
 // thread, accumulators in tensor memory) for every tile with a photon in
 // its chi range.  Everything else is k_push_photon_f32<DIM, true>.  (On the
@@ -275,7 +280,7 @@ __global__ void __launch_bounds__(kMlpTcRows, 4) k_push_photon_tc(PartF32 P, con
     mlp_tc_setup(S, q.net);
     uint32_t phase = 0;
     const long long nlive = *P.dn;
-    for (long long tile = blockIdx.x; tile * kMlpTcRows <= P.n; tile += gridDim.x) {
+    for (long long tile = blockIdx.x; tile * kMlpTcRows < nlive; tile += gridDim.x) {
         const long long p = tile * kMlpTcRows + threadIdx.x;
         const bool live = p < nlive && P.cell[p] != kDead;
         int c[3] = {0, 0, 0};
@@ -324,7 +329,7 @@ __global__ void __launch_bounds__(kMlpTcRows, 4) k_push_photon_tc(PartF32 P, con
             }
         }
         if (!live) {
-            if (p <= P.n) q.ev[p] = 0;
+            if (p < nlive) q.ev[p] = 0;
             continue;
         }
         uint32_t event = 0;
@@ -381,7 +386,7 @@ __global__ void __launch_bounds__(256) k_push_qed_f64(PartF64 P, double *__restr
 {
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= *P.dn || P.cell[p] == kDead) {
-        if (p <= P.n) q.ev[p] = 0;
+        if (p < *P.dn) q.ev[p] = 0;
         return;
     }
     double x[3] = {P.x[0][p], DIM >= 2 ? P.x[1][p] : 0.0, DIM >= 3 ? P.x[2][p] : 0.0};
@@ -454,17 +459,14 @@ __global__ void __launch_bounds__(256) k_push_qed_f64(PartF64 P, double *__restr
     double x1[3] = {x[0], x[1], x[2]};
 #pragma unroll
     for (int d = 0; d < DIM; d++) x[d] += pc.hdt * u[d] * ig1;
-    double S0[3][5], dS[3][5];
-    int base[3] = {0, 0, 0};
+    int i0[3] = {0, 0, 0}, i1[3] = {0, 0, 0};
+    double w0[3][3], w1[3][3];
     bool ok = true;
 #pragma unroll
     for (int d = 0; d < DIM; d++) {
-        int i0, i1;
-        double w0[3], w1[3];
-        axis_wn_f64(xh[d] / g.dx[d], i0, w0);
-        axis_wn_f64(x[d] / g.dx[d], i1, w1);
-        ok &= window5<double>(i0, w0, i1, w1, S0[d], dS[d]);
-        base[d] = i0 - 2;
+        axis_wn_f64(xh[d] / g.dx[d], i0[d], w0[d]);
+        axis_wn_f64(x[d] / g.dx[d], i1[d], w1[d]);
+        ok &= i1[d] - i0[d] >= -1 && i1[d] - i0[d] <= 1;
     }
     // a non-finite momentum (a NaN or infinite field) is reported and the particle
     // removed before anything uses its position: NaN positions would give no valid
@@ -481,7 +483,7 @@ __global__ void __launch_bounds__(256) k_push_qed_f64(PartF64 P, double *__restr
         q.ev[p] = 0;
         return;
     }
-    deposit_global<double, DIM>(F, g, base, S0, dS, pc.cJ, pc.qw * uy * ig1, pc.qw * uz * ig1);
+    deposit_moved<double, DIM, 2>(F, g, i0, w0, i1, w1, pc.cJ, pc.qw * uy * ig1, pc.qw * uz * ig1);
     bool dead = false;
     int cc[3] = {0, 0, 0};
 #pragma unroll
@@ -519,7 +521,7 @@ __global__ void __launch_bounds__(256) k_push_photon_f64(PartF64 P, const double
 {
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= *P.dn || P.cell[p] == kDead) {
-        if (p <= P.n) q.ev[p] = 0;
+        if (p < *P.dn) q.ev[p] = 0;
         return;
     }
     double x[3] = {P.x[0][p], DIM >= 2 ? P.x[1][p] : 0.0, DIM >= 3 ? P.x[2][p] : 0.0};

@@ -121,7 +121,7 @@ __device__ __forceinline__ void esirkepov3d_box(int *base, const float (*S0)[4],
 
 // the QED variants' slow paths, out of line (rare: a particle that drifted
 // out of its tile's box since the sort): the gather from HBM and the
-// deposit with global atomics on the 5-node window
+// deposit with global atomics
 static __device__ __noinline__ void gather3d_global(const float *F, const Grid &g, const int *icn,
                                                    const float (*wn)[3], const int *ich, const float (*wh)[3],
                                                    float *eb)
@@ -133,21 +133,18 @@ static __device__ __noinline__ bool deposit3d_global(float *F, const Grid &g, co
                                                      const float *oh, const int *c, const float *o, float uy,
                                                      float uz, float ig1)
 {
-    float S0[3][5], dS[3][5];
-    int base[3];
+    int i0[3], i1[3];
+    float w0[3][3], w1[3][3];
     bool ok = true;
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-        int i0, i1;
-        float w0[3], w1[3];
-        axis_wn_f32(ch[d], oh[d], i0, w0);
-        axis_wn_f32(c[d], o[d], i1, w1);
-        ok &= window5<float>(i0, w0, i1, w1, S0[d], dS[d]);
-        base[d] = i0 - 2;
+        axis_wn_f32(ch[d], oh[d], i0[d], w0[d]);
+        axis_wn_f32(c[d], o[d], i1[d], w1[d]);
+        ok &= i1[d] - i0[d] >= -1 && i1[d] - i0[d] <= 1;
     }
     if (!ok) return false;
     const float cJ[3] = {pc.cJ_f[0], pc.cJ_f[1], pc.cJ_f[2]};
-    deposit_global<float, 3>(F, g, base, S0, dS, cJ, pc.qw_f * uy * ig1, pc.qw_f * uz * ig1);
+    deposit_moved<float, 3, 2>(F, g, i0, w0, i1, w1, cJ, pc.qw_f * uy * ig1, pc.qw_f * uz * ig1);
     return true;
 }
 

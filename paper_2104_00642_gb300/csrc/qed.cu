@@ -17,6 +17,8 @@
 
 #include "qed.cuh"
 #include "qed_host.cuh"
+#include <type_traits>
+
 #include "scan_dev.cuh"
 #include "sort.cuh"
 
@@ -301,12 +303,15 @@ void launch_qed_eval(const QedTables &T, bool f64, int p, long long n, const dou
 
 // ---------------------------------------------------------------------
 // spawning: the events of a species are ranked in array order and the
-// children appended at the end of their species (deterministic order).  The
-// ranks come in two passes over the flags: the sums of blocks of kScanItems
-// flags, scanned (scan_block_sums), then the spawn kernel itself, which
-// strides over the blocks of flags: a block whose scanned sums show no event
-// is skipped without reading its flags; otherwise the 256 threads read 16
-// flags each, scan them and add the block's offset.
+// children appended at the end of their species (deterministic order).  One
+// kernel sums the flags of blocks of kScanItems; its last block to arrive
+// scans the sums, reserves the children's places and moves the counts.  The
+// spawn kernel strides over the blocks of flags: a block whose scanned sums
+// show no event is skipped without reading its flags; otherwise its events
+// are listed in array order in shared memory and taken one per thread.  (Two
+// launches an emitting species; sums, their scan, the children and the count
+// used to be four, and a thread made the children of its own 16 flags one
+// after the other.)
 // ---------------------------------------------------------------------
 constexpr int kSpawnThreads = 256, kSpawnPer = kScanItems / kSpawnThreads;
 
@@ -318,21 +323,14 @@ inline int spawn_grid(long long m)
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     }
-    return (int)std::min<long long>(scan_blocks(m), 4ll * nsm);
+    return (int)std::min<long long>((m + kScanItems - 1) / kScanItems, 4ll * nsm);
 }
 
-// the flags (0 or 1) of block b, kSpawnPer per thread from p0, as a bit mask,
-// and the rank of this thread's first event; false (block-uniform) when the
-// block has no event.  m: the flags' end (the parents' device count: the
-// slots past it count as no event, as in the block sums)
-__device__ __forceinline__ bool spawn_ranks(const uint32_t *__restrict__ ev, long long m,
-                                            const uint32_t *__restrict__ bsum, long long b, long long &p0,
-                                            uint32_t &bits, uint32_t &run)
+// this thread's kSpawnPer flags (0 or 1) of block b from p0 as a bit mask;
+// m: the flags' end (the parents' device count: what lies past it is no event)
+__device__ __forceinline__ uint32_t flag_bits(const uint32_t *__restrict__ ev, long long m, long long p0)
 {
-    __shared__ uint32_t sh[32];
-    if (bsum[b + 1] == bsum[b]) return false;
-    p0 = b * kScanItems + (long long)threadIdx.x * kSpawnPer;
-    bits = 0;
+    uint32_t bits = 0;
     if (p0 + kSpawnPer <= m && (reinterpret_cast<uintptr_t>(ev) & 15u) == 0) {
 #pragma unroll
         for (int k = 0; k < kSpawnPer; k += 4) {
@@ -344,27 +342,99 @@ __device__ __forceinline__ bool spawn_ranks(const uint32_t *__restrict__ ev, lon
         for (int k = 0; k < kSpawnPer; k++)
             if (p0 + k < m && ev[p0 + k]) bits |= 1u << k;
     }
-    uint32_t tot;
-    run = block_excl_scan<kSpawnThreads>((uint32_t)__popc(bits), sh, tot) + bsum[b];
-    return true;
+    return bits;
+}
+
+// bsum[b] = events before block b, bsum[nb] = all of them; then the children's
+// first places ctl.base (one or two target species) and the new counts.  A
+// pair is created only where both its electron and its positron find room, so
+// both counts advance by the same number.
+__global__ void __launch_bounds__(kSpawnThreads) k_flag_sums(const uint32_t *__restrict__ ev, long long m,
+                                                             const long long *__restrict__ dn, uint32_t *bsum,
+                                                             SpawnCtl *ctl, long long *count0, long long cap0,
+                                                             long long *count1, long long cap1, int *err)
+{
+    __shared__ uint32_t sh[32];
+    __shared__ bool last;
+    m = max(0ll, min(m, *dn));
+    const long long nb = (m + kScanItems - 1) / kScanItems;
+    for (long long b = blockIdx.x; b < nb; b += gridDim.x) {
+        const uint32_t bits = flag_bits(ev, m, b * kScanItems + (long long)threadIdx.x * kSpawnPer);
+        uint32_t tot;
+        block_excl_scan<kSpawnThreads>((uint32_t)__popc(bits), sh, tot);
+        if (threadIdx.x == 0) bsum[b] = tot;
+    }
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&ctl->done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    uint32_t carry = 0;
+    for (long long b0 = 0; b0 < nb; b0 += kSpawnThreads * 8) {
+        uint32_t v[8], s = 0, tot;
+        const long long i0 = b0 + threadIdx.x * 8;
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            v[k] = i0 + k < nb ? __ldcg(bsum + i0 + k) : 0u;
+            s += v[k];
+        }
+        uint32_t run = carry + block_excl_scan<kSpawnThreads>(s, sh, tot);
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            if (i0 + k < nb) bsum[i0 + k] = run;
+            run += v[k];
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) {
+        bsum[nb] = carry;
+        long long n = carry;
+        ctl->base[0] = *count0;
+        bool over = *count0 + n > cap0;
+        long long take = min(n, cap0 - *count0);
+        if (count1) {
+            ctl->base[1] = *count1;
+            over |= *count1 + n > cap1;
+            take = min(take, cap1 - *count1);
+        }
+        if (over) atomicOr(err, ERR_CAPACITY);
+        take = max(take, 0ll);
+        *count0 += take;
+        if (count1) *count1 += take;
+        ctl->done = 0u;
+    }
+}
+
+// the events of block b listed in array order (their places in the block);
+// returns their number (block-uniform)
+__device__ __forceinline__ int list_events(const uint32_t *__restrict__ ev, long long m,
+                                           const uint32_t *__restrict__ bsum, long long b, uint16_t *list)
+{
+    __shared__ uint32_t sh[32];
+    if (bsum[b + 1] == bsum[b]) return 0;
+    __syncthreads();  // (the list of the block before is done with)
+    uint32_t bits = flag_bits(ev, m, b * kScanItems + (long long)threadIdx.x * kSpawnPer), tot;
+    uint32_t run = block_excl_scan<kSpawnThreads>((uint32_t)__popc(bits), sh, tot);
+    for (; bits; bits &= bits - 1) list[run++] = (uint16_t)(threadIdx.x * kSpawnPer + __ffs(bits) - 1);
+    __syncthreads();
+    return (int)tot;
 }
 
 __global__ void __launch_bounds__(kSpawnThreads) k_spawn_photons_f32(PartF32 parent, const uint32_t *__restrict__ bsum,
-                                    const uint32_t *__restrict__ total, long long m, QedParams q, PartF32 ph, double *ph_tau,
-                                    uint64_t *ph_id, uint32_t *ph_ev, long long *ph_count, long long ph_cap, int dim,
-                                    int *err)
+                                    const SpawnCtl *__restrict__ ctl, long long m, QedParams q, PartF32 ph, double *ph_tau,
+                                    uint64_t *ph_id, uint32_t *ph_ev, long long ph_cap, int dim)
 {
-    const long long base = *ph_count;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && base + *total > ph_cap) atomicOr(err, ERR_CAPACITY);
+    __shared__ uint16_t list[kScanItems];
+    const long long base = ctl->base[0];
     m = min(m, *parent.dn);  // (past the parents' device count: no event)
     const long long nb = (m + kScanItems - 1) / kScanItems;
     for (long long b = blockIdx.x; b < nb; b += gridDim.x) {
-        long long p0;
-        uint32_t bits, run;
-        if (!spawn_ranks(q.ev, m, bsum, b, p0, bits, run)) continue;
-        for (; bits; bits &= bits - 1) {
-            const long long p = p0 + (__ffs(bits) - 1);
-            const uint32_t rank = run++;
+        const int n = list_events(q.ev, m, bsum, b, list);
+        for (int e = threadIdx.x; e < n; e += kSpawnThreads) {
+            const long long p = b * kScanItems + list[e];
+            const uint32_t rank = bsum[b] + e;
             const long long dst = base + rank;
             if (dst >= ph_cap) continue;
             uint32_t w[4];
@@ -385,23 +455,20 @@ __global__ void __launch_bounds__(kSpawnThreads) k_spawn_photons_f32(PartF32 par
     }
 }
 
-__global__ void __launch_bounds__(kSpawnThreads) k_spawn_pairs_f32(PartF32 phot, const uint32_t *__restrict__ bsum, const uint32_t *__restrict__ total, long long m,
+__global__ void __launch_bounds__(kSpawnThreads) k_spawn_pairs_f32(PartF32 phot, const uint32_t *__restrict__ bsum, const SpawnCtl *__restrict__ ctl, long long m,
                                   QedParams q, PartF32 el, double *el_tau, uint64_t *el_id, uint32_t *el_ev,
-                                  long long *el_count, long long el_cap, PartF32 po, double *po_tau, uint64_t *po_id,
-                                  uint32_t *po_ev, long long *po_count, long long po_cap, int dim, int *err)
+                                  long long el_cap, PartF32 po, double *po_tau, uint64_t *po_id,
+                                  uint32_t *po_ev, long long po_cap, int dim)
 {
-    const long long be = *el_count, bp = *po_count;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && (be + *total > el_cap || bp + *total > po_cap))
-        atomicOr(err, ERR_CAPACITY);
+    __shared__ uint16_t list[kScanItems];
+    const long long be = ctl->base[0], bp = ctl->base[1];
     m = min(m, *phot.dn);  // (past the photons' device count: no event)
     const long long nb = (m + kScanItems - 1) / kScanItems;
     for (long long b = blockIdx.x; b < nb; b += gridDim.x) {
-        long long p0;
-        uint32_t bits, run;
-        if (!spawn_ranks(q.ev, m, bsum, b, p0, bits, run)) continue;
-        for (; bits; bits &= bits - 1) {
-            const long long p = p0 + (__ffs(bits) - 1);
-            const uint32_t rank = run++;
+        const int n = list_events(q.ev, m, bsum, b, list);
+        for (int e = threadIdx.x; e < n; e += kSpawnThreads) {
+            const long long p = b * kScanItems + list[e];
+            const uint32_t rank = bsum[b] + e;
             const long long de = be + rank, dp = bp + rank;
             if (de >= el_cap || dp >= po_cap) continue;
             uint32_t w[4];
@@ -443,35 +510,32 @@ __global__ void __launch_bounds__(kSpawnThreads) k_spawn_pairs_f32(PartF32 phot,
 
 // FP64 plain form: absolute positions, event data as 4 doubles per particle
 __global__ void __launch_bounds__(kSpawnThreads) k_spawn_photons_f64(PartF64 parent, const uint32_t *__restrict__ bsum,
-                                    const uint32_t *__restrict__ total, long long m, QedParams q, PartF64 ph, double *ph_tau,
-                                    uint64_t *ph_id, uint32_t *ph_ev, long long *ph_count, long long ph_cap, int dim,
-                                    int *err)
+                                    const SpawnCtl *__restrict__ ctl, long long m, QedParams q, PartF64 ph, double *ph_tau,
+                                    uint64_t *ph_id, uint32_t *ph_ev, long long ph_cap, int dim)
 {
-    const long long base = *ph_count;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && base + *total > ph_cap) atomicOr(err, ERR_CAPACITY);
+    __shared__ uint16_t list[kScanItems];
+    const long long base = ctl->base[0];
     m = min(m, *parent.dn);  // (past the parents' device count: no event)
     const long long nb = (m + kScanItems - 1) / kScanItems;
     for (long long b = blockIdx.x; b < nb; b += gridDim.x) {
-        long long p0;
-        uint32_t bits, run;
-        if (!spawn_ranks(q.ev, m, bsum, b, p0, bits, run)) continue;
-        for (; bits; bits &= bits - 1) {
-            const long long p = p0 + (__ffs(bits) - 1);
-            const uint32_t rank = run++;
+        const int n = list_events(q.ev, m, bsum, b, list);
+        for (int e = threadIdx.x; e < n; e += kSpawnThreads) {
+            const long long p = b * kScanItems + list[e];
+            const uint32_t rank = bsum[b] + e;
             const long long dst = base + rank;
             if (dst >= ph_cap) continue;
             uint32_t w[4];
             const uint64_t pid = q.id[p];
             philox4x32_10((uint32_t)pid, (uint32_t)(pid >> 32), q.step, QP_EMIT, q.key[0], q.key[1], w);
             const uint64_t cid = ((uint64_t)w[3] << 32) | w[2];
-            const double4 e = reinterpret_cast<const double4 *>(q.evk)[p];
+            const double4 ed = reinterpret_cast<const double4 *>(q.evk)[p];
             ph.cell[dst] = parent.cell[p];
 #pragma unroll
             for (int d = 0; d < 3; d++)
                 if (d < dim) ph.x[d][dst] = parent.x[d][p];
-            ph.u[0][dst] = e.x;
-            ph.u[1][dst] = e.y;
-            ph.u[2][dst] = e.z;
+            ph.u[0][dst] = ed.x;
+            ph.u[1][dst] = ed.y;
+            ph.u[2][dst] = ed.z;
             ph_id[dst] = cid;
             ph_tau[dst] = initial_tau(cid, q.key);
             ph_ev[dst] = 0;
@@ -479,31 +543,28 @@ __global__ void __launch_bounds__(kSpawnThreads) k_spawn_photons_f64(PartF64 par
     }
 }
 
-__global__ void __launch_bounds__(kSpawnThreads) k_spawn_pairs_f64(PartF64 phot, const uint32_t *__restrict__ bsum, const uint32_t *__restrict__ total, long long m,
+__global__ void __launch_bounds__(kSpawnThreads) k_spawn_pairs_f64(PartF64 phot, const uint32_t *__restrict__ bsum, const SpawnCtl *__restrict__ ctl, long long m,
                                   QedParams q, PartF64 el, double *el_tau, uint64_t *el_id, uint32_t *el_ev,
-                                  long long *el_count, long long el_cap, PartF64 po, double *po_tau, uint64_t *po_id,
-                                  uint32_t *po_ev, long long *po_count, long long po_cap, int dim, int *err)
+                                  long long el_cap, PartF64 po, double *po_tau, uint64_t *po_id,
+                                  uint32_t *po_ev, long long po_cap, int dim)
 {
-    const long long be = *el_count, bp = *po_count;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && (be + *total > el_cap || bp + *total > po_cap))
-        atomicOr(err, ERR_CAPACITY);
+    __shared__ uint16_t list[kScanItems];
+    const long long be = ctl->base[0], bp = ctl->base[1];
     m = min(m, *phot.dn);  // (past the photons' device count: no event)
     const long long nb = (m + kScanItems - 1) / kScanItems;
     for (long long b = blockIdx.x; b < nb; b += gridDim.x) {
-        long long p0;
-        uint32_t bits, run;
-        if (!spawn_ranks(q.ev, m, bsum, b, p0, bits, run)) continue;
-        for (; bits; bits &= bits - 1) {
-            const long long p = p0 + (__ffs(bits) - 1);
-            const uint32_t rank = run++;
+        const int n = list_events(q.ev, m, bsum, b, list);
+        for (int e = threadIdx.x; e < n; e += kSpawnThreads) {
+            const long long p = b * kScanItems + list[e];
+            const uint32_t rank = bsum[b] + e;
             const long long de = be + rank, dp = bp + rank;
             if (de >= el_cap || dp >= po_cap) continue;
             uint32_t w[4];
             const uint64_t pid = q.id[p];
             philox4x32_10((uint32_t)pid, (uint32_t)(pid >> 32), q.step, QP_PAIR, q.key[0], q.key[1], w);
             const uint64_t eid = ((uint64_t)w[3] << 32) | w[2], pid2 = eid + 1;
-            const double4 e = reinterpret_cast<const double4 *>(q.evk)[p];
-            const double k = sqrt(e.x * e.x + e.y * e.y + e.z * e.z);
+            const double4 ed = reinterpret_cast<const double4 *>(q.evk)[p];
+            const double k = sqrt(ed.x * ed.x + ed.y * ed.y + ed.z * ed.z);
             const uint32_t cell = phot.cell[p];
 #pragma unroll
             for (int d = 0; d < 3; d++) {
@@ -514,15 +575,15 @@ __global__ void __launch_bounds__(kSpawnThreads) k_spawn_pairs_f64(PartF64 phot,
             el.cell[de] = cell;
             po.cell[dp] = cell;
             phot.cell[p] = kDead;
-            const double ep = e.w * k, em = (1.0 - e.w) * k;
+            const double ep = ed.w * k, em = (1.0 - ed.w) * k;
             const double pm = sqrt(fmax(em * em - 1.0, 0.0)), pp = sqrt(fmax(ep * ep - 1.0, 0.0));
             const double inv = k > 0.0 ? 1.0 / k : 0.0;
-            el.u[0][de] = pm * e.x * inv;
-            el.u[1][de] = pm * e.y * inv;
-            el.u[2][de] = pm * e.z * inv;
-            po.u[0][dp] = pp * e.x * inv;
-            po.u[1][dp] = pp * e.y * inv;
-            po.u[2][dp] = pp * e.z * inv;
+            el.u[0][de] = pm * ed.x * inv;
+            el.u[1][de] = pm * ed.y * inv;
+            el.u[2][de] = pm * ed.z * inv;
+            po.u[0][dp] = pp * ed.x * inv;
+            po.u[1][dp] = pp * ed.y * inv;
+            po.u[2][dp] = pp * ed.z * inv;
             el_id[de] = eid;
             po_id[dp] = pid2;
             el_tau[de] = initial_tau(eid, q.key);
@@ -531,25 +592,6 @@ __global__ void __launch_bounds__(kSpawnThreads) k_spawn_pairs_f64(PartF64 phot,
             po_ev[dp] = 0;
         }
     }
-}
-
-__global__ void k_add_count(long long *count, const uint32_t *total, long long cap)
-{
-    const long long c = *count + *total;
-    *count = c > cap ? cap : c;
-}
-
-// a pair is created only where both its electron and its positron find room
-// (the spawn kernels skip the rest), so both counts advance by the same number
-__global__ void k_add_pair_counts(long long *el_count, long long *po_count, const uint32_t *total, long long el_cap,
-                                  long long po_cap)
-{
-    long long n = *total;
-    n = min(n, el_cap - *el_count);
-    n = min(n, po_cap - *po_count);
-    if (n < 0) n = 0;
-    *el_count += n;
-    *po_count += n;
 }
 
 __global__ void k_init_qed(long long first, long long n, uint64_t id0, uint64_t *id, double *tau, uint32_t k0,
@@ -571,54 +613,56 @@ void launch_init_qed(long long first, long long n, uint64_t id0, uint64_t *id, d
     k_init_qed<<<div_up(n, 256), 256, 0, st>>>(first, n, id0, id, tau, key[0], key[1]);
 }
 
-void launch_spawn_photons(const PartF32 &parent, const uint32_t *bsum, const uint32_t *total, long long m,
-                          const QedParams &q,
-                          const PartF32 &ph, double *ph_tau, uint64_t *ph_id, uint32_t *ph_ev, long long *ph_count,
-                          long long ph_cap, int dim, int *err, cudaStream_t st)
+// block sums in bsum (scan_blocks(m) + 1 words)
+static void flag_sums(const uint32_t *ev, long long m, const long long *dn, uint32_t *bsum, SpawnCtl *ctl,
+                      long long *count0, long long cap0, long long *count1, long long cap1, int *err, cudaStream_t st)
 {
-    if (parent.n == 0 || m <= 0) return;
-    note_launch(2);
-    k_spawn_photons_f32<<<spawn_grid(m), kSpawnThreads, 0, st>>>(parent, bsum, total, m, q, ph, ph_tau, ph_id, ph_ev,
-                                                              ph_count, ph_cap, dim, err);
-    k_add_count<<<1, 1, 0, st>>>(ph_count, total, ph_cap);
+    note_launch();
+    k_flag_sums<<<spawn_grid(m), kSpawnThreads, 0, st>>>(ev, m, dn, bsum, ctl, count0, cap0, count1, cap1, err);
 }
 
-void launch_spawn_pairs(const PartF32 &phot, const uint32_t *bsum, const uint32_t *total, long long m,
-                        const QedParams &q,
-                        const PartF32 &el, double *el_tau, uint64_t *el_id, uint32_t *el_ev, long long *el_count,
-                        long long el_cap, const PartF32 &po, double *po_tau, uint64_t *po_id, uint32_t *po_ev,
+template <class P_t>
+void launch_spawn_photons(const P_t &parent, uint32_t *bsum, SpawnCtl *ctl, const QedParams &q, const P_t &ph,
+                          uint32_t *ph_ev, long long *ph_count, long long ph_cap, int dim, int *err, cudaStream_t st)
+{
+    const long long m = parent.n;
+    if (m <= 0) return;
+    flag_sums(q.ev, m, parent.dn, bsum, ctl, ph_count, ph_cap, nullptr, 0, err, st);
+    note_launch();
+    if constexpr (std::is_same_v<P_t, PartF32>)
+        k_spawn_photons_f32<<<spawn_grid(m), kSpawnThreads, 0, st>>>(parent, bsum, ctl, m, q, ph, ph.tau, ph.id, ph_ev, ph_cap,
+                                                                    dim);
+    else
+        k_spawn_photons_f64<<<spawn_grid(m), kSpawnThreads, 0, st>>>(parent, bsum, ctl, m, q, ph, ph.tau, ph.id, ph_ev, ph_cap,
+                                                                    dim);
+}
+
+template <class P_t>
+void launch_spawn_pairs(const P_t &phot, uint32_t *bsum, SpawnCtl *ctl, const QedParams &q, const P_t &el,
+                        uint32_t *el_ev, long long *el_count, long long el_cap, const P_t &po, uint32_t *po_ev,
                         long long *po_count, long long po_cap, int dim, int *err, cudaStream_t st)
 {
-    if (phot.n == 0 || m <= 0) return;
-    note_launch(2);
-    k_spawn_pairs_f32<<<spawn_grid(m), kSpawnThreads, 0, st>>>(phot, bsum, total, m, q, el, el_tau, el_id, el_ev, el_count,
-                                                          el_cap, po, po_tau, po_id, po_ev, po_count, po_cap, dim, err);
-    k_add_pair_counts<<<1, 1, 0, st>>>(el_count, po_count, total, el_cap, po_cap);
+    const long long m = phot.n;
+    if (m <= 0) return;
+    flag_sums(q.ev, m, phot.dn, bsum, ctl, el_count, el_cap, po_count, po_cap, err, st);
+    note_launch();
+    if constexpr (std::is_same_v<P_t, PartF32>)
+        k_spawn_pairs_f32<<<spawn_grid(m), kSpawnThreads, 0, st>>>(phot, bsum, ctl, m, q, el, el.tau, el.id, el_ev, el_cap, po,
+                                                                  po.tau, po.id, po_ev, po_cap, dim);
+    else
+        k_spawn_pairs_f64<<<spawn_grid(m), kSpawnThreads, 0, st>>>(phot, bsum, ctl, m, q, el, el.tau, el.id, el_ev, el_cap, po,
+                                                                  po.tau, po.id, po_ev, po_cap, dim);
 }
 
-void launch_spawn_photons(const PartF64 &parent, const uint32_t *bsum, const uint32_t *total, long long m,
-                          const QedParams &q,
-                          const PartF64 &ph, double *ph_tau, uint64_t *ph_id, uint32_t *ph_ev, long long *ph_count,
-                          long long ph_cap, int dim, int *err, cudaStream_t st)
-{
-    if (parent.n == 0 || m <= 0) return;
-    note_launch(2);
-    k_spawn_photons_f64<<<spawn_grid(m), kSpawnThreads, 0, st>>>(parent, bsum, total, m, q, ph, ph_tau, ph_id, ph_ev,
-                                                              ph_count, ph_cap, dim, err);
-    k_add_count<<<1, 1, 0, st>>>(ph_count, total, ph_cap);
-}
-
-void launch_spawn_pairs(const PartF64 &phot, const uint32_t *bsum, const uint32_t *total, long long m,
-                        const QedParams &q,
-                        const PartF64 &el, double *el_tau, uint64_t *el_id, uint32_t *el_ev, long long *el_count,
-                        long long el_cap, const PartF64 &po, double *po_tau, uint64_t *po_id, uint32_t *po_ev,
-                        long long *po_count, long long po_cap, int dim, int *err, cudaStream_t st)
-{
-    if (phot.n == 0 || m <= 0) return;
-    note_launch(2);
-    k_spawn_pairs_f64<<<spawn_grid(m), kSpawnThreads, 0, st>>>(phot, bsum, total, m, q, el, el_tau, el_id, el_ev, el_count,
-                                                          el_cap, po, po_tau, po_id, po_ev, po_count, po_cap, dim, err);
-    k_add_pair_counts<<<1, 1, 0, st>>>(el_count, po_count, total, el_cap, po_cap);
-}
+template void launch_spawn_photons<PartF32>(const PartF32 &, uint32_t *, SpawnCtl *, const QedParams &, const PartF32 &,
+                                            uint32_t *, long long *, long long, int, int *, cudaStream_t);
+template void launch_spawn_photons<PartF64>(const PartF64 &, uint32_t *, SpawnCtl *, const QedParams &, const PartF64 &,
+                                            uint32_t *, long long *, long long, int, int *, cudaStream_t);
+template void launch_spawn_pairs<PartF32>(const PartF32 &, uint32_t *, SpawnCtl *, const QedParams &, const PartF32 &,
+                                          uint32_t *, long long *, long long, const PartF32 &, uint32_t *, long long *,
+                                          long long, int, int *, cudaStream_t);
+template void launch_spawn_pairs<PartF64>(const PartF64 &, uint32_t *, SpawnCtl *, const QedParams &, const PartF64 &,
+                                          uint32_t *, long long *, long long, const PartF64 &, uint32_t *, long long *,
+                                          long long, int, int *, cudaStream_t);
 
 }  // namespace pic

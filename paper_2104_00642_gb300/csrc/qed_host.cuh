@@ -12,23 +12,20 @@ void launch_qed_eval(const QedTables &T, bool f64, int p, long long n, const dou
                      double *out, cudaStream_t st);
 void launch_init_qed(long long first, long long n, uint64_t id0, uint64_t *id, double *tau, const uint32_t *key,
                      cudaStream_t st);
-void launch_spawn_photons(const PartF32 &parent, const uint32_t *bsum, const uint32_t *total, long long m,
-                          const QedParams &q,
-                          const PartF32 &ph, double *ph_tau, uint64_t *ph_id, uint32_t *ph_ev, long long *ph_count,
-                          long long ph_cap, int dim, int *err, cudaStream_t st);
-void launch_spawn_pairs(const PartF32 &phot, const uint32_t *bsum, const uint32_t *total, long long m,
-                        const QedParams &q,
-                        const PartF32 &el, double *el_tau, uint64_t *el_id, uint32_t *el_ev, long long *el_count,
-                        long long el_cap, const PartF32 &po, double *po_tau, uint64_t *po_id, uint32_t *po_ev,
-                        long long *po_count, long long po_cap, int dim, int *err, cudaStream_t st);
-void launch_spawn_photons(const PartF64 &parent, const uint32_t *bsum, const uint32_t *total, long long m,
-                          const QedParams &q,
-                          const PartF64 &ph, double *ph_tau, uint64_t *ph_id, uint32_t *ph_ev, long long *ph_count,
-                          long long ph_cap, int dim, int *err, cudaStream_t st);
-void launch_spawn_pairs(const PartF64 &phot, const uint32_t *bsum, const uint32_t *total, long long m,
-                        const QedParams &q,
-                        const PartF64 &el, double *el_tau, uint64_t *el_id, uint32_t *el_ev, long long *el_count,
-                        long long el_cap, const PartF64 &po, double *po_tau, uint64_t *po_id, uint32_t *po_ev,
+// places of a step's children (k_flag_sums): the block counter (zero between
+// launches) and the first place in each target species
+struct SpawnCtl {
+    unsigned done, pad;
+    long long base[2];
+};
+// the children of the flagged particles (q.ev), appended in array order;
+// bsum: scan_blocks(n) + 1 words of scratch
+template <class P_t>
+void launch_spawn_photons(const P_t &parent, uint32_t *bsum, SpawnCtl *ctl, const QedParams &q, const P_t &ph,
+                          uint32_t *ph_ev, long long *ph_count, long long ph_cap, int dim, int *err, cudaStream_t st);
+template <class P_t>
+void launch_spawn_pairs(const P_t &phot, uint32_t *bsum, SpawnCtl *ctl, const QedParams &q, const P_t &el,
+                        uint32_t *el_ev, long long *el_count, long long el_cap, const P_t &po, uint32_t *po_ev,
                         long long *po_count, long long po_cap, int dim, int *err, cudaStream_t st);
 void launch_push_qed_f64(const PartF64 &P, double *F, const Grid &g, const PushConst &pc, const QedParams &q,
                          int *err, double *e_abs, cudaStream_t st);

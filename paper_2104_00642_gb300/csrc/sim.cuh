@@ -79,6 +79,7 @@ struct pic_sim {
     double *diag_scratch = nullptr;
     double *diag_out = nullptr;  // 32 doubles
     int *d_err = nullptr;
+    pic::SpawnCtl *spawn_ctl = nullptr;
     double *d_eabs = nullptr;
     long long step = 0;
     pic::Laser laser{};

@@ -157,11 +157,8 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_radix_scatter(const uint32_
 // ---------------------------------------------------------------------
 // device-wide exclusive scan of u32 (reduce, scan of block sums, downsweep)
 // ---------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_scan_reduce(const uint32_t *__restrict__ in, long long m, uint32_t *sums,
-                                                     bool zero_end = false, const long long *__restrict__ dn = nullptr)
+__global__ void __launch_bounds__(1024) k_scan_reduce(const uint32_t *__restrict__ in, long long m, uint32_t *sums)
 {
-    if (zero_end && blockIdx.x == 0 && threadIdx.x == 0) sums[gridDim.x] = 0u;  // the slot that scans to the total
-    if (dn && *dn < m) m = *dn < 0 ? 0 : *dn;  // words past the device count read as zero
     __shared__ uint32_t sh[32];
     long long b0 = (long long)blockIdx.x * kScanItems + threadIdx.x * 4;
     uint32_t s = 0;
@@ -202,22 +199,6 @@ size_t scan_scratch_words(long long m)
     }
     return w + 32;
 }
-
-// the exclusive scan of the sums of in's blocks of kScanItems words:
-// bsum[b] = sum of in[0, b kScanItems), bsum[nb] = the total (nb + 1 words,
-// scratch past them as for scan_exclusive); dn (device, optional): the
-// words from *dn on count as zero
-void scan_block_sums(const uint32_t *in, long long m, uint32_t *bsum, uint32_t *scratch, cudaStream_t st,
-                     const long long *dn)
-{
-    if (m <= 0) return;
-    const long long nb = (m + kScanItems - 1) / kScanItems;
-    note_launch();
-    k_scan_reduce<<<(int)nb, 1024, 0, st>>>(in, m, bsum, true, dn);
-    scan_exclusive(bsum, bsum, nb + 1, scratch, st);
-}
-
-long long scan_blocks(long long m) { return (m + kScanItems - 1) / kScanItems; }
 
 // exclusive scan of m words, in may equal out
 void scan_exclusive(const uint32_t *in, uint32_t *out, long long m, uint32_t *scratch, cudaStream_t st)

@@ -8,9 +8,6 @@ namespace pic {
 size_t sort_scratch_bytes(long long cap);
 size_t scan_scratch_words(long long m);
 void scan_exclusive(const uint32_t *in, uint32_t *out, long long m, uint32_t *scratch, cudaStream_t st);
-void scan_block_sums(const uint32_t *in, long long m, uint32_t *bsum, uint32_t *scratch, cudaStream_t st,
-                     const long long *dn = nullptr);
-long long scan_blocks(long long m);  // blocks of the scan of m words (kScanItems each)
 // a sort's outcome in its scratch: the permutation (new -> old), the sorted
 // keys and the number of entries (device)
 struct SortResult {

@@ -1255,17 +1255,20 @@ int mlp_net_alloc(pic_sim *s, MlpNet &net)
 int mlp_scratch(pic_sim *s, long long B)
 {
     MlpScratch &S = s->ms;
-    if (!S.it) {
+    if (!S.acc) {
         void *small = nullptr;
-        int rc = dalloc(s, &small, 64 + kMlpValAcc * sizeof(double));
+        int rc = dalloc(s, &small, 128 + kMlpValAcc * sizeof(double));
         if (rc) return rc;
-        S.loss = (float *)small;                  // 2 floats
-        S.it = (int *)((char *)small + 16);
-        S.acc = (double *)((char *)small + 64);   // kMlpValAcc doubles
+        S.loss = (float *)small;  // 2 floats
+        for (int q = 0; q < 2; q++) {
+            S.slot[q].it = (int *)((char *)small + 16 + 4 * q);
+            S.slot[q].sched = (double *)((char *)small + 32 + 24 * q);
+        }
+        S.acc = (double *)((char *)small + 128);  // kMlpValAcc doubles
     }
     if (B <= S.B) return PIC_OK;
     void *buf = nullptr;
-    const size_t per_row = (size_t)(3 * 2 + 6 * kMlpH) * sizeof(float);
+    const size_t per_row = (size_t)(5 * 2 + 6 * kMlpH) * sizeof(float);
     int rc = dalloc(s, &buf, per_row * (size_t)B + mlp_partial_floats(B) * sizeof(float));
     if (rc) return rc;
     float *f = (float *)buf;
@@ -1276,7 +1279,9 @@ int mlp_scratch(pic_sim *s, long long B)
         S.Z.z[l] = f + 6 * B + (size_t)l * kMlpH * B;
         S.D.z[l] = f + 6 * B + (size_t)(3 + l) * kMlpH * B;
     }
-    S.partials = f + 6 * B + (size_t)6 * kMlpH * B;
+    S.XT[0] = S.X;  // (and S.T behind it)
+    S.XT[1] = f + 6 * B + (size_t)6 * kMlpH * B;
+    S.partials = S.XT[1] + 4 * B;
     S.B = B;
     return PIC_OK;
 }
@@ -1389,36 +1394,41 @@ int pic_mlp_train(pic_sim *s, int p, const pic_mlp_train_opts *o, pic_mlp_report
         CK(cudaMemsetAsync(net.M, 0, 3 * (size_t)kMlpNParams * sizeof(float), s->st));  // M, V, G
     }
     launch_mlp_image(net.P, net.img, s->st);
-    CK(cudaMemsetAsync(s->ms.it, 0, sizeof(int), s->st));
+    CK(cudaMemsetAsync(s->ms.slot[0].it, 0, 2 * sizeof(int), s->st));
     CK(cudaMemsetAsync(s->ms.loss, 0, 2 * sizeof(float), s->st));
     CK(cudaStreamSynchronize(s->st));
     MlpAdam a{iters, o->lr > 0 ? o->lr : 1e-2, o->lr_final > 0 ? o->lr_final : 1e-4, 0.9f, 0.999f, 1e-8f};
     const float w_rate = (float)(o->rate_weight > 0 ? o->rate_weight : 4.0);
-    const uint32_t key[2] = {(uint32_t)o->seed, (uint32_t)(o->seed >> 32)};
-    // one iteration captured as a graph on a private stream, replayed
+    const MlpTraining tr{s->T, p, {(uint32_t)o->seed, (uint32_t)(o->seed >> 32)}, a, w_rate};
+    // one iteration per slot captured as a graph on a private stream, replayed
+    // in turn
     cudaStream_t ts = nullptr;
-    cudaGraph_t gr = nullptr;
-    cudaGraphExec_t ge = nullptr;
+    cudaGraph_t gr[2] = {nullptr, nullptr};
+    cudaGraphExec_t ge[2] = {nullptr, nullptr};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaStreamCreateWithFlags(&ts, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaStreamBeginCapture(ts, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        mlp_train_iteration(net, s->ms, s->T, p, key, a, w_rate, ts);
-        e = cudaStreamEndCapture(ts, &gr);
-    }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&ge, gr, 0);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    for (int q = 0; q < 2 && e == cudaSuccess; q++) {
+        e = cudaStreamBeginCapture(ts, cudaStreamCaptureModeThreadLocal);
+        if (e != cudaSuccess) break;
+        mlp_train_iteration(net, s->ms, tr, q, ts);
+        e = cudaStreamEndCapture(ts, &gr[q]);
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&ge[q], gr[q], 0);
+    }
     if (e == cudaSuccess) e = cudaEventRecord(e0, ts);
-    for (long long i = 0; i < iters && e == cudaSuccess; i++) e = cudaGraphLaunch(ge, ts);
-    note_launch(7 * (iters - 1));  // the captured iteration counted its seven launches once
+    if (e == cudaSuccess) launch_mlp_data(net, s->ms, tr, ts);
+    for (long long i = 0; i < iters && e == cudaSuccess; i++) e = cudaGraphLaunch(ge[i & 1], ts);
+    note_launch(4 * (iters - 2));  // (the two captured iterations counted theirs)
     if (e == cudaSuccess) e = cudaEventRecord(e1, ts);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ts);
     float ms = 0.f, loss[2] = {0.f, 0.f};
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
     if (e == cudaSuccess) e = cudaMemcpy(loss, s->ms.loss, sizeof loss, cudaMemcpyDeviceToHost);
-    if (ge) cudaGraphExecDestroy(ge);
-    if (gr) cudaGraphDestroy(gr);
+    for (int q = 0; q < 2; q++) {
+        if (ge[q]) cudaGraphExecDestroy(ge[q]);
+        if (gr[q]) cudaGraphDestroy(gr[q]);
+    }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (ts) cudaStreamDestroy(ts);

@@ -16,13 +16,27 @@ struct MlpNet {
     bool ready = false;
 };
 
+struct MlpAdam {
+    long long iters;
+    double lr0, lr_final;
+    float beta1, beta2, eps;
+};
+
+// the iteration whose samples a slot holds, and its learning rate and bias
+// corrections (device)
+struct MlpSlot {
+    int *it = nullptr;
+    double *sched = nullptr;  // 3
+};
+
 // training scratch for a batch of B rows (B a multiple of 128)
 struct MlpScratch {
     long long B = 0;
     float *X = nullptr, *T = nullptr, *Y = nullptr;  // [B][2]
+    float *XT[2] = {nullptr, nullptr};               // training: inputs and targets of the iteration in slot 0, 1
+    MlpSlot slot[2];
     MlpZ Z{}, D{};                                   // [B][64] each
     float *loss = nullptr;                           // [0] this iteration, [1] the last one
-    int *it = nullptr;                               // iteration counter
     double *acc = nullptr;                           // validation accumulators (kMlpValAcc)
     float *partials = nullptr;                       // per-block / per-warp gradient partials
 };
@@ -36,11 +50,6 @@ constexpr int kMlpValAcc = 4 + 2 * kMlpValRows;
 // floats of gradient partials a batch of B rows needs (mlp_partial_floats)
 size_t mlp_partial_floats(long long B);
 
-struct MlpAdam {
-    long long iters;
-    double lr0, lr_final;
-    float beta1, beta2, eps;
-};
 
 // (both staged images stay below the 48 KB default dynamic shared memory)
 static_assert(kMlpTrainStageBytes <= 48 * 1024, "no opt-in needed");
@@ -51,8 +60,19 @@ void launch_mlp_forward(const MlpImage *img, long long B, const float *X, const 
 void launch_mlp_backward(const MlpImage *img, long long B, const float *X, const float *Tg, const float *Y,
                          const MlpZ &Z, const MlpZ &D, float *partials, float *grad, float w_rate, float *loss,
                          cudaStream_t st);
-void mlp_train_iteration(MlpNet &net, MlpScratch &S, const QedTables &T, int p, const uint32_t *key,
-                         const MlpAdam &a, float w_rate, cudaStream_t st);
+// what a training run keeps fixed
+struct MlpTraining {
+    QedTables T;
+    int p;
+    uint32_t key[2];
+    MlpAdam a;
+    float w_rate;
+};
+// the samples of iteration 0 (its number is in slot 0) into slot 0
+void launch_mlp_data(const MlpNet &net, MlpScratch &S, const MlpTraining &t, cudaStream_t st);
+// one training iteration on the samples of a slot, drawing the next
+// iteration's into the other slot
+void mlp_train_iteration(MlpNet &net, MlpScratch &S, const MlpTraining &t, int slot, cudaStream_t st);
 void launch_mlp_eval(const MlpImage *img, long long n, const float *X, float *Y, cudaStream_t st);
 // the same evaluation on the tcgen05 tensor cores (mlp_tc.cu); a timeout of
 // the tensor cores sets ERR_TIMEOUT in *err

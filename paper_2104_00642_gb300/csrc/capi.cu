@@ -465,6 +465,7 @@ int step_loop(pic_sim *s, int64_t nsteps)
     const Grid &g = s->g;
     const double h = 0.5 * g.dt;
     R *F = (R *)s->F;
+    const bool one = fields_in_one_block<R>(g);
     for (int64_t it = 0; it < nsteps; it++) {
         if (s->sort_interval > 0 && s->step % s->sort_interval == 0) {
             ph_begin(s);
@@ -477,8 +478,12 @@ int step_loop(pic_sim *s, int64_t nsteps)
         const double t0 = (double)s->step * g.dt;
         if (it == 0) {
             ph_begin(s);
-            launch_update_E<R>(F, g, h, false, true, s->st);  // E^{n+1/2}, then J := 0
-            launch_update_B<R>(F, g, h, t0 + h, laser_at(s, t0 + h), s->st);
+            if (one) {
+                launch_fields_1d<R>(F, g, h, true, false, Laser{}, laser_at(s, t0 + h), s->st);
+            } else {
+                launch_update_E<R>(F, g, h, false, true, s->st);  // E^{n+1/2}, then J := 0
+                launch_update_B<R>(F, g, h, laser_at(s, t0 + h), false, s->st);
+            }
             ph_end(s, PIC_PHASE_FIELDS);
         }
         ph_begin(s);
@@ -499,16 +504,18 @@ int step_loop(pic_sim *s, int64_t nsteps)
         }
         qed_spawn(s);
         ph_end(s, PIC_PHASE_PUSH);
+        const bool last = it == nsteps - 1;
         ph_begin(s);
-        launch_fold<R>(F, g, s->st);
-        ph_end(s, PIC_PHASE_FOLD);
-        ph_begin(s);
-        launch_update_B<R>(F, g, h, t0 + g.dt, laser_at(s, t0 + g.dt), s->st);  // B^{n+1}
-        if (it == nsteps - 1) {
-            launch_update_E<R>(F, g, h, false, false, s->st);  // E^{n+1}
+        if (one) {
+            launch_fields_1d<R>(F, g, h, false, last, laser_at(s, t0 + g.dt), laser_at(s, t0 + g.dt + h), s->st);
         } else {
-            launch_update_E<R>(F, g, h, true, true, s->st);  // E^{n+3/2}, then J := 0
-            launch_update_B<R>(F, g, h, t0 + g.dt + h, laser_at(s, t0 + g.dt + h), s->st);  // B^{n+3/2}
+            launch_update_B<R>(F, g, h, laser_at(s, t0 + g.dt), true, s->st);  // the fold, B^{n+1}
+            if (last) {
+                launch_update_E<R>(F, g, h, false, false, s->st);  // E^{n+1}
+            } else {
+                launch_update_E<R>(F, g, h, true, true, s->st);  // E^{n+3/2}, then J := 0
+                launch_update_B<R>(F, g, h, laser_at(s, t0 + g.dt + h), false, s->st);  // B^{n+3/2}
+            }
         }
         ph_end(s, PIC_PHASE_FIELDS);
         CK(cudaGetLastError());

@@ -2,9 +2,15 @@
 // absorbing faces with the laser entering through x-min, and the current
 // fold of the ghost layers.
 //
-// One thread per padded cell on a (x, y, z) thread grid, x fastest: rows are
-// read and written with unit stride (coalesced) and no thread does integer
-// division.  Each thread updates the three components of its cell.  Along
+// One thread per padded cell, x fastest within a block: rows are read and
+// written with unit stride (coalesced) and no thread does integer division.
+// Blocks run through y before x: the ones at the x-min face, where the
+// laser's sines are a long chain in one lane of a warp, start first and hide
+// behind the others (2048 x 1024 cells, absorbing x faces and a laser: the
+// field launches of a step took 55.6 us with the rows' blocks in their order,
+// now 49.4; in FP64 242 and 209 us).  What bounds an update otherwise is
+// memory: 277 MB a step in 42 us on periodic axes.
+// Each thread updates the three components of its cell.  Along
 // periodic axes the ghost layers are computed directly (a neighbour that
 // falls off the padded box is taken one period away), so they stay
 // bit-identical copies of their images without a separate exchange.
@@ -55,11 +61,17 @@ __device__ __forceinline__ Phys phys_of(const Grid &g, int i, int j, int k)
     return r;
 }
 
-__device__ __forceinline__ bool thread_cell(const Grid &g, int &i, int &j, int &k)
+// thread blocks: 256 along x in 1D, else kBlockX by kBlockY
+constexpr unsigned kBlockX = 64, kBlockY = 4;
+
+// (nf: leading blocks of the launch that fold instead)
+__device__ __forceinline__ bool thread_cell(const Grid &g, int &i, int &j, int &k, unsigned nf = 0)
 {
-    i = blockIdx.x * blockDim.x + threadIdx.x;
-    j = blockIdx.y * blockDim.y + threadIdx.y;
-    k = blockIdx.z;
+    const unsigned ny = ((unsigned)g.ext[1] + kBlockY - 1) / kBlockY;
+    const unsigned b = blockIdx.x - nf, bx = b / ny;  // (1D: ny = 1)
+    i = bx * blockDim.x + threadIdx.x;
+    j = (b - bx * ny) * blockDim.y + threadIdx.y;
+    k = blockIdx.y;
     if (i >= g.ext[0] || j >= g.ext[1]) return false;
     i -= g.G[0];
     j -= g.G[1];
@@ -72,13 +84,122 @@ __device__ __forceinline__ int loff(const Grid &g, int i, int j, int k)
     return (int)g.origin + k * (int)g.sz + j * (int)g.sy + i;
 }
 
+// A set of ncomp arrays (base + q*stride) with per-component staggering
+// masks (bit d set = half node along axis d), e.g. Jx,Jy,Jz or rho.
+struct FoldSet {
+    int ncomp;
+    long long stride;
+    int mask[3];
+};
+
+// The fold of every axis at once.  Along a
+// periodic axis what was deposited into a ghost belongs to its image, and both
+// end up holding the sum (image + ghost, fixed order: x first); along an
+// absorbing axis what was deposited outside the physical range leaves the
+// domain and is discarded.  One thread per root cell: its coordinate along a
+// periodic axis lies in [0, N), along another anywhere in the padded range,
+// and along at least one axis it is in the shell that has work (the first such
+// axis owns it).
+struct FoldGrid {
+    int shell[3], rest[3];   // roots per axis in and outside the shell
+    unsigned first[4];       // first thread of each axis' share
+};
+
+__device__ __forceinline__ int shell_at(const Grid &g, int d, int u)
+{
+    if (g.bc[d] == PERIODIC) return u < g.G[d] ? u : g.n[d] - 2 * g.G[d] + u;
+    return u < g.G[d] ? u - g.G[d] : g.n[d] + (u - g.G[d]);
+}
+__device__ __forceinline__ int rest_at(const Grid &g, int d, int u) { return g.bc[d] == PERIODIC ? u + g.G[d] : u; }
+
+template <typename R, int DIM>
+__device__ __forceinline__ void fold_root(R *base, const FoldSet &fs, const Grid &g, const FoldGrid &fg, unsigned t)
+{
+    int d = 0;
+    unsigned u = t;
+#pragma unroll
+    for (int a = 1; a < DIM; a++)
+        if (t >= fg.first[a]) {
+            d = a;
+            u = t - fg.first[a];
+        }
+    int p[3] = {0, 0, 0}, step[3] = {0, 0, 0};  // step: to the partner along a periodic axis
+#pragma unroll
+    for (int a = 0; a < DIM; a++) {
+        const int in = fg.shell[a], out = fg.rest[a];
+        const unsigned m = a == d ? in : (a < d ? out : in + out);
+        const int v = (int)(u % m);
+        u /= m;
+        // (past the owning axis: the shell's roots, then the others)
+        p[a] = a == d || (a > d && v < in) ? shell_at(g, a, v) : rest_at(g, a, a > d ? v - in : v);
+        if (g.bc[a] == PERIODIC) step[a] = p[a] < g.G[a] ? g.n[a] : (p[a] >= g.n[a] - g.G[a] ? -g.n[a] : 0);
+    }
+    const int s[3] = {1, (int)g.sy, (int)g.sz};
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        if (q >= fs.ncomp) break;
+        bool gone = false;
+#pragma unroll
+        for (int a = 0; a < DIM; a++)
+            if (g.bc[a] != PERIODIC) gone |= p[a] < 0 || p[a] > (((fs.mask[q] >> a) & 1) ? g.n[a] - 1 : g.n[a]);
+        R *J = base + q * fs.stride + loff(g, p[0], p[1], p[2]);
+        // the root and its partners, x pairs first
+        R v[1 << DIM];
+#pragma unroll
+        for (int m = 0; m < 1 << DIM; m++) {
+            int o = 0;
+            bool is = true;
+#pragma unroll
+            for (int a = 0; a < DIM; a++)
+                if ((m >> a) & 1) {
+                    is &= step[a] != 0;
+                    o += step[a] * s[a];
+                }
+            v[m] = is ? J[o] : R(0);
+        }
+#pragma unroll
+        for (int a = 0; a < DIM; a++)
+#pragma unroll
+            for (int m = 0; m < 1 << DIM; m++)
+                if (!((m >> a) & 1) && (m & ((1 << a) - 1)) == 0 && step[a]) v[m] = v[m] + v[m | 1 << a];
+        const R sum = gone ? R(0) : v[0];
+#pragma unroll
+        for (int m = 0; m < 1 << DIM; m++) {
+            int o = 0;
+            bool is = true;
+#pragma unroll
+            for (int a = 0; a < DIM; a++)
+                if ((m >> a) & 1) {
+                    is &= step[a] != 0;
+                    o += step[a] * s[a];
+                }
+            if (is) J[o] = sum;
+        }
+    }
+}
+
+// The fold of J needs neither E nor B: its blocks lead the launch of the B half
+// step after a push (nb of them in each of the gridDim.y z layers; none: no
+// fold).  As a launch for each axis the fold cost a 2D step of 2048 x 1024
+// cells 5.3 us (periodic: 47.4 before, 42.0 now) and a small one 4 us.
+struct FoldBlocks {
+    unsigned nb;
+    FoldSet fs;
+    FoldGrid fg;
+};
+
+template <typename R, int DIM>
+__device__ __forceinline__ void fold_block(R *F, const Grid &g, const FoldBlocks &fb)
+{
+    const unsigned t = (blockIdx.y * fb.nb + blockIdx.x) * (blockDim.x * blockDim.y) + threadIdx.y * blockDim.x + threadIdx.x;
+    if (t < fb.fg.first[DIM]) fold_root<R, DIM>(F + JX * g.vol, fb.fs, g, fb.fg, t);
+}
+
 // E += h (curl B - J), once (mode 0) or twice (mode 1); then J = 0 when
 // zeroJ (J^n is no longer needed once the first half step of step n used it)
 template <typename R, int DIM>
-__global__ void __launch_bounds__(256) k_update_E(R *__restrict__ F, Grid g, R h, int twice, int zeroJ)
+__device__ __forceinline__ void cell_E(R *F, const Grid &g, R h, int twice, int zeroJ, int i, int j, int k)
 {
-    int i, j, k;
-    if (!thread_cell(g, i, j, k)) return;
     const int o = loff(g, i, j, k);
     const long long V = g.vol;
     const R *__restrict__ Bx = F + BX * V;
@@ -108,6 +229,13 @@ __global__ void __launch_bounds__(256) k_update_E(R *__restrict__ F, Grid g, R h
     if (ph.comp(EY)) { R e = Ey[o] + ay; if (twice) e += ay; Ey[o] = e; }
     if (ph.comp(EZ)) { R e = Ez[o] + az; if (twice) e += az; Ez[o] = e; }
     if (zeroJ) { Jx[o] = 0; Jy[o] = 0; Jz[o] = 0; }
+}
+
+template <typename R, int DIM>
+__global__ void __launch_bounds__(256) k_update_E(R *__restrict__ F, Grid g, R h, int twice, int zeroJ)
+{
+    int i, j, k;
+    if (thread_cell(g, i, j, k)) cell_E<R, DIM>(F, g, h, twice, zeroJ, i, j, k);
 }
 
 // incident B of the laser (a +x wave: Bz = Ey, By = -Ez) at time point q
@@ -149,10 +277,8 @@ __device__ __forceinline__ void mur_faces(R *const *B, const Grid &g, R h, const
 // s_ghost(new) = s_inner(old) + (a-1)/(a+1) (s_inner(new) - s_ghost(old)),
 // a = h/dx.  The thread owning the first inner value writes the ghost.
 template <typename R, int DIM>
-__global__ void __launch_bounds__(256) k_update_B(R *__restrict__ F, Grid g, R h, double t_new, Laser L)
+__device__ __forceinline__ void cell_B(R *F, const Grid &g, R h, const Laser &L, int i, int j, int k)
 {
-    int i, j, k;
-    if (!thread_cell(g, i, j, k)) return;
     const int o = loff(g, i, j, k);
     const long long V = g.vol;
     const R *__restrict__ Ex = F + EX * V;
@@ -185,45 +311,76 @@ __global__ void __launch_bounds__(256) k_update_B(R *__restrict__ F, Grid g, R h
     mur_faces<R, DIM>(B, g, h, L, i, j, k, o, oldv);
 }
 
+template <typename R, int DIM>
+__global__ void __launch_bounds__(256) k_update_B(R *__restrict__ F, Grid g, R h, Laser L, FoldBlocks fb)
+{
+    int i, j, k;
+    if (blockIdx.x < fb.nb) {
+        fold_block<R, DIM>(F, g, fb);
+        return;
+    }
+    if (thread_cell(g, i, j, k, fb.nb)) cell_B<R, DIM>(F, g, h, L, i, j, k);
+}
+
 // the Mur ghosts of cell (i, j, k) at offset o, after its B update (oldv:
-// its B before the update)
+// its B before the update).  Component c is staggered along the two axes
+// other than c; a ghost beyond two faces at once belongs to the cell inside
+// both, which takes the passes along the axes in their order, so the result
+// does not depend on the order of the blocks.
 template <typename R, int DIM>
 __device__ __forceinline__ void mur_faces(R *const *B, const Grid &g, R h, const Laser &L, int i, int j, int k, int o,
                                           const R *oldv)
 {
-    int p[3] = {i, j, k};
+    const int p[3] = {i, j, k};
 #pragma unroll
-    for (int d = 0; d < DIM; d++) {
-        if (g.bc[d] != ABSORB) continue;
-        const bool lo = p[d] == 0, hi = p[d] == g.n[d] - 1;
-        if (!lo && !hi) continue;
-        // the transverse position must itself be a swept (updated) one
-        bool ok = true;
-#pragma unroll
-        for (int e = 0; e < DIM; e++)
-            if (e != d && g.bc[e] == ABSORB && (p[e] < 0 || p[e] > g.n[e])) ok = false;
-        if (!ok) continue;
-        const R a = h * pic::rdx<R>(g, d);
-        const R c1 = (a - R(1)) / (a + R(1));
-        const int s = d == 0 ? 1 : (d == 1 ? (int)g.sy : (int)g.sz);
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            if (!stag(BX + c, d)) continue;
-            for (int face = 0; face < 2; face++) {
-                if ((face == 0 && !lo) || (face == 1 && !hi)) continue;
-                const int og = o + (face == 0 ? -s : s);
-                R ig_new = 0, ig_old = 0, ii_new = 0, ii_old = 0;
-                if (face == 0 && d == 0 && L.on) {
-                    ig_new = incident_B<R>(g, L, BX + c, 0, j, k);
-                    ig_old = incident_B<R>(g, L, BX + c, 1, j, k);
-                    ii_new = incident_B<R>(g, L, BX + c, 2, j, k);
-                    ii_old = incident_B<R>(g, L, BX + c, 3, j, k);
-                }
-                const R sg_old = B[c][og] - ig_old;
-                const R si_old = oldv[c] - ii_old;
-                const R si_new = B[c][o] - ii_new;
-                B[c][og] = ig_new + si_old + c1 * (si_new - sg_old);
+    for (int c = 0; c < 3; c++) {
+        const int d1 = c == 0 ? 1 : 0, d2 = c == 2 ? 1 : 2;
+        if (d1 >= DIM) continue;
+        // a swept (updated) position along the axis c, and inside the faces along the other two
+        if (c < DIM && g.bc[c] == ABSORB && (p[c] < 0 || p[c] > g.n[c])) continue;
+        const bool ab1 = g.bc[d1] == ABSORB, ab2 = d2 < DIM && g.bc[d2] == ABSORB;
+        if ((ab1 && (p[d1] < 0 || p[d1] >= g.n[d1])) || (ab2 && (p[d2] < 0 || p[d2] >= g.n[d2]))) continue;
+        const bool at1 = ab1 && (p[d1] == 0 || p[d1] == g.n[d1] - 1), at2 = ab2 && (p[d2] == 0 || p[d2] == g.n[d2] - 1);
+        if (!at1 && !at2) continue;
+        const int s1 = d1 == 0 ? 1 : (int)g.sy, s2 = d2 == 1 ? (int)g.sy : (int)g.sz;
+        const R a1 = h * pic::rdx<R>(g, d1), a2 = d2 < DIM ? h * pic::rdx<R>(g, d2) : R(0);
+        const R m1 = at1 ? (a1 - R(1)) / (a1 + R(1)) : R(0), m2 = at2 ? (a2 - R(1)) / (a2 + R(1)) : R(0);
+        R *Bc = B[c] + o;
+        for (int f1 = 0; f1 < 3; f1++) {  // faces of axis d1: low, high, none
+            if (f1 == 0 && !(ab1 && p[d1] == 0)) continue;
+            if (f1 == 1 && !(ab1 && p[d1] == g.n[d1] - 1)) continue;
+            if (f1 == 2 && !at2) continue;
+            const int o1 = f1 == 0 ? -s1 : (f1 == 1 ? s1 : 0);
+            R ig_new = 0, ig_old = 0, ii_new = 0, ii_old = 0;
+            if (f1 == 0 && d1 == 0 && L.on) {
+                ig_new = incident_B<R>(g, L, BX + c, 0, j, k);
+                ig_old = incident_B<R>(g, L, BX + c, 1, j, k);
+                ii_new = incident_B<R>(g, L, BX + c, 2, j, k);
+                ii_old = incident_B<R>(g, L, BX + c, 3, j, k);
             }
+            R g1_old = 0, g1_new = 0;
+            if (f1 < 2) {
+                g1_old = Bc[o1];
+                const R sg_old = g1_old - ig_old;
+                const R si_old = oldv[c] - ii_old;
+                const R si_new = Bc[0] - ii_new;
+                g1_new = ig_new + si_old + m1 * (si_new - sg_old);
+            }
+            for (int f2 = 0; f2 < 2; f2++) {
+                if (!(ab2 && p[d2] == (f2 == 0 ? 0 : g.n[d2] - 1))) continue;
+                const int o2 = f2 == 0 ? -s2 : s2;
+                const R g2_old = Bc[o2];
+                if (f1 == 2) {
+                    Bc[o2] = oldv[c] + m2 * (Bc[0] - g2_old);
+                    continue;
+                }
+                // beyond both faces: along d1 at the swept row (the high one), then along d2 likewise
+                R v = Bc[o1 + o2];
+                if (f2 == 1) v = g2_old + m1 * (g2_old - v);
+                if (f1 == 1) v = g1_old + m2 * (g1_new - v);
+                Bc[o1 + o2] = v;
+            }
+            if (f1 < 2) Bc[o1] = g1_new;
         }
     }
 }
@@ -249,11 +406,13 @@ __device__ __forceinline__ void unpack4(const float4 &a, float (&v)[4])
     v[3] = a.w;
 }
 
-__device__ __forceinline__ bool thread_cell4(const Grid &g, int &i, int &j, int &k)
+__device__ __forceinline__ bool thread_cell4(const Grid &g, int &i, int &j, int &k, unsigned nf = 0)
 {
-    i = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-    j = blockIdx.y * blockDim.y + threadIdx.y;
-    k = blockIdx.z;
+    const unsigned ny = ((unsigned)g.ext[1] + kBlockY - 1) / kBlockY;
+    const unsigned b = blockIdx.x - nf, bx = b / ny;
+    i = 4 * (bx * blockDim.x + threadIdx.x);
+    j = (b - bx * ny) * blockDim.y + threadIdx.y;
+    k = blockIdx.y;
     if (i >= g.ext[0] || j >= g.ext[1]) return false;
     i -= g.G[0];
     j -= g.G[1];
@@ -346,10 +505,14 @@ __global__ void __launch_bounds__(256) k_update_E4(float *__restrict__ F, Grid g
 }
 
 template <int DIM>
-__global__ void __launch_bounds__(256) k_update_B4(float *__restrict__ F, Grid g, float h, Laser L)
+__global__ void __launch_bounds__(256) k_update_B4(float *__restrict__ F, Grid g, float h, Laser L, FoldBlocks fb)
 {
     int i, j, k;
-    if (!thread_cell4(g, i, j, k)) return;
+    if (blockIdx.x < fb.nb) {
+        fold_block<float, DIM>(F, g, fb);
+        return;
+    }
+    if (!thread_cell4(g, i, j, k, fb.nb)) return;
     const int o = loff(g, i, j, k);
     const long long V = g.vol;
     const float *__restrict__ Ex = F + EX * V;
@@ -422,65 +585,38 @@ __global__ void __launch_bounds__(256) k_update_B4(float *__restrict__ F, Grid g
     }
 }
 
-// A set of ncomp arrays (base + q*stride) with per-component staggering
-// masks (bit d set = half node along axis d), e.g. Jx,Jy,Jz or rho.
-struct FoldSet {
-    int ncomp;
-    long long stride;
-    int mask[3];
+// (the charge density's, on its own)
+template <int DIM>
+__global__ void __launch_bounds__(256) k_fold(double *__restrict__ base, FoldSet fs, Grid g, FoldGrid fg)
+{
+    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < fg.first[DIM]) fold_root<double, DIM>(base, fs, g, fg, t);
+}
+
+// A 1D grid's share of a step between two pushes in one CTA: the fold, B half,
+// E (once, or twice between steps), B half, with a barrier where the launches
+// of larger grids end (256 cells: 16.6 us a step as four launches, 6.3 as one).
+struct Fields1d {
+    int fold, b1, twice, zeroJ, b2;
 };
 
-// thread grid over the padded box with axis d replaced by its 2G shell
-__device__ __forceinline__ bool shell_cell(const Grid &g, int d, int *p)
-{
-    int e[3] = {g.ext[0], g.ext[1], g.ext[2]};
-    e[d] = 2 * g.G[d];
-    p[0] = blockIdx.x * blockDim.x + threadIdx.x;
-    p[1] = blockIdx.y * blockDim.y + threadIdx.y;
-    p[2] = blockIdx.z;
-    if (p[0] >= e[0] || p[1] >= e[1]) return false;
-    for (int a = 0; a < 3; a++) p[a] -= (a == d) ? 0 : g.G[a];
-    return true;
-}
-
-// periodic fold along axis d: what was deposited into a ghost belongs to
-// its image; both end up holding the sum (image + ghost, fixed order)
 template <typename R>
-__global__ void k_fold_periodic(R *__restrict__ base, FoldSet fs, Grid g, int d)
+__global__ void __launch_bounds__(1024) k_fields_1d(R *__restrict__ F, Grid g, R h, Fields1d what, FoldSet fs, FoldGrid fg,
+                                                    Laser L1, Laser L2)
 {
-    int p[3];
-    if (!shell_cell(g, d, p)) return;
-    const int G = g.G[d], N = g.n[d];
-    const int s = p[d];
-    const int in = s < G ? s : N - 2 * G + s;
-    const int partner = in < G ? in + N : in - N;
-    p[d] = in;
-    const long long oi = goff(g, p[0], p[1], p[2]);
-    p[d] = partner;
-    const long long op = goff(g, p[0], p[1], p[2]);
-    for (int q = 0; q < fs.ncomp; q++) {
-        R *J = base + q * fs.stride;
-        R v = J[oi] + J[op];
-        J[oi] = v;
-        J[op] = v;
+    if (what.fold) {
+        for (unsigned t = threadIdx.x; t < fg.first[1]; t += blockDim.x) fold_root<R, 1>(F + JX * g.vol, fs, g, fg, t);
+        // (the update of E reads J after the next barrier)
     }
-}
-
-// absorbing axis d: what was deposited outside the physical range leaves
-// the domain and is discarded
-template <typename R>
-__global__ void k_discard_absorb(R *__restrict__ base, FoldSet fs, Grid g, int d)
-{
-    int p[3];
-    if (!shell_cell(g, d, p)) return;
-    const int G = g.G[d], N = g.n[d];
-    const int s = p[d];
-    p[d] = s < G ? s - G : N + (s - G);  // [-G,0) and [N, N+G)
-    const long long o = goff(g, p[0], p[1], p[2]);
-    for (int q = 0; q < fs.ncomp; q++) {
-        int hi = ((fs.mask[q] >> d) & 1) ? N - 1 : N;
-        if (p[d] < 0 || p[d] > hi) base[q * fs.stride + o] = 0;
+    if (what.b1) {
+        for (int i = threadIdx.x - g.G[0]; i < g.n[0] + g.G[0]; i += blockDim.x) cell_B<R, 1>(F, g, h, L1, i, 0, 0);
     }
+    __syncthreads();
+    for (int i = threadIdx.x - g.G[0]; i < g.n[0] + g.G[0]; i += blockDim.x)
+        cell_E<R, 1>(F, g, h, what.twice, what.zeroJ, i, 0, 0);
+    if (!what.b2) return;
+    __syncthreads();
+    for (int i = threadIdx.x - g.G[0]; i < g.n[0] + g.G[0]; i += blockDim.x) cell_B<R, 1>(F, g, h, L2, i, 0, 0);
 }
 
 // ---------------------------------------------------------------------
@@ -490,8 +626,8 @@ __global__ void k_discard_absorb(R *__restrict__ base, FoldSet fs, Grid g, int d
 static void grid_dims(const Grid &g, int e0, int e1, int e2, dim3 &blk, dim3 &grd)
 {
     if (g.dim == 1) blk = dim3(256, 1, 1);
-    else blk = dim3(64, 4, 1);
-    grd = dim3((unsigned)div_up(e0, blk.x), (unsigned)div_up(e1, blk.y), (unsigned)e2);
+    else blk = dim3(kBlockX, kBlockY, 1);
+    grd = dim3((unsigned)div_up(e1, blk.y) * (unsigned)div_up(e0, blk.x), (unsigned)e2);
 }
 
 static bool vec4_ok(const Grid &g) { return g.n[0] % 4 == 0 && g.G[0] % 4 == 0; }
@@ -516,58 +652,91 @@ void launch_update_E(R *F, const Grid &g, double h, bool twice, bool zeroJ, cuda
     else k_update_E<R, 3><<<n, b, 0, st>>>(F, g, (R)h, twice, zeroJ);
 }
 
-template <typename R>
-void launch_update_B(R *F, const Grid &g, double h, double t_new, const Laser &L, cudaStream_t st)
+static FoldGrid fold_grid(const Grid &g)
 {
+    FoldGrid fg{};
+    long long e[3] = {1, 1, 1};
+    for (int d = 0; d < g.dim; d++) {
+        const bool per = g.bc[d] == PERIODIC;
+        fg.shell[d] = 2 * g.G[d];
+        e[d] = per ? g.n[d] : g.n[d] + 2 * g.G[d];
+        fg.rest[d] = (int)(e[d] - fg.shell[d]);
+    }
+    for (int d = 0; d < g.dim; d++) {
+        long long m = fg.shell[d];
+        for (int a = 0; a < g.dim; a++) m *= a < d ? fg.rest[a] : (a > d ? e[a] : 1);
+        fg.first[d + 1] = fg.first[d] + (unsigned)m;  // (a grid has less than 2^31 cells)
+    }
+    return fg;
+}
+
+static FoldSet fold_j(const Grid &g) { return FoldSet{3, g.vol, {1, 2, 4}}; }
+
+template <typename R>
+void launch_update_B(R *F, const Grid &g, double h, const Laser &L, bool fold, cudaStream_t st)
+{
+    FoldBlocks fb{};
+    if (fold) {
+        fb.fs = fold_j(g);
+        fb.fg = fold_grid(g);
+        fb.nb = (unsigned)div_up(fb.fg.first[g.dim], 256ll * g.ext[2]);
+    }
     dim3 b, n;
     note_launch();
     if constexpr (sizeof(R) == 4) {
         if (vec4_ok(g)) {
             grid_dims(g, g.ext[0] / 4, g.ext[1], g.ext[2], b, n);
-            if (g.dim == 1) k_update_B4<1><<<n, b, 0, st>>>(F, g, (float)h, L);
-            else if (g.dim == 2) k_update_B4<2><<<n, b, 0, st>>>(F, g, (float)h, L);
-            else k_update_B4<3><<<n, b, 0, st>>>(F, g, (float)h, L);
+            n.x += fb.nb;
+            if (g.dim == 1) k_update_B4<1><<<n, b, 0, st>>>(F, g, (float)h, L, fb);
+            else if (g.dim == 2) k_update_B4<2><<<n, b, 0, st>>>(F, g, (float)h, L, fb);
+            else k_update_B4<3><<<n, b, 0, st>>>(F, g, (float)h, L, fb);
             return;
         }
     }
     grid_dims(g, g.ext[0], g.ext[1], g.ext[2], b, n);
-    if (g.dim == 1) k_update_B<R, 1><<<n, b, 0, st>>>(F, g, (R)h, t_new, L);
-    else if (g.dim == 2) k_update_B<R, 2><<<n, b, 0, st>>>(F, g, (R)h, t_new, L);
-    else k_update_B<R, 3><<<n, b, 0, st>>>(F, g, (R)h, t_new, L);
+    n.x += fb.nb;
+    if (g.dim == 1) k_update_B<R, 1><<<n, b, 0, st>>>(F, g, (R)h, L, fb);
+    else if (g.dim == 2) k_update_B<R, 2><<<n, b, 0, st>>>(F, g, (R)h, L, fb);
+    else k_update_B<R, 3><<<n, b, 0, st>>>(F, g, (R)h, L, fb);
 }
 
+// FP32 up to 2048 cells, FP64 up to 512: a step's field launches take (in one
+// block / in three launches, us) 6.3 / 12.5 on 256 cells, 10.5 / 12.5 on 2048,
+// 14.5 / 12.5 on 4096; in FP64 one SM's rate binds sooner, 8.4 / 12.5 on 256
+// cells, 12.1 / 12.5 on 512 (24.1 / 28.9 with a laser), 18.7 / 12.5 on 1024
 template <typename R>
-void launch_fold_set(R *base, const FoldSet &fs, const Grid &g, cudaStream_t st)
-{
-    for (int d = 0; d < g.dim; d++) {
-        int e[3] = {g.ext[0], g.ext[1], g.ext[2]};
-        e[d] = 2 * g.G[d];
-        dim3 b, n;
-        grid_dims(g, e[0], e[1], e[2], b, n);
-        note_launch();
-        if (g.bc[d] == PERIODIC) k_fold_periodic<R><<<n, b, 0, st>>>(base, fs, g, d);
-        else k_discard_absorb<R><<<n, b, 0, st>>>(base, fs, g, d);
-    }
-}
+bool fields_in_one_block(const Grid &g) { return g.dim == 1 && g.n[0] <= (sizeof(R) == 4 ? 2048 : 512); }
+template bool fields_in_one_block<float>(const Grid &);
+template bool fields_in_one_block<double>(const Grid &);
 
 template <typename R>
-void launch_fold(R *F, const Grid &g, cudaStream_t st)
+void launch_fields_1d(R *F, const Grid &g, double h, bool begin, bool last, const Laser &L1, const Laser &L2,
+                      cudaStream_t st)
 {
-    FoldSet fs{3, g.vol, {1, 2, 4}};
-    launch_fold_set<R>(F + JX * g.vol, fs, g, st);
+    Fields1d w{};
+    w.fold = w.b1 = begin ? 0 : 1;
+    w.twice = begin || last ? 0 : 1;
+    w.zeroJ = w.b2 = begin || !last ? 1 : 0;
+    note_launch();
+    k_fields_1d<R><<<1, g.ext[0] <= 256 ? 256 : 1024, 0, st>>>(F, g, (R)h, w, fold_j(g), fold_grid(g), L1, L2);
 }
+template void launch_fields_1d<float>(float *, const Grid &, double, bool, bool, const Laser &, const Laser &, cudaStream_t);
+template void launch_fields_1d<double>(double *, const Grid &, double, bool, bool, const Laser &, const Laser &, cudaStream_t);
 
 void launch_fold_rho(double *rho, const Grid &g, cudaStream_t st)
 {
-    FoldSet fs{1, 0, {0, 0, 0}};
-    launch_fold_set<double>(rho, fs, g, st);
+    const FoldSet fs{1, g.vol, {0}};
+    const FoldGrid fg = fold_grid(g);
+    const int nb = div_up(fg.first[g.dim], 256);
+    note_launch();
+    if (g.dim == 1) k_fold<1><<<nb, 256, 0, st>>>(rho, fs, g, fg);
+    else if (g.dim == 2) k_fold<2><<<nb, 256, 0, st>>>(rho, fs, g, fg);
+    else k_fold<3><<<nb, 256, 0, st>>>(rho, fs, g, fg);
 }
 
 template void launch_update_E<float>(float *, const Grid &, double, bool, bool, cudaStream_t);
 template void launch_update_E<double>(double *, const Grid &, double, bool, bool, cudaStream_t);
-template void launch_update_B<float>(float *, const Grid &, double, double, const Laser &, cudaStream_t);
-template void launch_update_B<double>(double *, const Grid &, double, double, const Laser &, cudaStream_t);
-template void launch_fold<float>(float *, const Grid &, cudaStream_t);
-template void launch_fold<double>(double *, const Grid &, cudaStream_t);
+template void launch_update_B<float>(float *, const Grid &, double, const Laser &, bool, cudaStream_t);
+template void launch_update_B<double>(double *, const Grid &, double, const Laser &, bool, cudaStream_t);
 
 }  // namespace pic

@@ -424,7 +424,9 @@ int pic_gather(pic_sim *sim, int sp, int64_t cap, double *out6);
 int pic_sync(pic_sim *sim);
 
 /* Phases of pic_step timed by pic_profile.  (The fold's blocks are part of the
- * fields' launches and are counted there: PIC_PHASE_FOLD stays 0.) */
+ * fields' launches and are counted there: PIC_PHASE_FOLD stays 0.  While timing
+ * is on every species' push is a launch of its own, so that it can be timed;
+ * otherwise the one-thread pushes of the QED species share one.) */
 enum { PIC_PHASE_SORT = 0, PIC_PHASE_FIELDS, PIC_PHASE_PUSH, PIC_PHASE_FOLD, PIC_NPHASE };
 
 /* Enable (1) or disable (0) per-phase timing of pic_step: CUDA events are

@@ -337,9 +337,27 @@ QedParams qed_params(pic_sim *s, int i)
     return q;
 }
 
-void push_species(pic_sim *s, int i, float *F)
+// the one-thread QED pushes of a step that go into one launch
+struct QedPushes {
+    int n = 0;
+    QedPush p[PIC_MAX_SPECIES];
+};
+
+void push_qed_pending(pic_sim *s, QedPushes &set, float *F)
+{
+    launch_push_qed_set(set.p, set.n, F, s->g, s->d_err, s->d_eabs, s->st);
+    set.n = 0;
+}
+void push_qed_pending(pic_sim *, QedPushes &, double *) {}
+
+void push_species(pic_sim *s, int i, float *F, QedPushes &set)
 {
     SpeciesState &p = s->sp[i];
+    auto one_thread = [&](const PartF32 &P, const QedParams &q, const uint32_t *first, bool photon) {
+        if (q.on && q.net) return false;  // (the network's pushes stage it in shared memory: their own launches)
+        if (P.n > 0) set.p[set.n++] = QedPush{P, push_const(s, p), q, first, photon ? 1 : 0, 0};
+        return true;
+    };
     if (p.kind == PIC_KIND_PHOTON) {
         const QedParams q = qed_params(s, i);
         const PartF32 P = view32(s, i, p.cur);
@@ -355,7 +373,7 @@ void push_species(pic_sim *s, int i, float *F)
             launch_push_photon_tile2d(P, p.tail_items, p.tail_nitems, (long long)tail_items_capacity(p.n_hi), F, s->g,
                                       push_const(s, p), q, s->d_err, s->st);
             launch_photon_resolve(q, P, s->d_err, s->st);
-        } else {
+        } else if (!one_thread(P, q, nullptr, true)) {
             launch_push_photon_f32(P, F, s->g, push_const(s, p), q, s->d_err, s->st,
                                    s->push_variant == PIC_PUSH_MLP_TC);
         }
@@ -374,9 +392,10 @@ void push_species(pic_sim *s, int i, float *F)
             else
                 launch_push_qed_tile2d(P, p.items, p.nitems, max_items, F, s->g, push_const(s, p), s->d_err,
                                        s->d_eabs, s->st, q);
-            launch_push_qed_f32(P, F, s->g, push_const(s, p), q, s->d_err, s->d_eabs, s->st,
-                                p.tile_start + s->g.ntiles);
-        } else {
+            if (!one_thread(P, q, p.tile_start + s->g.ntiles, false))
+                launch_push_qed_f32(P, F, s->g, push_const(s, p), q, s->d_err, s->d_eabs, s->st,
+                                    p.tile_start + s->g.ntiles);
+        } else if (!one_thread(P, q, nullptr, false)) {
             launch_push_qed_f32(P, F, s->g, push_const(s, p), q, s->d_err, s->d_eabs, s->st);
         }
         return;
@@ -393,7 +412,7 @@ void push_species(pic_sim *s, int i, float *F)
         launch_push_f32(view32(s, i, p.cur), F, s->g, push_const(s, p), s->d_err, s->d_eabs, s->st);
 }
 
-void push_species(pic_sim *s, int i, double *F)
+void push_species(pic_sim *s, int i, double *F, QedPushes &)
 {
     SpeciesState &p = s->sp[i];
     if (p.kind == PIC_KIND_PHOTON) {
@@ -415,17 +434,43 @@ void push_species(pic_sim *s, int i, double *F)
 template <typename R>
 void qed_spawn_views(pic_sim *s)
 {
-    auto view = [&](int i) {
+    using P_t = std::conditional_t<sizeof(R) == 8, PartF64, PartF32>;
+    auto view = [&](int i) -> P_t {
         if constexpr (sizeof(R) == 8) return view64(s, i, s->sp[i].cur);
         else return view32(s, i, s->sp[i].cur);
     };
-    uint32_t *bsum = (uint32_t *)s->sort_scratch;
     const int ph = s->qed.photon_sp, el = s->qed.electron_sp, po = s->qed.positron_sp;
-    const int dim = s->g.dim;
-    if (ph >= 0 && el >= 0 && po >= 0 && s->sp[ph].n_hi > 0) {
-        SpeciesState &P = s->sp[ph], &E = s->sp[el], &O = s->sp[po];
-        launch_spawn_pairs(view(ph), bsum, s->spawn_ctl, qed_params(s, ph), view(el), E.ev, E.d_count, E.cap, view(po),
-                           O.ev, O.d_count, O.cap, dim, s->d_err, s->st);
+    if (ph < 0) return;
+    SpawnSet<P_t> S{};
+    S.dim = s->g.dim;
+    S.ctl = s->spawn_ctl;
+    S.err = s->d_err;
+    auto target = [&](int i) { return SpawnTarget<P_t>{view(i), s->sp[i].ev, s->sp[i].d_count, s->sp[i].cap}; };
+    auto source = [&](int i) {
+        const QedParams q = qed_params(s, i);
+        S.key[0] = q.key[0];
+        S.key[1] = q.key[1];
+        S.step = q.step;
+        S.src[S.n++] = SpawnSource<P_t>{view(i), q.ev, q.evk, nullptr};
+    };
+    S.ph = target(ph);
+    SpeciesState &P = s->sp[ph];
+    if (el >= 0 && po >= 0 && P.n_hi > 0) {
+        S.pairs = 1;
+        S.el = target(el);
+        S.po = target(po);
+        source(ph);
+    }
+    for (int i = 0; i < s->nsp; i++)
+        if (s->sp[i].kind != PIC_KIND_PHOTON && s->sp[i].qed && s->sp[i].n_hi > 0) source(i);
+    launch_spawn(S, (uint32_t *)s->sort_scratch, s->st);
+    // the host's bounds: each emitter adds at most its own particles (the pairs
+    // of this step have not emitted yet), each photon a pair
+    long long emitted = 0;
+    for (int i = 0; i < s->nsp; i++)
+        if (s->sp[i].kind != PIC_KIND_PHOTON && s->sp[i].qed) emitted += s->sp[i].n_hi;
+    if (S.pairs) {
+        SpeciesState &E = s->sp[el], &O = s->sp[po];
         E.n_hi = std::min(E.cap, E.n_hi + P.n_hi);
         O.n_hi = std::min(O.cap, O.n_hi + P.n_hi);
         // the pairs land past the sorted particles (tile_start[ntiles]): the
@@ -434,17 +479,9 @@ void qed_spawn_views(pic_sim *s)
         if (!E.qed) E.items_valid = false;
         if (!O.qed) O.items_valid = false;
     }
-    if (ph < 0) return;
-    for (int i = 0; i < s->nsp; i++) {
-        SpeciesState &p = s->sp[i];
-        if (p.kind == PIC_KIND_PHOTON || !p.qed || p.n_hi == 0) continue;
-        SpeciesState &P = s->sp[ph];
-        launch_spawn_photons(view(i), bsum, s->spawn_ctl, qed_params(s, i), view(ph), P.ev, P.d_count, P.cap, dim,
-                             s->d_err, s->st);
-        P.n_hi = std::min(P.cap, P.n_hi + p.n_hi);
-        // (the photons land past the sorted ones: the photon push takes them
-        // as items of consecutive photons, the sort's work items stay valid)
-    }
+    // (the photons land past the sorted ones: the photon push takes them
+    // as items of consecutive photons, the sort's work items stay valid)
+    P.n_hi = std::min(P.cap, P.n_hi + emitted);
 }
 
 void qed_spawn(pic_sim *s)
@@ -487,6 +524,7 @@ int step_loop(pic_sim *s, int64_t nsteps)
             ph_end(s, PIC_PHASE_FIELDS);
         }
         ph_begin(s);
+        QedPushes pending;
         for (int i = 0; i < s->nsp; i++) {
             if (s->sp[i].n_hi) s->prof_push++;
             cudaEvent_t sa = nullptr;
@@ -494,7 +532,8 @@ int step_loop(pic_sim *s, int64_t nsteps)
                 cudaEventCreate(&sa);
                 cudaEventRecord(sa, s->st);
             }
-            push_species(s, i, F);
+            push_species(s, i, F, pending);
+            if (s->prof) push_qed_pending(s, pending, F);  // (a launch for each species, so that each is timed)
             if (sa) {
                 cudaEvent_t sb;
                 cudaEventCreate(&sb);
@@ -502,6 +541,7 @@ int step_loop(pic_sim *s, int64_t nsteps)
                 s->marks.push_back({PIC_NPHASE + i, sa, sb});
             }
         }
+        push_qed_pending(s, pending, F);
         qed_spawn(s);
         ph_end(s, PIC_PHASE_PUSH);
         const bool last = it == nsteps - 1;

@@ -251,10 +251,10 @@ __device__ __forceinline__ void deposit_moved(R *__restrict__ F, const Grid &g, 
     }
 }
 
-// FP32 offset drift with face crossing
-__device__ __forceinline__ void drift_f32(int &c, float &o, float d)
+// FP32 offset drift with face crossing: offset on (after a drift of less than a
+// cell) back into [0, 1) and its cell
+__device__ __forceinline__ void drift_to(int &c, float &o, float on)
 {
-    float on = o + d;
     if (on >= 1.0f) {
         on -= 1.0f;
         c += 1;
@@ -268,4 +268,5 @@ __device__ __forceinline__ void drift_f32(int &c, float &o, float d)
     }
     o = on;
 }
+__device__ __forceinline__ void drift_f32(int &c, float &o, float d) { drift_to(c, o, o + d); }
 }  // namespace pic

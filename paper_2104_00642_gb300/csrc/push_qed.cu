@@ -27,7 +27,9 @@ namespace pic {
 // first (optional, device): the particles below it are pushed by the tiled
 // kernel (the ones sorted into its work items); this launch takes the rest
 // (those appended since the sort) and owns their event flags.
-// one particle of k_push_qed_f32 (p0: the first particle it owns)
+// one particle of k_push_qed_f32 (p0: the first particle it owns).  The drifts
+// say whether their product is rounded before the sum: left to the compiler
+// that changes with the kernel around them, and with it, now and then, an event.
 template <int DIM, bool SURR>
 __device__ __forceinline__ void k_push_qed_f32_one(PartF32 &P, float *__restrict__ F, const Grid &g, const PushConst &pc, const QedParams &q, int *err, double *e_abs, const unsigned char *smem, long long p, long long p0)
 {
@@ -54,7 +56,7 @@ __device__ __forceinline__ void k_push_qed_f32_one(PartF32 &P, float *__restrict
     float u[3] = {ux, uy, uz};
     float ig = inv_gamma(ux, uy, uz);
 #pragma unroll
-    for (int d = 0; d < DIM; d++) drift_f32(c[d], o[d], pc.hdx_f[d] * u[d] * ig);
+    for (int d = 0; d < DIM; d++) drift_to(c[d], o[d], __fmaf_rn(pc.hdx_f[d] * u[d], ig, o[d]));
     const int ch[3] = {c[0], c[1], c[2]};
     const float oh[3] = {o[0], o[1], o[2]};
     int icn[3] = {0, 0, 0}, ich[3] = {0, 0, 0};
@@ -78,11 +80,11 @@ __device__ __forceinline__ void k_push_qed_f32_one(PartF32 &P, float *__restrict
     u[1] = uy;
     u[2] = uz;
 #pragma unroll
-    for (int d = 0; d < DIM; d++) drift_f32(c[d], o[d], pc.hdx_f[d] * u[d] * ig1);
+    for (int d = 0; d < DIM; d++) drift_to(c[d], o[d], __fadd_rn(o[d], __fmul_rn(pc.hdx_f[d] * u[d], ig1)));
     int c1[3] = {c[0], c[1], c[2]};
     const float o1[3] = {o[0], o[1], o[2]};
 #pragma unroll
-    for (int d = 0; d < DIM; d++) drift_f32(c[d], o[d], pc.hdx_f[d] * u[d] * ig1);
+    for (int d = 0; d < DIM; d++) drift_to(c[d], o[d], __fadd_rn(o[d], __fmul_rn(pc.hdx_f[d] * u[d], ig1)));
     int i0[3] = {0, 0, 0}, i1[3] = {0, 0, 0};
     float w0[3][3], w1[3][3];
     bool ok = true;
@@ -260,6 +262,41 @@ __global__ void __launch_bounds__(256, SURR ? 2 : 1) k_push_photon_f32(PartF32 P
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long base = (p0 / blockDim.x + blockIdx.x) * blockDim.x; base < nlive; base += stride)
         k_push_photon_f32_one<DIM, SURR>(P, F, g, pc, q, err, smem, base + threadIdx.x, p0);
+}
+
+// The one-thread pushes of a step's QED species (no network) in one launch:
+// the species' pushes are independent (each deposits into J), and for the few
+// thousand particles of a cascade each is one latency chain of about 17 us
+// whatever its size.  Side by side the three take 26 us.  Two lepton species
+// and the photons, each in code of its own.  CTAs per SM: the photons' global
+// gathers in 3D want them (200k electrons and 130k photons, 8 steps: 7.4 ms
+// with one, 5.8 with two, 5.5 with three, 5.6 with four); in 1D and 2D a third
+// spills (the cascade: 24.6, 24.5, 25.7, 26.7 ms).
+static_assert(3 * sizeof(QedPush) <= 3584, "kernel parameters");
+
+template <int DIM, bool PHOTON>
+__device__ __forceinline__ void push_qed_blocks(const QedPush &s, int b, float *F, const Grid &g, int *err, double *e_abs)
+{
+    const long long nlive = *s.P.dn, p0 = s.first ? (long long)*s.first : 0;
+    const long long stride = s.first ? (long long)s.nb * 256 : nlive;
+    PartF32 P = s.P;
+    // (first: a block-uniform stride over [first, count); else one pass)
+    for (long long base = (p0 / 256 + b) * 256; base < nlive; base += stride) {
+        if constexpr (PHOTON)
+            k_push_photon_f32_one<DIM, false>(P, F, g, s.pc, s.q, err, nullptr, base + threadIdx.x, p0);
+        else
+            k_push_qed_f32_one<DIM, false>(P, F, g, s.pc, s.q, err, e_abs, nullptr, base + threadIdx.x, p0);
+    }
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(256, DIM == 3 ? 3 : 2) k_push_qed_set(QedPush s0, QedPush s1, QedPush ph, float *__restrict__ F, Grid g,
+                                                         int *err, double *e_abs)
+{
+    const int b = blockIdx.x;
+    if (b < s0.nb) push_qed_blocks<DIM, false>(s0, b, F, g, err, e_abs);
+    else if (b < s0.nb + s1.nb) push_qed_blocks<DIM, false>(s1, b - s0.nb, F, g, err, e_abs);
+    else push_qed_blocks<DIM, true>(ph, b - s0.nb - s1.nb, F, g, err, e_abs);
 }
 
 // The photon push with the pair network on the tcgen05 tensor cores:
@@ -672,6 +709,34 @@ void launch_push_photon_f32(const PartF32 &P, const float *F, const Grid &g, con
         else if (g.dim == 2) k_push_photon_f32<2, false><<<nb, 256, 0, st>>>(P, F, g, pc, q, err, first);
         else k_push_photon_f32<3, false><<<nb, 256, 0, st>>>(P, F, g, pc, q, err, first);
     }
+}
+
+void launch_push_qed_set(QedPush *p, int n, float *F, const Grid &g, int *err, double *e_abs, cudaStream_t st)
+{
+    QedPush S[3] = {};  // two lepton species, photons
+    int used = 0, nb = 0;
+    auto flush = [&] {
+        if (nb == 0) return;
+        note_launch();
+        if (g.dim == 1) k_push_qed_set<1><<<nb, 256, 0, st>>>(S[0], S[1], S[2], F, g, err, e_abs);
+        else if (g.dim == 2) k_push_qed_set<2><<<nb, 256, 0, st>>>(S[0], S[1], S[2], F, g, err, e_abs);
+        else k_push_qed_set<3><<<nb, 256, 0, st>>>(S[0], S[1], S[2], F, g, err, e_abs);
+        for (QedPush &q : S) q = QedPush{};
+        used = nb = 0;
+    };
+    for (int k = 0; k < n; k++) {
+        if (p[k].P.n == 0) continue;
+        int at = p[k].photon ? 2 : ((used & 1) ? 1 : 0);
+        if ((used >> at) & 1) {  // (more species than places)
+            flush();
+            at = p[k].photon ? 2 : 0;
+        }
+        QedPush &s = S[at] = p[k];
+        s.nb = s.first ? (int)std::min<long long>(div_up(s.P.n + 1, 256), 152ll * 8) : div_up(s.P.n + 1, 256);
+        used |= 1 << at;
+        nb += s.nb;
+    }
+    flush();
 }
 
 }  // namespace pic

@@ -303,15 +303,15 @@ void launch_qed_eval(const QedTables &T, bool f64, int p, long long n, const dou
 
 // ---------------------------------------------------------------------
 // spawning: the events of a species are ranked in array order and the
-// children appended at the end of their species (deterministic order).  One
-// kernel sums the flags of blocks of kScanItems; its last block to arrive
-// scans the sums, reserves the children's places and moves the counts.  The
-// spawn kernel strides over the blocks of flags: a block whose scanned sums
-// show no event is skipped without reading its flags; otherwise its events
-// are listed in array order in shared memory and taken one per thread.  (Two
-// launches an emitting species; sums, their scan, the children and the count
-// used to be four, and a thread made the children of its own 16 flags one
-// after the other.)
+// children appended at the end of their species (deterministic order: the
+// pairs, then each emitting species' photons).  One kernel sums the flags of
+// blocks of kScanItems of every source; its last block to arrive scans the
+// sums, reserves the children's places and moves the counts.  The spawn kernel
+// strides over the blocks of flags: a block whose scanned sums show no event
+// is skipped without reading its flags; otherwise its events are listed in
+// array order in shared memory and taken one per thread.  (Two launches a
+// step: two an emitting species took 38 us of a 120 us step of the cascade of
+// 2000 replicas, all of it latency, now 17.)
 // ---------------------------------------------------------------------
 constexpr int kSpawnThreads = 256, kSpawnPer = kScanItems / kSpawnThreads;
 
@@ -345,66 +345,87 @@ __device__ __forceinline__ uint32_t flag_bits(const uint32_t *__restrict__ ev, l
     return bits;
 }
 
-// bsum[b] = events before block b, bsum[nb] = all of them; then the children's
-// first places ctl.base (one or two target species) and the new counts.  A
+// Source blockIdx.y: bsum[b] = events before block b, bsum[nb] = all of them;
+// then, source by source, the flags that were summed (ctl.m), the children's
+// first places (ctl.base; two target species for pairs) and the new counts.  A
 // pair is created only where both its electron and its positron find room, so
 // both counts advance by the same number.
-__global__ void __launch_bounds__(kSpawnThreads) k_flag_sums(const uint32_t *__restrict__ ev, long long m,
-                                                             const long long *__restrict__ dn, uint32_t *bsum,
-                                                             SpawnCtl *ctl, long long *count0, long long cap0,
-                                                             long long *count1, long long cap1, int *err)
+template <class P_t>
+__global__ void __launch_bounds__(kSpawnThreads) k_flag_sums(const __grid_constant__ SpawnSet<P_t> S)
 {
     __shared__ uint32_t sh[32];
     __shared__ bool last;
-    m = max(0ll, min(m, *dn));
-    const long long nb = (m + kScanItems - 1) / kScanItems;
-    for (long long b = blockIdx.x; b < nb; b += gridDim.x) {
-        const uint32_t bits = flag_bits(ev, m, b * kScanItems + (long long)threadIdx.x * kSpawnPer);
-        uint32_t tot;
-        block_excl_scan<kSpawnThreads>((uint32_t)__popc(bits), sh, tot);
-        if (threadIdx.x == 0) bsum[b] = tot;
+    {
+        const SpawnSource<P_t> &src = S.src[blockIdx.y];
+        uint32_t *bsum = src.bsum;
+        const long long m = max(0ll, min(src.p.n, *src.p.dn));
+        const long long nb = (m + kScanItems - 1) / kScanItems;
+        for (long long b = blockIdx.x; b < nb; b += gridDim.x) {
+            const uint32_t bits = flag_bits(src.ev, m, b * kScanItems + (long long)threadIdx.x * kSpawnPer);
+            uint32_t tot;
+            block_excl_scan<kSpawnThreads>((uint32_t)__popc(bits), sh, tot);
+            if (threadIdx.x == 0) bsum[b] = tot;
+        }
     }
     if (threadIdx.x == 0) {
         __threadfence();
-        last = atomicAdd(&ctl->done, 1u) == gridDim.x - 1;
+        last = atomicAdd(&S.ctl->done, 1u) == gridDim.x * gridDim.y - 1;
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    uint32_t carry = 0;
-    for (long long b0 = 0; b0 < nb; b0 += kSpawnThreads * 8) {
-        uint32_t v[8], s = 0, tot;
-        const long long i0 = b0 + threadIdx.x * 8;
+    uint32_t total[kSpawnSources];
 #pragma unroll
-        for (int k = 0; k < 8; k++) {
-            v[k] = i0 + k < nb ? __ldcg(bsum + i0 + k) : 0u;
-            s += v[k];
-        }
-        uint32_t run = carry + block_excl_scan<kSpawnThreads>(s, sh, tot);
+    for (int q = 0; q < kSpawnSources; q++) {
+        if (q >= S.n) break;
+        uint32_t *bsum = S.src[q].bsum;
+        const long long m = max(0ll, min(S.src[q].p.n, *S.src[q].p.dn));
+        const long long nb = (m + kScanItems - 1) / kScanItems;
+        uint32_t carry = 0;
+        for (long long b0 = 0; b0 < nb; b0 += kSpawnThreads * 8) {
+            uint32_t v[8], s = 0, tot;
+            const long long i0 = b0 + threadIdx.x * 8;
 #pragma unroll
-        for (int k = 0; k < 8; k++) {
-            if (i0 + k < nb) bsum[i0 + k] = run;
-            run += v[k];
+            for (int k = 0; k < 8; k++) {
+                v[k] = i0 + k < nb ? __ldcg(bsum + i0 + k) : 0u;
+                s += v[k];
+            }
+            uint32_t run = carry + block_excl_scan<kSpawnThreads>(s, sh, tot);
+#pragma unroll
+            for (int k = 0; k < 8; k++) {
+                if (i0 + k < nb) bsum[i0 + k] = run;
+                run += v[k];
+            }
+            carry += tot;
         }
-        carry += tot;
+        total[q] = carry;
+        if (threadIdx.x == 0) {
+            bsum[nb] = carry;
+            S.ctl->m[q] = m;  // (before any count moves)
+        }
     }
-    if (threadIdx.x == 0) {
-        bsum[nb] = carry;
-        long long n = carry;
-        ctl->base[0] = *count0;
-        bool over = *count0 + n > cap0;
-        long long take = min(n, cap0 - *count0);
-        if (count1) {
-            ctl->base[1] = *count1;
-            over |= *count1 + n > cap1;
-            take = min(take, cap1 - *count1);
+    if (threadIdx.x != 0) return;
+#pragma unroll
+    for (int q = 0; q < kSpawnSources; q++) {
+        if (q >= S.n) break;
+        const bool pair = q == 0 && S.pairs;
+        const SpawnTarget<P_t> &a = pair ? S.el : S.ph;
+        const long long n = total[q], n0 = *a.count;
+        S.ctl->base[q][0] = n0;
+        bool over = n0 + n > a.cap;
+        long long take = min(n, a.cap - n0);
+        if (pair) {
+            const long long n1 = *S.po.count;
+            S.ctl->base[q][1] = n1;
+            over |= n1 + n > S.po.cap;
+            take = min(take, S.po.cap - n1);
         }
-        if (over) atomicOr(err, ERR_CAPACITY);
+        if (over) atomicOr(S.err, ERR_CAPACITY);
         take = max(take, 0ll);
-        *count0 += take;
-        if (count1) *count1 += take;
-        ctl->done = 0u;
+        *a.count += take;
+        if (pair) *S.po.count += take;
     }
+    S.ctl->done = 0u;
 }
 
 // the events of block b listed in array order (their places in the block);
@@ -422,174 +443,121 @@ __device__ __forceinline__ int list_events(const uint32_t *__restrict__ ev, long
     return (int)tot;
 }
 
-__global__ void __launch_bounds__(kSpawnThreads) k_spawn_photons_f32(PartF32 parent, const uint32_t *__restrict__ bsum,
-                                    const SpawnCtl *__restrict__ ctl, long long m, QedParams q, PartF32 ph, double *ph_tau,
-                                    uint64_t *ph_id, uint32_t *ph_ev, long long ph_cap, int dim)
+// The photon emitted by particle p of src: its event data, at the parent's
+// x^{n+1}; FP32 event data are 4 floats per particle, FP64 4 doubles.
+template <class P_t>
+__device__ __forceinline__ void spawn_photon(const SpawnSet<P_t> &S, const SpawnSource<P_t> &src, long long p,
+                                             long long dst)
 {
-    __shared__ uint16_t list[kScanItems];
-    const long long base = ctl->base[0];
-    m = min(m, *parent.dn);  // (past the parents' device count: no event)
-    const long long nb = (m + kScanItems - 1) / kScanItems;
-    for (long long b = blockIdx.x; b < nb; b += gridDim.x) {
-        const int n = list_events(q.ev, m, bsum, b, list);
-        for (int e = threadIdx.x; e < n; e += kSpawnThreads) {
-            const long long p = b * kScanItems + list[e];
-            const uint32_t rank = bsum[b] + e;
-            const long long dst = base + rank;
-            if (dst >= ph_cap) continue;
-            uint32_t w[4];
-            const uint64_t pid = q.id[p];
-            philox4x32_10((uint32_t)pid, (uint32_t)(pid >> 32), q.step, QP_EMIT, q.key[0], q.key[1], w);
-            const uint64_t cid = ((uint64_t)w[3] << 32) | w[2];
-            ph.cell[dst] = parent.cell[p];  // the parent's x^{n+1}
+    const P_t &parent = src.p, &ph = S.ph.p;
+    uint32_t w[4];
+    const uint64_t pid = src.p.id[p];
+    philox4x32_10((uint32_t)pid, (uint32_t)(pid >> 32), S.step, QP_EMIT, S.key[0], S.key[1], w);
+    const uint64_t cid = ((uint64_t)w[3] << 32) | w[2];
+    ph.cell[dst] = parent.cell[p];
+    if constexpr (std::is_same_v<P_t, PartF32>) {
+        const float *evk = reinterpret_cast<const float *>(src.evk);
 #pragma unroll
-            for (int d = 0; d < 3; d++)
-                if (d < dim) ph.off[d][dst] = parent.off[d][p];  // (constant indices: the views stay in registers)
-            ph.u[0][dst] = q.evk[4 * p];
-            ph.u[1][dst] = q.evk[4 * p + 1];
-            ph.u[2][dst] = q.evk[4 * p + 2];
-            ph_id[dst] = cid;
-            ph_tau[dst] = initial_tau_f32(cid, q.key);
-            ph_ev[dst] = 0;
-        }
+        for (int d = 0; d < 3; d++)
+            if (d < S.dim) ph.off[d][dst] = parent.off[d][p];
+        ph.u[0][dst] = evk[4 * p];
+        ph.u[1][dst] = evk[4 * p + 1];
+        ph.u[2][dst] = evk[4 * p + 2];
+        ph.tau[dst] = initial_tau_f32(cid, S.key);
+    } else {
+        const double4 ed = reinterpret_cast<const double4 *>(src.evk)[p];
+#pragma unroll
+        for (int d = 0; d < 3; d++)
+            if (d < S.dim) ph.x[d][dst] = parent.x[d][p];
+        ph.u[0][dst] = ed.x;
+        ph.u[1][dst] = ed.y;
+        ph.u[2][dst] = ed.z;
+        ph.tau[dst] = initial_tau(cid, S.key);
     }
+    ph.id[dst] = cid;
+    S.ph.ev[dst] = 0;
 }
 
-__global__ void __launch_bounds__(kSpawnThreads) k_spawn_pairs_f32(PartF32 phot, const uint32_t *__restrict__ bsum, const SpawnCtl *__restrict__ ctl, long long m,
-                                  QedParams q, PartF32 el, double *el_tau, uint64_t *el_id, uint32_t *el_ev,
-                                  long long el_cap, PartF32 po, double *po_tau, uint64_t *po_id,
-                                  uint32_t *po_ev, long long po_cap, int dim)
+// The pair of photon p of src (event data: its momentum k and the positron
+// fraction v), born where the photon converted (its x^{n+1}); the photon dies.
+template <class P_t>
+__device__ __forceinline__ void spawn_pair(const SpawnSet<P_t> &S, const SpawnSource<P_t> &src, long long p, long long de,
+                                           long long dp)
+{
+    const P_t &phot = src.p, &el = S.el.p, &po = S.po.p;
+    uint32_t w[4];
+    const uint64_t pid = src.p.id[p];
+    philox4x32_10((uint32_t)pid, (uint32_t)(pid >> 32), S.step, QP_PAIR, S.key[0], S.key[1], w);
+    const uint64_t eid = ((uint64_t)w[3] << 32) | w[2], pid2 = eid + 1;
+    double kx, ky, kz, v;
+    if constexpr (std::is_same_v<P_t, PartF32>) {
+        const float *evk = reinterpret_cast<const float *>(src.evk);
+        kx = evk[4 * p], ky = evk[4 * p + 1], kz = evk[4 * p + 2], v = evk[4 * p + 3];
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            if (d >= S.dim) break;
+            el.off[d][de] = phot.off[d][p];
+            po.off[d][dp] = phot.off[d][p];
+        }
+    } else {
+        const double4 ed = reinterpret_cast<const double4 *>(src.evk)[p];
+        kx = ed.x, ky = ed.y, kz = ed.z, v = ed.w;
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            if (d >= S.dim) break;
+            el.x[d][de] = phot.x[d][p];
+            po.x[d][dp] = phot.x[d][p];
+        }
+    }
+    const double k = sqrt(kx * kx + ky * ky + kz * kz);
+    const uint32_t cell = phot.cell[p];
+    el.cell[de] = cell;
+    po.cell[dp] = cell;
+    phot.cell[p] = kDead;
+    const double ep = v * k, em = (1.0 - v) * k;  // eps_+ and eps_- (m c^2)
+    const double pm = sqrt(fmax(em * em - 1.0, 0.0)), pp = sqrt(fmax(ep * ep - 1.0, 0.0));
+    const double inv = k > 0.0 ? 1.0 / k : 0.0;
+    using R = std::remove_reference_t<decltype(*el.u[0])>;
+    el.u[0][de] = (R)(pm * kx * inv);
+    el.u[1][de] = (R)(pm * ky * inv);
+    el.u[2][de] = (R)(pm * kz * inv);
+    po.u[0][dp] = (R)(pp * kx * inv);
+    po.u[1][dp] = (R)(pp * ky * inv);
+    po.u[2][dp] = (R)(pp * kz * inv);
+    el.id[de] = eid;
+    po.id[dp] = pid2;
+    if constexpr (std::is_same_v<P_t, PartF32>) {
+        el.tau[de] = initial_tau_f32(eid, S.key);
+        po.tau[dp] = initial_tau_f32(pid2, S.key);
+    } else {
+        el.tau[de] = initial_tau(eid, S.key);
+        po.tau[dp] = initial_tau(pid2, S.key);
+    }
+    S.el.ev[de] = 0;
+    S.po.ev[dp] = 0;
+}
+
+// source blockIdx.y; the children land past every source's summed flags, so
+// the sources do not meet
+template <class P_t>
+__global__ void __launch_bounds__(kSpawnThreads) k_spawn(const __grid_constant__ SpawnSet<P_t> S)
 {
     __shared__ uint16_t list[kScanItems];
-    const long long be = ctl->base[0], bp = ctl->base[1];
-    m = min(m, *phot.dn);  // (past the photons' device count: no event)
+    const int k = blockIdx.y;
+    const SpawnSource<P_t> &src = S.src[k];
+    const bool pair = k == 0 && S.pairs;
+    const long long m = S.ctl->m[k], base = S.ctl->base[k][0], base1 = pair ? S.ctl->base[k][1] : 0;
     const long long nb = (m + kScanItems - 1) / kScanItems;
     for (long long b = blockIdx.x; b < nb; b += gridDim.x) {
-        const int n = list_events(q.ev, m, bsum, b, list);
+        const int n = list_events(src.ev, m, src.bsum, b, list);
         for (int e = threadIdx.x; e < n; e += kSpawnThreads) {
             const long long p = b * kScanItems + list[e];
-            const uint32_t rank = bsum[b] + e;
-            const long long de = be + rank, dp = bp + rank;
-            if (de >= el_cap || dp >= po_cap) continue;
-            uint32_t w[4];
-            const uint64_t pid = q.id[p];
-            philox4x32_10((uint32_t)pid, (uint32_t)(pid >> 32), q.step, QP_PAIR, q.key[0], q.key[1], w);
-            const uint64_t eid = ((uint64_t)w[3] << 32) | w[2], pid2 = eid + 1;
-            // event data: the photon's momentum k and the positron fraction v
-            const double kx = q.evk[4 * p], ky = q.evk[4 * p + 1], kz = q.evk[4 * p + 2], v = q.evk[4 * p + 3];
-            const double k = sqrt(kx * kx + ky * ky + kz * kz);
-            // the pair is born where the photon converted (its x^{n+1}); the photon dies
-            const uint32_t cell = phot.cell[p];
-#pragma unroll
-            for (int d = 0; d < 3; d++) {
-                if (d >= dim) break;
-                el.off[d][de] = phot.off[d][p];
-                po.off[d][dp] = phot.off[d][p];
+            const uint32_t rank = src.bsum[b] + e;
+            if (pair) {
+                if (base + rank < S.el.cap && base1 + rank < S.po.cap) spawn_pair(S, src, p, base + rank, base1 + rank);
+            } else if (base + rank < S.ph.cap) {
+                spawn_photon(S, src, p, base + rank);
             }
-            el.cell[de] = cell;
-            po.cell[dp] = cell;
-            phot.cell[p] = kDead;
-            const double ep = v * k, em = (1.0 - v) * k;  // eps_+ and eps_- (m c^2)
-            const double pm = sqrt(fmax(em * em - 1.0, 0.0)), pp = sqrt(fmax(ep * ep - 1.0, 0.0));
-            const double inv = k > 0.0 ? 1.0 / k : 0.0;
-            el.u[0][de] = (float)(pm * kx * inv);
-            el.u[1][de] = (float)(pm * ky * inv);
-            el.u[2][de] = (float)(pm * kz * inv);
-            po.u[0][dp] = (float)(pp * kx * inv);
-            po.u[1][dp] = (float)(pp * ky * inv);
-            po.u[2][dp] = (float)(pp * kz * inv);
-            el_id[de] = eid;
-            po_id[dp] = pid2;
-            el_tau[de] = initial_tau_f32(eid, q.key);
-            po_tau[dp] = initial_tau_f32(pid2, q.key);
-            el_ev[de] = 0;
-            po_ev[dp] = 0;
-        }
-    }
-}
-
-// FP64 plain form: absolute positions, event data as 4 doubles per particle
-__global__ void __launch_bounds__(kSpawnThreads) k_spawn_photons_f64(PartF64 parent, const uint32_t *__restrict__ bsum,
-                                    const SpawnCtl *__restrict__ ctl, long long m, QedParams q, PartF64 ph, double *ph_tau,
-                                    uint64_t *ph_id, uint32_t *ph_ev, long long ph_cap, int dim)
-{
-    __shared__ uint16_t list[kScanItems];
-    const long long base = ctl->base[0];
-    m = min(m, *parent.dn);  // (past the parents' device count: no event)
-    const long long nb = (m + kScanItems - 1) / kScanItems;
-    for (long long b = blockIdx.x; b < nb; b += gridDim.x) {
-        const int n = list_events(q.ev, m, bsum, b, list);
-        for (int e = threadIdx.x; e < n; e += kSpawnThreads) {
-            const long long p = b * kScanItems + list[e];
-            const uint32_t rank = bsum[b] + e;
-            const long long dst = base + rank;
-            if (dst >= ph_cap) continue;
-            uint32_t w[4];
-            const uint64_t pid = q.id[p];
-            philox4x32_10((uint32_t)pid, (uint32_t)(pid >> 32), q.step, QP_EMIT, q.key[0], q.key[1], w);
-            const uint64_t cid = ((uint64_t)w[3] << 32) | w[2];
-            const double4 ed = reinterpret_cast<const double4 *>(q.evk)[p];
-            ph.cell[dst] = parent.cell[p];
-#pragma unroll
-            for (int d = 0; d < 3; d++)
-                if (d < dim) ph.x[d][dst] = parent.x[d][p];
-            ph.u[0][dst] = ed.x;
-            ph.u[1][dst] = ed.y;
-            ph.u[2][dst] = ed.z;
-            ph_id[dst] = cid;
-            ph_tau[dst] = initial_tau(cid, q.key);
-            ph_ev[dst] = 0;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kSpawnThreads) k_spawn_pairs_f64(PartF64 phot, const uint32_t *__restrict__ bsum, const SpawnCtl *__restrict__ ctl, long long m,
-                                  QedParams q, PartF64 el, double *el_tau, uint64_t *el_id, uint32_t *el_ev,
-                                  long long el_cap, PartF64 po, double *po_tau, uint64_t *po_id,
-                                  uint32_t *po_ev, long long po_cap, int dim)
-{
-    __shared__ uint16_t list[kScanItems];
-    const long long be = ctl->base[0], bp = ctl->base[1];
-    m = min(m, *phot.dn);  // (past the photons' device count: no event)
-    const long long nb = (m + kScanItems - 1) / kScanItems;
-    for (long long b = blockIdx.x; b < nb; b += gridDim.x) {
-        const int n = list_events(q.ev, m, bsum, b, list);
-        for (int e = threadIdx.x; e < n; e += kSpawnThreads) {
-            const long long p = b * kScanItems + list[e];
-            const uint32_t rank = bsum[b] + e;
-            const long long de = be + rank, dp = bp + rank;
-            if (de >= el_cap || dp >= po_cap) continue;
-            uint32_t w[4];
-            const uint64_t pid = q.id[p];
-            philox4x32_10((uint32_t)pid, (uint32_t)(pid >> 32), q.step, QP_PAIR, q.key[0], q.key[1], w);
-            const uint64_t eid = ((uint64_t)w[3] << 32) | w[2], pid2 = eid + 1;
-            const double4 ed = reinterpret_cast<const double4 *>(q.evk)[p];
-            const double k = sqrt(ed.x * ed.x + ed.y * ed.y + ed.z * ed.z);
-            const uint32_t cell = phot.cell[p];
-#pragma unroll
-            for (int d = 0; d < 3; d++) {
-                if (d >= dim) break;
-                el.x[d][de] = phot.x[d][p];
-                po.x[d][dp] = phot.x[d][p];
-            }
-            el.cell[de] = cell;
-            po.cell[dp] = cell;
-            phot.cell[p] = kDead;
-            const double ep = ed.w * k, em = (1.0 - ed.w) * k;
-            const double pm = sqrt(fmax(em * em - 1.0, 0.0)), pp = sqrt(fmax(ep * ep - 1.0, 0.0));
-            const double inv = k > 0.0 ? 1.0 / k : 0.0;
-            el.u[0][de] = pm * ed.x * inv;
-            el.u[1][de] = pm * ed.y * inv;
-            el.u[2][de] = pm * ed.z * inv;
-            po.u[0][dp] = pp * ed.x * inv;
-            po.u[1][dp] = pp * ed.y * inv;
-            po.u[2][dp] = pp * ed.z * inv;
-            el_id[de] = eid;
-            po_id[dp] = pid2;
-            el_tau[de] = initial_tau(eid, q.key);
-            po_tau[dp] = initial_tau(pid2, q.key);
-            el_ev[de] = 0;
-            po_ev[dp] = 0;
         }
     }
 }
@@ -613,56 +581,22 @@ void launch_init_qed(long long first, long long n, uint64_t id0, uint64_t *id, d
     k_init_qed<<<div_up(n, 256), 256, 0, st>>>(first, n, id0, id, tau, key[0], key[1]);
 }
 
-// block sums in bsum (scan_blocks(m) + 1 words)
-static void flag_sums(const uint32_t *ev, long long m, const long long *dn, uint32_t *bsum, SpawnCtl *ctl,
-                      long long *count0, long long cap0, long long *count1, long long cap1, int *err, cudaStream_t st)
-{
-    note_launch();
-    k_flag_sums<<<spawn_grid(m), kSpawnThreads, 0, st>>>(ev, m, dn, bsum, ctl, count0, cap0, count1, cap1, err);
-}
-
 template <class P_t>
-void launch_spawn_photons(const P_t &parent, uint32_t *bsum, SpawnCtl *ctl, const QedParams &q, const P_t &ph,
-                          uint32_t *ph_ev, long long *ph_count, long long ph_cap, int dim, int *err, cudaStream_t st)
+void launch_spawn(SpawnSet<P_t> &S, uint32_t *scratch, cudaStream_t st)
 {
-    const long long m = parent.n;
-    if (m <= 0) return;
-    flag_sums(q.ev, m, parent.dn, bsum, ctl, ph_count, ph_cap, nullptr, 0, err, st);
-    note_launch();
-    if constexpr (std::is_same_v<P_t, PartF32>)
-        k_spawn_photons_f32<<<spawn_grid(m), kSpawnThreads, 0, st>>>(parent, bsum, ctl, m, q, ph, ph.tau, ph.id, ph_ev, ph_cap,
-                                                                    dim);
-    else
-        k_spawn_photons_f64<<<spawn_grid(m), kSpawnThreads, 0, st>>>(parent, bsum, ctl, m, q, ph, ph.tau, ph.id, ph_ev, ph_cap,
-                                                                    dim);
+    if (S.n == 0) return;
+    long long most = 0;
+    for (int k = 0; k < S.n; k++) {
+        S.src[k].bsum = scratch;
+        scratch += (S.src[k].p.n + kScanItems - 1) / kScanItems + 1;
+        most = std::max(most, S.src[k].p.n);
+    }
+    const dim3 grid(spawn_grid(most), S.n);
+    note_launch(2);
+    k_flag_sums<P_t><<<grid, kSpawnThreads, 0, st>>>(S);
+    k_spawn<P_t><<<grid, kSpawnThreads, 0, st>>>(S);
 }
-
-template <class P_t>
-void launch_spawn_pairs(const P_t &phot, uint32_t *bsum, SpawnCtl *ctl, const QedParams &q, const P_t &el,
-                        uint32_t *el_ev, long long *el_count, long long el_cap, const P_t &po, uint32_t *po_ev,
-                        long long *po_count, long long po_cap, int dim, int *err, cudaStream_t st)
-{
-    const long long m = phot.n;
-    if (m <= 0) return;
-    flag_sums(q.ev, m, phot.dn, bsum, ctl, el_count, el_cap, po_count, po_cap, err, st);
-    note_launch();
-    if constexpr (std::is_same_v<P_t, PartF32>)
-        k_spawn_pairs_f32<<<spawn_grid(m), kSpawnThreads, 0, st>>>(phot, bsum, ctl, m, q, el, el.tau, el.id, el_ev, el_cap, po,
-                                                                  po.tau, po.id, po_ev, po_cap, dim);
-    else
-        k_spawn_pairs_f64<<<spawn_grid(m), kSpawnThreads, 0, st>>>(phot, bsum, ctl, m, q, el, el.tau, el.id, el_ev, el_cap, po,
-                                                                  po.tau, po.id, po_ev, po_cap, dim);
-}
-
-template void launch_spawn_photons<PartF32>(const PartF32 &, uint32_t *, SpawnCtl *, const QedParams &, const PartF32 &,
-                                            uint32_t *, long long *, long long, int, int *, cudaStream_t);
-template void launch_spawn_photons<PartF64>(const PartF64 &, uint32_t *, SpawnCtl *, const QedParams &, const PartF64 &,
-                                            uint32_t *, long long *, long long, int, int *, cudaStream_t);
-template void launch_spawn_pairs<PartF32>(const PartF32 &, uint32_t *, SpawnCtl *, const QedParams &, const PartF32 &,
-                                          uint32_t *, long long *, long long, const PartF32 &, uint32_t *, long long *,
-                                          long long, int, int *, cudaStream_t);
-template void launch_spawn_pairs<PartF64>(const PartF64 &, uint32_t *, SpawnCtl *, const QedParams &, const PartF64 &,
-                                          uint32_t *, long long *, long long, const PartF64 &, uint32_t *, long long *,
-                                          long long, int, int *, cudaStream_t);
+template void launch_spawn<PartF32>(SpawnSet<PartF32> &, uint32_t *, cudaStream_t);
+template void launch_spawn<PartF64>(SpawnSet<PartF64> &, uint32_t *, cudaStream_t);
 
 }  // namespace pic

@@ -1,5 +1,6 @@
 // qed_host.cuh -- host entry points of the QED module (qed.cu).
 #pragma once
+#include "../../include/pic.h"
 #include "push.cuh"
 #include "qed.cuh"
 
@@ -12,25 +13,55 @@ void launch_qed_eval(const QedTables &T, bool f64, int p, long long n, const dou
                      double *out, cudaStream_t st);
 void launch_init_qed(long long first, long long n, uint64_t id0, uint64_t *id, double *tau, const uint32_t *key,
                      cudaStream_t st);
-// places of a step's children (k_flag_sums): the block counter (zero between
-// launches) and the first place in each target species
+// A step's children.  Sources: the converting photons (first, when pairs), then
+// the emitting species; targets: the photon species, and the pair's two.
+constexpr int kSpawnSources = PIC_MAX_SPECIES;
+// device state: the block counter (zero between launches), and per source the
+// flags summed and the first place in each target species
 struct SpawnCtl {
     unsigned done, pad;
-    long long base[2];
+    long long m[kSpawnSources], base[kSpawnSources][2];
 };
-// the children of the flagged particles (q.ev), appended in array order;
-// bsum: scan_blocks(n) + 1 words of scratch
 template <class P_t>
-void launch_spawn_photons(const P_t &parent, uint32_t *bsum, SpawnCtl *ctl, const QedParams &q, const P_t &ph,
-                          uint32_t *ph_ev, long long *ph_count, long long ph_cap, int dim, int *err, cudaStream_t st);
+struct SpawnSource {
+    P_t p;               // (p.n: the host's bound on the count)
+    const uint32_t *ev;  // event flags
+    const void *evk;     // event data
+    uint32_t *bsum;      // set by launch_spawn
+};
 template <class P_t>
-void launch_spawn_pairs(const P_t &phot, uint32_t *bsum, SpawnCtl *ctl, const QedParams &q, const P_t &el,
-                        uint32_t *el_ev, long long *el_count, long long el_cap, const P_t &po, uint32_t *po_ev,
-                        long long *po_count, long long po_cap, int dim, int *err, cudaStream_t st);
+struct SpawnTarget {
+    P_t p;
+    uint32_t *ev;
+    long long *count, cap;
+};
+template <class P_t>
+struct SpawnSet {
+    int n, pairs, dim;
+    uint32_t key[2], step;
+    SpawnCtl *ctl;
+    int *err;
+    SpawnTarget<P_t> ph, el, po;
+    SpawnSource<P_t> src[kSpawnSources];
+};
+// the children of the flagged particles, appended in the sources' order and in
+// array order; scratch: scan_blocks(n) + 1 words per source
+template <class P_t>
+void launch_spawn(SpawnSet<P_t> &S, uint32_t *scratch, cudaStream_t st);
 void launch_push_qed_f64(const PartF64 &P, double *F, const Grid &g, const PushConst &pc, const QedParams &q,
                          int *err, double *e_abs, cudaStream_t st);
 void launch_push_photon_f64(const PartF64 &P, const double *F, const Grid &g, const PushConst &pc,
                             const QedParams &q, int *err, cudaStream_t st);
+// one species' one-thread-per-particle push with QED (photon: launch_push_photon_f32)
+struct QedPush {
+    PartF32 P;
+    PushConst pc;
+    QedParams q;
+    const uint32_t *first;
+    int photon, nb;  // nb: set by the launch
+};
+// the pushes of several species (none with a network) in one launch
+void launch_push_qed_set(QedPush *p, int n, float *F, const Grid &g, int *err, double *e_abs, cudaStream_t st);
 // (first: see k_push_qed_f32 -- nullptr pushes every particle)
 void launch_push_qed_f32(const PartF32 &P, float *F, const Grid &g, const PushConst &pc, const QedParams &q,
                          int *err, double *e_abs, cudaStream_t st, const uint32_t *first = nullptr);

@@ -138,8 +138,8 @@ __device__ __forceinline__ void k_push_qed_f32_one(PartF32 &P, float *__restrict
     if (event) reinterpret_cast<float4 *>(q.evk)[p] = evd;
 }
 
-template <int DIM, bool SURR>
-__global__ void __launch_bounds__(256, SURR ? 2 : 1) k_push_qed_f32(PartF32 P, float *__restrict__ F, Grid g, PushConst pc,
+template <int DIM>
+__global__ void __launch_bounds__(256, 2) k_push_qed_f32(PartF32 P, float *__restrict__ F, Grid g, PushConst pc,
                                                       QedParams q, int *err, double *e_abs,
                                                       const uint32_t *__restrict__ first)
 {
@@ -148,12 +148,10 @@ __global__ void __launch_bounds__(256, SURR ? 2 : 1) k_push_qed_f32(PartF32 P, f
     // (a block without particles leaves before it stages the network: the grid
     // covers the host's bound on the count)
     if (((first ? (long long)*first / blockDim.x : 0) + blockIdx.x) * blockDim.x >= nlive) return;
-    if constexpr (SURR) {
-        mlp_stage(smem, q.net, kMlpStageBytes);
-        __syncthreads();
-    }
+    mlp_stage(smem, q.net, kMlpStageBytes);
+    __syncthreads();
     if (!first) {
-        k_push_qed_f32_one<DIM, SURR>(P, F, g, pc, q, err, e_abs, smem, (long long)blockIdx.x * blockDim.x + threadIdx.x, 0);
+        k_push_qed_f32_one<DIM, true>(P, F, g, pc, q, err, e_abs, smem, (long long)blockIdx.x * blockDim.x + threadIdx.x, 0);
         return;
     }
     // the tail after the tiled kernel's particles: a block-uniform grid
@@ -162,7 +160,7 @@ __global__ void __launch_bounds__(256, SURR ? 2 : 1) k_push_qed_f32(PartF32 P, f
     const long long p0 = (long long)*first;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long base = (p0 / blockDim.x + blockIdx.x) * blockDim.x; base < nlive; base += stride)
-        k_push_qed_f32_one<DIM, SURR>(P, F, g, pc, q, err, e_abs, smem, base + threadIdx.x, p0);
+        k_push_qed_f32_one<DIM, true>(P, F, g, pc, q, err, e_abs, smem, base + threadIdx.x, p0);
 }
 
 // SURR: the pair network inside its chi range, as in k_push_qed_f32
@@ -238,8 +236,8 @@ __device__ __forceinline__ void k_push_photon_f32_one(PartF32 &P, const float *_
     if (event) reinterpret_cast<float4 *>(q.evk)[p] = evd;
 }
 
-template <int DIM, bool SURR>
-__global__ void __launch_bounds__(256, SURR ? 2 : 1) k_push_photon_f32(PartF32 P, const float *__restrict__ F, Grid g, PushConst pc,
+template <int DIM>
+__global__ void __launch_bounds__(256, 2) k_push_photon_f32(PartF32 P, const float *__restrict__ F, Grid g, PushConst pc,
                                                          QedParams q, int *err, const uint32_t *__restrict__ first)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -247,12 +245,10 @@ __global__ void __launch_bounds__(256, SURR ? 2 : 1) k_push_photon_f32(PartF32 P
     // (a block without particles leaves before it stages the network: the grid
     // covers the host's bound on the count)
     if (((first ? (long long)*first / blockDim.x : 0) + blockIdx.x) * blockDim.x >= nlive) return;
-    if constexpr (SURR) {
-        mlp_stage(smem, q.net, kMlpStageBytes);
-        __syncthreads();
-    }
+    mlp_stage(smem, q.net, kMlpStageBytes);
+    __syncthreads();
     if (!first) {
-        k_push_photon_f32_one<DIM, SURR>(P, F, g, pc, q, err, smem, (long long)blockIdx.x * blockDim.x + threadIdx.x, 0);
+        k_push_photon_f32_one<DIM, true>(P, F, g, pc, q, err, smem, (long long)blockIdx.x * blockDim.x + threadIdx.x, 0);
         return;
     }
     // the tail after the tiled kernel's particles: a block-uniform grid
@@ -261,7 +257,7 @@ __global__ void __launch_bounds__(256, SURR ? 2 : 1) k_push_photon_f32(PartF32 P
     const long long p0 = (long long)*first;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long base = (p0 / blockDim.x + blockIdx.x) * blockDim.x; base < nlive; base += stride)
-        k_push_photon_f32_one<DIM, SURR>(P, F, g, pc, q, err, smem, base + threadIdx.x, p0);
+        k_push_photon_f32_one<DIM, true>(P, F, g, pc, q, err, smem, base + threadIdx.x, p0);
 }
 
 // The one-thread pushes of a step's QED species (no network) in one launch:
@@ -304,7 +300,7 @@ __global__ void __launch_bounds__(256, DIM == 3 ? 3 : 2) k_push_qed_set(QedPush 
 // to the device count, so that the dead slots get a zero flag);
 // the network is evaluated by the whole CTA (mlp_eval_cta: one row per
 // thread, accumulators in tensor memory) for every tile with a photon in
-// its chi range.  Everything else is k_push_photon_f32<DIM, true>.  (On the
+// its chi range.  Everything else is k_push_photon_f32<DIM>.  (On the
 // QED collision it runs at the speed of the warp-level kernel, 2 % behind:
 // the network's cost is its per-row SiLU and FP32 work, which both share;
 // the push uses it when asked for, PIC_PUSH_MLP_TC.)
@@ -661,16 +657,10 @@ void launch_push_qed_f32(const PartF32 &P, float *F, const Grid &g, const PushCo
     if (P.n == 0) return;
     note_launch();
     const int nb = first ? (int)std::min<long long>(div_up(P.n + 1, 256), 152ll * 8) : div_up(P.n + 1, 256);
-    if (q.on && q.net) {
-        const int sm = kMlpStageBytes;
-        if (g.dim == 1) k_push_qed_f32<1, true><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, e_abs, first);
-        else if (g.dim == 2) k_push_qed_f32<2, true><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, e_abs, first);
-        else k_push_qed_f32<3, true><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, e_abs, first);
-    } else {
-        if (g.dim == 1) k_push_qed_f32<1, false><<<nb, 256, 0, st>>>(P, F, g, pc, q, err, e_abs, first);
-        else if (g.dim == 2) k_push_qed_f32<2, false><<<nb, 256, 0, st>>>(P, F, g, pc, q, err, e_abs, first);
-        else k_push_qed_f32<3, false><<<nb, 256, 0, st>>>(P, F, g, pc, q, err, e_abs, first);
-    }
+    const int sm = kMlpStageBytes;
+    if (g.dim == 1) k_push_qed_f32<1><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, e_abs, first);
+    else if (g.dim == 2) k_push_qed_f32<2><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, e_abs, first);
+    else k_push_qed_f32<3><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, e_abs, first);
 }
 
 void launch_push_photon_f32(const PartF32 &P, const float *F, const Grid &g, const PushConst &pc,
@@ -679,7 +669,7 @@ void launch_push_photon_f32(const PartF32 &P, const float *F, const Grid &g, con
     if (P.n == 0) return;
     note_launch();
     const int nb = first ? (int)std::min<long long>(div_up(P.n + 1, 256), 152ll * 8) : div_up(P.n + 1, 256);
-    if (q.on && q.net && tc && !first) {
+    if (tc && !first) {
         const int sm = (int)mlp_tc_smem_bytes();
         static bool attr = false;
         if (!attr) {
@@ -699,15 +689,11 @@ void launch_push_photon_f32(const PartF32 &P, const float *F, const Grid &g, con
         if (g.dim == 1) k_push_photon_tc<1><<<grid, kMlpTcRows, sm, st>>>(P, F, g, pc, q, err);
         else if (g.dim == 2) k_push_photon_tc<2><<<grid, kMlpTcRows, sm, st>>>(P, F, g, pc, q, err);
         else k_push_photon_tc<3><<<grid, kMlpTcRows, sm, st>>>(P, F, g, pc, q, err);
-    } else if (q.on && q.net) {
-        const int sm = kMlpStageBytes;
-        if (g.dim == 1) k_push_photon_f32<1, true><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, first);
-        else if (g.dim == 2) k_push_photon_f32<2, true><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, first);
-        else k_push_photon_f32<3, true><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, first);
     } else {
-        if (g.dim == 1) k_push_photon_f32<1, false><<<nb, 256, 0, st>>>(P, F, g, pc, q, err, first);
-        else if (g.dim == 2) k_push_photon_f32<2, false><<<nb, 256, 0, st>>>(P, F, g, pc, q, err, first);
-        else k_push_photon_f32<3, false><<<nb, 256, 0, st>>>(P, F, g, pc, q, err, first);
+        const int sm = kMlpStageBytes;
+        if (g.dim == 1) k_push_photon_f32<1><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, first);
+        else if (g.dim == 2) k_push_photon_f32<2><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, first);
+        else k_push_photon_f32<3><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, first);
     }
 }
 

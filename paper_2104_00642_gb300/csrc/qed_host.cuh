@@ -62,6 +62,7 @@ struct QedPush {
 };
 // the pushes of several species (none with a network) in one launch
 void launch_push_qed_set(QedPush *p, int n, float *F, const Grid &g, int *err, double *e_abs, cudaStream_t st);
+// The pushes with a network (q.on, q.net).
 // (first: see k_push_qed_f32 -- nullptr pushes every particle)
 void launch_push_qed_f32(const PartF32 &P, float *F, const Grid &g, const PushConst &pc, const QedParams &q,
                          int *err, double *e_abs, cudaStream_t st, const uint32_t *first = nullptr);

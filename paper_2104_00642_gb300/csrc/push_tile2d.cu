@@ -211,7 +211,8 @@ __device__ __forceinline__ void deposit_row2d(const float *sR, int *sJ, int j, i
 //
 // Fixed point: the units of the item's current box come from its particles,
 // about 2^31 for the sum over them of the most that each can add to one node
-// (|q w v_d| times the shapes' largest values), so no node can overflow, and
+// (|q w| times the largest values of the shapes times |v_d| and what the FP32
+// offsets round a move by, see box_units), so no node can overflow, and
 // wrapped intermediate sums are exact.
 //
 // The field box of an item is one TMA tile copy (tmap: the six field
@@ -447,10 +448,11 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         // |q w v_d|: along x and y the prefix of the shape difference times the
         // other axis' shape, along z both shapes; then 1/2^31 of the sum)
         constexpr float kW = ORDER == 2 ? 0.75f : 115.0f / 192.0f, kP = ORDER == 2 ? 1.0f : 2.0f / 3.0f;
-        const float scx = box_units(sSum[0], fabsf(qw) * (kP * kW)), scy = box_units(sSum[1], fabsf(qw) * (kP * kW)),
-                    scz = box_units(sSum[2], fabsf(qw) * (kW * kW));
+        const int nk = sCnt[0], nc = sCnt[1];
+        const float scx = box_units(sSum[0], qw, nk + nc, cjx, kP * kW), scy = box_units(sSum[1], qw, nk + nc, cjy, kP * kW),
+                    scz = box_units(sSum[2], qw, 0, 0.f, kW * kW);  // (v_z itself is in the record)
         const float sjx = cjx * scx, sjy = cjy * scy, sqw = qw * scz;
-        const int nk = sCnt[0], nc = sCnt[1], Sk = deposit_rows(nk), Sc = deposit_rows(nc);
+        const int Sk = deposit_rows(nk), Sc = deposit_rows(nc);
         for (int j = next_row(&sCnt[2]); j < Sc + Sk; j = next_row(&sCnt[2])) {
             if (j < Sc) deposit_row2d<T, ORDER, AGG, true>(sR, sJ, j, Sc, nc, sjx, sjy, sqw);
             else deposit_row2d<T, ORDER, AGG, false>(sR, sJ, j - Sc, Sk, nk, sjx, sjy, sqw);

@@ -367,13 +367,14 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         // deposit phase
         // (a node's share of a particle's |q w v_d|: at most the square of the
         // largest weight, 3/4)
+        const int nk = sCnt[0], nc = sCnt[1];
         float sc[3], cj[3];
 #pragma unroll
         for (int d = 0; d < 3; d++) {
-            sc[d] = box_units(sSum[d], fabsf(pc.qw_f) * 0.5625f);
+            sc[d] = box_units(sSum[d], pc.qw_f, nk + nc, pc.cJ_f[d], 0.5625f);
             cj[d] = pc.cJ_f[d] * sc[d];
         }
-        const int nk = sCnt[0], nc = sCnt[1], Sk = deposit_rows(nk), Sc = deposit_rows(nc);
+        const int Sk = deposit_rows(nk), Sc = deposit_rows(nc);
         for (int j = next_row(&sCnt[2]); j < Sc + Sk; j = next_row(&sCnt[2])) {
             if (j < Sc) deposit_row3d<T, true>(sR, sJ, j, Sc, nc, cj);
             else deposit_row3d<T, false>(sR, sJ, j - Sc, Sk, nk, cj);

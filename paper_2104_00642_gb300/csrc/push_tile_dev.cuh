@@ -75,16 +75,21 @@ __device__ __forceinline__ void warp_sums(float *v, float (*sum)[kPushThreads / 
     }
 }
 
-// fixed-point units per unit of current for an item whose particles' sum of
-// |v_d| is in sum (per warp), each adding at most most |v_d| to a node: 2^31
-// less a margin for the roundings (at most half a unit per particle, and
-// FP32's in the sums)
-__device__ __forceinline__ float box_units(const float *sum, float most)
+// Fixed-point units per unit of current for an item of n records whose
+// particles' sum of |v_d| is in sum (per warp), each adding at most
+// shape |q w v_d| to a node: 2^31 less a margin for the roundings (at most half
+// a unit per particle, and FP32's in the sums).  What a record adds along an
+// active axis is not q w v_d but q w dx_d / dt (cj) times the difference of
+// two weights at FP32 offsets: two drifts, each rounded by up to 2^-24 cells,
+// and weights good to about 2^-22 (order 4).  For slow particles that is most
+// of the move, so every record counts with 2^-20 cells more; of a thermal
+// particle's move it is 1e-5.
+__device__ __forceinline__ float box_units(const float *sum, float qw, int n, float cj, float shape)
 {
     float v = 0.f;
 #pragma unroll
     for (int w = 0; w < kPushThreads / 32; w++) v += sum[w];
-    return 2.14e9f / fmaxf(most * v, 1e-28f);
+    return 2.14e9f / fmaxf(shape * fmaf(fabsf(qw), v, (float)n * fabsf(cj * 9.5367432e-7f)), 1e-28f);
 }
 
 // the deposit phase's rows of 32 records (an odd number: see deposit_row2d),

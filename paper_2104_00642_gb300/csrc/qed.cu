@@ -367,6 +367,8 @@ __global__ void __launch_bounds__(kSpawnThreads) k_flag_sums(const __grid_consta
             if (threadIdx.x == 0) bsum[b] = tot;
         }
     }
+    // (all of the block has read its source's count: the last block moves it)
+    __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         last = atomicAdd(&S.ctl->done, 1u) == gridDim.x * gridDim.y - 1;
@@ -404,6 +406,9 @@ __global__ void __launch_bounds__(kSpawnThreads) k_flag_sums(const __grid_consta
             S.ctl->m[q] = m;  // (before any count moves)
         }
     }
+    // (a source without a particle has no barrier in its scan: a warp that read
+    // its count after thread 0 moved it would scan alone)
+    __syncthreads();
     if (threadIdx.x != 0) return;
 #pragma unroll
     for (int q = 0; q < kSpawnSources; q++) {

@@ -168,13 +168,13 @@ __device__ __forceinline__ void deposit_row2d(const float *sR, int *sJ, int j, i
                     const float s0 = o0 ? (k >= 1 ? w0[k - 1] : 0.f) : (k < PN ? w0[k] : 0.f);
                     const float s1 = o1 ? (k >= 1 ? w1[k - 1] : 0.f) : (k < PN ? w1[k] : 0.f);
                     S0[d][k] = s0;
-                    dS[d][k] = s1 - s0;
+                    dS[d][k] = weight_step<ORDER == 4>(s1, s0);
                 }
             } else {
 #pragma unroll
                 for (int k = 0; k < W; k++) {
                     S0[d][k] = w0[k];
-                    dS[d][k] = w1[k] - w0[k];
+                    dS[d][k] = weight_step<ORDER == 4>(w1[k], w0[k]);
                 }
             }
         }
@@ -209,6 +209,12 @@ __device__ __forceinline__ void deposit_row2d(const float *sR, int *sJ, int j, i
 // 4 (262,144 particles at rest on a 128 x 128 grid) 201 us on the
 // one-thread-per-particle kernel -> 39 us.
 //
+// Order 4 was the one-thread push's: it keeps that kernel's root and quotients
+// and takes the finer units (EXACT and SIGNED in push_tile_dev.cuh), so that
+// nothing is less precise than there (1 keV, 128 x 128 cells, 16 steps: E
+// 9.3e-7 off 64 bits with the fast ones, 5.4e-7 now, 6.1e-7 one thread per
+// particle), for 4 % of that case's time.
+//
 // Fixed point: the units of the item's current box come from its particles,
 // about 2^31 for the sum over them of the most that each can add to one node
 // (|q w| times the largest values of the shapes times |v_d| and what the FP32
@@ -233,7 +239,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     extern __shared__ __align__(16) float smem_raw[];
     __shared__ uint64_t mbar;
     __shared__ int sCnt[3];                      // records filed from the front (node unmoved) and the back; rows taken
-    __shared__ float sSum[3][kPushThreads / 32];  // sum of |v_d| per warp
+    __shared__ int2 sSum[3][kPushThreads / 32];  // sums of v_d per warp
     // the TMA destination starts on a 128-byte boundary
     // (offset from the shared array itself, so that the compiler keeps every
     // access below in the shared address space)
@@ -309,7 +315,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         }
         // push phase (the records are filed by the warp; a warp without
         // particles skips its passes)
-        float vsum[3] = {0.f, 0.f, 0.f};
+        float vsum[3] = {0.f, 0.f, 0.f}, vabs[3] = {0.f, 0.f, 0.f};
         for (uint32_t pbase = m.start + 32 * warp; pbase < pend; pbase += kPushThreads, p += kPushThreads) {
             const uint32_t cp = ncell;
             float ux = nst[2], uy = nst[3], uz = nst[4];
@@ -325,7 +331,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             if (act) {
                 int dummy;
                 unpack_cell(g, cp, c[0], c[1], dummy);
-                float ig = inv_gamma_fast(ux, uy, uz);
+                float ig = inv_gamma_tile<ORDER == 4>(ux, uy, uz);
                 drift_sel_f32(c[0], o[0], hdx0, ux, ig);
                 drift_sel_f32(c[1], o[1], hdx1, uy, ig);
                 oh[0] = o[0];
@@ -339,8 +345,8 @@ __global__ void __launch_bounds__(kPushThreads, 3)
                 if (gin) gather2d<ORDER>(sF, B::N, B::WX, bx0, by0, icn, wn, ich, wh, eb);
                 else gather2d<ORDER>(Fg, V, rs, 0, 0, icn, wn, ich, wh, eb);
                 if (pc.pusher) vay<float>(ux, uy, uz, k * eb[0], k * eb[1], k * eb[2], k * eb[3], k * eb[4], k * eb[5]);
-                else boris_fast(ux, uy, uz, k * eb[0], k * eb[1], k * eb[2], k * eb[3], k * eb[4], k * eb[5]);
-                ig1 = inv_gamma_fast(ux, uy, uz);
+                else boris_tile<ORDER == 4>(ux, uy, uz, k * eb[0], k * eb[1], k * eb[2], k * eb[3], k * eb[4], k * eb[5]);
+                ig1 = inv_gamma_tile<ORDER == 4>(ux, uy, uz);
                 drift_sel_f32(c[0], o[0], hdx0, ux, ig1);
                 drift_sel_f32(c[1], o[1], hdx1, uy, ig1);
                 c1[0] = c[0];
@@ -387,7 +393,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
                         const float s0 = s0u ? (a >= 1 ? w0[a - 1] : 0.f) : (a < PN ? w0[a] : 0.f);
                         const float s1 = s1u ? (a >= 1 ? w1[a - 1] : 0.f) : (a < PN ? w1[a] : 0.f);
                         S0[d][a] = s0;
-                        dS[d][a] = s1 - s0;
+                        dS[d][a] = weight_step<ORDER == 4>(s1, s0);
                     }
                 }
                 AccGlobal acc{Fg + JX * V + (long long)u0[1] * rs + u0[0], V, rs};
@@ -412,9 +418,12 @@ __global__ void __launch_bounds__(kPushThreads, 3)
                 for (int d = 0; d < 2; d++)
                     pk |= (uint32_t)(icn[d] - H - u0[d]) << (16 + 2 * d) | (uint32_t)(i1[d] - H - u0[d]) << (17 + 2 * d);
                 sR[5 * kChunkMax + slot] = __uint_as_float(pk);
-                vsum[0] += fabsf(ux) * ig1;
-                vsum[1] += fabsf(uy) * ig1;
-                vsum[2] += fabsf(vz);
+                const float v[3] = {ux * ig1, uy * ig1, vz};
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    if (ORDER == 4) vsum[d] += v[d];
+                    vabs[d] += fabsf(v[d]);
+                }
             }
             if (!act) continue;
             // boundaries
@@ -439,7 +448,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             P.u[1][p] = uy;
             P.u[2][p] = uz;
         }
-        warp_sums(vsum, sSum);
+        warp_sums<ORDER == 4>(vabs, vsum, sSum);
         __syncthreads();
         // the next item's field box, while this one's records are deposited
         if (use_tma && threadIdx.x == 0 && it + (int)gridDim.x < nit) stage_box(items[it + gridDim.x].tile);

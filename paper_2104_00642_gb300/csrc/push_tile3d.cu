@@ -119,7 +119,7 @@ __device__ __forceinline__ void esirkepov3d_box(int *base, const float (*S0)[W],
 }
 
 // one row of the deposits (as deposit_row2d of push_tile2d.cu)
-template <int T, bool CROSS>
+template <int T, bool EXACT, bool CROSS>
 __device__ __forceinline__ void deposit_row3d(const float *sR, int *sJ, int j, int S, int n, const float *cj)
 {
     constexpr int W = CROSS ? 4 : 3;
@@ -140,7 +140,7 @@ __device__ __forceinline__ void deposit_row3d(const float *sR, int *sJ, int j, i
             const float s0 = o0 ? (k >= 1 ? w0[k - 1] : 0.f) : (k < 3 ? w0[k < 3 ? k : 0] : 0.f);
             const float s1 = o1 ? (k >= 1 ? w1[k - 1] : 0.f) : (k < 3 ? w1[k < 3 ? k : 0] : 0.f);
             S0[d][k] = s0;
-            dS[d][k] = s1 - s0;
+            dS[d][k] = weight_step<EXACT>(s1, s0);
         }
     }
     esirkepov3d_box<T, W>(sJ + (pk & 0xffffu), S0, dS, cj);
@@ -166,7 +166,7 @@ __device__ __forceinline__ void deposit_row3d(const float *sR, int *sJ, int j, i
 // afterwards on the global path (launch_push_list_f32).  Nothing of the
 // particle is written before that decision, and a warp never waits on one
 // lane's slow path.
-template <int T>
+template <int T, bool EXACT>
 __global__ void __launch_bounds__(kPushThreads, 3)
     k_push_tile3d(PartF32 P, const TileItem *__restrict__ items, const uint32_t *__restrict__ nitems,
                   float *__restrict__ F, Grid g, PushConst pc, int *err, double *e_abs, uint32_t *defer,
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     extern __shared__ __align__(16) float smem_raw[];
     __shared__ uint64_t mbar;
     __shared__ int sCnt[3];                    // records filed from the front (node unmoved) and the back; rows taken
-    __shared__ float sSum[3][kPushThreads / 32];  // sum of |v_d| per warp
+    __shared__ int2 sSum[3][kPushThreads / 32];  // sums of v_d per warp
     // the TMA destination starts on a 128-byte boundary
     // (offset from the shared array itself, so that the compiler keeps every
     // access below in the shared address space)
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             return;
         }
         // push phase (a warp without particles skips its passes)
-        float vsum[3] = {0.f, 0.f, 0.f};
+        float vsum[3] = {0.f, 0.f, 0.f}, vabs[3] = {0.f, 0.f, 0.f};
         for (uint32_t pbase = m.start + 32 * warp; pbase < pend; pbase += kPushThreads, p += kPushThreads) {
             const uint32_t cp = ncell;
             float o[3] = {nst[0], nst[1], nst[2]};
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             bool din = false, cross = false;
             if (act) {
                 unpack_cell(g, cp, c[0], c[1], c[2]);
-                const float ig = inv_gamma_fast(ux, uy, uz);
+                const float ig = inv_gamma_tile<EXACT>(ux, uy, uz);
                 const float u[3] = {ux, uy, uz};
                 int ich[3];
                 float wn[3][3], wh[3][3];
@@ -285,8 +285,8 @@ __global__ void __launch_bounds__(kPushThreads, 3)
                     float eb[6];
                     gather3d_box<T>(sF, o0, icn, wn, ich, wh, eb);
                     if (pc.pusher) vay<float>(ux, uy, uz, k * eb[0], k * eb[1], k * eb[2], k * eb[3], k * eb[4], k * eb[5]);
-                    else boris_fast(ux, uy, uz, k * eb[0], k * eb[1], k * eb[2], k * eb[3], k * eb[4], k * eb[5]);
-                    ig1 = inv_gamma_fast(ux, uy, uz);
+                    else boris_tile<EXACT>(ux, uy, uz, k * eb[0], k * eb[1], k * eb[2], k * eb[3], k * eb[4], k * eb[5]);
+                    ig1 = inv_gamma_tile<EXACT>(ux, uy, uz);
                     const float un[3] = {ux, uy, uz};
                     // Esirkepov on x^{n+1/2} -> x^{n+3/2}: the window of both end points
                     bool ok = true;
@@ -335,9 +335,12 @@ __global__ void __launch_bounds__(kPushThreads, 3)
                 pk |= (uint32_t)(icn[d] - 1 - u0[d]) << (16 + 2 * d) | (uint32_t)(i1[d] - 1 - u0[d]) << (17 + 2 * d);
             }
             sR[6 * kChunk3Max + slot] = __uint_as_float(pk);
-            vsum[0] += fabsf(ux) * ig1;
-            vsum[1] += fabsf(uy) * ig1;
-            vsum[2] += fabsf(uz) * ig1;
+            const float v[3] = {ux * ig1, uy * ig1, uz * ig1};
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                if (EXACT) vsum[d] += v[d];
+                vabs[d] += fabsf(v[d]);
+            }
             // boundaries
             int cc[3] = {c1[0], c1[1], c1[2]};
             bool dead = false;
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             P.u[1][p] = uy;
             P.u[2][p] = uz;
         }
-        warp_sums(vsum, sSum);
+        warp_sums<EXACT>(vabs, vsum, sSum);
         __syncthreads();
         // the next item's field box, while this one's records are deposited
         if (use_tma && threadIdx.x == 0 && it + (int)gridDim.x < nit) stage_box(items[it + gridDim.x].tile);
@@ -376,8 +379,8 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         }
         const int Sk = deposit_rows(nk), Sc = deposit_rows(nc);
         for (int j = next_row(&sCnt[2]); j < Sc + Sk; j = next_row(&sCnt[2])) {
-            if (j < Sc) deposit_row3d<T, true>(sR, sJ, j, Sc, nc, cj);
-            else deposit_row3d<T, false>(sR, sJ, j - Sc, Sk, nk, cj);
+            if (j < Sc) deposit_row3d<T, EXACT, true>(sR, sJ, j, Sc, nc, cj);
+            else deposit_row3d<T, EXACT, false>(sR, sJ, j - Sc, Sk, nk, cj);
         }
         __syncthreads();
         if (threadIdx.x == 0) sCnt[0] = sCnt[1] = sCnt[2] = 0;
@@ -399,20 +402,20 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     }
 }
 
-void launch_push_tile3d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
-                        float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, uint32_t *defer,
-                        uint32_t *ndefer, cudaStream_t st)
+template <bool EXACT>
+static void launch_exact(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items, float *F,
+                         const Grid &g, const PushConst &pc, int *err, double *e_abs, uint32_t *defer, uint32_t *ndefer,
+                         cudaStream_t st)
 {
-    if (P.n == 0) return;
     constexpr int T = 4;
     constexpr int smem = Box3p<T>::SMEM + 128;  // + alignment of the TMA destination
     static int nsm = 0, per_sm = 0;
     if (!per_sm) {
-        cudaFuncSetAttribute(k_push_tile3d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaFuncSetAttribute(k_push_tile3d<T, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         int dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_push_tile3d<T>, kPushThreads, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_push_tile3d<T, EXACT>, kPushThreads, smem);
         if (per_sm < 1) per_sm = 1;
     }
     // the six field components as one 4D tensor (x, y, z, component)
@@ -424,9 +427,24 @@ void launch_push_tile3d(const PartF32 &P, const TileItem *items, const uint32_t 
     if (grid < 1) grid = 1;
     cudaMemsetAsync(ndefer, 0, sizeof(uint32_t), st);
     note_launch();
-    k_push_tile3d<T><<<(int)grid, kPushThreads, smem, st>>>(P, items, nitems, F, g, pc, err, e_abs, defer, ndefer, tmap,
-                                                            tma ? 1 : 0);
+    k_push_tile3d<T, EXACT><<<(int)grid, kPushThreads, smem, st>>>(P, items, nitems, F, g, pc, err, e_abs, defer, ndefer,
+                                                                   tmap, tma ? 1 : 0);
     launch_push_list_f32(P, defer, ndefer, P.n, F, g, pc, err, e_abs, st);
+}
+
+void launch_push_tile3d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
+                        float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, uint32_t *defer,
+                        uint32_t *ndefer, cudaStream_t st)
+{
+    if (P.n == 0) return;
+    // Sizes that are not multiples of 4 were the one-thread push's: these take its
+    // root and quotients and the finer units, so that nothing of them is less
+    // precise than there (61 x 45 x 39 cells, 8 steps: E 4.1e-7 off 64 bits with
+    // the fast ones, 3.3e-7 now, 3.8e-7 one thread per particle; the case takes
+    // 1.56 ms instead of 1.54).
+    const bool whole = g.n[0] % 4 == 0 && g.n[1] % 4 == 0 && g.n[2] % 4 == 0;
+    if (whole) launch_exact<false>(P, items, nitems, max_items, F, g, pc, err, e_abs, defer, ndefer, st);
+    else launch_exact<true>(P, items, nitems, max_items, F, g, pc, err, e_abs, defer, ndefer, st);
 }
 
 bool tile3d_push_supported(const Grid &g)

@@ -64,32 +64,48 @@ __device__ __forceinline__ void drift_sel_f32(int &c, float &o, float h, float u
     c += (up ? 1 : 0) - (dn && !face ? 1 : 0);
 }
 
-// per-warp sums of |v_d| over the records a thread filed
-__device__ __forceinline__ void warp_sums(float *v, float (*sum)[kPushThreads / 32])
+// Per-warp sums of v_d over the records a thread filed, from its sums of |v_d|
+// and (SIGNED) of v_d: of the positive ones (x) and of the negative ones (y), or
+// of all |v_d| (x).  In units of 2^-20, rounded up per thread (an item's 1024
+// records stay below 2^30), so that one integer reduction a value does it.
+template <bool SIGNED>
+__device__ __forceinline__ void warp_sums(const float *vabs, const float *v, int2 (*sum)[kPushThreads / 32])
 {
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-#pragma unroll
-        for (int s = 16; s > 0; s >>= 1) v[d] += __shfl_xor_sync(0xffffffffu, v[d], s);
-        if ((threadIdx.x & 31u) == 0) sum[d][threadIdx.x >> 5] = v[d];
+        int2 t = make_int2(0, 0);
+        if constexpr (SIGNED) {
+            t.x = __reduce_add_sync(0xffffffffu, __float2int_ru((vabs[d] + v[d]) * 524288.0f));
+            t.y = __reduce_add_sync(0xffffffffu, __float2int_ru((vabs[d] - v[d]) * 524288.0f));
+        } else {
+            t.x = __reduce_add_sync(0xffffffffu, __float2int_ru(vabs[d] * 1048576.0f));
+        }
+        if ((threadIdx.x & 31u) == 0) sum[d][threadIdx.x >> 5] = t;
     }
 }
 
 // Fixed-point units per unit of current for an item of n records whose
-// particles' sum of |v_d| is in sum (per warp), each adding at most
-// shape |q w v_d| to a node: 2^31 less a margin for the roundings (at most half
-// a unit per particle, and FP32's in the sums).  What a record adds along an
-// active axis is not q w v_d but q w dx_d / dt (cj) times the difference of
-// two weights at FP32 offsets: two drifts, each rounded by up to 2^-24 cells,
-// and weights good to about 2^-22 (order 4).  For slow particles that is most
-// of the move, so every record counts with 2^-20 cells more; of a thermal
-// particle's move it is 1e-5.
-__device__ __forceinline__ float box_units(const float *sum, float qw, int n, float cj, float shape)
+// particles' sums of v_d are in sum (per warp), each adding values of the sign
+// of q w v_d, at most shape |q w v_d| to a node: a node's value lies between the
+// sums of the particles of either sign, so the larger of the two takes 2^31
+// less a margin for the roundings (at most half a unit per particle, and FP32's
+// in the sums).  In a plasma that is half the sum of all |v_d|, which does for
+// the others, and half the rounding of a node.
+//
+// What a record adds along an active axis is not q w v_d but q w dx_d / dt
+// (cj) times the difference of two weights at FP32 offsets: two drifts, each
+// rounded by up to 2^-24 cells, and weights good to about 2^-22 (order 4).  For
+// slow particles that is most of the move, so every record counts with 2^-20
+// cells more; of a thermal particle's move it is 1e-5.
+__device__ __forceinline__ float box_units(const int2 *sum, float qw, int n, float cj, float shape)
 {
-    float v = 0.f;
+    int p = 0, m = 0;
 #pragma unroll
-    for (int w = 0; w < kPushThreads / 32; w++) v += sum[w];
-    return 2.14e9f / fmaxf(shape * fmaf(fabsf(qw), v, (float)n * fabsf(cj * 9.5367432e-7f)), 1e-28f);
+    for (int w = 0; w < kPushThreads / 32; w++) {
+        p += sum[w].x;
+        m += sum[w].y;
+    }
+    return 2.14e9f / fmaxf(shape * 9.5367432e-7f * fmaf(fabsf(qw), (float)max(p, m), (float)n * fabsf(cj)), 1e-28f);
 }
 
 // the deposit phase's rows of 32 records (an odd number: see deposit_row2d),
@@ -136,6 +152,36 @@ __device__ __forceinline__ float inv_gamma_fast(float ux, float uy, float uz)
     float u2 = ux * ux + uy * uy + uz * uz;
     if (u2 < 1e8f) return rsqrtf(1.0f + u2);
     return inv_gamma_island(ux, uy, uz);
+}
+
+// The difference of an end point's weight and a start point's.  A step's end
+// point is the next step's start point, so that what its weights round off
+// cancels over the steps -- if it rounds alike in both places.  EXACT says so;
+// left to the compiler the end point's last product is contracted into the
+// difference and the roundings add up (E of a 1 keV plasma at order 4, 16
+// steps: 9.3e-7 off 64 bits instead of 5.4e-7).
+template <bool EXACT>
+__device__ __forceinline__ float weight_step(float w1, float w0)
+{
+    return EXACT ? __fsub_rn(w1, w0) : w1 - w0;
+}
+
+// 1/gamma and Boris' update of a tiled push.  EXACT: with the correctly rounded
+// root and quotients, as the one-thread pushes have them.
+template <bool EXACT>
+__device__ __forceinline__ float inv_gamma_tile(float ux, float uy, float uz)
+{
+    if constexpr (!EXACT) return inv_gamma_fast(ux, uy, uz);
+    const float u2 = ux * ux + uy * uy + uz * uz;
+    if (u2 < 1e8f) return 1.0f / sqrtf(1.0f + u2);
+    return inv_gamma_island(ux, uy, uz);
+}
+template <bool EXACT>
+__device__ __forceinline__ void boris_tile(float &ux, float &uy, float &uz, float ex, float ey, float ez, float bx,
+                                           float by, float bz)
+{
+    if constexpr (EXACT) boris<float>(ux, uy, uz, ex, ey, ez, bx, by, bz);
+    else boris_fast(ux, uy, uz, ex, ey, ez, bx, by, bz);
 }
 
 }  // namespace pic

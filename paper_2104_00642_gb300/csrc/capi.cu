@@ -1313,7 +1313,7 @@ int mlp_scratch(pic_sim *s, long long B)
         }
         S.acc = (double *)((char *)small + 128);  // kMlpValAcc doubles
     }
-    if (B <= S.B) return PIC_OK;
+    if (B <= S.rows) return PIC_OK;
     void *buf = nullptr;
     const size_t per_row = (size_t)(5 * 2 + 6 * kMlpH) * sizeof(float);
     int rc = dalloc(s, &buf, per_row * (size_t)B + mlp_partial_floats(B) * sizeof(float));
@@ -1329,7 +1329,7 @@ int mlp_scratch(pic_sim *s, long long B)
     S.XT[0] = S.X;  // (and S.T behind it)
     S.XT[1] = f + 6 * B + (size_t)6 * kMlpH * B;
     S.partials = S.XT[1] + 4 * B;
-    S.B = B;
+    S.rows = B;
     return PIC_OK;
 }
 
@@ -1446,7 +1446,7 @@ int pic_mlp_train(pic_sim *s, int p, const pic_mlp_train_opts *o, pic_mlp_report
     CK(cudaStreamSynchronize(s->st));
     MlpAdam a{iters, o->lr > 0 ? o->lr : 1e-2, o->lr_final > 0 ? o->lr_final : 1e-4, 0.9f, 0.999f, 1e-8f};
     const float w_rate = (float)(o->rate_weight > 0 ? o->rate_weight : 4.0);
-    const MlpTraining tr{s->T, p, {(uint32_t)o->seed, (uint32_t)(o->seed >> 32)}, a, w_rate};
+    const MlpTraining tr{s->T, p, {(uint32_t)o->seed, (uint32_t)(o->seed >> 32)}, a, w_rate, B};
     // one iteration per slot captured as a graph on a private stream, replayed
     // in turn
     cudaStream_t ts = nullptr;

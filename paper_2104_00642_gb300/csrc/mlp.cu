@@ -607,25 +607,25 @@ void launch_mlp_backward(const MlpImage *img, long long B, const float *X, const
 
 static MlpData data_of(const MlpNet &net, MlpScratch &S, const MlpTraining &t, int from, int add, int to)
 {
-    return {t.T, t.p, net.nrm, t.key[0], t.key[1], S.slot[from].it, add, t.a, S.slot[to], S.B, S.XT[to], S.XT[to] + 2 * S.B};
+    return {t.T, t.p, net.nrm, t.key[0], t.key[1], S.slot[from].it, add, t.a, S.slot[to], t.B, S.XT[to], S.XT[to] + 2 * S.rows};
 }
 
 void launch_mlp_data(const MlpNet &net, MlpScratch &S, const MlpTraining &t, cudaStream_t st)
 {
     note_launch();
-    k_mlp_data<<<div_up_i(S.B, 256), 256, 0, st>>>(data_of(net, S, t, 0, 0, 0));
+    k_mlp_data<<<div_up_i(t.B, 256), 256, 0, st>>>(data_of(net, S, t, 0, 0, 0));
 }
 
 void mlp_train_iteration(MlpNet &net, MlpScratch &S, const MlpTraining &t, int slot, cudaStream_t st)
 {
-    float *X = S.XT[slot], *Tg = X + 2 * S.B;
+    float *X = S.XT[slot], *Tg = X + 2 * S.rows;
     float *part = S.partials, *head = S.partials + (size_t)kWgBlocks * kOffW3;
-    launch_mlp_forward(net.img, S.B, X, S.Z, S.Y, st);
+    launch_mlp_forward(net.img, t.B, X, S.Z, S.Y, st);
     note_launch(3);
-    launch_bwd(net.img, S.B, Tg, S.Y, S.Z, S.D, head, t.w_rate, st);
-    const int nb = std::min(div_up_i(S.B, kWgRows), kWgBlocks);
-    k_mlp_wgrad<<<dim3(nb, 4), 256, 0, st>>>(S.B, X, S.Z, S.D, part, data_of(net, S, t, slot, 1, 1 - slot));
-    k_mlp_update<<<kRedBlk0 + kRedBlk1, kRedThreads, 0, st>>>(part, nb, head, (int)(S.B / 32), net.P, net.M, net.V,
+    launch_bwd(net.img, t.B, Tg, S.Y, S.Z, S.D, head, t.w_rate, st);
+    const int nb = std::min(div_up_i(t.B, kWgRows), kWgBlocks);
+    k_mlp_wgrad<<<dim3(nb, 4), 256, 0, st>>>(t.B, X, S.Z, S.D, part, data_of(net, S, t, slot, 1, 1 - slot));
+    k_mlp_update<<<kRedBlk0 + kRedBlk1, kRedThreads, 0, st>>>(part, nb, head, (int)(t.B / 32), net.P, net.M, net.V,
                                                              net.img, S.slot[slot].sched, t.a, S.loss + 1);
 }
 

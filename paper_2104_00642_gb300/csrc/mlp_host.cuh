@@ -29,13 +29,14 @@ struct MlpSlot {
     double *sched = nullptr;  // 3
 };
 
-// training scratch for a batch of B rows (B a multiple of 128)
+// training scratch for batches of up to `rows` rows (grows to the largest batch
+// so far; a launch's own batch is its argument)
 struct MlpScratch {
-    long long B = 0;
-    float *X = nullptr, *T = nullptr, *Y = nullptr;  // [B][2]
+    long long rows = 0;
+    float *X = nullptr, *T = nullptr, *Y = nullptr;  // [rows][2]
     float *XT[2] = {nullptr, nullptr};               // training: inputs and targets of the iteration in slot 0, 1
     MlpSlot slot[2];
-    MlpZ Z{}, D{};                                   // [B][64] each
+    MlpZ Z{}, D{};                                   // [rows][64] each
     float *loss = nullptr;                           // [0] this iteration, [1] the last one
     double *acc = nullptr;                           // validation accumulators (kMlpValAcc)
     float *partials = nullptr;                       // per-block / per-warp gradient partials
@@ -67,6 +68,7 @@ struct MlpTraining {
     uint32_t key[2];
     MlpAdam a;
     float w_rate;
+    long long B;  // samples an iteration (a multiple of 128)
 };
 // the samples of iteration 0 (its number is in slot 0) into slot 0
 void launch_mlp_data(const MlpNet &net, MlpScratch &S, const MlpTraining &t, cudaStream_t st);

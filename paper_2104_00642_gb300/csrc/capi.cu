@@ -215,25 +215,33 @@ void out_box(const Grid &g, long long *m)
 }
 
 // one component to and from the host in the exchange layout, staged in a
-// dense device block: s->rho (the diagnostics' array, free between them), or
-// a temporary one when rho itself leaves
+// dense device block, s->rho (the diagnostics' array, free between them)
 template <typename R>
 int copy_comp_out(pic_sim *s, const R *dev, double *host_out)
 {
     long long m[3];
     out_box(s->g, m);
-    const size_t bytes = (size_t)(m[0] * m[1] * m[2]) * sizeof(double);
-    double *stage = s->rho, *tmp = nullptr;
-    if ((const void *)dev == (const void *)s->rho) {
-        if (int rc = talloc(s, (void **)&tmp, bytes)) return rc;
-        stage = tmp;
-    }
-    field_pack<R>(dev, s->g, m, stage, s->st);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(host_out, stage, bytes, cudaMemcpyDeviceToHost, s->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
-    tfree(s, tmp);
-    if (e != cudaSuccess) return fail(s, PIC_ERR_CUDA, "field copy: %s", cudaGetErrorString(e));
+    field_pack<R>(dev, s->g, m, s->rho, s->st);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(host_out, s->rho, (size_t)(m[0] * m[1] * m[2]) * sizeof(double), cudaMemcpyDeviceToHost, s->st));
+    CK(cudaStreamSynchronize(s->st));
+    return PIC_OK;
+}
+
+// rho itself, row by row out of its padded array: there is no other block to
+// stage it in
+int copy_rho_out(pic_sim *s, double *host_out)
+{
+    const Grid &g = s->g;
+    long long m[3];
+    out_box(g, m);
+    cudaMemcpy3DParms p{};
+    p.srcPtr = make_cudaPitchedPtr(s->rho + g.origin, (size_t)g.sy * sizeof(double), (size_t)g.sy * sizeof(double), g.ext[1]);
+    p.dstPtr = make_cudaPitchedPtr(host_out, (size_t)m[0] * sizeof(double), (size_t)m[0] * sizeof(double), (size_t)m[1]);
+    p.extent = make_cudaExtent((size_t)m[0] * sizeof(double), (size_t)m[1], (size_t)m[2]);
+    p.kind = cudaMemcpyDeviceToHost;
+    CK(cudaMemcpy3DAsync(&p, s->st));
+    CK(cudaStreamSynchronize(s->st));
     return PIC_OK;
 }
 
@@ -1103,7 +1111,7 @@ int pic_fields(pic_sim *s, int comp, double *host_out)
     if (comp == PIC_RHO) {
         int rc = compute_rho(s);
         if (rc) return rc;
-        return copy_comp_out<double>(s, s->rho, host_out);
+        return copy_rho_out(s, host_out);
     }
     if (s->precision == PIC_PREC_FP64_PLAIN)
         return copy_comp_out<double>(s, (const double *)s->F + comp * s->g.vol, host_out);

@@ -188,13 +188,14 @@ __device__ __forceinline__ void boris_fp64(double &ux, double &uy, double &uz, d
 }
 
 // the cell of x in [0, n dx): floor(x / dx), divided out only where the
-// product with 1/dx lies within rounding of a cell face
+// product with 1/dx lies within rounding of a cell face (1e-7: three roundings
+// of at most 2^24 cells are below 6e-9)
 __device__ __forceinline__ int cell_fp64(double x, const Grid &g, int d)
 {
     const double q = x * g.rdx_d[d];
     int i;
     const double f = q - nearest_fp64(q - 0.5, i);  // in [0, 1]
-    if (f < 1e-9 || f > 1.0 - 1e-9) i = (int)floor(x / g.dx[d]);
+    if (f < 1e-7 || f > 1.0 - 1e-7) i = (int)floor(x / g.dx[d]);
     return i < 0 ? 0 : (i >= g.n[d] ? g.n[d] - 1 : i);
 }
 

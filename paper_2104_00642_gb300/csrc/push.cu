@@ -156,18 +156,30 @@ __device__ __forceinline__ void shape_w_fp64(double delta, double *w)
     }
 }
 
+// the node nearest to X, of two the upper one, and X less it.  (Of two by their
+// parity, a particle that goes a cell less a rounding from one half node to the
+// next would go two nodes.)
+__device__ __forceinline__ double node_fp64(double X, int &i)
+{
+    double delta = X - nearest_fp64(X, i);
+    if (__double2hiint(delta) == 0x3fe00000 && __double2loint(delta) == 0) {  // 1/2 (compared by its bits)
+        delta = -0.5;
+        i++;
+    }
+    return delta;
+}
+
 // nearest nodes and weights of both staggerings at X = x / dx
 template <int ORDER>
 __device__ __forceinline__ void axis_w_near(double X, int &icn, double *wn, int &ich, double *wh)
 {
-    shape_w_fp64<ORDER>(X - nearest_fp64(X, icn), wn);
-    const double Y = X - 0.5;  // half nodes: the nearest to X - 1/2
-    shape_w_fp64<ORDER>(Y - nearest_fp64(Y, ich), wh);
+    shape_w_fp64<ORDER>(node_fp64(X, icn), wn);
+    shape_w_fp64<ORDER>(node_fp64(X - 0.5, ich), wh);  // half nodes: the nearest to X - 1/2
 }
 template <int ORDER>
 __device__ __forceinline__ void axis_wn_near(double X, int &icn, double *wn)
 {
-    shape_w_fp64<ORDER>(X - nearest_fp64(X, icn), wn);
+    shape_w_fp64<ORDER>(node_fp64(X, icn), wn);
 }
 
 // Boris (Eqs. (13)-(16)) with the FP64 root and quotient of fp64_dev.cuh

@@ -3,10 +3,13 @@
 // positions that bracket the integer step, and the Gauss residual
 // max |div E - rho - rho_bg| (Eq. (1) in the units of Eq. (8)).
 //
-// Sums use a fixed reduction tree: a fixed grid of blocks, each reducing a
-// fixed strided set of elements in a fixed shuffle order into one partial,
-// and the block that finishes last summing the partials in index order, so
-// results do not depend on scheduling.
+// Sums use a fixed reduction tree: blocks that each reduce a fixed strided set
+// of elements in a fixed shuffle order into one partial, and the block that
+// finishes last summing the partials in index order, so results do not depend
+// on scheduling.  Nor on the number of blocks, which follows the host's bound
+// on the elements: as long as it is below kRedBlocks a thread has one element
+// at most, its block's partial is the same whatever the grid, and the blocks
+// left out are those whose partials would be zero.
 //
 // FP64 runs at 1/73 of the FP32 rate here and bounds these kernels: the roots
 // and quotients are Newton iterations from an FP32 seed, FP32 inputs become

@@ -297,14 +297,15 @@ constexpr int kBwdSmem = kMlpTrainStageBytes + 4 * 36 * 32 * (int)sizeof(float);
 // broadcasts, its A two banks a lane (4 x 4 tiles, 16 lanes apart in j, took
 // twice the shared-memory wavefronts).
 // Each block writes its partial sums (packed parameter order, layers 0-2)
-// to its own row of `part`; k_mlp_reduce adds the rows in a fixed order.
-constexpr int kWgRows = 64;
-constexpr int kWgBlocks = 64;
+// to its own row of `part`; k_mlp_update (k_mlp_reduce for a gradient alone)
+// adds the rows in a fixed order.
 //
 // The blocks past the three layers (blockIdx.y = 3, training) draw the next
 // iteration's samples: they need nothing of this one, and the FP64 units they
 // keep busy are idle otherwise (19 us as a kernel of its own; 10 us on a
 // second branch of the graph, for its fork and join).
+constexpr int kWgRows = 64;
+constexpr int kWgBlocks = 64;
 __global__ void __launch_bounds__(256) k_mlp_wgrad(long long B, const float *__restrict__ X, MlpZ Z, MlpZ D,
                                                    float *__restrict__ part, MlpData next)
 {

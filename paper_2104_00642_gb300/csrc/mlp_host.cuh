@@ -51,8 +51,8 @@ constexpr int kMlpValAcc = 4 + 2 * kMlpValRows;
 // floats of gradient partials a batch of B rows needs (mlp_partial_floats)
 size_t mlp_partial_floats(long long B);
 
-
-// (both staged images stay below the 48 KB default dynamic shared memory)
+// (the staged images alone stay below the 48 KB of dynamic shared memory that
+// need no opt-in; k_mlp_bwd stages more beside them and opts in)
 static_assert(kMlpTrainStageBytes <= 48 * 1024, "no opt-in needed");
 void launch_mlp_image(const float *P, MlpImage *img, cudaStream_t st);
 void launch_mlp_forward(const MlpImage *img, long long B, const float *X, const MlpZ &Z, float *Y, cudaStream_t st);

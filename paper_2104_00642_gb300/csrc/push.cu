@@ -461,12 +461,23 @@ void launch_push_f32(const PartF32 &P, float *F, const Grid &g, const PushConst 
     else k_push_f32<3, 2><<<nb, bs, 0, st>>>(P, F, g, pc, err, e_abs);
 }
 
+int sm_count()
+{
+    static const int n = [] {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        return sms > 0 ? sms : 1;
+    }();
+    return n;
+}
+
 void launch_push_list_f32(const PartF32 &P, const uint32_t *list, const uint32_t *count, long long max_n, float *F,
                           const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st)
 {
     if (max_n <= 0) return;
     note_launch();
-    const int nb = (int)std::min<long long>(div_up(max_n, 256), 152LL * 8);
+    const int nb = (int)std::min<long long>(div_up(max_n, 256), 8ll * sm_count());
     if (g.dim == 1) k_push_list_f32<1><<<nb, 256, 0, st>>>(P, list, count, F, g, pc, err, e_abs);
     else if (g.dim == 2) k_push_list_f32<2><<<nb, 256, 0, st>>>(P, list, count, F, g, pc, err, e_abs);
     else k_push_list_f32<3><<<nb, 256, 0, st>>>(P, list, count, F, g, pc, err, e_abs);

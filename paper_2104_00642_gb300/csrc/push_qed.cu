@@ -163,17 +163,15 @@ __global__ void __launch_bounds__(256, 2) k_push_qed_f32(PartF32 P, float *__res
         k_push_qed_f32_one<DIM, true>(P, F, g, pc, q, err, e_abs, smem, base + threadIdx.x, p0);
 }
 
-// SURR: the pair network inside its chi range, as in k_push_qed_f32
-// (first: as in k_push_qed_f32 -- the photons below it are the tiled kernel's)
-// one particle of k_push_photon_f32 (p0: the first particle it owns)
+// one particle of k_push_photon_f32 (SURR: the pair network inside its chi
+// range, as in k_push_qed_f32)
 template <int DIM, bool SURR>
-__device__ __forceinline__ void k_push_photon_f32_one(PartF32 &P, const float *__restrict__ F, const Grid &g, const PushConst &pc, const QedParams &q, int *err, const unsigned char *smem, long long p, long long p0)
+__device__ __forceinline__ void k_push_photon_f32_one(PartF32 &P, const float *__restrict__ F, const Grid &g, const PushConst &pc, const QedParams &q, int *err, const unsigned char *smem, long long p)
 {
-    const bool mine = p >= p0;
-    const bool live = mine && p < *P.dn && P.cell[p] != kDead;
+    const bool live = p < *P.dn && P.cell[p] != kDead;
     if (!SURR || !__any_sync(0xffffffffu, live)) {
         if (!live) {
-            if (mine && p < *P.dn) q.ev[p] = 0;  // a dead slot (flags past the device count are never read)
+            if (p < *P.dn) q.ev[p] = 0;  // a dead slot (flags past the device count are never read)
             return;
         }
     }
@@ -205,11 +203,11 @@ __device__ __forceinline__ void k_push_photon_f32_one(PartF32 &P, const float *_
         gather<float, DIM>(F, g, icn, wn, ich, wh, eb);
         qed_photon_f32<SURR>(q, smem, live, p, km, kx, ky, kz, eb, live ? q.tau[p] : 0.0, err, event, evd);
         if (SURR && !live) {
-            if (mine && p < *P.dn) q.ev[p] = 0;
+            if (p < *P.dn) q.ev[p] = 0;
             return;
         }
     } else if (SURR && !live) {
-        if (mine && p < *P.dn) q.ev[p] = 0;
+        if (p < *P.dn) q.ev[p] = 0;
         return;
     }
 #pragma unroll
@@ -238,26 +236,15 @@ __device__ __forceinline__ void k_push_photon_f32_one(PartF32 &P, const float *_
 
 template <int DIM>
 __global__ void __launch_bounds__(256, 2) k_push_photon_f32(PartF32 P, const float *__restrict__ F, Grid g, PushConst pc,
-                                                         QedParams q, int *err, const uint32_t *__restrict__ first)
+                                                         QedParams q, int *err)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const long long nlive = *P.dn;
     // (a block without particles leaves before it stages the network: the grid
     // covers the host's bound on the count)
-    if (((first ? (long long)*first / blockDim.x : 0) + blockIdx.x) * blockDim.x >= nlive) return;
+    if ((long long)blockIdx.x * blockDim.x >= *P.dn) return;
     mlp_stage(smem, q.net, kMlpStageBytes);
     __syncthreads();
-    if (!first) {
-        k_push_photon_f32_one<DIM, true>(P, F, g, pc, q, err, smem, (long long)blockIdx.x * blockDim.x + threadIdx.x, 0);
-        return;
-    }
-    // the tail after the tiled kernel's particles: a block-uniform grid
-    // stride over [first, count) (a grid over the whole range would launch a
-    // block per 256 slots only to find most of them the tiled kernel's)
-    const long long p0 = (long long)*first;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long base = (p0 / blockDim.x + blockIdx.x) * blockDim.x; base < nlive; base += stride)
-        k_push_photon_f32_one<DIM, true>(P, F, g, pc, q, err, smem, base + threadIdx.x, p0);
+    k_push_photon_f32_one<DIM, true>(P, F, g, pc, q, err, smem, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // The one-thread pushes of a step's QED species (no network) in one launch:
@@ -279,7 +266,7 @@ __device__ __forceinline__ void push_qed_blocks(const QedPush &s, int b, float *
     // (first: a block-uniform stride over [first, count); else one pass)
     for (long long base = (p0 / 256 + b) * 256; base < nlive; base += stride) {
         if constexpr (PHOTON)
-            k_push_photon_f32_one<DIM, false>(P, F, g, s.pc, s.q, err, nullptr, base + threadIdx.x, p0);
+            k_push_photon_f32_one<DIM, false>(P, F, g, s.pc, s.q, err, nullptr, base + threadIdx.x);
         else
             k_push_qed_f32_one<DIM, false>(P, F, g, s.pc, s.q, err, e_abs, nullptr, base + threadIdx.x, p0);
     }
@@ -656,7 +643,7 @@ void launch_push_qed_f32(const PartF32 &P, float *F, const Grid &g, const PushCo
 {
     if (P.n == 0) return;
     note_launch();
-    const int nb = first ? (int)std::min<long long>(div_up(P.n + 1, 256), 152ll * 8) : div_up(P.n + 1, 256);
+    const int nb = first ? (int)std::min<long long>(div_up(P.n + 1, 256), 8ll * sm_count()) : div_up(P.n + 1, 256);
     const int sm = kMlpStageBytes;
     if (g.dim == 1) k_push_qed_f32<1><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, e_abs, first);
     else if (g.dim == 2) k_push_qed_f32<2><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, e_abs, first);
@@ -664,12 +651,11 @@ void launch_push_qed_f32(const PartF32 &P, float *F, const Grid &g, const PushCo
 }
 
 void launch_push_photon_f32(const PartF32 &P, const float *F, const Grid &g, const PushConst &pc,
-                            const QedParams &q, int *err, cudaStream_t st, bool tc, const uint32_t *first)
+                            const QedParams &q, int *err, cudaStream_t st, bool tc)
 {
     if (P.n == 0) return;
     note_launch();
-    const int nb = first ? (int)std::min<long long>(div_up(P.n + 1, 256), 152ll * 8) : div_up(P.n + 1, 256);
-    if (tc && !first) {
+    if (tc) {
         const int sm = (int)mlp_tc_smem_bytes();
         static bool attr = false;
         if (!attr) {
@@ -678,22 +664,16 @@ void launch_push_photon_f32(const PartF32 &P, const float *F, const Grid &g, con
             cudaFuncSetAttribute(k_push_photon_tc<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
             attr = true;
         }
-        static int nsm = 0;
-        if (!nsm) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        }
         const long long tiles = P.n / kMlpTcRows + 1;  // slots 0..P.n
-        const int grid = (int)std::min<long long>(tiles, 4ll * nsm);
+        const int grid = (int)std::min<long long>(tiles, 4ll * sm_count());
         if (g.dim == 1) k_push_photon_tc<1><<<grid, kMlpTcRows, sm, st>>>(P, F, g, pc, q, err);
         else if (g.dim == 2) k_push_photon_tc<2><<<grid, kMlpTcRows, sm, st>>>(P, F, g, pc, q, err);
         else k_push_photon_tc<3><<<grid, kMlpTcRows, sm, st>>>(P, F, g, pc, q, err);
     } else {
-        const int sm = kMlpStageBytes;
-        if (g.dim == 1) k_push_photon_f32<1><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, first);
-        else if (g.dim == 2) k_push_photon_f32<2><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, first);
-        else k_push_photon_f32<3><<<nb, 256, sm, st>>>(P, F, g, pc, q, err, first);
+        const int sm = kMlpStageBytes, nb = div_up(P.n, 256);
+        if (g.dim == 1) k_push_photon_f32<1><<<nb, 256, sm, st>>>(P, F, g, pc, q, err);
+        else if (g.dim == 2) k_push_photon_f32<2><<<nb, 256, sm, st>>>(P, F, g, pc, q, err);
+        else k_push_photon_f32<3><<<nb, 256, sm, st>>>(P, F, g, pc, q, err);
     }
 }
 
@@ -718,7 +698,7 @@ void launch_push_qed_set(QedPush *p, int n, float *F, const Grid &g, int *err, d
             at = p[k].photon ? 2 : 0;
         }
         QedPush &s = S[at] = p[k];
-        s.nb = s.first ? (int)std::min<long long>(div_up(s.P.n + 1, 256), 152ll * 8) : div_up(s.P.n + 1, 256);
+        s.nb = s.first ? (int)std::min<long long>(div_up(s.P.n + 1, 256), 8ll * sm_count()) : div_up(s.P.n + 1, 256);
         used |= 1 << at;
         nb += s.nb;
     }

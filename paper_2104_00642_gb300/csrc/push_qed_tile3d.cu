@@ -10,6 +10,10 @@
 
 namespace pic {
 
+// this file's own boxes, gathers and deposits (those of the other tiled pushes
+// have the same names)
+namespace {
+
 // ---------------------------------------------------------------------
 // 3D: tiles of T^3 cells, the same scheme with a 3D box
 //   x: [t0-4, t0+T+4) (float4-aligned rows), y and z: [t0-3, t0+T+3);
@@ -147,6 +151,8 @@ static __device__ __noinline__ bool deposit3d_global(float *F, const Grid &g, co
     deposit_moved<float, 3, 2>(F, g, i0, w0, i1, w1, cJ, pc.qw_f * uy * ig1, pc.qw_f * uz * ig1);
     return true;
 }
+
+}  // namespace
 
 // QM (QED leptons): 1 = the Monte Carlo of Sec. IV with the tables, 2 = with
 // the surrogate network (its image after the boxes), as in the 2D kernel;

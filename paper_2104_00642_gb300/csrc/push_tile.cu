@@ -29,6 +29,10 @@ namespace pic {
 // 32 banks
 constexpr int kPSlot = 33 * (kChunk / 32);
 
+// this file's own boxes, gathers and deposits (those of the other tiled pushes
+// have the same names)
+namespace {
+
 template <int T>
 struct Box2 {
     static constexpr int WX = T + 12;  // x: [t0-4, t0+T+8), a multiple of 4 floats
@@ -112,6 +116,8 @@ struct AccGlobal {
         if (v != 0.f) atomicAdd(base + c * cs + (long long)b * rs + a, v);
     }
 };
+
+}  // namespace
 
 // With use_tma the field box of an item is one TMA tile copy (tmap: the six
 // field components as a 3D tensor, x fastest), issued by one thread and
@@ -681,8 +687,8 @@ __global__ void k_item_write(const uint32_t *__restrict__ starts, const uint32_t
 }
 
 // Particles per work item at most.  2D without QED: kChunkMax (the records
-// fit) while that leaves each of the 456 resident CTAs an item and a half,
-// less for fewer particles.  (A hot plasma of 1,048,576 particles: 59 us a
+// fit) while that leaves each of the resident CTAs (three an SM) an item and a
+// half, less for fewer particles.  (A hot plasma of 1,048,576 particles: 59 us a
 // push with items of 352, 48 with 512 or 1024; an item's fixed cost is the
 // flush of its current box, ~210 instructions a warp.)
 int tile_chunk(const Grid &g, bool qed, long long n)
@@ -692,7 +698,7 @@ int tile_chunk(const Grid &g, bool qed, long long n)
     // (order 4 spreads a particle over 25 nodes: half the particles an item
     // keep its fixed-point units as fine against them)
     for (int c = g.order == 4 ? kChunkMax / 2 : kChunkMax; c > kPushThreads; c /= 2)
-        if (2 * n >= 3ll * 456 * c) return c;
+        if (2 * n >= 9ll * sm_count() * c) return c;
     return kPushThreads;
 }
 
@@ -706,11 +712,6 @@ void build_tile_items(const uint32_t *starts, long long ntiles, int chunk, uint3
     k_item_counts<<<div_up(ntiles + 1, 256), 256, 0, st>>>(starts, ntiles, c, grain, cnt_scratch);
     scan_exclusive(cnt_scratch, cnt_scratch, ntiles + 1, scan_scratch, st);
     k_item_write<<<div_up(ntiles + 1, 256), 256, 0, st>>>(starts, cnt_scratch, ntiles, c, grain, items, nitems);
-}
-
-bool tile_push_supported(const Grid &g, int tile_edge)
-{
-    return g.dim == 2 && (1 << g.tile_log2[0]) == tile_edge && (1 << g.tile_log2[1]) == tile_edge;
 }
 
 template <int T, int QM>

@@ -1,4 +1,5 @@
-// push_tile.cuh -- tiled 2D push (push_tile.cu) and its work items.
+// push_tile.cuh -- the tiled pushes (push_tile2d.cu, push_tile3d.cu; of the QED
+// species push_tile.cu, push_qed_tile3d.cu) and their work items (push_tile.cu).
 #pragma once
 #include "push.cuh"
 #include "sort.cuh"
@@ -28,7 +29,6 @@ int tile_chunk(const Grid &g, bool qed, long long n);
 size_t tile_items_capacity(long long cap, long long ntiles);
 void build_tile_items(const uint32_t *starts, long long ntiles, int chunk, uint32_t *cnt_scratch,
                       uint32_t *scan_scratch, TileItem *items, uint32_t *nitems, cudaStream_t st);
-bool tile_push_supported(const Grid &g, int tile_edge);
 // 2D, shape orders 2 and 4 (agg: the warp-aggregated deposit, order 2); and
 // with a QED lepton species' Monte Carlo q fused in (order 2; q.on; the
 // particles appended since the sort, and their event flags, are left to
@@ -40,13 +40,12 @@ void launch_push_qed_tile2d(const PartF32 &P, const TileItem *items, const uint3
                             float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st,
                             const QedParams &q);
 // the tiled photon push (2D, FP32; tiles of 8 or 16 cells): the photons of
-// the work items, their pair Monte Carlo with q; the photons appended since
-// the sort are left to launch_push_photon_f32
+// the work items, their pair Monte Carlo with q
 void launch_push_photon_tile2d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
                                const float *F, const Grid &g, const PushConst &pc, const QedParams &q, int *err,
                                cudaStream_t st);
-// 2D photons: work items over the photons appended since the sort ([*first,
-// *P.dn), kChunk each)
+// work items for it over the photons appended since the sort ([*first, *P.dn),
+// kChunk each)
 size_t tail_items_capacity(long long cap);
 void launch_tail_items(const PartF32 &P, const uint32_t *first, const Grid &g, TileItem *items, uint32_t *nitems,
                        cudaStream_t st);

@@ -23,6 +23,10 @@
 
 namespace pic {
 
+// this file's own boxes, gathers and deposits (those of the other tiled pushes
+// have the same names)
+namespace {
+
 template <int T>
 struct Box2p {
     static constexpr int WX = T + 12;  // x: [t0-4, t0+T+8), a multiple of 4 floats
@@ -191,6 +195,8 @@ __device__ __forceinline__ void deposit_row2d(const float *sR, int *sJ, int j, i
         esirkepov2d<W>(S0, dS, sjx, sjy, jvz, acc);
     }
 }
+
+}  // namespace
 
 // One item in two phases.
 //   push:    consecutive lanes on consecutive particles -- state read and

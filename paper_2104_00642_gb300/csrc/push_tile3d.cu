@@ -8,6 +8,10 @@
 
 namespace pic {
 
+// this file's own boxes, gathers and deposits (those of the other tiled pushes
+// have the same names)
+namespace {
+
 // Tiles of T^3 cells.  The box holds x in [t0-4, t0+T+4) (float4-aligned
 // rows) and y, z in [t0-3, t0+T+4): a particle within two cells below or one
 // above its tile's faces after the half drift finds all its nodes there.  In
@@ -145,6 +149,8 @@ __device__ __forceinline__ void deposit_row3d(const float *sR, int *sJ, int j, i
     }
     esirkepov3d_box<T, W>(sJ + (pk & 0xffffu), S0, dS, cj);
 }
+
+}  // namespace
 
 // One item in the two phases of k_push_tile2d (push_tile2d.cu): push with
 // consecutive lanes on consecutive particles, then the lane-strided deposit of

@@ -1,5 +1,5 @@
-// push_tile_dev.cuh -- device helpers shared by the tiled pushes (2D in
-// push_tile.cu, 3D in push_tile3d.cu).
+// push_tile_dev.cuh -- device helpers shared by the tiled pushes (push_tile2d.cu
+// and push_tile3d.cu; of the QED species push_tile.cu and push_qed_tile3d.cu).
 #pragma once
 #include "push_dev.cuh"
 #include "push_tile.cuh"

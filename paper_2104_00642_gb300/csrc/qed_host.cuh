@@ -45,7 +45,7 @@ struct SpawnSet {
     SpawnSource<P_t> src[kSpawnSources];
 };
 // the children of the flagged particles, appended in the sources' order and in
-// array order; scratch: scan_blocks(n) + 1 words per source
+// array order; scratch: a word for each kScanItems flags and one more per source
 template <class P_t>
 void launch_spawn(SpawnSet<P_t> &S, uint32_t *scratch, cudaStream_t st);
 void launch_push_qed_f64(const PartF64 &P, double *F, const Grid &g, const PushConst &pc, const QedParams &q,
@@ -66,11 +66,9 @@ void launch_push_qed_set(QedPush *p, int n, float *F, const Grid &g, int *err, d
 // (first: see k_push_qed_f32 -- nullptr pushes every particle)
 void launch_push_qed_f32(const PartF32 &P, float *F, const Grid &g, const PushConst &pc, const QedParams &q,
                          int *err, double *e_abs, cudaStream_t st, const uint32_t *first = nullptr);
-// (tc: with the surrogate, evaluate the pair network per CTA on the tcgen05
-// tensor cores instead of per warp with mma.sync)
-// (first: see k_push_photon_f32 -- nullptr pushes every photon; tc is not
-// taken with first)
+// (tc: evaluate the pair network per CTA on the tcgen05 tensor cores instead
+// of per warp with mma.sync)
 void launch_push_photon_f32(const PartF32 &P, const float *F, const Grid &g, const PushConst &pc,
-                            const QedParams &q, int *err, cudaStream_t st, bool tc, const uint32_t *first = nullptr);
+                            const QedParams &q, int *err, cudaStream_t st, bool tc);
 
 }  // namespace pic

@@ -150,7 +150,11 @@ enum { PIC_PUSHER_BORIS = 0, PIC_PUSHER_VAY = 1 };
  * x = 0 at t_peak.  pol: linear along y or circular (both components of
  * amplitude a0).  It enters through the scattered-field Mur condition on the
  * x-min face (the paper uses absorbing faces and lasers from the left
- * boundary, Sec. III(a), without giving the method). */
+ * boundary, Sec. III(a), without giving the method).  The wave enters on rows
+ * 0 .. n-1 of a transverse axis.  Where that axis absorbs, the field components
+ * that sit on its nodes have one row more, n, on the domain's edge, and no wave
+ * enters there (B_y for circular light; B_z with an absorbing z axis): the
+ * axis should be wide enough for the beam to have died away at its ends. */
 typedef struct {
     double a0, waist, fwhm, t_peak, x_focus, yc, zc;
     int pol;

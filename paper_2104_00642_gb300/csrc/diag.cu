@@ -323,55 +323,56 @@ template void diag_gauss<double>(const double *, const double *, const Grid &, d
 // exchange layout (FP64, x fastest, [0, N) or [0, N] per axis) <-> padded
 // component: one thread per padded cell of a row, so that a component crosses
 // to the host as one dense block and the host walks no arrays.  The blocks of
-// all rows and planes are numbered along x (a launch's y and z hold 65535, and
-// a grid may have more rows than four times that, or more planes)
+// a plane are numbered along x and planes are strided over (a launch's y and z
+// hold 65535 blocks, and a grid may have more rows than four times that, or more
+// planes)
 // ---------------------------------------------------------------------
 struct ExBox {
     int m[3];
 };
 
-// this thread's cell of a box of e0 x e1 x (the launch's blocks) cells
-__device__ __forceinline__ bool ex_cell(int e0, int e1, int &i, int &j, int &k)
+// this thread's row and column of a plane of e0 x e1 cells
+__device__ __forceinline__ bool ex_cell(int e0, int e1, int &i, int &j)
 {
-    const unsigned nx = (e0 + blockDim.x - 1) / blockDim.x, ny = (e1 + blockDim.y - 1) / blockDim.y;
-    const unsigned r = blockIdx.x / nx;
-    i = (blockIdx.x - r * nx) * blockDim.x + threadIdx.x;
-    k = r / ny;
-    j = (r - k * ny) * blockDim.y + threadIdx.y;
+    const unsigned ny = (e1 + blockDim.y - 1) / blockDim.y, bx = blockIdx.x / ny;
+    i = bx * blockDim.x + threadIdx.x;
+    j = (blockIdx.x - bx * ny) * blockDim.y + threadIdx.y;
     return i < e0 && j < e1;
 }
 
 template <typename R>
 __global__ void __launch_bounds__(256) k_pack(const R *__restrict__ comp, Grid g, ExBox b, double *__restrict__ out)
 {
-    int i, j, k;
-    if (!ex_cell(b.m[0], b.m[1], i, j, k)) return;
-    out[((long long)k * b.m[1] + j) * b.m[0] + i] = (double)comp[goff(g, i, j, k)];
+    int i, j;
+    if (!ex_cell(b.m[0], b.m[1], i, j)) return;
+    for (int k = blockIdx.y; k < b.m[2]; k += gridDim.y)
+        out[((long long)k * b.m[1] + j) * b.m[0] + i] = (double)comp[goff(g, i, j, k)];
 }
 
 // every padded cell whose (periodic image of the) index lies in the box
 template <typename R>
-__global__ void __launch_bounds__(256) k_unpack(const double *__restrict__ in, Grid g, ExBox b, R *__restrict__ comp)
+__global__ void __launch_bounds__(256) k_unpack(const double *__restrict__ src, Grid g, ExBox b, R *__restrict__ comp)
 {
-    int p[3];
-    if (!ex_cell(g.ext[0], g.ext[1], p[0], p[1], p[2])) return;
+    int i, j;
+    if (!ex_cell(g.ext[0], g.ext[1], i, j)) return;
+    for (int k = blockIdx.y; k < g.ext[2]; k += gridDim.y) {
+        int p[3] = {i - g.G[0], j - g.G[1], k - g.G[2]};
+        const long long o = goff(g, p[0], p[1], p[2]);
+        bool in = true;
 #pragma unroll
-    for (int d = 0; d < 3; d++) p[d] -= g.G[d];
-    const long long o = goff(g, p[0], p[1], p[2]);
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-        if (d >= g.dim) continue;
-        if (g.bc[d] == PERIODIC) p[d] = (p[d] % g.n[d] + g.n[d]) % g.n[d];
-        else if (p[d] < 0 || p[d] >= b.m[d]) return;
+        for (int d = 0; d < 3; d++) {
+            if (d >= g.dim) continue;
+            if (g.bc[d] == PERIODIC) p[d] = (p[d] % g.n[d] + g.n[d]) % g.n[d];
+            else in &= p[d] >= 0 && p[d] < b.m[d];
+        }
+        if (in) comp[o] = (R)src[((long long)p[2] * b.m[1] + p[1]) * b.m[0] + p[0]];
     }
-    comp[o] = (R)in[((long long)p[2] * b.m[1] + p[1]) * b.m[0] + p[0]];
 }
 
 static dim3 ex_block(const Grid &g) { return g.dim == 1 ? dim3(256, 1, 1) : dim3(64, 4, 1); }
-// (below 2^31: a padded component holds fewer cells than that)
-static unsigned ex_blocks(const dim3 &blk, long long e0, long long e1, long long e2)
+static dim3 ex_grid(const dim3 &blk, long long e0, long long e1, long long e2)
 {
-    return (unsigned)((long long)div_up(e0, blk.x) * div_up(e1, blk.y) * e2);
+    return dim3((unsigned)div_up(e0, blk.x) * (unsigned)div_up(e1, blk.y), (unsigned)std::min(e2, 65535ll));
 }
 
 template <typename R>
@@ -379,7 +380,7 @@ void field_pack(const R *comp, const Grid &g, const long long *m, double *out, c
 {
     const ExBox b{{(int)m[0], (int)m[1], (int)m[2]}};
     const dim3 blk = ex_block(g);
-    k_pack<R><<<ex_blocks(blk, m[0], m[1], m[2]), blk, 0, st>>>(comp, g, b, out);
+    k_pack<R><<<ex_grid(blk, m[0], m[1], m[2]), blk, 0, st>>>(comp, g, b, out);
 }
 template void field_pack<float>(const float *, const Grid &, const long long *, double *, cudaStream_t);
 template void field_pack<double>(const double *, const Grid &, const long long *, double *, cudaStream_t);
@@ -389,7 +390,7 @@ void field_unpack(const double *in, const Grid &g, const long long *m, R *comp, 
 {
     const ExBox b{{(int)m[0], (int)m[1], (int)m[2]}};
     const dim3 blk = ex_block(g);
-    k_unpack<R><<<ex_blocks(blk, g.ext[0], g.ext[1], g.ext[2]), blk, 0, st>>>(in, g, b, comp);
+    k_unpack<R><<<ex_grid(blk, g.ext[0], g.ext[1], g.ext[2]), blk, 0, st>>>(in, g, b, comp);
 }
 template void field_unpack<float>(const double *, const Grid &, const long long *, float *, cudaStream_t);
 template void field_unpack<double>(const double *, const Grid &, const long long *, double *, cudaStream_t);

@@ -169,8 +169,9 @@ int sort_species(pic_sim *s, int i)
         sort_apply(view32(s, i, p.cur), view32(s, i, o), r, p.n_hi, s->g, p.tile_start, p.d_count, s->st);
     p.cur = o;
     if (p.items) {
-        build_tile_items(p.tile_start, s->g.ntiles, tile_chunk(s->g, p.has_qed_arrays(), p.n_hi), p.item_cnt,
-                         p.item_scan, p.items, p.nitems, s->st);
+        build_tile_items(p.tile_start, s->g.ntiles, tile_chunk(s->g, p.has_qed_arrays(), p.n_hi), least_of(s, p),
+                         p.item_cnt, p.item_scan, p.items, p.nitems, s->st);
+        p.maybe_sparse = least_of(s, p) > 0;
         p.items_valid = true;
     }
     CK(cudaGetLastError());
@@ -411,11 +412,14 @@ void push_species(pic_sim *s, int i, float *F, QedPushes &set)
     if (use_tile_push(s, p)) {
         const long long max_items = (long long)tile_items_capacity(p.n_hi, s->g.ntiles);
         if (s->g.dim == 3)
-            launch_push_tile3d(view32(s, i, p.cur), p.items, p.nitems, max_items, F, s->g, push_const(s, p), s->d_err,
-                               s->d_eabs, p.defer + 1, p.defer, s->st);
+            launch_push_tile3d(view32(s, i, p.cur), p.items, p.nitems + 1, max_items, F, s->g, push_const(s, p), s->d_err,
+                               s->d_eabs, p.defer + 1, p.defer, p.maybe_sparse, s->st);
         else
-            launch_push_tile2d(view32(s, i, p.cur), p.items, p.nitems, max_items, F, s->g, push_const(s, p), s->d_err,
+            launch_push_tile2d(view32(s, i, p.cur), p.items, p.nitems + 1, max_items, F, s->g, push_const(s, p), s->d_err,
                                s->d_eabs, s->st, s->push_variant == PIC_PUSH_TILE_AGG);
+        if (p.maybe_sparse && s->g.dim == 2)
+            launch_push_unless_f32(view32(s, i, p.cur), F, s->g, push_const(s, p), s->d_err, s->d_eabs, p.nitems + 1,
+                                   s->st);
     } else
         launch_push_f32(view32(s, i, p.cur), F, s->g, push_const(s, p), s->d_err, s->d_eabs, s->st);
 }
@@ -725,7 +729,7 @@ int pic_create(const pic_grid *grid, double dt, const pic_species *species, int 
         if (prec == PIC_PREC_FP32_CELLOFF && (g.dim == 2 || (g.dim == 3 && tile3d_push_supported(g)))) {
             p.items_cap = (long long)tile_items_capacity(p.cap, g.ntiles);
             rc = rc ? rc : dalloc(s, (void **)&p.items, (size_t)p.items_cap * sizeof(TileItem));
-            rc = rc ? rc : dalloc(s, (void **)&p.nitems, sizeof(uint32_t));
+            rc = rc ? rc : dalloc(s, (void **)&p.nitems, 2 * sizeof(uint32_t));
             rc = rc ? rc : dalloc(s, (void **)&p.item_cnt, (size_t)(g.ntiles + 1) * sizeof(uint32_t));
             rc = rc ? rc : dalloc(s, (void **)&p.item_scan, scan_scratch_words(g.ntiles + 1) * sizeof(uint32_t));
             if (g.dim == 3) rc = rc ? rc : dalloc(s, (void **)&p.defer, (size_t)(p.cap + 1) * sizeof(uint32_t));

@@ -282,8 +282,10 @@ int pic_restore(pic_sim *s, const char *path)
             CK(cudaMemcpyAsync(p.nitems, &nit, 4, cudaMemcpyHostToDevice, s->st));
             p.items_valid = true;
         }
-        CK(cudaStreamSynchronize(s->st));
         p.n_hi = n_hi;
+        p.maybe_sparse = items && least_of(s, p) > 0;
+        if (items) launch_item_counts(p.tile_start, s->g.ntiles, least_of(s, p), p.nitems, s->st);
+        CK(cudaStreamSynchronize(s->st));
     }
     for (int q = 0; q < 2; q++) {
         int ready = 0;

@@ -37,15 +37,28 @@ __global__ void __launch_bounds__(256) k_push_f32(PartF32 P, float *__restrict__
     push_one_f32<DIM, ORDER>(P, p, F, g, pc, err, e_abs);
 }
 
-// the particles of a list (the tiled push's deferred ones), grid-stride
+// the same unless *unless (a kernel of its own: k_push_f32 reads no flag)
+template <int DIM, int ORDER>
+__global__ void __launch_bounds__(256) k_push_unless_f32(PartF32 P, float *__restrict__ F, Grid g, PushConst pc,
+                                                         int *err, double *e_abs, const uint32_t *__restrict__ unless)
+{
+    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (*unless || p >= *P.dn) return;
+    push_one_f32<DIM, ORDER>(P, p, F, g, pc, err, e_abs);
+}
+
+// the particles of a list (the tiled push's deferred ones), grid-stride; all of
+// them where unless is given and *unless is zero
 template <int DIM>
 __global__ void __launch_bounds__(256) k_push_list_f32(PartF32 P, const uint32_t *__restrict__ list,
                                                        const uint32_t *__restrict__ count, float *__restrict__ F,
-                                                       Grid g, PushConst pc, int *err, double *e_abs)
+                                                       Grid g, PushConst pc, int *err, double *e_abs,
+                                                       const uint32_t *__restrict__ unless)
 {
-    const uint32_t n = *count;
+    const bool all = unless && *unless == 0u;
+    const uint32_t n = all ? (uint32_t)*P.dn : *count;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        push_one_f32<DIM>(P, list[i], F, g, pc, err, e_abs);
+        push_one_f32<DIM>(P, all ? i : list[i], F, g, pc, err, e_abs);
 }
 
 // one particle: half drift, gather (HBM), Boris, drifts, Esirkepov (global
@@ -461,6 +474,16 @@ void launch_push_f32(const PartF32 &P, float *F, const Grid &g, const PushConst 
     else k_push_f32<3, 2><<<nb, bs, 0, st>>>(P, F, g, pc, err, e_abs);
 }
 
+void launch_push_unless_f32(const PartF32 &P, float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs,
+                            const uint32_t *unless, cudaStream_t st)
+{
+    if (P.n == 0) return;
+    note_launch();
+    const int nb = div_up(P.n, 256);
+    if (g.order == 4) k_push_unless_f32<2, 4><<<nb, 256, 0, st>>>(P, F, g, pc, err, e_abs, unless);
+    else k_push_unless_f32<2, 2><<<nb, 256, 0, st>>>(P, F, g, pc, err, e_abs, unless);
+}
+
 int sm_count()
 {
     static const int n = [] {
@@ -473,14 +496,15 @@ int sm_count()
 }
 
 void launch_push_list_f32(const PartF32 &P, const uint32_t *list, const uint32_t *count, long long max_n, float *F,
-                          const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st)
+                          const Grid &g, const PushConst &pc, int *err, double *e_abs, const uint32_t *unless,
+                          cudaStream_t st)
 {
     if (max_n <= 0) return;
     note_launch();
     const int nb = (int)std::min<long long>(div_up(max_n, 256), 8ll * sm_count());
-    if (g.dim == 1) k_push_list_f32<1><<<nb, 256, 0, st>>>(P, list, count, F, g, pc, err, e_abs);
-    else if (g.dim == 2) k_push_list_f32<2><<<nb, 256, 0, st>>>(P, list, count, F, g, pc, err, e_abs);
-    else k_push_list_f32<3><<<nb, 256, 0, st>>>(P, list, count, F, g, pc, err, e_abs);
+    if (g.dim == 1) k_push_list_f32<1><<<nb, 256, 0, st>>>(P, list, count, F, g, pc, err, e_abs, unless);
+    else if (g.dim == 2) k_push_list_f32<2><<<nb, 256, 0, st>>>(P, list, count, F, g, pc, err, e_abs, unless);
+    else k_push_list_f32<3><<<nb, 256, 0, st>>>(P, list, count, F, g, pc, err, e_abs, unless);
 }
 
 void launch_push_f64(const PartF64 &P, double *F, const Grid &g, const PushConst &pc, int *err, double *e_abs,

@@ -667,12 +667,20 @@ __global__ void k_item_counts(const uint32_t *__restrict__ starts, long long nti
     cnt[t] = (n + s - 1) / s;
 }
 
+// nitems[0]: the items; nitems[1]: those the tiled push without QED takes, none
+// where n particles are at most `least` an item (see tile_least)
+__device__ __forceinline__ void put_item_counts(uint32_t *nitems, uint32_t all, uint32_t n, uint32_t least)
+{
+    nitems[0] = all;
+    nitems[1] = (unsigned long long)n <= (unsigned long long)least * all ? 0u : all;
+}
+
 __global__ void k_item_write(const uint32_t *__restrict__ starts, const uint32_t *__restrict__ off, long long ntiles,
-                             uint32_t chunk, uint32_t grain, TileItem *items, uint32_t *nitems)
+                             uint32_t chunk, uint32_t grain, uint32_t least, TileItem *items, uint32_t *nitems)
 {
     long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= ntiles) {
-        if (t == ntiles) *nitems = off[ntiles];
+        if (t == ntiles) put_item_counts(nitems, off[ntiles], starts[ntiles], least);
         return;
     }
     const uint32_t s = starts[t], n = starts[t + 1] - s, o = off[t], sz = item_size(n, chunk, grain);
@@ -702,16 +710,46 @@ int tile_chunk(const Grid &g, bool qed, long long n)
     return kPushThreads;
 }
 
+__global__ void k_item_counts_again(const uint32_t *__restrict__ starts, long long ntiles, uint32_t least,
+                                    uint32_t *nitems)
+{
+    put_item_counts(nitems, nitems[0], starts[ntiles], least);
+}
+
+// Particles per item up to which the one-thread push is the faster one (0: not
+// asked).  An item costs its boxes' staging and flush whatever is in it, 11 ns of
+// the chip in 3D (0.35 ns a particle saved on it), 6 ns in 2D (0.07; order 4: 9
+// and 0.16), and asking costs a launch without items, 5 us, which grids of few
+// tiles don't save.  Uniform plasma, 8 steps a sort, us a step, tiled / this rule: 3D
+// 96^3 at 0.1 a cell 268 / 120, 0.3 279 / 203, 0.6 290 / 290 (one thread 307);
+// 95 x 93 x 91 at 0.1 300 / 143, 0.45 318 / 259; 2D 768^2 at 0.1 a cell 64 / 57,
+// 0.2 68 / 66, 0.3 70 / 70 (one thread 65 + 5); with 8 x 8 tiles at 0.1 105 / 56, 1
+// 122 / 113, 1.5 127 / 127 (133 + 5); order 4 at 0.1 86 / 73, 0.2 95 / 92.
+int tile_least(const Grid &g)
+{
+    if (g.ntiles < (g.dim == 3 ? 512 : 1536)) return 0;
+    if (g.dim == 3) return 34;
+    if (g.order == 4) return 60;
+    return g.tile_log2[0] == 4 ? 64 : 86;
+}
+
 size_t tile_items_capacity(long long cap, long long ntiles) { return (size_t)(ntiles + cap / 256 + 2); }
 
-void build_tile_items(const uint32_t *starts, long long ntiles, int chunk, uint32_t *cnt_scratch,
+void launch_item_counts(const uint32_t *starts, long long ntiles, int least, uint32_t *nitems, cudaStream_t st)
+{
+    note_launch();
+    k_item_counts_again<<<1, 1, 0, st>>>(starts, ntiles, (uint32_t)least, nitems);
+}
+
+void build_tile_items(const uint32_t *starts, long long ntiles, int chunk, int least, uint32_t *cnt_scratch,
                       uint32_t *scan_scratch, TileItem *items, uint32_t *nitems, cudaStream_t st)
 {
     const uint32_t c = (uint32_t)chunk, grain = chunk % kPushThreads == 0 ? kPushThreads : 32u;
     note_launch(2);
     k_item_counts<<<div_up(ntiles + 1, 256), 256, 0, st>>>(starts, ntiles, c, grain, cnt_scratch);
     scan_exclusive(cnt_scratch, cnt_scratch, ntiles + 1, scan_scratch, st);
-    k_item_write<<<div_up(ntiles + 1, 256), 256, 0, st>>>(starts, cnt_scratch, ntiles, c, grain, items, nitems);
+    k_item_write<<<div_up(ntiles + 1, 256), 256, 0, st>>>(starts, cnt_scratch, ntiles, c, grain, (uint32_t)least, items,
+                                                        nitems);
 }
 
 template <int T, int QM>

@@ -27,8 +27,14 @@ constexpr int kChunk3 = 256;
 // (qed: photons and the leptons of the Monte Carlo)
 int tile_chunk(const Grid &g, bool qed, long long n);
 size_t tile_items_capacity(long long cap, long long ntiles);
-void build_tile_items(const uint32_t *starts, long long ntiles, int chunk, uint32_t *cnt_scratch,
+// nitems (two words): all items, and those of the tiled push without QED, none
+// where there are at most `least` particles an item (0: no such rule; see
+// least_of in sim.cuh): the one-thread push runs instead
+int tile_least(const Grid &g);
+void build_tile_items(const uint32_t *starts, long long ntiles, int chunk, int least, uint32_t *cnt_scratch,
                       uint32_t *scan_scratch, TileItem *items, uint32_t *nitems, cudaStream_t st);
+// nitems[1] for items that are there already
+void launch_item_counts(const uint32_t *starts, long long ntiles, int least, uint32_t *nitems, cudaStream_t st);
 // 2D, shape orders 2 and 4 (agg: the warp-aggregated deposit, order 2); and
 // with a QED lepton species' Monte Carlo q fused in (order 2; q.on; the
 // particles appended since the sort, and their event flags, are left to
@@ -53,11 +59,11 @@ void launch_tail_items(const PartF32 &P, const uint32_t *first, const Grid &g, T
 void launch_photon_resolve(const QedParams &q, const PartF32 &P, int *err, cudaStream_t st);
 // 3D, tiles of 4^3 cells (defer: a list of capacity >= the particle count,
 // ndefer its device count; the particles the tiled kernel defers are pushed
-// after it on the global path)
+// after it on the global path, with maybe_sparse all of them if *nitems is zero)
 bool tile3d_push_supported(const Grid &g);
 void launch_push_tile3d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
                         float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, uint32_t *defer,
-                        uint32_t *ndefer, cudaStream_t st);
+                        uint32_t *ndefer, bool maybe_sparse, cudaStream_t st);
 // and with a QED lepton species' Monte Carlo q fused in (q.on; every n_d a
 // multiple of 4); nothing is deferred, and the particles appended since the
 // sort are left to launch_push_qed_f32

@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     int *sJ = reinterpret_cast<int *>(smem + 6 * B::N);  // 3 components, fixed point
     float *sR = smem + 6 * B::N + 3 * B::NJ;             // records: oh_x, oh_y, oe_x, oe_y, v_z, window
     const int nit = (int)*nitems;
+    if ((int)blockIdx.x >= nit) return;
     const long long V = g.vol;
     const float hdx0 = pc.hdx_f[0], hdx1 = pc.hdx_f[1];
     const float k = pc.qmdt2_f;
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         sCnt[0] = sCnt[1] = sCnt[2] = 0;
         if (use_tma) {
             mbar_init(&mbar, 1);
-            if ((int)blockIdx.x < nit) stage_box(items[blockIdx.x].tile);
+            stage_box(items[blockIdx.x].tile);
         }
     }
     for (int e = threadIdx.x; e < 3 * B::NJ / 4; e += kPushThreads) reinterpret_cast<int4 *>(sJ)[e] = make_int4(0, 0, 0, 0);

@@ -191,6 +191,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     int *sJ = reinterpret_cast<int *>(smem + 6 * B::N);  // 3 components, fixed point
     float *sR = smem + 9 * B::N;                         // records: oh (3), oe (3), window
     const int nit = (int)*nitems;
+    if ((int)blockIdx.x >= nit) return;
     const long long V = g.vol;
     const float hdx[3] = {pc.hdx_f[0], pc.hdx_f[1], pc.hdx_f[2]};
     const float k = pc.qmdt2_f;
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         sCnt[0] = sCnt[1] = sCnt[2] = 0;
         if (use_tma) {
             mbar_init(&mbar, 1);
-            if ((int)blockIdx.x < nit) stage_box(items[blockIdx.x].tile);
+            stage_box(items[blockIdx.x].tile);
         }
     }
     for (int e4 = threadIdx.x; e4 < 3 * B::N / 4; e4 += kPushThreads)
@@ -411,7 +412,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
 template <bool EXACT>
 static void launch_exact(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items, float *F,
                          const Grid &g, const PushConst &pc, int *err, double *e_abs, uint32_t *defer, uint32_t *ndefer,
-                         cudaStream_t st)
+                         bool maybe_sparse, cudaStream_t st)
 {
     constexpr int T = 4;
     constexpr int smem = Box3p<T>::SMEM + 128;  // + alignment of the TMA destination
@@ -435,12 +436,12 @@ static void launch_exact(const PartF32 &P, const TileItem *items, const uint32_t
     note_launch();
     k_push_tile3d<T, EXACT><<<(int)grid, kPushThreads, smem, st>>>(P, items, nitems, F, g, pc, err, e_abs, defer, ndefer,
                                                                    tmap, tma ? 1 : 0);
-    launch_push_list_f32(P, defer, ndefer, P.n, F, g, pc, err, e_abs, st);
+    launch_push_list_f32(P, defer, ndefer, P.n, F, g, pc, err, e_abs, maybe_sparse ? nitems : nullptr, st);
 }
 
 void launch_push_tile3d(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items,
                         float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, uint32_t *defer,
-                        uint32_t *ndefer, cudaStream_t st)
+                        uint32_t *ndefer, bool maybe_sparse, cudaStream_t st)
 {
     if (P.n == 0) return;
     // Sizes that are not multiples of 4 were the one-thread push's: these take its
@@ -449,8 +450,8 @@ void launch_push_tile3d(const PartF32 &P, const TileItem *items, const uint32_t 
     // the fast ones, 3.3e-7 now, 3.8e-7 one thread per particle; the case takes
     // 1.56 ms instead of 1.54).
     const bool whole = g.n[0] % 4 == 0 && g.n[1] % 4 == 0 && g.n[2] % 4 == 0;
-    if (whole) launch_exact<false>(P, items, nitems, max_items, F, g, pc, err, e_abs, defer, ndefer, st);
-    else launch_exact<true>(P, items, nitems, max_items, F, g, pc, err, e_abs, defer, ndefer, st);
+    if (whole) launch_exact<false>(P, items, nitems, max_items, F, g, pc, err, e_abs, defer, ndefer, maybe_sparse, st);
+    else launch_exact<true>(P, items, nitems, max_items, F, g, pc, err, e_abs, defer, ndefer, maybe_sparse, st);
 }
 
 bool tile3d_push_supported(const Grid &g)

@@ -28,12 +28,13 @@ struct SpeciesState {
     uint32_t *tile_start = nullptr;  // ntiles + 1
     // work items of the tiled push (rebuilt after every sort)
     TileItem *items = nullptr;
-    uint32_t *nitems = nullptr;
+    uint32_t *nitems = nullptr;     // 2 words (see build_tile_items)
     uint32_t *item_cnt = nullptr;   // ntiles + 1
     uint32_t *item_scan = nullptr;  // scan scratch
     uint32_t *defer = nullptr;      // 3D: particles the tiled push leaves to the global path ([0] = count)
     long long items_cap = 0;
     bool items_valid = false;
+    bool maybe_sparse = false;      // the tiled push may find no items (see least_of)
     // 2D photons: work items over the photons appended since the sort (rebuilt every step)
     TileItem *tail_items = nullptr;
     uint32_t *tail_nitems = nullptr;
@@ -120,6 +121,16 @@ int dalloc(pic_sim *s, void **p, size_t bytes);
 // temporary device memory of one call (released by tfree before it returns)
 int talloc(pic_sim *s, void **p, size_t bytes);
 void tfree(pic_sim *s, void *p);
+// particles per work item up to which a species goes to the one-thread push
+// instead (build_tile_items), 0: whatever they are, because the tiled push was
+// asked for, the push is a QED one, or there are too many particles for it
+// however they lie (an item a tile; more items only where tiles are full)
+inline int least_of(const pic_sim *s, const SpeciesState &p)
+{
+    if (s->push_variant != PIC_PUSH_AUTO || p.has_qed_arrays()) return 0;
+    const int least = tile_least(s->g);
+    return p.n_hi <= (long long)least * s->g.ntiles ? least : 0;
+}
 inline size_t rsize(const pic_sim *s) { return s->precision == PIC_PREC_FP64_PLAIN ? 8 : 4; }
 
 }  // namespace pic

@@ -723,14 +723,14 @@ __global__ void k_item_counts_again(const uint32_t *__restrict__ starts, long lo
 // tiles don't save.  Uniform plasma, 8 steps a sort, us a step, tiled / this rule: 3D
 // 96^3 at 0.1 a cell 268 / 120, 0.3 279 / 203, 0.6 290 / 290 (one thread 307);
 // 95 x 93 x 91 at 0.1 300 / 143, 0.45 318 / 259; 2D 768^2 at 0.1 a cell 64 / 57,
-// 0.2 68 / 66, 0.3 70 / 70 (one thread 65 + 5); with 8 x 8 tiles at 0.1 105 / 56, 1
-// 122 / 113, 1.5 127 / 127 (133 + 5); order 4 at 0.1 86 / 73, 0.2 95 / 92.
+// 0.2 68 / 66, 0.3 70 / 70 (one thread 65 + 5); with 8 x 8 tiles at 0.1 81 / 56,
+// 0.6 95 / 91, 0.8 99 / 99 (96 + 5); order 4 at 0.1 86 / 73, 0.2 95 / 92.
 int tile_least(const Grid &g)
 {
     if (g.ntiles < (g.dim == 3 ? 512 : 1536)) return 0;
     if (g.dim == 3) return 34;
-    if (g.order == 4) return 60;
-    return g.tile_log2[0] == 4 ? 64 : 86;
+    if (g.order == 4) return g.tile_log2[0] == 4 ? 60 : 50;
+    return g.tile_log2[0] == 4 ? 64 : 46;
 }
 
 size_t tile_items_capacity(long long cap, long long ntiles) { return (size_t)(ntiles + cap / 256 + 2); }

@@ -9,7 +9,7 @@ namespace pic {
 struct QedParams;
 
 constexpr int kChunkMax = 1024;    // particles per work item at most (2D)
-constexpr int kPushThreads = 256;  // threads per CTA of the 2D push
+constexpr int kPushThreads = 256;  // threads per CTA of the 2D push (tiles of 8 x 8 cells: 128 on large grids)
 constexpr int kChunk = 384;        // particles per work item at most (2D, QED species)
 constexpr int kTileThreads = 128;  // threads per CTA of the QED species' pushes and the 3D push
 constexpr int kTileMinBlocks = 6;  // CTAs per SM of the 2D QED pushes: 80 registers, 35 KB shared memory each (measured best)

@@ -234,8 +234,8 @@ __device__ __forceinline__ void deposit_row2d(const float *sR, int *sJ, int j, i
 //
 // AGG: the deposit phase walks consecutive records and sums the lanes that
 // share a window before one atomic per value.
-template <int T, int ORDER, bool AGG>
-__global__ void __launch_bounds__(kPushThreads, 3)
+template <int T, int ORDER, bool AGG, int NT>
+__global__ void __launch_bounds__(NT, 768 / NT)
     k_push_tile2d(PartF32 P, const TileItem *__restrict__ items, const uint32_t *__restrict__ nitems,
                   float *__restrict__ F, Grid g, PushConst pc, int *err, double *e_abs,
                   const __grid_constant__ CUtensorMap tmap, int use_tma)
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     extern __shared__ __align__(16) float smem_raw[];
     __shared__ uint64_t mbar;
     __shared__ int sCnt[3];                      // records filed from the front (node unmoved) and the back; rows taken
-    __shared__ int2 sSum[3][kPushThreads / 32];  // sums of v_d per warp
+    __shared__ int2 sSum[3][NT / 32];  // sums of v_d per warp
     // the TMA destination starts on a 128-byte boundary
     // (offset from the shared array itself, so that the compiler keeps every
     // access below in the shared address space)
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             stage_box(items[blockIdx.x].tile);
         }
     }
-    for (int e = threadIdx.x; e < 3 * B::NJ / 4; e += kPushThreads) reinterpret_cast<int4 *>(sJ)[e] = make_int4(0, 0, 0, 0);
+    for (int e = threadIdx.x; e < 3 * B::NJ / 4; e += NT) reinterpret_cast<int4 *>(sJ)[e] = make_int4(0, 0, 0, 0);
     __syncthreads();
     uint32_t phase = 0;
     for (int it = blockIdx.x; it < nit; it += gridDim.x) {
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             landed = mbar_wait(&mbar, phase, 1 << 22);
             phase ^= 1u;
         } else {
-            for (int e = threadIdx.x; e < 6 * B::N; e += kPushThreads) {
+            for (int e = threadIdx.x; e < 6 * B::N; e += NT) {
                 const int c = e / B::N, r = e - c * B::N;
                 const int y = r / B::WX, x = r - y * B::WX;
                 const int gx = bx0 + x, gy = by0 + y;
@@ -323,11 +323,11 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         // push phase (the records are filed by the warp; a warp without
         // particles skips its passes)
         float vsum[3] = {0.f, 0.f, 0.f}, vabs[3] = {0.f, 0.f, 0.f};
-        for (uint32_t pbase = m.start + 32 * warp; pbase < pend; pbase += kPushThreads, p += kPushThreads) {
+        for (uint32_t pbase = m.start + 32 * warp; pbase < pend; pbase += NT, p += NT) {
             const uint32_t cp = ncell;
             float ux = nst[2], uy = nst[3], uz = nst[4];
             float o[2] = {nst[0], nst[1]};
-            fetch(p + kPushThreads);
+            fetch(p + NT);
             bool act = cp != kDead;  // a live particle of this item
             int c[2] = {0, 0}, c1[2] = {0, 0}, u0[2] = {0, 0};
             float o1[2] = {0.f, 0.f}, oh[2] = {0.f, 0.f};
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             P.u[1][p] = uy;
             P.u[2][p] = uz;
         }
-        warp_sums<ORDER == 4>(vabs, vsum, sSum);
+        warp_sums<ORDER == 4, NT / 32>(vabs, vsum, sSum);
         __syncthreads();
         // the next item's field box, while this one's records are deposited
         if (use_tma && threadIdx.x == 0 && it + (int)gridDim.x < nit) stage_box(items[it + gridDim.x].tile);
@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         if (threadIdx.x == 0) sCnt[0] = sCnt[1] = sCnt[2] = 0;
         // flush the current box, four values at a time, and leave it zero
         const float unit[3] = {1.0f / scx, 1.0f / scy, 1.0f / scz};
-        for (int v4 = threadIdx.x; v4 < 3 * B::WY * (B::WX / 4); v4 += kPushThreads) {
+        for (int v4 = threadIdx.x; v4 < 3 * B::WY * (B::WX / 4); v4 += NT) {
             const int row = v4 / (B::WX / 4), x = 4 * (v4 - row * (B::WX / 4));
             const int c = row / B::WY, y = row - c * B::WY;
             int4 *cellv = reinterpret_cast<int4 *>(sJ + c * B::NJ + y * B::RJ + x);
@@ -503,18 +503,18 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     }
 }
 
-template <int T, int ORDER, bool AGG>
+template <int T, int ORDER, bool AGG, int NT = kPushThreads>
 static void launch_T(const PartF32 &P, const TileItem *items, const uint32_t *nitems, long long max_items, float *F,
                      const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st)
 {
     constexpr int smem = Box2p<T>::SMEM + 128;  // + alignment of the TMA destination
     static int nsm = 0, per_sm = 0;  // resident CTAs per SM
     if (!per_sm) {
-        cudaFuncSetAttribute(k_push_tile2d<T, ORDER, AGG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaFuncSetAttribute(k_push_tile2d<T, ORDER, AGG, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         int dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_push_tile2d<T, ORDER, AGG>, kPushThreads, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_push_tile2d<T, ORDER, AGG, NT>, NT, smem);
         if (per_sm < 1) per_sm = 1;
     }
     // the six field components as one 3D tensor (x, y, component); tiles of
@@ -526,7 +526,7 @@ static void launch_T(const PartF32 &P, const TileItem *items, const uint32_t *ni
     long long grid = std::min<long long>(max_items, (long long)nsm * per_sm);  // one resident wave
     if (grid < 1) grid = 1;
     note_launch();
-    k_push_tile2d<T, ORDER, AGG><<<(int)grid, kPushThreads, smem, st>>>(P, items, nitems, F, g, pc, err, e_abs, tmap,
+    k_push_tile2d<T, ORDER, AGG, NT><<<(int)grid, NT, smem, st>>>(P, items, nitems, F, g, pc, err, e_abs, tmap,
                                                                        tma ? 1 : 0);
 }
 
@@ -535,6 +535,16 @@ static void launch_variant(const PartF32 &P, const TileItem *items, const uint32
                            float *F, const Grid &g, const PushConst &pc, int *err, double *e_abs, cudaStream_t st,
                            bool agg)
 {
+    if constexpr (T == 8)
+        // tiles of 8 x 8 cells hold few particles: CTAs of 128 threads, six an SM,
+        // where there are tiles for all of them (768 x 768 cells, 1.5 a cell: 127 us
+        // a step with 256 threads, 107 with 128, 2 a cell 137 and 122; order 4 275
+        // and 211; 96 x 96 cells, 144 tiles, 8 a cell: 35 and 38)
+        if (!agg && g.ntiles >= 6ll * sm_count()) {
+            if (g.order == 4) launch_T<T, 4, false, 128>(P, items, nitems, max_items, F, g, pc, err, e_abs, st);
+            else launch_T<T, 2, false, 128>(P, items, nitems, max_items, F, g, pc, err, e_abs, st);
+            return;
+        }
     if (g.order == 4) launch_T<T, 4, false>(P, items, nitems, max_items, F, g, pc, err, e_abs, st);
     else if (agg) launch_T<T, 2, true>(P, items, nitems, max_items, F, g, pc, err, e_abs, st);
     else launch_T<T, 2, false>(P, items, nitems, max_items, F, g, pc, err, e_abs, st);

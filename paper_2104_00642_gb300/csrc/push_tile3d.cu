@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             P.u[1][p] = uy;
             P.u[2][p] = uz;
         }
-        warp_sums<EXACT>(vabs, vsum, sSum);
+        warp_sums<EXACT, kPushThreads / 32>(vabs, vsum, sSum);
         __syncthreads();
         // the next item's field box, while this one's records are deposited
         if (use_tma && threadIdx.x == 0 && it + (int)gridDim.x < nit) stage_box(items[it + gridDim.x].tile);

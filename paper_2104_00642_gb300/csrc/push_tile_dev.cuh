@@ -68,8 +68,8 @@ __device__ __forceinline__ void drift_sel_f32(int &c, float &o, float h, float u
 // and (SIGNED) of v_d: of the positive ones (x) and of the negative ones (y), or
 // of all |v_d| (x).  In units of 2^-20, rounded up per thread (an item's 1024
 // records stay below 2^30), so that one integer reduction a value does it.
-template <bool SIGNED>
-__device__ __forceinline__ void warp_sums(const float *vabs, const float *v, int2 (*sum)[kPushThreads / 32])
+template <bool SIGNED, int NW>
+__device__ __forceinline__ void warp_sums(const float *vabs, const float *v, int2 (*sum)[NW])
 {
 #pragma unroll
     for (int d = 0; d < 3; d++) {
@@ -97,11 +97,12 @@ __device__ __forceinline__ void warp_sums(const float *vabs, const float *v, int
 // rounded by up to 2^-24 cells, and weights good to about 2^-22 (order 4).  For
 // slow particles that is most of the move, so every record counts with 2^-20
 // cells more; of a thermal particle's move it is 1e-5.
-__device__ __forceinline__ float box_units(const int2 *sum, float qw, int n, float cj, float shape)
+template <int NW>
+__device__ __forceinline__ float box_units(const int2 (&sum)[NW], float qw, int n, float cj, float shape)
 {
     int p = 0, m = 0;
 #pragma unroll
-    for (int w = 0; w < kPushThreads / 32; w++) {
+    for (int w = 0; w < NW; w++) {
         p += sum[w].x;
         m += sum[w].y;
     }

@@ -14,7 +14,8 @@ A, P = W.ABSORB, W.PERIODIC
 # per tile: the line, its neighbours, next to nothing, and far beyond
 # (and a grid of too few tiles to ask)
 GRIDS = [((32, 32, 32), 2, (4, 4, 4), 34), ((33, 31, 30), 2, (4, 4, 4), 34), ((640, 624), 2, (16, 16, 1), 64),
-         ((320, 312), 2, (8, 8, 1), 86), ((640, 624), 4, (16, 16, 1), 60), ((16, 16, 12), 2, (4, 4, 4), 34)]
+         ((320, 312), 2, (8, 8, 1), 46), ((640, 624), 4, (16, 16, 1), 60),
+         ((320, 312), 4, (8, 8, 1), 50), ((16, 16, 12), 2, (4, 4, 4), 34)]
 
 
 def _workload(n, per_tile, tile, lie, bc, seed):

@@ -106,7 +106,8 @@ __device__ __forceinline__ float box_units(const int2 (&sum)[NW], float qw, int 
         p += sum[w].x;
         m += sum[w].y;
     }
-    return 2.14e9f / fmaxf(shape * 9.5367432e-7f * fmaf(fabsf(qw), (float)max(p, m), (float)n * fabsf(cj)), 1e-28f);
+    constexpr float u = 9.5367432e-7f;  // 2^-20
+    return 2.14e9f / fmaxf(shape * fmaf(fabsf(qw), (float)max(p, m) * u, (float)n * fabsf(cj * u)), 1e-28f);
 }
 
 // the deposit phase's rows of 32 records (an odd number: see deposit_row2d),

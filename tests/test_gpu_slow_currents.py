@@ -46,3 +46,26 @@ def test_current_of_a_rounded_up_move(dim, n, order, k, tol, axis, count):
     assert np.max(np.abs(want)) > 0.0
     assert np.max(np.abs(sim.pic_fields(c) - want)) <= tol * np.max(np.abs(want))
     sim.close()
+
+
+@pytest.mark.parametrize("dim,n,order", [(2, (32, 32), 2), (2, (32, 32), 4), (3, (16, 12, 8), 2), (3, (13, 10, 9), 2)])
+@pytest.mark.parametrize("power", [-70, 108])
+def test_current_scales_with_the_weight(dim, n, order, power):
+    """a weight times a power of two: the same fixed-point values, in units that
+    many times larger"""
+    w, _ = random_state(dim, n, (0.1,) * dim, 0.05, 8, seed=5, fields=False)
+    J = []
+    for p in (0, power):
+        w.species[0].w = 0.125 * 2.0 ** p
+        sim = pic.from_workload(w, precision=pic.FP32_CELLOFF, sort_interval=1, tile=(4, 4, 4) if dim == 3 else (16, 16, 1),
+                                order=order)
+        try:
+            sim.pic_step(1)
+        except pic.PicError:
+            pass  # (fields of 1e30 may be reported; the current is there)
+        J.append([sim.pic_fields(c) * 2.0 ** -p for c in (pic.JX, pic.JY, pic.JZ)])
+        sim.close()
+    for a, b in zip(*J):
+        assert np.max(np.abs(a)) > 0.0
+        # (the items' sums meet in FP32, in any order)
+        assert np.max(np.abs(a - b)) <= 1e-5 * np.max(np.abs(a))

@@ -209,11 +209,12 @@ __device__ __forceinline__ void deposit_row2d(const float *sR, int *sJ, int j, i
 //            node moved (4 x 4, 40 atomics).
 // A single pass (gather, push and atomics per particle, lane-strided) was
 // bound by the shared-memory pipe (85 %; 250 bank-conflict wavefronts per 32
-// particles, lanes sharing cells) with ~1030 instructions per particle; now
-// issue-bound, ~890 instructions, 70 conflict wavefronts: the laser-foil's
-// 2,097,152 electrons 101 -> 89 us, its protons 97 -> 82 us a push.  At order
-// 4 (262,144 particles at rest on a 128 x 128 grid) 201 us on the
-// one-thread-per-particle kernel -> 39 us.
+// particles, lanes sharing cells); now issue is its first bound (60 % of the
+// slots, 1170 instructions and 122 conflict wavefronts per 32 of the foil's heated
+// electrons): its 2,097,152 electrons 101 -> 89 us, its protons 97 -> 82 us a push
+// while the pulse comes up.  At order 4 (262,144 particles of 1 keV on a 128 x
+// 128 grid) 201 us on the one-thread-per-particle kernel -> 39 us (2070
+// instructions per 32 particles, 55 % of the issue slots).
 //
 // Order 4 was the one-thread push's: it keeps that kernel's root and quotients
 // and takes the finer units (EXACT and SIGNED in push_tile_dev.cuh), so that

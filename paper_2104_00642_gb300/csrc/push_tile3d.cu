@@ -158,10 +158,10 @@ __device__ __forceinline__ void deposit_row3d(const float *sR, int *sJ, int j, i
 // atomics), the others on 4^3 (144); units of the current box from the item's
 // particles.
 //
-// Bound: the shared-memory pipe (78 %; 162 field loads and 54 to 144 atomics a
-// particle, about two wavefronts each) and issue (57 %).  256^3-style thermal
+// Bound: the shared-memory pipe (76 %; 162 field loads and 54 to 144 atomics a
+// particle, about two wavefronts each) and issue (60 %).  256^3-style thermal
 // plasma, 16,777,216 particles at 200 keV: 2.63 ms a push in one pass over
-// consecutive lanes (eight lanes on one cell) and its deferred list, now 1.73
+// consecutive lanes (eight lanes on one cell) and its deferred list, now 1.72
 // ms; 856,440 particles on a 61 x 45 x 39 grid: 757 us one thread per
 // particle, now 130 us.  The box's row above the tile is two cells deep: 7 %
 // fewer cells (six rows and planes around the tile) deferred enough particles

@@ -135,8 +135,10 @@ typedef struct {
 } pic_options;
 
 /* Push kernels: AUTO uses the tiled shared-memory kernel wherever it exists
- * (2D grids, FP32 form, 8x8 or 16x16 tiles, particles sorted at least once)
- * and the simple kernel elsewhere; SIMPLE always uses the simple kernel;
+ * (FP32 form, particles sorted since they were loaded; 2D grids with 8x8 or
+ * 16x16 tiles, 3D grids with 4x4x4 tiles at order 2) and is the faster one (a
+ * species without QED on a grid of many tiles needs some tens of particles per
+ * occupied tile), and the simple kernel elsewhere; SIMPLE always uses the simple kernel;
  * TILE_AGG is AUTO with the 2D tiled kernel's warp-aggregated deposit (the
  * lanes of a warp on consecutive, cell-sorted particles; lanes sharing a
  * deposit window summed by warp reductions before one atomic per value). */
